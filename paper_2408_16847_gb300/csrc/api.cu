@@ -46,9 +46,7 @@ static int (*const kMultiOcc[TPCF_MAX_M + 1])(int) = {
     int map_fwd_tc_occupancy_m##m(int, int);                                                  \
     cudaError_t map_bwd_launch_m##m(const MapDev&, const MapCall&, int, int, cudaStream_t);    \
     int map_fwd_occupancy_m##m(int, int, int);                                                \
-    int map_bwd_occupancy_m##m(int, int);                                                     \
-    size_t map_fwd_smem_m##m(int);                                                            \
-    size_t map_bwd_smem_m##m(int);
+    int map_bwd_occupancy_m##m(int, int);
 TPCF_DECL_M(0) TPCF_DECL_M(1) TPCF_DECL_M(2) TPCF_DECL_M(3) TPCF_DECL_M(4) TPCF_DECL_M(5)
 TPCF_DECL_M(6) TPCF_DECL_M(7) TPCF_DECL_M(8) TPCF_DECL_M(9) TPCF_DECL_M(10) TPCF_DECL_M(11)
 TPCF_DECL_M(12) TPCF_DECL_M(13) TPCF_DECL_M(14) TPCF_DECL_M(15) TPCF_DECL_M(16)
@@ -75,11 +73,9 @@ struct MLaunch {
     cudaError_t (*bwd)(const MapDev&, const MapCall&, int, int, cudaStream_t);
     int (*fwd_occ)(int, int, int);
     int (*bwd_occ)(int, int);
-    size_t (*fwd_smem)(int);
-    size_t (*bwd_smem)(int);
 };
 #define TPCF_ROW_M(m) \
-    {map_fwd_launch_m##m, map_fwd_tc_launch_m##m, map_fwd_tc_occupancy_m##m, map_bwd_launch_m##m, map_fwd_occupancy_m##m, map_bwd_occupancy_m##m, map_fwd_smem_m##m, map_bwd_smem_m##m}
+    {map_fwd_launch_m##m, map_fwd_tc_launch_m##m, map_fwd_tc_occupancy_m##m, map_bwd_launch_m##m, map_fwd_occupancy_m##m, map_bwd_occupancy_m##m}
 static const MLaunch kLaunch[TPCF_MAX_M + 1] = {
     TPCF_ROW_M(0),  TPCF_ROW_M(1),  TPCF_ROW_M(2),  TPCF_ROW_M(3),  TPCF_ROW_M(4),  TPCF_ROW_M(5),
     TPCF_ROW_M(6),  TPCF_ROW_M(7),  TPCF_ROW_M(8),  TPCF_ROW_M(9),  TPCF_ROW_M(10), TPCF_ROW_M(11),
@@ -185,11 +181,14 @@ static tpcf_status build_map(tpcf_plan_s* P, int64_t nside, cudaStream_t s) {
     g.K = K;
     g.M = P->M;
     g.npix = 12 * nside * nside;
-    int64_t *first, *pair_off, *tile_off, *npairs_r, *ntiles_r, *tot;
+    int64_t *first, *pair_off, *tile_off, *wtile_off, *npairs_r, *ntiles_r, *nwtiles_r, *tot;
     int *npr, *shift;
     double *z, *sd, *th, *E, *theta;
     float *zf, *sf, *sf_lo, *rstep, *rstep_lo, *rinvn, *rinvn_lo;
     int2 *ring_range, *bin_range;
+    unsigned char* lin;  // the walk's ring classes (map_walk.cuh)
+    int* reach;
+    float4* rc;
     TRY_CUDA(P->alloc(&first, nrings));
     TRY_CUDA(P->alloc(&npr, nrings));
     TRY_CUDA(P->alloc(&shift, nrings));
@@ -209,33 +208,50 @@ static tpcf_status build_map(tpcf_plan_s* P, int64_t nside, cudaStream_t s) {
     TRY_CUDA(P->alloc(&tile_off, nrings));
     TRY_CUDA(P->alloc(&npairs_r, nrings));
     TRY_CUDA(P->alloc(&ntiles_r, nrings));
-    TRY_CUDA(P->alloc(&tot, 2));
+    TRY_CUDA(P->alloc(&wtile_off, nrings));
+    TRY_CUDA(P->alloc(&nwtiles_r, nrings));
+    TRY_CUDA(P->alloc(&lin, nrings));
+    TRY_CUDA(P->alloc(&reach, nrings));
+    TRY_CUDA(P->alloc(&rc, 2 * (size_t)nrings));
+    TRY_CUDA(P->alloc(&tot, 3));
     TRY_CUDA(P->alloc(&E, K + 1));
     TRY_CUDA(P->alloc(&theta, K + 1));
     TRY_CUDA(cudaMemcpyAsync(theta, P->edges.data(), sizeof(double) * (K + 1), cudaMemcpyHostToDevice, s));
     edges_kernel<<<1, 64, 0, s>>>(K, theta, E);
     ring_table_kernel<<<n_blocks(nrings, 128), 128, 0, s>>>((int)nside, nrings, first, npr, shift, z, sd, th,
-                                                            zf, sf, sf_lo, rstep, rstep_lo, rinvn, rinvn_lo);
-    ring_range_kernel<<<n_blocks(nrings, 128), 128, 0, s>>>(nrings, K, th, E, npr, ring_range, bin_range,
-                                                            npairs_r, ntiles_r);
+                                                            zf, sf, sf_lo, rstep, rstep_lo, rinvn, rinvn_lo, rc);
+    ring_range_kernel<<<n_blocks(nrings, 128), 128, 0, s>>>(nrings, K, th, sd, E, npr, shift, ring_range,
+                                                            bin_range, npairs_r, ntiles_r, nwtiles_r, lin, reach);
     exclusive_scan_kernel<<<1, 1024, 0, s>>>(npairs_r, pair_off, nrings, tot);
     exclusive_scan_kernel<<<1, 1024, 0, s>>>(ntiles_r, tile_off, nrings, tot + 1);
+    exclusive_scan_kernel<<<1, 1024, 0, s>>>(nwtiles_r, wtile_off, nrings, tot + 2);
     TRY_CUDA(cudaGetLastError());
-    int64_t totals[2];
+    int64_t totals[3];
     TRY_CUDA(cudaMemcpyAsync(totals, tot, sizeof(totals), cudaMemcpyDeviceToHost, s));
     TRY_CUDA(cudaStreamSynchronize(s));
-    const int64_t npairs = totals[0], ntiles = totals[1];
+    const int64_t npairs = totals[0], ntiles = totals[1], nwtiles = totals[2];
     P->tile_off_h.resize(nrings);
+    P->wtile_off_h.resize(nrings);
+    P->lin_h.resize(nrings);
     TRY_CUDA(cudaMemcpy(P->tile_off_h.data(), tile_off, sizeof(int64_t) * nrings, cudaMemcpyDeviceToHost));
+    TRY_CUDA(cudaMemcpy(P->wtile_off_h.data(), wtile_off, sizeof(int64_t) * nrings, cudaMemcpyDeviceToHost));
+    TRY_CUDA(cudaMemcpy(P->lin_h.data(), lin, nrings, cudaMemcpyDeviceToHost));
     float2* pair_A;
-    int2 *pair_T, *tiles;
+    int2 *pair_T, *tiles, *wtiles;
     TRY_CUDA(P->alloc(&pair_A, npairs));
     TRY_CUDA(P->alloc(&pair_T, (size_t)npairs * (K + 1)));
     TRY_CUDA(P->alloc(&tiles, ntiles));
+    TRY_CUDA(P->alloc(&wtiles, nwtiles));
     pair_table_kernel<<<n_blocks(npairs, 128), 128, 0, s>>>(nrings, K, pair_off, npairs, ring_range, th, sd,
                                                             npr, E, pair_A, pair_T);
-    tile_list_kernel<<<nrings, 128, 0, s>>>(nrings, tile_off, ntiles_r, tiles);
+    tile_list_kernel<<<nrings, 128, 0, s>>>(nrings, tile_off, ntiles_r, nullptr, tiles);
+    tile_list_kernel<<<nrings, 128, 0, s>>>(nrings, wtile_off, nwtiles_r, lin, wtiles);
     TRY_CUDA(cudaGetLastError());
+    g.lin = lin;
+    g.ring_reach = reach;
+    g.rc = rc;
+    g.wtiles = wtiles;
+    g.nwtiles = nwtiles;
     g.ring_first = first;
     g.ring_n = npr;
     g.ring_shift = shift;
@@ -267,16 +283,15 @@ static tpcf_status build_map(tpcf_plan_s* P, int64_t nside, cudaStream_t s) {
         return TPCF_ERR_UNSUPPORTED;
     }
     // slots for the largest grid any configuration launches
-    P->fwd_grid = (int)std::min<int64_t>(ntiles, (int64_t)P->num_sms * occ_f);
+    P->fwd_grid = (int)std::min<int64_t>(g.nwtiles, (int64_t)P->num_sms * occ_f);
     P->bwd_grid = (int)std::min<int64_t>(ntiles, (int64_t)P->num_sms * occ_b);
-    P->tune_fwd.ctas = tc ? occ_f : L.fwd_occ(K, self, 3);
-    P->tune_bwd.ctas = L.bwd_occ(K, 3);
-    if (P->tune_fwd.ctas < 1) P->tune_fwd.variant = 2, P->tune_fwd.ctas = L.fwd_occ(K, self, 2);
-    if (P->tune_bwd.ctas < 1) P->tune_bwd.variant = 2, P->tune_bwd.ctas = L.bwd_occ(K, 2);
+    P->tune_fwd.variant = P->tune_bwd.variant = 2;
+    P->tune_fwd.ctas = tc ? occ_f : L.fwd_occ(K, self, 2);
+    P->tune_bwd.ctas = L.bwd_occ(K, 2);
     if (P->fwd_grid < 1) P->fwd_grid = 1;
     if (P->bwd_grid < 1) P->bwd_grid = 1;
     P->nent = n_entries(K, P->M);
-    TRY_CUDA(P->alloc(&P->wdw, g.npix));
+    TRY_CUDA(P->alloc(&P->wdw, g.npix + 1));  // and a zero after the last pixel
     TRY_CUDA(P->alloc(&P->slots, (size_t)P->fwd_grid * P->nent));
     TRY_CUDA(P->alloc(&P->sums, P->nent));
     TRY_CUDA(P->alloc(&P->counter, 4));
@@ -388,25 +403,23 @@ static int64_t ring_first_pixel(int64_t nside, int64_t ri) {  // 0-based ring
     return 12 * nside * nside - 2 * rr * (rr + 1);
 }
 
-// Tiles [*tlo, *thi) that hold the pivots [lo, hi) (tiles are 32 consecutive pixels
-// of one ring, rings in order).
-// Tiles [tlo, thi) that can hold a pivot of [lo, hi).  Linear layout: the tiles of the
-// range's pixels.  Quadrant layout (the forward kernels): a partial ring's pivots are
-// spread over all of its tiles, so whole rings at the two ends.
-static void tile_range(const tpcf_plan_s* P, int64_t lo, int64_t hi, int64_t* tlo, int64_t* thi, bool quad) {
+// Tiles [*tlo, *thi) that can hold a pivot of [lo, hi).  Tiles of 32 consecutive pivots: those
+// of the range's pixels.  The walk's tiles: likewise on linear rings; on the others a
+// partial ring's pivots are spread over all of its tiles, so whole rings at the ends.
+static void tile_range(const tpcf_plan_s* P, int64_t lo, int64_t hi, int64_t* tlo, int64_t* thi, bool walk) {
     if (hi <= lo) {
         *tlo = *thi = 0;
         return;
     }
     const int64_t nside = P->map.nside;
     const int64_t ra = ring_of_pixel(nside, lo), rb = ring_of_pixel(nside, hi - 1);
-    if (quad) {
-        *tlo = P->tile_off_h[ra];
-        *thi = rb + 1 < (int64_t)P->tile_off_h.size() ? P->tile_off_h[rb + 1] : P->map.ntiles;
-        return;
-    }
-    *tlo = P->tile_off_h[ra] + (lo - ring_first_pixel(nside, ra)) / TILE;
-    *thi = P->tile_off_h[rb] + (hi - 1 - ring_first_pixel(nside, rb)) / TILE + 1;
+    const std::vector<int64_t>& off = walk ? P->wtile_off_h : P->tile_off_h;
+    *tlo = off[ra];
+    if (!walk || P->lin_h[ra]) *tlo += (lo - ring_first_pixel(nside, ra)) / TILE;
+    if (!walk || P->lin_h[rb])
+        *thi = off[rb] + (hi - 1 - ring_first_pixel(nside, rb)) / TILE + 1;
+    else
+        *thi = rb + 1 < (int64_t)off.size() ? off[rb + 1] : P->map.nwtiles;
 }
 
 static int launch_grid(const tpcf_plan_s* P, const tpcf_plan_s::Tune& t, int64_t ntiles, int cap) {
@@ -438,8 +451,7 @@ static tpcf_status map_forward(tpcf_plan_s* P, const float* d_delta, const float
         c.tile_lo = 0;
         c.tile_hi = P->ngtiles;
     } else {
-        c.quad = P->tune_fwd.quad;
-        tile_range(P, lo, hi, &c.tile_lo, &c.tile_hi, c.quad != 0);
+        tile_range(P, lo, hi, &c.tile_lo, &c.tile_hi, true);
     }
     const int grid = launch_grid(P, P->tune_fwd, c.tile_hi - c.tile_lo, P->fwd_grid);
     if (P->flags & TPCF_CONTRACT_TC)
@@ -535,11 +547,11 @@ extern "C" tpcf_status tpcf_forward_multi(tpcf_plan plan, const float* d_delta_a
                      "tpcf_forward_multi: three fields' moments (K=%d, m_max=%d) do not fit in shared memory", K, M);
             return TPCF_ERR_UNSUPPORTED;
         }
-        const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(g.ntiles, (int64_t)P->num_sms * occ));
+        const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(g.nwtiles, (int64_t)P->num_sms * occ));
         float2 *b, *c;
         double *sl, *su;
-        TRY_CUDA(P->alloc(&b, g.npix));
-        TRY_CUDA(P->alloc(&c, g.npix));
+        TRY_CUDA(P->alloc(&b, g.npix + 1));
+        TRY_CUDA(P->alloc(&c, g.npix + 1));
         TRY_CUDA(P->alloc(&sl, (size_t)grid * nent));
         TRY_CUDA(P->alloc(&su, (size_t)nent));
         P->wdw_c = c;

@@ -55,9 +55,12 @@ namespace {
 struct Group {
     int M = 0;
     std::vector<int> members;  // indices into the batch's plan list
-    BatchItem* d_items = nullptr;
+    BatchItem* d_items = nullptr;    // forward: the walk's tiles
+    BatchItem* d_items_b = nullptr;  // adjoint: tiles of 32 consecutive pivots
     long long total_tiles = 0;
     size_t fwd_smem = 0, bwd_smem = 0;
+    int fwd_cells = 0, bwd_cells = 0;  // cell tables of the walk
+    long long total_wtiles = 0;
     int fwd_grid = 0, bwd_grid = 0;
 };
 }  // namespace
@@ -105,7 +108,7 @@ static tpcf_status record(tpcf_batch_s* B, int num_sms, int max_nent, int max_no
     TRY_CUDA(cudaMemsetAsync(B->d_counters, 0, sizeof(unsigned long long) * 2 * B->groups.size(), s));
     for (size_t gi = 0; gi < B->groups.size(); ++gi) {
         const Group& G = B->groups[gi];
-        TRY_CUDA(kBatch[G.M].fwd(G.d_items, (int)G.members.size(), G.total_tiles, B->d_counters + 2 * gi,
+        TRY_CUDA(kBatch[G.M].fwd(G.d_items, (int)G.members.size(), G.total_wtiles, B->d_counters + 2 * gi,
                                  G.fwd_smem, G.fwd_grid, s));
         B->kernels += 1;
     }
@@ -117,7 +120,7 @@ static tpcf_status record(tpcf_batch_s* B, int num_sms, int max_nent, int max_no
         B->kernels += 1;
         for (size_t gi = 0; gi < B->groups.size(); ++gi) {
             const Group& G = B->groups[gi];
-            TRY_CUDA(kBatch[G.M].bwd(G.d_items, (int)G.members.size(), G.total_tiles, B->d_counters + 2 * gi + 1,
+            TRY_CUDA(kBatch[G.M].bwd(G.d_items_b, (int)G.members.size(), G.total_tiles, B->d_counters + 2 * gi + 1,
                                      G.bwd_smem, G.bwd_grid, s));
             B->kernels += 1;
         }
@@ -145,10 +148,19 @@ static tpcf_status batch_build(tpcf_batch_s* B, const tpcf_plan* plans, const fl
     std::vector<BatchIO> io(n);
     std::vector<int> grid_of(n, 0);
     for (Group& G : B->groups) {
+        size_t fwd_base = 0, bwd_base = 0;
         for (int i : G.members) {
             const tpcf_plan P = plans[i];
-            G.fwd_smem = std::max(G.fwd_smem, tile_floats_rt(P->K, P->M) * sizeof(float));
-            G.bwd_smem = std::max(G.bwd_smem, bwd_tile_floats_rt(P->K, P->M) * sizeof(float));
+            fwd_base = std::max(fwd_base, tile_floats_rt(P->K, P->M, true) * sizeof(float));
+            bwd_base = std::max(bwd_base, (tile_floats_rt(P->K, P->M, false) + TILE) * sizeof(float));
+        }
+        G.fwd_cells = walk_pick_cells(fwd_base, NWARPS);
+        G.bwd_cells = walk_pick_cells(bwd_base, NWARPS);
+        for (int i : G.members) {
+            const tpcf_plan P = plans[i];
+            G.fwd_smem = std::max(G.fwd_smem, tile_floats_rt(P->K, P->M, true) * sizeof(float) +
+                                                  walk_scratch_bytes(NWARPS, G.fwd_cells));
+            G.bwd_smem = std::max(G.bwd_smem, bwd_smem_bytes(P->K, P->M, false, G.bwd_cells));
         }
         const int of = kBatch[G.M].fwd_occ(G.fwd_smem);
         TRY_CUDA(cudaGetLastError());
@@ -196,8 +208,8 @@ static tpcf_status batch_build(tpcf_batch_s* B, const tpcf_plan* plans, const fl
     TRY_CUDA(B->alloc(&B->d_counters, 2 * B->groups.size()));
 
     for (Group& G : B->groups) {
-        std::vector<BatchItem> items;
-        long long t0 = 0;
+        std::vector<BatchItem> items, items_b;
+        long long t0 = 0, t0_b = 0;
         for (int i : G.members) {
             const tpcf_plan P = plans[i];
             BatchItem it{};
@@ -214,16 +226,24 @@ static tpcf_status batch_build(tpcf_batch_s* B, const tpcf_plan* plans, const fl
             it.c.grad = io[i].grad;
             it.c.self_subtract = io[i].self_subtract;
             it.c.flush = P->tune_fwd.flush;
-            it.c.quad = P->tune_fwd.quad;
+            it.c.cells = G.fwd_cells;
             it.c.tile_lo = 0;
-            it.c.tile_hi = P->map.ntiles;
+            it.c.tile_hi = P->map.nwtiles;
             it.tile0 = t0;
-            t0 += P->map.ntiles;
+            t0 += P->map.nwtiles;
             items.push_back(it);
+            it.c.cells = G.bwd_cells;
+            it.c.tile_hi = P->map.ntiles;
+            it.tile0 = t0_b;
+            t0_b += P->map.ntiles;
+            items_b.push_back(it);
         }
-        G.total_tiles = t0;
+        G.total_wtiles = t0;
+        G.total_tiles = t0_b;
         TRY_CUDA(B->alloc(&G.d_items, items.size()));
         TRY_CUDA(cudaMemcpy(G.d_items, items.data(), sizeof(BatchItem) * items.size(), cudaMemcpyHostToDevice));
+        TRY_CUDA(B->alloc(&G.d_items_b, items_b.size()));
+        TRY_CUDA(cudaMemcpy(G.d_items_b, items_b.data(), sizeof(BatchItem) * items_b.size(), cudaMemcpyHostToDevice));
     }
 
     TRY_CUDA(cudaStreamCreateWithFlags(&B->cap, cudaStreamNonBlocking));

@@ -17,7 +17,7 @@ namespace tpcf {
 
 __global__ void ring_table_kernel(int nside, int nrings, int64_t* first, int* npr, int* shift, double* z,
                                   double* s, double* th, float* zf, float* sf, float* sf_lo, float* step,
-                                  float* step_lo, float* invn, float* invn_lo) {
+                                  float* step_lo, float* invn, float* invn_lo, float4* rc) {
     const int ri = blockIdx.x * blockDim.x + threadIdx.x;
     if (ri >= nrings) return;
     const long long n = nside;
@@ -57,6 +57,9 @@ __global__ void ring_table_kernel(int nside, int nrings, int64_t* first, int* np
     step_lo[ri] = (float)(st - (double)(float)st);
     invn[ri] = (float)iv;
     invn_lo[ri] = (float)(iv - (double)(float)iv);
+    rc[2 * ri] = make_float4(sf[ri], sf_lo[ri], step[ri], step_lo[ri]);
+    rc[2 * ri + 1] = make_float4(invn[ri], invn_lo[ri], __int_as_float(2 * npr[ri] + shift[ri]),
+                                 __int_as_float((int)first[ri]));
 }
 
 // Rings r with sin^2((theta_r - theta_i)/2) < E form a contiguous range around i.
@@ -82,15 +85,28 @@ __device__ int2 ring_window(const double* th, int nrings, int i, double E) {
     return make_int2(rlo, lo);
 }
 
-__global__ void ring_range_kernel(int nrings, int K, const double* th, const double* E, const int* npr,
-                                  int2* ring_range, int2* bin_range, int64_t* npairs, int64_t* ntiles) {
+// Also the class of each ring for the walk (map_walk.cuh): linear when all its neighbour
+// rings have its own pixel count and the outer edge leaves part of each of them out (both
+// decided at the ends of the window: the pixel count and the sine of the colatitude rise and
+// fall once from pole to pole); reach bounds how far, in pixels, a linear tile's rows extend
+// beyond a pivot (offsets of at most T plus rounding).
+__global__ void ring_range_kernel(int nrings, int K, const double* th, const double* s, const double* E,
+                                  const int* npr, const int* shift, int2* ring_range, int2* bin_range,
+                                  int64_t* npairs, int64_t* ntiles, int64_t* nwtiles, unsigned char* lin, int* reach) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= nrings) return;
     const int2 rr = ring_window(th, nrings, i, E[K]);
     ring_range[i] = rr;
     for (int k = 0; k < K; ++k) bin_range[(size_t)i * K + k] = ring_window(th, nrings, i, E[k + 1]);
     npairs[i] = rr.y - rr.x + 1;
-    ntiles[i] = (npr[i] + TILE - 1) / TILE;
+    const int n = npr[i];
+    ntiles[i] = (n + TILE - 1) / TILE;
+    const double q = E[K] / (s[i] * fmin(s[rr.x], s[rr.y]));
+    const bool same = npr[rr.x] == n && npr[rr.y] == n && q <= 1.0;
+    lin[i] = same ? 1 : 0;
+    reach[i] = same ? (int)(n / M_PI * asin(sqrt(q))) + 4 : n;
+    const int norb = shift[i] ? ((n >> 2) + 1) >> 1 : (n >> 3) + 1;  // orbit_count(n, shift)
+    nwtiles[i] = same ? (n + TILE - 1) / TILE : (norb + TILE / 8 - 1) / (TILE / 8);
 }
 
 // Exclusive prefix sum of n int64 values by one block (n is at most 4 * 8192 - 1).
@@ -162,12 +178,16 @@ __global__ void pair_table_kernel(int nrings, int K, const int64_t* pair_off, in
     }
 }
 
-__global__ void tile_list_kernel(int nrings, const int64_t* tile_off, const int64_t* ntiles_ring, int2* tiles) {
+// lin: NULL for tiles of 32 consecutive pivots, else the walk's tiles (four orbits each on
+// rings that are not linear).
+__global__ void tile_list_kernel(int nrings, const int64_t* tile_off, const int64_t* ntiles_ring,
+                                 const unsigned char* lin, int2* tiles) {
     const int i = blockIdx.x;
     if (i >= nrings) return;
     const int64_t o = tile_off[i];
     const int64_t nt = ntiles_ring[i];
-    for (int64_t t = threadIdx.x; t < nt; t += blockDim.x) tiles[o + t] = make_int2(i, (int)(t * TILE));
+    const int per = lin == nullptr || lin[i] ? TILE : TILE / 8;
+    for (int64_t t = threadIdx.x; t < nt; t += blockDim.x) tiles[o + t] = make_int2(i, (int)(t * per));
 }
 
 __global__ void edges_kernel(int K, const double* theta, double* E) {

@@ -37,12 +37,25 @@ static int occupancy(Kern* k, size_t smem) {
     return nb;
 }
 
+// Shared memory of the forward tile (bytes) and the cell table of its walk.
+static size_t fwd_smem(int K, bool self, int* cells) {
+    const size_t base = tile_floats<TPCF_M>(K, self) * sizeof(float);
+    *cells = walk_pick_cells(base, NWARPS);
+    return base + walk_scratch_bytes(NWARPS, *cells);
+}
+
+static size_t bwd_smem(int K, bool self, int* cells) {
+    *cells = walk_pick_cells((tile_floats<TPCF_M>(K, self) + TILE) * sizeof(float), NWARPS);
+    return bwd_smem_bytes(K, TPCF_M, self, *cells);
+}
+
 // The forward pair kernel; variant 3 or 2 = CTAs per SM its registers are sized for.
-cudaError_t TPCF_CAT(map_fwd_launch_m, TPCF_M)(const MapDev& g, const MapCall& c, int grid, int variant,
+cudaError_t TPCF_CAT(map_fwd_launch_m, TPCF_M)(const MapDev& g, const MapCall& c0, int grid, int variant,
                                                cudaStream_t s) {
-    const size_t smem = tile_floats<TPCF_M>(g.K) * sizeof(float);
+    MapCall c = c0;
+    const size_t smem = fwd_smem(g.K, c.self_subtract != 0, &c.cells);
     if (c.group > 1)  // shared neighbour lists (self pairs kept)
-        return launch(map_fwd_kernel<TPCF_M, false, false, 3, true>, smem, grid, g, c, s);
+        return launch(map_fwd_kernel<TPCF_M, false, false, 2, true>, smem, grid, g, c, s);
     if (c.self_subtract)
         return variant == 2 ? launch(map_fwd_kernel<TPCF_M, true, false, 2>, smem, grid, g, c, s)
                             : launch(map_fwd_kernel<TPCF_M, true, false, 3>, smem, grid, g, c, s);
@@ -50,9 +63,10 @@ cudaError_t TPCF_CAT(map_fwd_launch_m, TPCF_M)(const MapDev& g, const MapCall& c
                         : launch(map_fwd_kernel<TPCF_M, false, false, 3>, smem, grid, g, c, s);
 }
 
-cudaError_t TPCF_CAT(map_bwd_launch_m, TPCF_M)(const MapDev& g, const MapCall& c, int grid, int variant,
+cudaError_t TPCF_CAT(map_bwd_launch_m, TPCF_M)(const MapDev& g, const MapCall& c0, int grid, int variant,
                                                cudaStream_t s) {
-    const size_t smem = bwd_tile_floats<TPCF_M>(g.K) * sizeof(float);
+    MapCall c = c0;
+    const size_t smem = bwd_smem(g.K, c.self_subtract != 0, &c.cells);
     if (c.self_subtract)
         return variant == 2 ? launch(map_bwd_kernel<TPCF_M, true, 2>, smem, grid, g, c, s)
                             : launch(map_bwd_kernel<TPCF_M, true, 3>, smem, grid, g, c, s);
@@ -62,7 +76,8 @@ cudaError_t TPCF_CAT(map_bwd_launch_m, TPCF_M)(const MapDev& g, const MapCall& c
 
 // Resident CTAs per SM of the forward variant (shared memory and registers).
 int TPCF_CAT(map_fwd_occupancy_m, TPCF_M)(int K, int self_subtract, int variant) {
-    const size_t smem = tile_floats<TPCF_M>(K) * sizeof(float);
+    int cells;
+    const size_t smem = fwd_smem(K, self_subtract != 0, &cells);
     if (self_subtract)
         return variant == 2 ? occupancy(map_fwd_kernel<TPCF_M, true, false, 2>, smem)
                             : occupancy(map_fwd_kernel<TPCF_M, true, false, 3>, smem);
@@ -72,21 +87,27 @@ int TPCF_CAT(map_fwd_occupancy_m, TPCF_M)(int K, int self_subtract, int variant)
 
 // Resident CTAs per SM of the adjoint variant (either self-pair mode).
 int TPCF_CAT(map_bwd_occupancy_m, TPCF_M)(int K, int variant) {
-    const size_t smem = bwd_tile_floats<TPCF_M>(K) * sizeof(float);
-    int a, b;
+    int cells, a, b;
+    const size_t smem = bwd_smem(K, false, &cells), smem_self = bwd_smem(K, true, &cells);
     if (variant == 2) {
         a = occupancy(map_bwd_kernel<TPCF_M, false, 2>, smem);
-        b = occupancy(map_bwd_kernel<TPCF_M, true, 2>, smem);
+        b = occupancy(map_bwd_kernel<TPCF_M, true, 2>, smem_self);
     } else {
         a = occupancy(map_bwd_kernel<TPCF_M, false, 3>, smem);
-        b = occupancy(map_bwd_kernel<TPCF_M, true, 3>, smem);
+        b = occupancy(map_bwd_kernel<TPCF_M, true, 3>, smem_self);
     }
     return a < b ? a : b;
 }
 
 // Forward with the split-precision tensor-core contraction.
-cudaError_t TPCF_CAT(map_fwd_tc_launch_m, TPCF_M)(const MapDev& g, const MapCall& c, int grid, cudaStream_t s) {
-    const size_t smem = tc_smem_bytes(g.K, TPCF_M, c.self_subtract != 0);
+static size_t tc_smem(int K, bool self, int* cells) {
+    *cells = walk_pick_cells((size_t)tc_layout(K, TPCF_M, self).offWalk * sizeof(float), NWARPS);
+    return tc_smem_bytes(K, TPCF_M, self, *cells);
+}
+
+cudaError_t TPCF_CAT(map_fwd_tc_launch_m, TPCF_M)(const MapDev& g, const MapCall& c0, int grid, cudaStream_t s) {
+    MapCall c = c0;
+    const size_t smem = tc_smem(g.K, c.self_subtract != 0, &c.cells);
     if (c.self_subtract) {
         auto* k = map_fwd_tc_kernel<TPCF_M, true>;
         cudaError_t e = prefer_shared(k, smem);
@@ -125,17 +146,26 @@ static int occupancy_by_resources(Kern* k, size_t smem) {
 }
 
 int TPCF_CAT(map_fwd_tc_occupancy_m, TPCF_M)(int K, int self_subtract) {
-    const size_t smem = tc_smem_bytes(K, TPCF_M, self_subtract != 0);
+    int cells;
+    const size_t smem = tc_smem(K, self_subtract != 0, &cells);
     const int nb = self_subtract ? occupancy_by_resources(map_fwd_tc_kernel<TPCF_M, true>, smem)
                                  : occupancy_by_resources(map_fwd_tc_kernel<TPCF_M, false>, smem);
     // at most 512 / TC_TMEM_COLS accumulators per SM; more resident CTAs would wait in tcgen05.alloc
     return nb < 512 / TC_TMEM_COLS ? nb : 512 / TC_TMEM_COLS;
 }
 
-// Multi-field forward (three fields on the same pixels).
-cudaError_t TPCF_CAT(map_fwd_multi_launch_m, TPCF_M)(const MapDev& g, const MapCall& c, const float2* wdwB,
+// Multi-field forward (three fields on the same pixels).  Without room for the walk's
+// scratch beside three fields' moments (cells = 0) the tiles take the per-lane walk.
+static size_t multi_smem(int K, int* cells) {
+    const size_t base = multi_tile_floats(K, TPCF_M) * sizeof(float);
+    *cells = walk_pick_cells(base, NWARPS);
+    return base + (*cells ? walk_scratch_bytes(NWARPS, *cells) : 0);
+}
+
+cudaError_t TPCF_CAT(map_fwd_multi_launch_m, TPCF_M)(const MapDev& g, const MapCall& c0, const float2* wdwB,
                                                      const float2* wdwC, int grid, cudaStream_t s) {
-    const size_t smem = multi_tile_floats(g.K, TPCF_M) * sizeof(float);
+    MapCall c = c0;
+    const size_t smem = multi_smem(g.K, &c.cells);
     auto* k = map_fwd_multi_kernel<TPCF_M>;
     cudaError_t e = prefer_shared(k, smem);
     if (e != cudaSuccess) return e;
@@ -144,7 +174,8 @@ cudaError_t TPCF_CAT(map_fwd_multi_launch_m, TPCF_M)(const MapDev& g, const MapC
 }
 
 int TPCF_CAT(map_fwd_multi_occupancy_m, TPCF_M)(int K) {
-    return occupancy(map_fwd_multi_kernel<TPCF_M>, multi_tile_floats(K, TPCF_M) * sizeof(float));
+    int cells;
+    return occupancy(map_fwd_multi_kernel<TPCF_M>, multi_smem(K, &cells));
 }
 
 // Multi-field forward on a catalogue.
@@ -163,18 +194,16 @@ int TPCF_CAT(cat_fwd_multi_occupancy_m, TPCF_M)(int K) {
 }
 
 // Forward that reads the caller's delta and w directly (no packed copy).
-cudaError_t TPCF_CAT(map_fwd_direct_launch_m, TPCF_M)(const MapDev& g, const MapCall& c, int grid,
+cudaError_t TPCF_CAT(map_fwd_direct_launch_m, TPCF_M)(const MapDev& g, const MapCall& c0, int grid,
                                                       cudaStream_t s) {
-    const size_t smem = tile_floats<TPCF_M>(g.K) * sizeof(float);
-    auto* k = map_fwd_kernel<TPCF_M, false, true>;
+    MapCall c = c0;
+    const size_t smem = fwd_smem(g.K, false, &c.cells);
+    auto* k = map_fwd_kernel<TPCF_M, false, true, 2>;
     cudaError_t e = prefer_shared(k, smem);
     if (e != cudaSuccess) return e;
     k<<<grid, NTHREADS, smem, s>>>(g, c);
     return cudaGetLastError();
 }
-
-size_t TPCF_CAT(map_fwd_smem_m, TPCF_M)(int K) { return tile_floats<TPCF_M>(K) * sizeof(float); }
-size_t TPCF_CAT(map_bwd_smem_m, TPCF_M)(int K) { return bwd_tile_floats<TPCF_M>(K) * sizeof(float); }
 
 // Batched forward / adjoint over all the plans of a batch whose largest m_max is this
 // M (the dynamic shared memory is the largest any of them needs).

@@ -3,10 +3,13 @@
 // which is compiled once per M.
 //
 // Work decomposition (forward):
-//   * a tile is 32 consecutive pivots of one HEALPix ring, one pivot per lane;
-//   * a CTA of 8 warps owns one tile at a time (persistent CTAs, 3 per SM, pull
-//     tiles from an atomic counter); for every radial bin k the warps split the
-//     neighbour rings that can hold bin-k pixels;
+//   * a tile is 32 pivots of one HEALPix ring; a CTA of 8 warps owns one tile at a time
+//     (persistent CTAs pull tiles from an atomic counter).  Its moments come from the
+//     shared-angle walk (map_walk.cuh); the points below describe the per-lane walk, one
+//     pivot per lane, that shared neighbour lists and the adjoint use on rings without
+//     common angles;
+//   * for every radial bin k the warps split the neighbour rings that can hold bin-k
+//     pixels;
 //   * on a neighbour ring the bin-k pixels of a pivot form at most two contiguous
 //     runs, found from the per-ring-pair edge offsets T_e built by the plan (an
 //     exact ring-range disc query); each lane walks its own runs, so the bin is
@@ -312,7 +315,9 @@ struct PackedLoad {
 struct DirectLoad {
     const float* __restrict__ d;
     const float* __restrict__ w;
+    long long n;  // pixels: entry n reads as zero, as in the packed array
     __device__ __forceinline__ float2 operator()(long long i) const {
+        if (i >= n) return make_float2(0.0f, 0.0f);
         const float wi = __ldg(w + i);
         return make_float2(wi * __ldg(d + i), wi);
     }
@@ -377,67 +382,6 @@ __device__ __forceinline__ void walk_run(const RingCtx& R, const L& ld, const La
         }
         idx = idx1 + 1 >= R.n ? idx1 + 1 - R.n : idx1 + 1;
     }
-}
-
-// walk_run for a tile in the quadrant layout (tile_pivot): the four lanes l, l + 8,
-// l + 16, l + 24 hold pivots a quarter turn apart, and since every ring has a multiple
-// of four pixels they see ring r at the same fractional offset, with runs of the same
-// length at the same offset from their own pivot, hence the same position angle at
-// every step.  Each lane of a group computes the (folded) angle of one of every four
-// steps and the group shares them by shuffles; every lane still sums its own pixels.
-// The caller has checked runs_quad().
-template <int M, bool FAST, bool SELF, class L>
-__device__ __forceinline__ void walk_run_quad(const RingCtx& R, const L& ld, const LaneC& c, int a, int len,
-                                              float2 (&acc)[M + 1], float& W, float& Q, float& QW, int mr = M) {
-    const int maxlen = __reduce_max_sync(0xffffffffu, len);
-    if (maxlen <= 0) return;
-    const int lane = threadIdx.x & 31, j = lane >> 3, gb = lane & 7;
-    const float i0 = (float)(a - c.cint);
-    const float xneg = -c.cfrac * R.step, uneg = -c.cfrac * R.inv_n;
-    const int last = max(len - 1, 0);
-    int idx = wrap_idx(a, R.n);
-    const auto row = ld.row(R.first);
-    for (int t0 = 0; t0 < maxlen; t0 += 4) {
-        Fold mine;
-        {
-            // steps past the run take its last offset, a valid direction (zero weight)
-            const int tj = min(t0 + j, last);
-            float cph, sph;
-            pixel_dir<FAST>(i0 + (float)tj, xneg, uneg, R, cph, sph);
-            mine = fold_angle(cph, sph);
-        }
-        // two steps at a time, so that only two shared angles are live
-#pragma unroll
-        for (int h = 0; h < 4; h += 2) {
-            const Fold fa = shfl_fold(mine, gb + 8 * h), fb = shfl_fold(mine, gb + 8 * h + 8);
-            const int i1 = idx + 1 >= R.n ? idx + 1 - R.n : idx + 1;
-            // (the index test is a guard: a run's indices always lie within the ring)
-            const bool ia = t0 + h < len && (unsigned)idx < (unsigned)R.n;
-            const bool ib = t0 + h + 1 < len && (unsigned)i1 < (unsigned)R.n;
-            const float2 va = ia ? row(idx) : make_float2(0.0f, 0.0f);
-            const float2 vb = ib ? row(i1) : make_float2(0.0f, 0.0f);
-            harmonics2f<M>(acc, fa, va.x, va.x, fb, vb.x, vb.x, mr);
-            W += va.y + vb.y;
-            if (SELF) {
-                Q = fmaf(va.x, va.x, fmaf(vb.x, vb.x, Q));
-                QW = fmaf(va.y, va.y, fmaf(vb.y, vb.y, QW));
-            }
-            idx = i1 + 1 >= R.n ? i1 + 1 - R.n : i1 + 1;
-        }
-    }
-}
-
-// True when each lane's run has the same offset from its pivot, the same length and
-// the same fractional pivot position as the other three lanes of its quadrant group
-// (an empty run matches any other empty run).  Every lane takes part in every shuffle.
-__device__ __forceinline__ bool runs_quad(const LaneC& c, int a, int len) {
-    const int gb = threadIdx.x & 7;
-    const int rel = len > 0 ? a - c.cint : 0;
-    const unsigned cf = __float_as_uint(c.cfrac);
-    const int rel0 = __shfl_sync(0xffffffffu, rel, gb);
-    const int len0 = __shfl_sync(0xffffffffu, len, gb);
-    const unsigned cf0 = __shfl_sync(0xffffffffu, cf, gb);
-    return __all_sync(0xffffffffu, rel == rel0 && len == len0 && cf == cf0);
 }
 
 // Walk the pixel pairs (p, mb - p), p in [a, a + len): mirror images about the
@@ -671,7 +615,7 @@ __device__ __forceinline__ ExactCtx exact_ctx(const MapDev& g, const PivotRing& 
 template <int M, bool SELF, class L>
 __device__ __forceinline__ void fwd_ring_bin(const MapDev& g, const PivotRing& P, int r, int k, int q,
                                              const L& ld, float2 (&acc)[M + 1], float& W,
-                                             float& Q, float& QW, int mr = M, bool quad = false) {
+                                             float& Q, float& QW, int mr = M) {
     const long long pr = P.pair0 + (r - P.rlo);
     const int2 Tk = g.pair_T[pr * (g.K + 1) + k];
     const int2 Tk1 = g.pair_T[pr * (g.K + 1) + k + 1];
@@ -706,16 +650,6 @@ __device__ __forceinline__ void fwd_ring_bin(const MapDev& g, const PivotRing& P
     }
     const float om = fmaxf(run_omax(c, b.a0, b.n0), run_omax(c, b.a1, b.n1));
     const bool fast = __all_sync(0xffffffffu, om * R.step <= FAST_XMAX);
-    if (quad && runs_quad(c, b.a0, b.n0) && runs_quad(c, b.a1, b.n1)) {
-        if (fast) {
-            walk_run_quad<M, true, SELF>(R, ld, c, b.a0, b.n0, acc, W, Q, QW, mr);
-            walk_run_quad<M, true, SELF>(R, ld, c, b.a1, b.n1, acc, W, Q, QW, mr);
-        } else {
-            walk_run_quad<M, false, SELF>(R, ld, c, b.a0, b.n0, acc, W, Q, QW, mr);
-            walk_run_quad<M, false, SELF>(R, ld, c, b.a1, b.n1, acc, W, Q, QW, mr);
-        }
-        return;
-    }
     if (fast) {
         walk_run<M, true, SELF>(R, ld, c, b.a0, b.n0, acc, W, Q, QW, mr);
         walk_run<M, true, SELF>(R, ld, c, b.a1, b.n1, acc, W, Q, QW, mr);
@@ -729,8 +663,8 @@ __device__ __forceinline__ void fwd_ring_bin(const MapDev& g, const PivotRing& P
 //   A[k][m][2][32] : sum w d cos(m phi), sum w d sin(m phi)   (a = re - i im)
 //   W[k][32], Q[k][32], QW[k][32], piv[2][32] (w d, w of the pivots)
 template <int M>
-__host__ __device__ inline size_t tile_floats(int K) {
-    return tile_floats_rt(K, M);
+__host__ __device__ inline size_t tile_floats(int K, bool self = true) {
+    return tile_floats_rt(K, M, self);
 }
 
 // Load the tile's pivot description; returns false if no lane has w != 0.
@@ -747,32 +681,11 @@ __device__ __forceinline__ PivotRing pivot_ring(const MapDev& g, int i) {
     return P;
 }
 
-// Pivot of a lane in tile (ring i, start = 32 j).  Linear layout: q = start + lane.
-// Quadrant layout (the forward kernels): q = 8 j + (lane & 7) + (lane >> 3) n_i / 4,
-// four groups of eight consecutive pivots a quarter turn apart (walk_run_quad); a ring
-// has ceil(n_i / 32) tiles either way.  `valid`: q is a pixel of the ring; lanes past
-// the end take the geometry qg of the last pivot (of their quadrant), which keeps every
-// unwrapped pixel index within [-n_r, 2 n_r).
-struct TilePivot {
-    int q, qg;
-    bool valid;
-};
+}  // namespace tpcf
 
-__device__ __forceinline__ TilePivot tile_pivot(int start, int n_i, bool quad) {
-    const int lane = threadIdx.x & 31;
-    TilePivot t;
-    if (quad) {
-        const int quarter = n_i >> 2, qq = (start >> 2) + (lane & 7), off = (lane >> 3) * quarter;
-        t.valid = qq < quarter;
-        t.q = qq + off;
-        t.qg = min(qq, quarter - 1) + off;
-    } else {
-        t.q = start + lane;
-        t.valid = t.q < n_i;
-        t.qg = min(t.q, n_i - 1);
-    }
-    return t;
-}
+#include "map_walk.cuh"
+
+namespace tpcf {
 
 // Where the tile's moments live in shared memory.  LayKM: A[k][m][re/im][32 pivots],
 // W[k][32], Q[k][32], QW[k][32] (the FP32 contraction and the adjoint read this).
@@ -791,7 +704,7 @@ struct LayKM {
 // Smem must be zeroed beforehand; it is complete after the caller's __syncthreads().
 template <int M, bool SELF, class L, class Lay>
 __device__ __forceinline__ void tile_moments_l(const MapDev& g, const PivotRing& P, int q, const L& ld,
-                                               const Lay& lay, int flush, int mr = M, bool quad = false) {
+                                               const Lay& lay, int flush, int mr = M) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (int k = 0; k < g.K; ++k) {
         const int2 br = g.bin_range[(long long)P.i * g.K + k];
@@ -805,7 +718,7 @@ __device__ __forceinline__ void tile_moments_l(const MapDev& g, const PivotRing&
         // sums short.
         int nr = 0;
         for (int r = br.x + warp; r <= br.y; r += NWARPS) {
-            fwd_ring_bin<M, SELF>(g, P, r, k, q, ld, acc, W, Q, QW, mr, quad);
+            fwd_ring_bin<M, SELF>(g, P, r, k, q, ld, acc, W, Q, QW, mr);
             if (++nr == flush || r + NWARPS > br.y) {
                 nr = 0;
 #pragma unroll
@@ -830,9 +743,8 @@ __device__ __forceinline__ void tile_moments_l(const MapDev& g, const PivotRing&
 
 template <int M, bool SELF, class L>
 __device__ __forceinline__ void tile_moments(const MapDev& g, const PivotRing& P, int q, const L& ld, float* sA,
-                                             float* sW, float* sQ, float* sQW, int flush, int mr = M,
-                                             bool quad = false) {
-    tile_moments_l<M, SELF>(g, P, q, ld, LayKM{sA, sW, sQ, sQW, mr + 1}, flush, mr, quad);
+                                             float* sW, float* sQ, float* sQW, int flush, int mr = M) {
+    tile_moments_l<M, SELF>(g, P, q, ld, LayKM{sA, sW, sQ, sQW, mr + 1}, flush, mr);
 }
 
 // Per-pivot normalisation of the tile's moments (Sec. 3.1): each lane's a_m^k is
@@ -873,9 +785,24 @@ __device__ __forceinline__ void tile_normalize(int K, float* sA, float* sW, int 
     __syncthreads();
 }
 
+// Block (b1 <= b2) number i of the CB x CB blocks of a triangle, columns first.
+__device__ __forceinline__ void tri_block(int i, int& b1, int& b2) {
+    b2 = (int)((sqrtf(8.0f * i + 1.0f) - 1.0f) * 0.5f);
+    while (b2 * (b2 + 1) / 2 > i) --b2;
+    while ((b2 + 1) * (b2 + 2) / 2 <= i) ++b2;
+    b1 = i - b2 * (b2 + 1) / 2;
+}
+
 // Per-tile partial sums into the CTA's FP64 slot (eq. zetamEst2 summed over the
 // tile's pivots).  Slot layout: for m, for pair (k1 <= k2): (Re S, Im S); then D for
 // pairs; then sum_i w_i d_i Q^k(i) and sum_i w_i QW^k(i) for k.
+//
+// A thread takes a 4 x 4 block of bin pairs of one multipole over half of the tile's pivots:
+// 17 shared-memory words feed 64 multiply-adds (one bin pair per thread needed 5 words for 8,
+// and the loads bounded it).  Neighbouring lanes hold the two halves; they add them, and
+// one of them adds the real part to the slot, the other the imaginary part.
+constexpr int CB = 4;  // bins on a side of a block
+
 template <int M>
 __device__ __forceinline__ void tile_contract(int K, const float* sA, const float* sW, const float* sQ,
                                               const float* sQW, const float* sPiv, double* slot,
@@ -884,44 +811,67 @@ __device__ __forceinline__ void tile_contract(int K, const float* sA, const floa
     const int nS = (mr + 1) * P;
     const float* wd = sPiv;
     const float* wt = sPiv + TILE;
-    for (int e = threadIdx.x; e < nS + P + (self ? K : 0); e += NTHREADS) {
-        if (e < nS) {
-            const int m = e / P;
-            const int pidx = e - m * P;
-            int k2 = (int)((sqrtf(8.0f * pidx + 1.0f) - 1.0f) * 0.5f);
-            while (k2 * (k2 + 1) / 2 > pidx) --k2;
-            while ((k2 + 1) * (k2 + 2) / 2 <= pidx) ++k2;
-            const int k1 = pidx - k2 * (k2 + 1) / 2;
-            const float* r1 = sA + ((size_t)k1 * (mr + 1) + m) * 2 * TILE;
-            const float* i1 = r1 + TILE;
-            const float* r2 = sA + ((size_t)k2 * (mr + 1) + m) * 2 * TILE;
-            const float* i2 = r2 + TILE;
-            float sr = 0.0f, si = 0.0f;
-            // start each thread at its own lane so a warp's 32 rows hit 32 banks
-#pragma unroll 8
-            for (int j = 0; j < TILE; ++j) {
-                const int l = (j + threadIdx.x) & (TILE - 1);
-                const float a = r1[l], b = i1[l], cc = r2[l], d = i2[l];
-                sr = fmaf(wd[l], fmaf(a, cc, b * d), sr);
-                si = fmaf(wd[l], fmaf(a, d, -b * cc), si);
+    const int nb = (K + CB - 1) / CB, nbp = nb * (nb + 1) / 2;
+    const int half = threadIdx.x & 1, l0 = threadIdx.x >> 1;
+    const size_t kstr = (size_t)(mr + 1) * 2 * TILE;
+    // both lanes of a pair take the same number of turns (2 (mr + 1) nbp is even)
+    for (int e = threadIdx.x; e < 2 * (mr + 1) * nbp; e += NTHREADS) {
+        const int m = (e >> 1) / nbp;
+        int b1, b2;
+        tri_block((e >> 1) - m * nbp, b1, b2);
+        const float *r1[CB], *r2[CB];
+#pragma unroll
+        for (int i = 0; i < CB; ++i) {  // bins past the last one repeat it and are not written
+            r1[i] = sA + min(CB * b1 + i, K - 1) * kstr + m * 2 * TILE + half * (TILE / 2);
+            r2[i] = sA + min(CB * b2 + i, K - 1) * kstr + m * 2 * TILE + half * (TILE / 2);
+        }
+        float2 acc[CB][CB];
+#pragma unroll
+        for (int i = 0; i < CB; ++i)
+#pragma unroll
+            for (int j = 0; j < CB; ++j) acc[i][j] = make_float2(0.0f, 0.0f);
+#pragma unroll 2
+        for (int t = 0; t < TILE / 2; ++t) {
+            const int l = (t + l0) & (TILE / 2 - 1);  // a warp's 32 reads of a word hit 32 banks
+            const float w = wd[half * (TILE / 2) + l];
+            float2 x[CB], y[CB], z[CB];
+#pragma unroll
+            for (int i = 0; i < CB; ++i) {
+                x[i] = make_float2(w * r1[i][l], w * r1[i][TILE + l]);
+                y[i] = make_float2(r2[i][l], r2[i][TILE + l]);
+                z[i] = make_float2(y[i].y, -y[i].x);
             }
-            red_add_f32(slot + 2 * e, sr);
-            red_add_f32(slot + 2 * e + 1, si);
-        } else if (e < nS + P) {
-            const int pidx = e - nS;
-            int k2 = (int)((sqrtf(8.0f * pidx + 1.0f) - 1.0f) * 0.5f);
-            while (k2 * (k2 + 1) / 2 > pidx) --k2;
-            while ((k2 + 1) * (k2 + 2) / 2 <= pidx) ++k2;
-            const int k1 = pidx - k2 * (k2 + 1) / 2;
+#pragma unroll
+            for (int i = 0; i < CB; ++i)
+#pragma unroll
+                for (int j = 0; j < CB; ++j)  // (a c + b d, a d - b c)
+                    acc[i][j] = __ffma2_rn(make_float2(x[i].x, x[i].x), y[j],
+                                           __ffma2_rn(make_float2(x[i].y, x[i].y), z[j], acc[i][j]));
+        }
+        const unsigned pair = 3u << (threadIdx.x & 30);
+#pragma unroll
+        for (int i = 0; i < CB; ++i)
+#pragma unroll
+            for (int j = 0; j < CB; ++j) {
+                const float2 v = acc[i][j];
+                const float s = (half ? v.y : v.x) + __shfl_xor_sync(pair, half ? v.x : v.y, 1);
+                const int k1 = CB * b1 + i, k2 = CB * b2 + j;
+                if (k1 <= k2 && k2 < K) red_add_f32(slot + 2 * (m * P + k2 * (k2 + 1) / 2 + k1) + half, s);
+            }
+    }
+    for (int e = threadIdx.x; e < P + (self ? K : 0); e += NTHREADS) {
+        if (e < P) {
+            int k1, k2;
+            tri_block(e, k1, k2);
             float s = 0.0f;
 #pragma unroll 8
             for (int j = 0; j < TILE; ++j) {
                 const int l = (j + threadIdx.x) & (TILE - 1);
                 s = fmaf(wt[l], sW[k1 * TILE + l] * sW[k2 * TILE + l], s);
             }
-            red_add_f32(slot + nS + e, s);
+            red_add_f32(slot + 2 * nS + e, s);
         } else {
-            const int k = e - nS - P;
+            const int k = e - P;
             float s1 = 0.0f, s2 = 0.0f;
             for (int j = 0; j < TILE; ++j) {
                 const int l = (j + threadIdx.x) & (TILE - 1);
@@ -966,7 +916,8 @@ struct TcLayout {
     int Rm, RD, NBm, NBd;  // rows per m block and of the W block; MMA N of each
     int x0, D0;            // first row of the moments; first row of the W block
     int offB, offPiv, offSc, offQ, offQW;
-    int total;             // floats
+    int offWalk;           // the walk's scratch (over the staging, which is used after it)
+    int total;             // floats, without the walk's scratch
 };
 
 __host__ __device__ inline TcLayout tc_layout(int K, int M, bool self) {
@@ -978,8 +929,6 @@ __host__ __device__ inline TcLayout tc_layout(int K, int M, bool self) {
     L.x0 = 0;
     L.D0 = (M + 1) * L.Rm;
     int off = (L.D0 + L.RD) * TILE;
-    L.offB = off;  // B hi rows, then B lo rows (NBm each); reused for the C^T staging
-    off += 2 * L.NBm * TILE;
     L.offPiv = off;  // (w d, w) of the pivots
     off += 2 * TILE;
     L.offSc = off;  // sqrt|w d|, sign(w d), sqrt w
@@ -987,6 +936,9 @@ __host__ __device__ inline TcLayout tc_layout(int K, int M, bool self) {
     L.offQ = off;
     L.offQW = off + (self ? K * TILE : 0);
     if (self) off += 2 * K * TILE;
+    L.offWalk = off;
+    L.offB = off;  // B hi rows, then B lo rows (NBm each); reused for the C^T staging
+    off += 2 * L.NBm * TILE;
     // the MMA of the last block reads 128 rows from its start
     const int need = (L.D0 + 128) * TILE;
     L.total = off > need ? off : need;
@@ -994,8 +946,11 @@ __host__ __device__ inline TcLayout tc_layout(int K, int M, bool self) {
 }
 
 // bytes of dynamic shared memory
-__host__ __device__ inline size_t tc_smem_bytes(int K, int M, bool self) {
-    return (size_t)tc_layout(K, M, self).total * sizeof(float);
+__host__ __device__ inline size_t tc_smem_bytes(int K, int M, bool self, int cells) {
+    const TcLayout L = tc_layout(K, M, self);
+    const size_t a = (size_t)L.total * sizeof(float);
+    const size_t b = (size_t)L.offWalk * sizeof(float) + walk_scratch_bytes(NWARPS, cells);
+    return a > b ? a : b;
 }
 
 // Position of (row r, pivot p) in the K-major canonical layout without swizzle: core
@@ -1258,45 +1213,55 @@ __device__ __forceinline__ void fwd_tile(const MapDev& g, const MapCall& c, int 
     const int K = g.K;
     float* sA = smem;
     float* sW = sA + (size_t)K * (mr + 1) * 2 * TILE;
-    float* sQ = sW + K * TILE;
+    float* sQ = sW + K * TILE;  // Q, QW with SELF only
     float* sQW = sQ + K * TILE;
-    float* sPiv = sQW + K * TILE;
+    float* sPiv = SELF ? sQW + K * TILE : sQ;
+    char* scratch = reinterpret_cast<char*>(sPiv + 2 * TILE);
     const int lane = threadIdx.x & 31;
-    const size_t nfl = tile_floats_rt(K, mr) - 2 * TILE;
+    const size_t nfl = tile_floats_rt(K, mr, SELF) - 2 * TILE;
     constexpr bool grouped = GROUPED;  // shared neighbour lists (c.group > 1): own instantiation
-    const int2 tq = grouped ? c.gtiles[tile] : g.tiles[tile];
+    const int2 tq = grouped ? c.gtiles[tile] : g.wtiles[tile];
     if (tq.x < 0 || tq.x >= g.nrings) {
         if (threadIdx.x == 0) atomicOr(c.status, ST_BAD_TILE);
         __syncthreads();
         return;
     }
     const PivotRing P = pivot_ring(g, tq.x);
+    const bool lin = g.lin[P.i] != 0;
     float2 pv = make_float2(0.0f, 0.0f);
-    int qg;  // the lane's geometry; lanes past the ring's end: zero weight, valid geometry
+    int qg, qa, qb;  // geometry of the lane's pivot, and of pivots lane & 15 and 16 + (lane & 15)
     if (grouped) {
         // shared neighbour lists: the lane stands for the run of c.group consecutive ring
         // pixels gi, sits at the run's middle pixel and carries the run's summed weights
         const int ng = (P.n_i + c.group - 1) / c.group;
+        auto middle = [&](int gi) {
+            const int s0 = min(gi, ng - 1) * c.group;
+            return s0 + (min(c.group, P.n_i - s0) - 1) / 2;
+        };
         const int gi = tq.y + lane;
         const int s0 = min(gi, ng - 1) * c.group, ln = min(c.group, P.n_i - s0);
-        qg = s0 + (ln - 1) / 2;
+        qg = middle(gi);
+        qa = middle(tq.y + (lane & 15));
+        qb = middle(tq.y + 16 + (lane & 15));
         if (gi < ng) {
             const long long f = g.ring_first[P.i] + s0;
             for (int u = 0; u < ln; ++u) {
                 const long long pix = f + u;
                 if (pix >= c.piv_lo && pix < c.piv_hi) {
-                    const float2 v = DIRECT ? DirectLoad{c.delta, c.w}(pix) : c.wdw[pix];
+                    const float2 v = DIRECT ? DirectLoad{c.delta, c.w, g.npix}(pix) : c.wdw[pix];
                     pv.x += v.x;
                     pv.y += v.y;
                 }
             }
         }
     } else {
-        const TilePivot tp = tile_pivot(tq.y, P.n_i, c.quad != 0);
+        const TileSlot tp = tile_slot(lin, P.n_i, P.s_i, tq.y, lane);
         const long long pix = g.ring_first[P.i] + tp.q;
         if (tp.valid && pix >= c.piv_lo && pix < c.piv_hi)
-            pv = DIRECT ? DirectLoad{c.delta, c.w}(pix) : c.wdw[pix];
-        qg = tp.qg;
+            pv = DIRECT ? DirectLoad{c.delta, c.w, g.npix}(pix) : c.wdw[pix];
+        qg = tp.q;
+        qa = tile_slot(lin, P.n_i, P.s_i, tq.y, lane & 15).q;
+        qb = tile_slot(lin, P.n_i, P.s_i, tq.y, 16 + (lane & 15)).q;
     }
     if (!__syncthreads_or(pv.y != 0.0f)) return;
     for (size_t e = threadIdx.x; e < nfl; e += NTHREADS) sA[e] = 0.0f;
@@ -1305,11 +1270,18 @@ __device__ __forceinline__ void fwd_tile(const MapDev& g, const MapCall& c, int 
         sPiv[TILE + lane] = pv.y;
     }
     __syncthreads();
-    if (DIRECT)
-        tile_moments<M, SELF>(g, P, qg, DirectLoad{c.delta, c.w}, sA, sW, sQ, sQW, c.flush, mr,
-                              !grouped && c.quad);
+    auto moments = [&](const auto& ld) {
+        // runs of pixels on other rings have no common angles: one pivot per lane
+        if (grouped && !lin)
+            tile_moments<M, SELF>(g, P, qg, ld, sA, sW, sQ, sQW, c.flush, mr);
+        else
+            walk_tile<M, SELF>(g, P, lin, qa, qb, tq.y, ld, LayKM{sA, sW, sQ, sQW, mr + 1}, scratch, c.cells, c.flush,
+                               mr);
+    };
+    if constexpr (DIRECT)
+        moments(DirectLoad{c.delta, c.w, g.npix});
     else
-        tile_moments<M, SELF>(g, P, qg, PackedLoad{c.wdw}, sA, sW, sQ, sQW, c.flush, mr, !grouped && c.quad);
+        moments(PackedLoad{c.wdw});
     __syncthreads();
     if (c.norm != NORM_NONE) tile_normalize<M>(K, sA, sW, c.norm, mr);
     tile_contract<M>(K, sA, sW, sQ, sQW, sPiv, slot, SELF && c.self_subtract, mr);
@@ -1323,19 +1295,19 @@ __device__ __forceinline__ void fwd_tile_tc(const MapDev& g, const MapCall& c, i
                                             TcState& tc) {
     const int K = g.K;
     const int lane = threadIdx.x & 31;
-    const int2 tq = g.tiles[tile];
+    const int2 tq = g.wtiles[tile];
     if (tq.x < 0 || tq.x >= g.nrings) {
         if (threadIdx.x == 0) atomicOr(c.status, ST_BAD_TILE);
         __syncthreads();
         return;
     }
     const PivotRing P = pivot_ring(g, tq.x);
-    const TilePivot tp = tile_pivot(tq.y, P.n_i, c.quad != 0);
+    const bool lin = g.lin[P.i] != 0;
+    const TileSlot tp = tile_slot(lin, P.n_i, P.s_i, tq.y, lane);
     const long long pix = g.ring_first[P.i] + tp.q;
     const bool in = tp.valid && pix >= c.piv_lo && pix < c.piv_hi;
     float2 pv = make_float2(0.0f, 0.0f);
     if (in) pv = c.wdw[pix];
-    const int qg = tp.qg;
     if (!__syncthreads_or(pv.y != 0.0f)) return;
     {
         const TcLayout L = tc_layout(K, M, SELF);
@@ -1352,8 +1324,10 @@ __device__ __forceinline__ void fwd_tile_tc(const MapDev& g, const MapCall& c, i
     {
         const int Rm = (2 * K + 7) & ~7, D0 = (M + 1) * Rm;
         const TcLayout L = tc_layout(K, M, SELF);
-        tile_moments_l<M, SELF>(g, P, qg, PackedLoad{c.wdw}, LayTC{base, base + L.offQ, base + L.offQW, Rm, D0},
-                                c.flush, M, c.quad != 0);
+        walk_tile<M, SELF>(g, P, lin, tile_slot(lin, P.n_i, P.s_i, tq.y, lane & 15).q,
+                           tile_slot(lin, P.n_i, P.s_i, tq.y, 16 + (lane & 15)).q, tq.y, PackedLoad{c.wdw},
+                           LayTC{base, base + L.offQ, base + L.offQW, Rm, D0},
+                           reinterpret_cast<char*>(base + L.offWalk), c.cells, c.flush, M);
     }
     __syncthreads();
     tile_contract_tc<M, SELF>(K, base, slot, tc, c.status);
@@ -1379,7 +1353,7 @@ __global__ void __launch_bounds__(NTHREADS, OCC) map_fwd_kernel(MapDev g, MapCal
 // The forward with the tensor-core contraction (3 CTAs per SM where the shared
 // memory allows it; 128 accumulator columns each, so at most 4 fit an SM's TMEM).
 template <int M, bool SELF>
-__global__ void __launch_bounds__(NTHREADS, 3) map_fwd_tc_kernel(MapDev g, MapCall c) {
+__global__ void __launch_bounds__(NTHREADS, 2) map_fwd_tc_kernel(MapDev g, MapCall c) {
     extern __shared__ __align__(16) float smem_tc[];
     __shared__ int s_tile;
     __shared__ uint32_t s_tmem;
@@ -1507,14 +1481,15 @@ __global__ void __launch_bounds__(NTHREADS, 2) map_fwd_multi_kernel(MapDev g, Ma
         __syncthreads();
         const long long tile = c.tile_lo + s_tile;
         if (tile >= c.tile_hi) break;
-        const int2 tq = g.tiles[tile];
+        const int2 tq = g.wtiles[tile];
         if (tq.x < 0 || tq.x >= g.nrings) {
             if (threadIdx.x == 0) atomicOr(c.status, ST_BAD_TILE);
             __syncthreads();
             continue;
         }
         const PivotRing P = pivot_ring(g, tq.x);
-        const TilePivot tp = tile_pivot(tq.y, P.n_i, true);
+        const bool lin = g.lin[P.i] != 0;
+        const TileSlot tp = tile_slot(lin, P.n_i, P.s_i, tq.y, lane);
         const long long pix = g.ring_first[P.i] + tp.q;
         const bool in = tp.valid && pix >= c.piv_lo && pix < c.piv_hi;
         float2 pv[3];
@@ -1524,7 +1499,8 @@ __global__ void __launch_bounds__(NTHREADS, 2) map_fwd_multi_kernel(MapDev g, Ma
             pv[f] = in ? arr[f][pix] : make_float2(0.0f, 0.0f);
             live = live || pv[f].y != 0.0f;
         }
-        const int qg = tp.qg;
+        const int qa = tile_slot(lin, P.n_i, P.s_i, tq.y, lane & 15).q;
+        const int qb = tile_slot(lin, P.n_i, P.s_i, tq.y, 16 + (lane & 15)).q;
         if (!__syncthreads_or(live)) continue;
         for (size_t e = threadIdx.x; e < 3 * fsz; e += NTHREADS) sF[e] = 0.0f;
         if (threadIdx.x < TILE) {
@@ -1537,8 +1513,12 @@ __global__ void __launch_bounds__(NTHREADS, 2) map_fwd_multi_kernel(MapDev g, Ma
         __syncthreads();
         for (int f = 0; f < 3; ++f) {
             float* sA = sF + f * fsz;
-            tile_moments<M, false>(g, P, qg, PackedLoad{arr[f]}, sA, sA + (size_t)K * (M + 1) * 2 * TILE, nullptr,
-                                   nullptr, c.flush, M, true);
+            float* sW = sA + (size_t)K * (M + 1) * 2 * TILE;
+            if (c.cells > 0)
+                walk_tile<M, false>(g, P, lin, qa, qb, tq.y, PackedLoad{arr[f]}, LayKM{sA, sW, nullptr, nullptr, M + 1},
+                                    reinterpret_cast<char*>(sPiv + 6 * TILE), c.cells, c.flush, M);
+            else  // the walk's scratch does not fit beside three fields' moments
+                tile_moments<M, false>(g, P, tp.q, PackedLoad{arr[f]}, sA, sW, nullptr, nullptr, c.flush, M);
         }
         __syncthreads();
         tile_contract_multi<M>(K, sF, sPiv, slot);
@@ -1932,14 +1912,6 @@ __device__ __forceinline__ void adj_ring(const MapDev& g, const PivotRing& P, in
     }
 }
 
-// Shared memory of an adjoint tile: phases 1-2 use the moments A, W, Q, QW, the
-// pivot values, the primary-term sums and one m of H; phase 3 keeps only A (now h)
-// and puts the warps' row buffers where W and the rest were.
-template <int M>
-__host__ __device__ inline size_t bwd_tile_floats(int K) {
-    return bwd_tile_floats_rt(K, M);
-}
-
 // One adjoint tile (all three phases).  Called by every thread of the CTA.  With
 // SELF (self-pair subtraction) the subtracted diagonal adds, per bin k with
 // cdiag_k = sum_m Re C_m(k,k), -w_p Q^k(p) cdiag_k to a pivot and
@@ -1951,12 +1923,13 @@ __device__ __forceinline__ void bwd_tile(const MapDev& g, const MapCall& c, int 
     float* sW = sA + (size_t)K * (mr + 1) * 2 * TILE;
     float* sQ = sW + K * TILE;
     float* sQW = sQ + K * TILE;
-    float* sPiv = sQW + K * TILE;
+    float* sPiv = SELF ? sQW + K * TILE : sQ;
     float* sPrim = sPiv + 2 * TILE;
-    float* sHm = sPrim + TILE;                  // [K][K][2] one m at a time
-    float* sRow = sW;                           // [NWARPS][ROW], phase 3 only
+    char* scratch = reinterpret_cast<char*>(sPrim + TILE);
+    float* sHm = reinterpret_cast<float*>(scratch);   // phase 2: [K][K][2], one m at a time
+    float* sRow = reinterpret_cast<float*>(scratch);  // phase 3: [NWARPS][ROW]
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const size_t nfl = (size_t)K * (mr + 1) * 2 * TILE + 3 * (size_t)K * TILE;
+    const size_t nfl = tile_floats_rt(K, mr, SELF) - 2 * TILE;
 
     const int2 tq = g.tiles[tile];
     if (tq.x < 0 || tq.x >= g.nrings) {
@@ -1979,7 +1952,12 @@ __device__ __forceinline__ void bwd_tile(const MapDev& g, const MapCall& c, int 
     }
     __syncthreads();
     // phase 1: the tile's moments, exactly as in the forward
-    tile_moments<M, SELF>(g, P, qg, PackedLoad{c.wdw}, sA, sW, sQ, sQW, c.flush, mr);
+    if (g.lin[P.i])
+        walk_tile<M, SELF>(g, P, true, tile_slot(true, P.n_i, P.s_i, tq.y, lane & 15).q,
+                           tile_slot(true, P.n_i, P.s_i, tq.y, 16 + (lane & 15)).q, tq.y, PackedLoad{c.wdw},
+                           LayKM{sA, sW, sQ, sQW, mr + 1}, scratch, c.cells, c.flush, mr);
+    else
+        tile_moments<M, SELF>(g, P, qg, PackedLoad{c.wdw}, sA, sW, sQ, sQW, c.flush, mr);
     __syncthreads();
     // phase 2: h = H conj(a) per m, in place; primary term (1/2) sum Re[a h]
     for (int m = 0; m <= mr; ++m) {

@@ -39,11 +39,14 @@ struct tpcf_plan_s {
     std::vector<void*> allocs;  // everything freed by destroy
     MapDev map{};
     tpcf::CatDev cat{};
-    std::vector<int64_t> tile_off_h;  // map plans: first tile of each ring (host copy)
+    std::vector<int64_t> tile_off_h;   // map plans: first tile of each ring (host copy)
+    std::vector<int64_t> wtile_off_h;  // map plans: first walk tile of each ring
+    std::vector<unsigned char> lin_h;  // map plans: ring has linear walk tiles
     // launch configuration of the map pair kernels (defaults, or picked by the autotuner):
     // register variant (CTAs per SM the registers are sized for), CTAs per SM launched,
     // rings summed in registers per shared-memory flush
-    // and, for the forward, the tile layout (1: quarter-turn runs, 0: consecutive pivots)
+    // and, for the forward, a tile-layout choice that is kept for callers that store configurations
+    // (the layout follows from the ring, map_walk.cuh)
     struct Tune {
         int variant = 3, ctas = 0, flush = 8, quad = 0;
     } tune_fwd, tune_bwd;

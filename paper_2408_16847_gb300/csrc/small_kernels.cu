@@ -4,7 +4,8 @@
 
 namespace tpcf {
 
-// (w d, w) per point, so the pair loops read one 8-byte word per neighbour.
+// (w d, w) per point, so the pair loops read one 8-byte word per neighbour; a zero after
+// the last one (entries without a pixel point there).
 __global__ void pack_kernel(const float* __restrict__ delta, const float* __restrict__ w, float2* wdw,
                             int64_t n) {
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
@@ -12,6 +13,7 @@ __global__ void pack_kernel(const float* __restrict__ delta, const float* __rest
         const float wi = w[i];
         wdw[i] = make_float2(wi * delta[i], wi);
     }
+    if (blockIdx.x == 0 && threadIdx.x == 0) wdw[n] = make_float2(0.0f, 0.0f);
 }
 
 __global__ void zero_f32_kernel(float* p, int64_t n) {
@@ -140,6 +142,7 @@ __global__ void batch_pack_kernel(const BatchIO* __restrict__ io) {
         const float wi = b.w[i];
         b.wdw[i] = make_float2(wi * b.delta[i], wi);
     }
+    if (blockIdx.x == 0 && threadIdx.x == 0) b.wdw[b.npix] = make_float2(0.0f, 0.0f);
 }
 
 // Zeroes each plan's CTA slots and, when `with_grad`, its gradient.

@@ -38,8 +38,13 @@ struct MapDev {
     const int64_t* pair_off;    // [nrings] first (i, r) pair index of pivot ring i
     const float2* pair_A;       // [npairs] sin(theta_i - theta_r) as fp32 (hi, lo) from fp64
     const int2* pair_T;         // [npairs * (K+1)] edge offsets T_e in ring-r pixels
-    const int2* tiles;          // [ntiles] (ring, first pivot index in ring)
+    const int2* tiles;          // [ntiles] (ring, first pivot index in ring): 32 consecutive pivots
     int64_t ntiles;
+    const int2* wtiles;         // [nwtiles] (ring, first pivot or orbit): the walk's tiles (map_walk.cuh)
+    int64_t nwtiles;
+    const unsigned char* lin;   // [nrings] 1: linear walk tiles (every neighbour ring has n_i pixels)
+    const int* ring_reach;      // [nrings] pixels that a linear tile's rows reach beyond a pivot
+    const float4* rc;           // [2 * nrings] (s, s_lo, step, step_lo), (1/n, its lo, 2 n + shift, first)
     const double* E;            // [K+1] sin^2(theta_e / 2)
 };
 
@@ -82,7 +87,7 @@ struct MapCall {
     int flush;              // rings summed in registers before a shared-memory flush (tuned)
     int64_t tile_lo, tile_hi;  // tiles that can hold a pivot of [piv_lo, piv_hi)
     int norm;               // NORM_*: per-pivot normalisation of the moments before the contraction
-    int quad;               // forward tiles in the quarter-turn layout (tile_pivot)
+    int cells;              // cell table of the walk (map_walk.cuh); 0: the per-lane path
     int group;              // > 1: shared neighbour lists, one lane per run of `group` ring pixels
     const int2* gtiles;     // group > 1: tiles (ring, first run of the tile)
 };
@@ -119,18 +124,43 @@ constexpr int ROW = 512;  // floats per warp row buffer of the adjoint (wider ro
 
 // Shared memory (floats) of a map forward tile with runtime m_max mr: moments
 // A[k][m][re/im][32], W, Q, QW [k][32], the pivots' (w d, w).
-__host__ __device__ inline size_t tile_floats_rt(int K, int mr) {
-    return (size_t)K * (mr + 1) * 2 * TILE + 3 * (size_t)K * TILE + 2 * TILE;
+// (Q, QW: self-pair subtraction only.)
+__host__ __device__ inline size_t tile_floats_rt(int K, int mr, bool self) {
+    return (size_t)K * (mr + 1) * 2 * TILE + (self ? 3 : 1) * (size_t)K * TILE + 2 * TILE;
 }
 
-// Shared memory (floats) of a map adjoint tile: phases 1-2 use the moments, W, Q, QW,
-// the pivots, the primary-term sums and one m of H; phase 3 keeps the moments (then
-// h) and the warps' row buffers.
-__host__ __device__ inline size_t bwd_tile_floats_rt(int K, int mr) {
-    const size_t a = (size_t)K * (mr + 1) * 2 * TILE;
-    const size_t p12 = a + 3 * (size_t)K * TILE + 2 * TILE + TILE + (size_t)K * K * 2;
-    const size_t p3 = a + (size_t)NWARPS * ROW;
-    return p12 > p3 ? p12 : p3;
+// The shared-angle walk (map_walk.cuh).
+constexpr int WALK_CELLS = 4096;      // largest cell table (shared memory: 10 bytes per cell)
+constexpr int WALK_HEAD = 640;        // bytes of the small tables in front of it
+
+// Bytes between staged entries: up to eight pixel indices and the angle; an odd number of
+// 16-byte words, so that eight different entries fall in different banks.
+constexpr int WALK_STRIDE = 48;
+
+__host__ __device__ inline size_t walk_scratch_bytes(int nwarps, int cells) {
+    return WALK_HEAD + (size_t)cells * 10 + 16 + (size_t)nwarps * 32 * WALK_STRIDE;
+}
+
+// Cell table of the walk for a kernel with `base` other bytes of dynamic shared memory: the
+// largest that leaves room for two CTAs per SM (228 KB, 1 KB reserved per CTA and about 1 KB of
+// static tables), else the largest that fits one; 0 if none fits.
+inline int walk_pick_cells(size_t base, int nwarps) {
+    const size_t limit[2] = {114000, 231000};
+    for (int i = 0; i < 2; ++i)
+        for (int cells = WALK_CELLS; cells >= 256; cells /= 2)
+            if (base + walk_scratch_bytes(nwarps, cells) <= limit[i]) return cells;
+    return 0;
+}
+
+// Shared memory (bytes) of an adjoint tile with runtime m_max mr: the moments (then h), W,
+// Q and QW, the pivots' values, the primary-term sums, and one region used in turn by the
+// walk, by one m of H and by the warps' row buffers.
+__host__ __device__ inline size_t bwd_smem_bytes(int K, int mr, bool self, int cells) {
+    const size_t a = walk_scratch_bytes(NWARPS, cells), b = (size_t)K * K * 2 * sizeof(float),
+                 c = (size_t)NWARPS * ROW * sizeof(float);
+    size_t u = a > b ? a : b;
+    u = u > c ? u : c;
+    return (tile_floats_rt(K, mr, self) + TILE) * sizeof(float) + u;
 }
 
 // Device status bits.
