@@ -20,7 +20,7 @@ namespace tpcf {
 #define TPCF_DECL_MULTI(m)                                                                                    \
     cudaError_t map_fwd_multi_launch_m##m(const MapDev&, const MapCall&, const float2*, const float2*, int, \
                                           cudaStream_t);                                                  \
-    int map_fwd_multi_occupancy_m##m(int);
+    int map_fwd_multi_occupancy_m##m();
 TPCF_DECL_MULTI(0) TPCF_DECL_MULTI(1) TPCF_DECL_MULTI(2) TPCF_DECL_MULTI(3) TPCF_DECL_MULTI(4) TPCF_DECL_MULTI(5)
 TPCF_DECL_MULTI(6) TPCF_DECL_MULTI(7) TPCF_DECL_MULTI(8) TPCF_DECL_MULTI(9) TPCF_DECL_MULTI(10)
 TPCF_DECL_MULTI(11) TPCF_DECL_MULTI(12) TPCF_DECL_MULTI(13) TPCF_DECL_MULTI(14) TPCF_DECL_MULTI(15)
@@ -33,7 +33,7 @@ static const multi_fn kMulti[TPCF_MAX_M + 1] = {
     map_fwd_multi_launch_m8,  map_fwd_multi_launch_m9,  map_fwd_multi_launch_m10, map_fwd_multi_launch_m11,
     map_fwd_multi_launch_m12, map_fwd_multi_launch_m13, map_fwd_multi_launch_m14, map_fwd_multi_launch_m15,
     map_fwd_multi_launch_m16};
-static int (*const kMultiOcc[TPCF_MAX_M + 1])(int) = {
+static int (*const kMultiOcc[TPCF_MAX_M + 1])() = {
     map_fwd_multi_occupancy_m0,  map_fwd_multi_occupancy_m1,  map_fwd_multi_occupancy_m2,
     map_fwd_multi_occupancy_m3,  map_fwd_multi_occupancy_m4,  map_fwd_multi_occupancy_m5,
     map_fwd_multi_occupancy_m6,  map_fwd_multi_occupancy_m7,  map_fwd_multi_occupancy_m8,
@@ -41,12 +41,12 @@ static int (*const kMultiOcc[TPCF_MAX_M + 1])(int) = {
     map_fwd_multi_occupancy_m12, map_fwd_multi_occupancy_m13, map_fwd_multi_occupancy_m14,
     map_fwd_multi_occupancy_m15, map_fwd_multi_occupancy_m16};
 #define TPCF_DECL_M(m)                                                                         \
-    cudaError_t map_fwd_launch_m##m(const MapDev&, const MapCall&, int, int, cudaStream_t);    \
+    cudaError_t map_fwd_launch_m##m(const MapDev&, const MapCall&, int, cudaStream_t);         \
     cudaError_t map_fwd_tc_launch_m##m(const MapDev&, const MapCall&, int, cudaStream_t);      \
     int map_fwd_tc_occupancy_m##m(int, int);                                                  \
-    cudaError_t map_bwd_launch_m##m(const MapDev&, const MapCall&, int, int, cudaStream_t);    \
-    int map_fwd_occupancy_m##m(int, int, int);                                                \
-    int map_bwd_occupancy_m##m(int, int);
+    cudaError_t map_bwd_launch_m##m(const MapDev&, const MapCall&, int, cudaStream_t);         \
+    int map_fwd_occupancy_m##m();                                                             \
+    int map_bwd_occupancy_m##m();
 TPCF_DECL_M(0) TPCF_DECL_M(1) TPCF_DECL_M(2) TPCF_DECL_M(3) TPCF_DECL_M(4) TPCF_DECL_M(5)
 TPCF_DECL_M(6) TPCF_DECL_M(7) TPCF_DECL_M(8) TPCF_DECL_M(9) TPCF_DECL_M(10) TPCF_DECL_M(11)
 TPCF_DECL_M(12) TPCF_DECL_M(13) TPCF_DECL_M(14) TPCF_DECL_M(15) TPCF_DECL_M(16)
@@ -67,12 +67,12 @@ tpcf_status catalog_forward_multi(tpcf_plan_s* P, const float* const* d_delta, c
 tpcf_status noalloc_prepare(int dev);
 
 struct MLaunch {
-    cudaError_t (*fwd)(const MapDev&, const MapCall&, int, int, cudaStream_t);
+    cudaError_t (*fwd)(const MapDev&, const MapCall&, int, cudaStream_t);
     cudaError_t (*fwd_tc)(const MapDev&, const MapCall&, int, cudaStream_t);
     int (*fwd_tc_occ)(int, int);
-    cudaError_t (*bwd)(const MapDev&, const MapCall&, int, int, cudaStream_t);
-    int (*fwd_occ)(int, int, int);
-    int (*bwd_occ)(int, int);
+    cudaError_t (*bwd)(const MapDev&, const MapCall&, int, cudaStream_t);
+    int (*fwd_occ)();
+    int (*bwd_occ)();
 };
 #define TPCF_ROW_M(m) \
     {map_fwd_launch_m##m, map_fwd_tc_launch_m##m, map_fwd_tc_occupancy_m##m, map_bwd_launch_m##m, map_fwd_occupancy_m##m, map_bwd_occupancy_m##m}
@@ -82,9 +82,9 @@ static const MLaunch kLaunch[TPCF_MAX_M + 1] = {
     TPCF_ROW_M(12), TPCF_ROW_M(13), TPCF_ROW_M(14), TPCF_ROW_M(15), TPCF_ROW_M(16)};
 #undef TPCF_ROW_M
 
-// resident CTAs per SM of each register variant (used by the autotuner, tune.cu)
-int map_fwd_occupancy(int M, int K, int self, int variant) { return kLaunch[M].fwd_occ(K, self, variant); }
-int map_bwd_occupancy(int M, int K, int variant) { return kLaunch[M].bwd_occ(K, variant); }
+// resident CTAs per SM (used by the autotuner, tune.cu)
+int map_fwd_occupancy(int M) { return kLaunch[M].fwd_occ(); }
+int map_bwd_occupancy(int M) { return kLaunch[M].bwd_occ(); }
 // applies a configuration cached by the autotuner (tune.cu)
 void tune_from_cache(tpcf_plan_s* P);
 }  // namespace tpcf
@@ -181,12 +181,12 @@ static tpcf_status build_map(tpcf_plan_s* P, int64_t nside, cudaStream_t s) {
     g.K = K;
     g.M = P->M;
     g.npix = 12 * nside * nside;
-    int64_t *first, *pair_off, *tile_off, *wtile_off, *npairs_r, *ntiles_r, *nwtiles_r, *tot;
+    int64_t *first, *pair_off, *tile_off, *lin_off, *orb_off, *npairs_r, *ntiles_r, *nlin_r, *norb_r, *tot;
     int *npr, *shift;
     double *z, *sd, *th, *E, *theta;
     float *zf, *sf, *sf_lo, *rstep, *rstep_lo, *rinvn, *rinvn_lo;
     int2 *ring_range, *bin_range;
-    unsigned char* lin;  // the walk's ring classes (map_walk.cuh)
+    unsigned char* lin;  // ring classes (map_block.cuh)
     int* reach;
     float4* rc;
     TRY_CUDA(P->alloc(&first, nrings));
@@ -208,50 +208,60 @@ static tpcf_status build_map(tpcf_plan_s* P, int64_t nside, cudaStream_t s) {
     TRY_CUDA(P->alloc(&tile_off, nrings));
     TRY_CUDA(P->alloc(&npairs_r, nrings));
     TRY_CUDA(P->alloc(&ntiles_r, nrings));
-    TRY_CUDA(P->alloc(&wtile_off, nrings));
-    TRY_CUDA(P->alloc(&nwtiles_r, nrings));
+    TRY_CUDA(P->alloc(&lin_off, nrings));
+    TRY_CUDA(P->alloc(&orb_off, nrings));
+    TRY_CUDA(P->alloc(&nlin_r, nrings));
+    TRY_CUDA(P->alloc(&norb_r, nrings));
     TRY_CUDA(P->alloc(&lin, nrings));
     TRY_CUDA(P->alloc(&reach, nrings));
     TRY_CUDA(P->alloc(&rc, 2 * (size_t)nrings));
-    TRY_CUDA(P->alloc(&tot, 3));
+    TRY_CUDA(P->alloc(&tot, 4));
     TRY_CUDA(P->alloc(&E, K + 1));
     TRY_CUDA(P->alloc(&theta, K + 1));
     TRY_CUDA(cudaMemcpyAsync(theta, P->edges.data(), sizeof(double) * (K + 1), cudaMemcpyHostToDevice, s));
     edges_kernel<<<1, 64, 0, s>>>(K, theta, E);
     ring_table_kernel<<<n_blocks(nrings, 128), 128, 0, s>>>((int)nside, nrings, first, npr, shift, z, sd, th,
                                                             zf, sf, sf_lo, rstep, rstep_lo, rinvn, rinvn_lo, rc);
-    ring_range_kernel<<<n_blocks(nrings, 128), 128, 0, s>>>(nrings, K, th, sd, E, npr, shift, ring_range,
-                                                            bin_range, npairs_r, ntiles_r, nwtiles_r, lin, reach);
+    const int np = walk_np(P->M);
+    ring_range_kernel<<<n_blocks(nrings, 128), 128, 0, s>>>(nrings, K, th, sd, E, npr, ring_range, bin_range,
+                                                            npairs_r, ntiles_r, nlin_r, norb_r, np, lin, reach);
     exclusive_scan_kernel<<<1, 1024, 0, s>>>(npairs_r, pair_off, nrings, tot);
     exclusive_scan_kernel<<<1, 1024, 0, s>>>(ntiles_r, tile_off, nrings, tot + 1);
-    exclusive_scan_kernel<<<1, 1024, 0, s>>>(nwtiles_r, wtile_off, nrings, tot + 2);
+    exclusive_scan_kernel<<<1, 1024, 0, s>>>(nlin_r, lin_off, nrings, tot + 2);
+    exclusive_scan_kernel<<<1, 1024, 0, s>>>(norb_r, orb_off, nrings, tot + 3);
     TRY_CUDA(cudaGetLastError());
-    int64_t totals[3];
+    int64_t totals[4];
     TRY_CUDA(cudaMemcpyAsync(totals, tot, sizeof(totals), cudaMemcpyDeviceToHost, s));
     TRY_CUDA(cudaStreamSynchronize(s));
-    const int64_t npairs = totals[0], ntiles = totals[1], nwtiles = totals[2];
+    const int64_t npairs = totals[0], ntiles = totals[1], nlin = totals[2], norb = totals[3];
     P->tile_off_h.resize(nrings);
-    P->wtile_off_h.resize(nrings);
+    P->lin_off_h.resize(nrings + 1);
+    P->orb_off_h.resize(nrings + 1);
     P->lin_h.resize(nrings);
     TRY_CUDA(cudaMemcpy(P->tile_off_h.data(), tile_off, sizeof(int64_t) * nrings, cudaMemcpyDeviceToHost));
-    TRY_CUDA(cudaMemcpy(P->wtile_off_h.data(), wtile_off, sizeof(int64_t) * nrings, cudaMemcpyDeviceToHost));
+    TRY_CUDA(cudaMemcpy(P->lin_off_h.data(), lin_off, sizeof(int64_t) * nrings, cudaMemcpyDeviceToHost));
+    TRY_CUDA(cudaMemcpy(P->orb_off_h.data(), orb_off, sizeof(int64_t) * nrings, cudaMemcpyDeviceToHost));
+    P->lin_off_h[nrings] = nlin;
+    P->orb_off_h[nrings] = norb;
     TRY_CUDA(cudaMemcpy(P->lin_h.data(), lin, nrings, cudaMemcpyDeviceToHost));
     float2* pair_A;
-    int2 *pair_T, *tiles, *wtiles;
+    int2 *pair_T, *tiles, *lin_list, *orb_list;
     TRY_CUDA(P->alloc(&pair_A, npairs));
     TRY_CUDA(P->alloc(&pair_T, (size_t)npairs * (K + 1)));
     TRY_CUDA(P->alloc(&tiles, ntiles));
-    TRY_CUDA(P->alloc(&wtiles, nwtiles));
+    TRY_CUDA(P->alloc(&lin_list, nlin));
+    TRY_CUDA(P->alloc(&orb_list, norb));
     pair_table_kernel<<<n_blocks(npairs, 128), 128, 0, s>>>(nrings, K, pair_off, npairs, ring_range, th, sd,
                                                             npr, E, pair_A, pair_T);
-    tile_list_kernel<<<nrings, 128, 0, s>>>(nrings, tile_off, ntiles_r, nullptr, tiles);
-    tile_list_kernel<<<nrings, 128, 0, s>>>(nrings, wtile_off, nwtiles_r, lin, wtiles);
+    tile_list_kernel<<<nrings, 128, 0, s>>>(nrings, tile_off, ntiles_r, TILE, tiles);
+    tile_list_kernel<<<nrings, 128, 0, s>>>(nrings, lin_off, nlin_r, BT * np, lin_list);
+    tile_list_kernel<<<nrings, 128, 0, s>>>(nrings, orb_off, norb_r, TILE, orb_list);
     TRY_CUDA(cudaGetLastError());
     g.lin = lin;
     g.ring_reach = reach;
     g.rc = rc;
-    g.wtiles = wtiles;
-    g.nwtiles = nwtiles;
+    g.lin_list = lin_list;
+    g.orb_list = orb_list;
     g.ring_first = first;
     g.ring_n = npr;
     g.ring_shift = shift;
@@ -276,25 +286,28 @@ static tpcf_status build_map(tpcf_plan_s* P, int64_t nside, cudaStream_t s) {
     const MLaunch& L = kLaunch[P->M];
     const int self = (P->flags & TPCF_SELF_PAIRS_SUBTRACT) ? 1 : 0;
     const bool tc = (P->flags & TPCF_CONTRACT_TC) != 0;
-    int occ_f = tc ? L.fwd_tc_occ(K, self) : std::max(L.fwd_occ(K, self, 3), L.fwd_occ(K, self, 2));
-    int occ_b = std::max(L.bwd_occ(K, 3), L.bwd_occ(K, 2));
+    const int occ_f = tc ? L.fwd_tc_occ(K, self) : L.fwd_occ();
+    const int occ_b = L.bwd_occ();
     if (occ_f < 1 || occ_b < 1) {
         snprintf(g_last_error, sizeof(g_last_error), "kernel does not fit (K=%d, M=%d)", K, P->M);
         return TPCF_ERR_UNSUPPORTED;
     }
     // slots for the largest grid any configuration launches
-    P->fwd_grid = (int)std::min<int64_t>(g.nwtiles, (int64_t)P->num_sms * occ_f);
-    P->bwd_grid = (int)std::min<int64_t>(ntiles, (int64_t)P->num_sms * occ_b);
+    P->fwd_grid = P->num_sms * ((occ_f + 1) / 2 * 2);
+    P->bwd_grid = P->num_sms * ((occ_b + 1) / 2 * 2);
     P->tune_fwd.variant = P->tune_bwd.variant = 2;
-    P->tune_fwd.ctas = tc ? occ_f : L.fwd_occ(K, self, 2);
-    P->tune_bwd.ctas = L.bwd_occ(K, 2);
-    if (P->fwd_grid < 1) P->fwd_grid = 1;
-    if (P->bwd_grid < 1) P->bwd_grid = 1;
+    P->tune_fwd.ctas = (occ_f + 1) / 2;
+    P->tune_bwd.ctas = (occ_b + 1) / 2;
+    // workspace: a block per CTA, or (calls with few blocks) one per block, see block_call
+    P->ws_slots = (int)std::max<int64_t>(1, std::min<int64_t>(2 * std::max(P->fwd_grid, P->bwd_grid), nlin + (norb + 1) / 2));
+    P->fwd_grid = (int)std::min<int64_t>(P->fwd_grid, 8 * (int64_t)P->ws_slots);
+    P->ws_floats = block_floats(K, P->M, P->M, self != 0);
+    TRY_CUDA(P->alloc(&P->ws, P->ws_floats * P->ws_slots));
     P->nent = n_entries(K, P->M);
     TRY_CUDA(P->alloc(&P->wdw, g.npix + 1));  // and a zero after the last pixel
     TRY_CUDA(P->alloc(&P->slots, (size_t)P->fwd_grid * P->nent));
     TRY_CUDA(P->alloc(&P->sums, P->nent));
-    TRY_CUDA(P->alloc(&P->counter, 4));
+    TRY_CUDA(P->alloc(&P->counter, 4 + P->ws_slots));  // work counter (4 words), then finished parts per block
     TRY_CUDA(P->alloc(&P->status, 4));
     TRY_CUDA(P->alloc(&P->H, (size_t)(P->M + 1) * K * K * 2 + K));  // H, then cdiag (self-pair mode)
     TRY_CUDA(cudaMemsetAsync(P->status, 0, sizeof(int) * 4, s));
@@ -403,38 +416,62 @@ static int64_t ring_first_pixel(int64_t nside, int64_t ri) {  // 0-based ring
     return 12 * nside * nside - 2 * rr * (rr + 1);
 }
 
-// Tiles [*tlo, *thi) that can hold a pivot of [lo, hi).  Tiles of 32 consecutive pivots: those
-// of the range's pixels.  The walk's tiles: likewise on linear rings; on the others a
-// partial ring's pivots are spread over all of its tiles, so whole rings at the ends.
-static void tile_range(const tpcf_plan_s* P, int64_t lo, int64_t hi, int64_t* tlo, int64_t* thi, bool walk) {
+// Tiles [*tlo, *thi) of 32 consecutive pivots that hold the pivots [lo, hi).
+static void tile_range(const tpcf_plan_s* P, int64_t lo, int64_t hi, int64_t* tlo, int64_t* thi) {
     if (hi <= lo) {
         *tlo = *thi = 0;
         return;
     }
     const int64_t nside = P->map.nside;
     const int64_t ra = ring_of_pixel(nside, lo), rb = ring_of_pixel(nside, hi - 1);
-    const std::vector<int64_t>& off = walk ? P->wtile_off_h : P->tile_off_h;
-    *tlo = off[ra];
-    if (!walk || P->lin_h[ra]) *tlo += (lo - ring_first_pixel(nside, ra)) / TILE;
-    if (!walk || P->lin_h[rb])
-        *thi = off[rb] + (hi - 1 - ring_first_pixel(nside, rb)) / TILE + 1;
-    else
-        *thi = rb + 1 < (int64_t)off.size() ? off[rb + 1] : P->map.nwtiles;
+    *tlo = P->tile_off_h[ra] + (lo - ring_first_pixel(nside, ra)) / TILE;
+    *thi = P->tile_off_h[rb] + (hi - 1 - ring_first_pixel(nside, rb)) / TILE + 1;
 }
 
-static int launch_grid(const tpcf_plan_s* P, const tpcf_plan_s::Tune& t, int64_t ntiles, int cap) {
-    const int64_t g = std::min<int64_t>(ntiles, (int64_t)P->num_sms * t.ctas);
-    return (int)std::max<int64_t>(1, std::min<int64_t>(g, cap));
+// Blocks, parts and workspace of a forward over lin_list [lin_lo, lin_lo + nlin) and orb_list
+// [orb_lo, orb_lo + norb) (map_block.cuh); returns the grid.  Warp tiles go four to a block (one
+// per warp), or two if that leaves fewer than four blocks per CTA of a full grid; a call with
+// fewer than three blocks per CTA splits each by bins, if the workspace has a slot for each block.
+static int block_shape(const tpcf_plan_s* P, const tpcf_plan_s::Tune& t, int cap, MapCall* c) {
+    const int64_t full = (int64_t)P->num_sms * 2 * t.ctas;
+    auto blocks = [&](int tiles) { return c->nlin + (c->norb + tiles - 1) / tiles; };
+    c->tiles = BW;
+    while (c->tiles > 2 && blocks(c->tiles) < 4 * full) c->tiles /= 2;
+    const int64_t n = blocks(c->tiles);
+    c->parts = 1;
+    if (n < 3 * full && n <= P->ws_slots && n > 0)
+        c->parts = (int)std::min<int64_t>(std::min(8, P->K), (4 * full + n - 1) / n);
+    c->ws = P->ws;
+    c->ws_floats = P->ws_floats;
+    c->done = P->counter + 4;
+    int64_t grid = std::min<int64_t>(std::min<int64_t>(n * c->parts, full), cap);
+    if (c->parts == 1) grid = std::min<int64_t>(grid, P->ws_slots);
+    return (int)std::max<int64_t>(1, grid);
 }
+
+static void block_range(const tpcf_plan_s* P, int64_t lo, int64_t hi, MapCall* c) {
+    c->lin_list = P->map.lin_list;
+    c->orb_list = P->map.orb_list;
+    c->lin_lo = c->nlin = c->orb_lo = c->norb = 0;
+    if (hi <= lo) return;
+    const int64_t nside = P->map.nside, per = (int64_t)BT * walk_np(P->M);
+    const int64_t ra = ring_of_pixel(nside, lo), rb = ring_of_pixel(nside, hi - 1);
+    c->lin_lo = P->lin_off_h[ra] + (P->lin_h[ra] ? (lo - ring_first_pixel(nside, ra)) / per : 0);
+    const int64_t end = P->lin_h[rb] ? P->lin_off_h[rb] + (hi - 1 - ring_first_pixel(nside, rb)) / per + 1
+                                     : P->lin_off_h[rb];
+    c->nlin = std::max<int64_t>(0, end - c->lin_lo);
+    c->orb_lo = P->orb_off_h[ra];  // a partial ring's pivots are spread over all of its warp tiles
+    c->norb = P->orb_off_h[rb + 1] - c->orb_lo;
+}
+
+// Ints of P->counter a launch needs zeroed: the work counter, and the blocks' finished parts.
+static int n_counters(const tpcf_plan_s* P, const MapCall& c) { return 4 + (c.parts > 1 ? P->ws_slots : 0); }
 
 // group > 1: shared neighbour lists over P->gtiles (tpcf_forward_grouped).
 static tpcf_status map_forward(tpcf_plan_s* P, const float* d_delta, const float* d_w, int64_t lo, int64_t hi,
                                double* d_zeta, double* d_norm, double* d_sums, cudaStream_t s, int group = 1) {
     const MapDev& g = P->map;
-    pack_kernel<<<P->num_sms * 8, 256, 0, s>>>(d_delta, d_w, P->wdw, g.npix);
-    P->launches += 4;  // pack, forward, reduce, finalize
-    TRY_CUDA(cudaMemsetAsync(P->slots, 0, sizeof(double) * (size_t)P->fwd_grid * P->nent, s));
-    TRY_CUDA(cudaMemsetAsync(P->counter, 0, sizeof(int), s));
+    P->launches += 4;  // prep, forward, reduce, finalize
     MapCall c{};
     c.wdw = P->wdw;
     c.piv_lo = lo;
@@ -445,20 +482,24 @@ static tpcf_status map_forward(tpcf_plan_s* P, const float* d_delta, const float
     c.self_subtract = (P->flags & TPCF_SELF_PAIRS_SUBTRACT) ? 1 : 0;
     c.norm = norm_of_flags(P->flags);
     c.flush = P->tune_fwd.flush;
-    if (group > 1) {  // every run tile; those without a pivot in range return at once
+    c.cells = LIN_CELLS;
+    if (group > 1) {  // every run's block; those without a pivot in range return at once
         c.group = group;
-        c.gtiles = P->gtiles;
-        c.tile_lo = 0;
-        c.tile_hi = P->ngtiles;
+        c.lin_list = P->gtiles;
+        c.orb_list = P->gtiles + P->nglin;
+        c.nlin = P->nglin;
+        c.norb = P->ngorb;
     } else {
-        tile_range(P, lo, hi, &c.tile_lo, &c.tile_hi, true);
+        block_range(P, lo, hi, &c);
     }
-    const int grid = launch_grid(P, P->tune_fwd, c.tile_hi - c.tile_lo, P->fwd_grid);
+    const int grid = block_shape(P, P->tune_fwd, P->fwd_grid, &c);
+    fwd_prep_kernel<<<P->num_sms * 8, 256, 0, s>>>(d_delta, d_w, P->wdw, g.npix, P->slots, (int64_t)grid * P->nent,
+                                                   P->counter, n_counters(P, c));
     if (P->flags & TPCF_CONTRACT_TC)
         TRY_CUDA(kLaunch[P->M].fwd_tc(g, c, grid, s));
     else
-        TRY_CUDA(kLaunch[P->M].fwd(g, c, grid, P->tune_fwd.variant, s));
-    reduce_slots_kernel<<<n_blocks(P->nent, 128), 128, 0, s>>>(P->slots, P->fwd_grid, P->nent, P->sums);
+        TRY_CUDA(kLaunch[P->M].fwd(g, c, grid, s));
+    reduce_slots_kernel<<<n_blocks(P->nent, 32), REDUCE_THREADS, 0, s>>>(P->slots, grid, P->nent, P->sums);
     const int nout = (P->M + 1) * P->K * P->K;
     finalize_kernel<<<n_blocks(nout, 128), 128, 0, s>>>(P->sums, P->K, P->M, c.self_subtract, 1.0, d_zeta,
                                                         d_norm, d_sums);
@@ -480,15 +521,20 @@ extern "C" tpcf_status tpcf_forward_grouped(tpcf_plan plan, const float* d_delta
     plan->last_stream = s;
     if (group == 1) return map_forward(plan, d_delta, d_w, pivot_begin, pivot_end, d_zeta, d_norm, d_sums, s);
     tpcf_plan_s* P = plan;
-    if (P->ggroup != group) {  // the tile list of this run length: ceil(ceil(n_i / group) / 32) per ring
+    if (P->ggroup != group) {  // the blocks of this run length
         const int64_t nside = P->map.nside;
-        std::vector<int2> t;
+        std::vector<int2> t, orb;
         for (int r = 0; r < P->map.nrings; ++r) {
             const int64_t ri = r + 1;
             const int64_t n = ri < nside ? 4 * ri : (ri <= 3 * nside ? 4 * nside : 4 * (4 * nside - ri));
             const int64_t ng = (n + group - 1) / group;
-            for (int64_t f = 0; f < ng; f += TILE) t.push_back(make_int2(r, (int)f));
+            if (P->lin_h[r])
+                for (int64_t f = 0; f < ng; f += BT * walk_np(P->M)) t.push_back(make_int2(r, (int)f));
+            else
+                for (int64_t f = 0; f < ng; f += TILE) orb.push_back(make_int2(r, (int)f));
         }
+        const int64_t nglin = (int64_t)t.size();
+        t.insert(t.end(), orb.begin(), orb.end());
         if ((int64_t)t.size() > P->gtiles_cap) {
             int2* buf = nullptr;
             TRY_CUDA(P->alloc(&buf, t.size()));
@@ -497,7 +543,8 @@ extern "C" tpcf_status tpcf_forward_grouped(tpcf_plan plan, const float* d_delta
         }
         TRY_CUDA(cudaMemcpyAsync(P->gtiles, t.data(), sizeof(int2) * t.size(), cudaMemcpyHostToDevice, s));
         TRY_CUDA(cudaStreamSynchronize(s));
-        P->ngtiles = (int64_t)t.size();
+        P->nglin = nglin;
+        P->ngorb = (int64_t)t.size() - nglin;
         P->ggroup = group;
     }
     return map_forward(P, d_delta, d_w, pivot_begin, pivot_end, d_zeta, d_norm, d_sums, s, group);
@@ -541,30 +588,30 @@ extern "C" tpcf_status tpcf_forward_multi(tpcf_plan plan, const float* d_delta_a
     const int K = P->K, M = P->M;
     const int nent = n_entries_multi(K, M);
     if (!P->wdw_b) {
-        const int occ = kMultiOcc[M](K);
-        if (occ < 1) {
+        // the three fields' moments of one tile have to fit an SM (as the catalogue's must)
+        if (((size_t)3 * (K * (M + 1) * 2 + K) * TILE + 6 * TILE) * sizeof(float) > 232448 || kMultiOcc[M]() < 1) {
             snprintf(g_last_error, sizeof(g_last_error),
                      "tpcf_forward_multi: three fields' moments (K=%d, m_max=%d) do not fit in shared memory", K, M);
             return TPCF_ERR_UNSUPPORTED;
         }
-        const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(g.nwtiles, (int64_t)P->num_sms * occ));
+        const int grid = (int)std::min<int64_t>(P->num_sms * kMultiOcc[M](), P->fwd_grid);
         float2 *b, *c;
         double *sl, *su;
         TRY_CUDA(P->alloc(&b, g.npix + 1));
         TRY_CUDA(P->alloc(&c, g.npix + 1));
         TRY_CUDA(P->alloc(&sl, (size_t)grid * nent));
         TRY_CUDA(P->alloc(&su, (size_t)nent));
+        float* w3;
+        TRY_CUDA(P->alloc(&w3, 3 * P->ws_floats * P->ws_slots));
+        P->ws3 = w3;
         P->wdw_c = c;
         P->mslots = sl;
         P->msums = su;
         P->multi_grid = grid;
         P->wdw_b = b;
     }
-    pack_kernel<<<P->num_sms * 8, 256, 0, s>>>(d_delta_a, d_w_a, P->wdw, g.npix);
     pack_kernel<<<P->num_sms * 8, 256, 0, s>>>(d_delta_b, d_w_b, P->wdw_b, g.npix);
     pack_kernel<<<P->num_sms * 8, 256, 0, s>>>(d_delta_c, d_w_c, P->wdw_c, g.npix);
-    TRY_CUDA(cudaMemsetAsync(P->mslots, 0, sizeof(double) * (size_t)P->multi_grid * nent, s));
-    TRY_CUDA(cudaMemsetAsync(P->counter, 0, sizeof(int), s));
     MapCall c{};
     c.wdw = P->wdw;
     c.piv_lo = pivot_begin;
@@ -573,13 +620,18 @@ extern "C" tpcf_status tpcf_forward_multi(tpcf_plan plan, const float* d_delta_a
     c.counter = P->counter;
     c.status = P->status;
     c.flush = P->tune_fwd.flush;
-    tile_range(P, pivot_begin, pivot_end, &c.tile_lo, &c.tile_hi, true);
-    const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(c.tile_hi - c.tile_lo, P->multi_grid));
+    c.cells = LIN_CELLS;
+    block_range(P, pivot_begin, pivot_end, &c);
+    const int grid = std::min(block_shape(P, P->tune_fwd, P->fwd_grid, &c), P->multi_grid);
+    c.ws = P->ws3;
+    c.ws_floats = 3 * P->ws_floats;
+    fwd_prep_kernel<<<P->num_sms * 8, 256, 0, s>>>(d_delta_a, d_w_a, P->wdw, g.npix, P->mslots, (int64_t)grid * nent,
+                                                   P->counter, n_counters(P, c));
     TRY_CUDA(kMulti[M](g, c, P->wdw_b, P->wdw_c, grid, s));
-    reduce_slots_kernel<<<n_blocks(nent, 128), 128, 0, s>>>(P->mslots, P->multi_grid, nent, P->msums);
+    reduce_slots_kernel<<<n_blocks(nent, 32), REDUCE_THREADS, 0, s>>>(P->mslots, grid, nent, P->msums);
     const int nout = (M + 1) * K * K;
     finalize_full_kernel<<<n_blocks(nout, 128), 128, 0, s>>>(P->msums, K, M, d_zeta, d_norm, d_sums);
-    P->launches += 6;  // three packs, the pair kernel, reduce, finalize
+    P->launches += 6;  // prep and two packs, the pair kernel, reduce, finalize
     TRY_CUDA(cudaGetLastError());
     return TPCF_OK;
 }
@@ -598,7 +650,7 @@ extern "C" tpcf_status tpcf_count_pairs(tpcf_plan plan, const float* d_w, int64_
     plan->launches += 2;
     TRY_CUDA(cudaMemsetAsync(d_counts, 0, 3 * sizeof(int64_t), s));
     int64_t tlo, thi;
-    tile_range(plan, pivot_begin, pivot_end, &tlo, &thi, false);
+    tile_range(plan, pivot_begin, pivot_end, &tlo, &thi);
     TRY_CUDA(map_count_launch(g, plan->wdw, pivot_begin, pivot_end, tlo, thi, (unsigned long long*)d_counts,
                               plan->num_sms * 4, s));
     return TPCF_OK;
@@ -607,13 +659,8 @@ extern "C" tpcf_status tpcf_count_pairs(tpcf_plan plan, const float* d_w, int64_
 static tpcf_status map_backward(tpcf_plan_s* P, const float* d_delta, const float* d_w, int64_t lo, int64_t hi,
                                 const double* d_norm, const double* d_dL, float* d_grad, cudaStream_t s) {
     const MapDev& g = P->map;
-    pack_kernel<<<P->num_sms * 8, 256, 0, s>>>(d_delta, d_w, P->wdw, g.npix);
-    const int nout = (P->M + 1) * P->K * P->K;
     const int self = (P->flags & TPCF_SELF_PAIRS_SUBTRACT) ? 1 : 0;
-    adjoint_prep_kernel<<<n_blocks(nout, 128), 128, 0, s>>>(d_dL, d_norm, P->K, P->M, P->H, self);
-    zero_f32_kernel<<<P->num_sms * 8, 256, 0, s>>>(d_grad, g.npix);
-    P->launches += 4;  // pack, prep, zero, adjoint
-    TRY_CUDA(cudaMemsetAsync(P->counter, 0, sizeof(int), s));
+    P->launches += 2;  // prep, adjoint
     MapCall c{};
     c.wdw = P->wdw;
     c.piv_lo = lo;
@@ -624,9 +671,19 @@ static tpcf_status map_backward(tpcf_plan_s* P, const float* d_delta, const floa
     c.grad = d_grad;
     c.self_subtract = self;
     c.flush = P->tune_bwd.flush;
-    tile_range(P, lo, hi, &c.tile_lo, &c.tile_hi, false);
-    const int grid = launch_grid(P, P->tune_bwd, c.tile_hi - c.tile_lo, P->bwd_grid);
-    TRY_CUDA(kLaunch[P->M].bwd(g, c, grid, P->tune_bwd.variant, s));
+    c.cells = LIN_CELLS;
+    block_range(P, lo, hi, &c);
+    const int grid = block_shape(P, P->tune_bwd, P->bwd_grid, &c);
+    bwd_prep_kernel<<<P->num_sms * 8, 256, 0, s>>>(d_delta, d_w, P->wdw, d_grad, g.npix, d_dL, d_norm, P->K, P->M, P->H,
+                                                   self, P->counter, n_counters(P, c));
+    c.step = c.parts > 1 ? 1 : 0;
+    TRY_CUDA(kLaunch[P->M].bwd(g, c, grid, s));
+    if (c.step == 1) {  // the blocks' h are in the workspace: the neighbour legs, again in parts
+        TRY_CUDA(cudaMemsetAsync(P->counter, 0, sizeof(int), s));
+        c.step = 2;
+        TRY_CUDA(kLaunch[P->M].bwd(g, c, grid, s));
+        P->launches += 1;
+    }
     return TPCF_OK;
 }
 

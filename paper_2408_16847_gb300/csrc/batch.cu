@@ -55,12 +55,11 @@ namespace {
 struct Group {
     int M = 0;
     std::vector<int> members;  // indices into the batch's plan list
-    BatchItem* d_items = nullptr;    // forward: the walk's tiles
-    BatchItem* d_items_b = nullptr;  // adjoint: tiles of 32 consecutive pivots
-    long long total_tiles = 0;
+    BatchItem* d_items = nullptr;
     size_t fwd_smem = 0, bwd_smem = 0;
-    int fwd_cells = 0, bwd_cells = 0;  // cell tables of the walk
-    long long total_wtiles = 0;
+    long long total_blocks = 0;  // work items of a pass
+    float* ws = nullptr;         // workspace: one block per CTA
+    size_t ws_floats = 0;
     int fwd_grid = 0, bwd_grid = 0;
 };
 }  // namespace
@@ -108,11 +107,11 @@ static tpcf_status record(tpcf_batch_s* B, int num_sms, int max_nent, int max_no
     TRY_CUDA(cudaMemsetAsync(B->d_counters, 0, sizeof(unsigned long long) * 2 * B->groups.size(), s));
     for (size_t gi = 0; gi < B->groups.size(); ++gi) {
         const Group& G = B->groups[gi];
-        TRY_CUDA(kBatch[G.M].fwd(G.d_items, (int)G.members.size(), G.total_wtiles, B->d_counters + 2 * gi,
+        TRY_CUDA(kBatch[G.M].fwd(G.d_items, (int)G.members.size(), G.total_blocks, B->d_counters + 2 * gi,
                                  G.fwd_smem, G.fwd_grid, s));
         B->kernels += 1;
     }
-    batch_reduce_kernel<<<dim3(n_blocks(max_nent, 128), n), 128, 0, s>>>(B->d_io);
+    batch_reduce_kernel<<<dim3(n_blocks(max_nent, 32), n), REDUCE_THREADS, 0, s>>>(B->d_io);
     batch_finalize_kernel<<<dim3(n_blocks(max_nout, 128), n), 128, 0, s>>>(B->d_io);
     B->kernels += 2;
     if (B->with_bwd) {
@@ -120,7 +119,7 @@ static tpcf_status record(tpcf_batch_s* B, int num_sms, int max_nent, int max_no
         B->kernels += 1;
         for (size_t gi = 0; gi < B->groups.size(); ++gi) {
             const Group& G = B->groups[gi];
-            TRY_CUDA(kBatch[G.M].bwd(G.d_items_b, (int)G.members.size(), G.total_tiles, B->d_counters + 2 * gi + 1,
+            TRY_CUDA(kBatch[G.M].bwd(G.d_items, (int)G.members.size(), G.total_blocks, B->d_counters + 2 * gi + 1,
                                      G.bwd_smem, G.bwd_grid, s));
             B->kernels += 1;
         }
@@ -148,20 +147,10 @@ static tpcf_status batch_build(tpcf_batch_s* B, const tpcf_plan* plans, const fl
     std::vector<BatchIO> io(n);
     std::vector<int> grid_of(n, 0);
     for (Group& G : B->groups) {
-        size_t fwd_base = 0, bwd_base = 0;
-        for (int i : G.members) {
-            const tpcf_plan P = plans[i];
-            fwd_base = std::max(fwd_base, tile_floats_rt(P->K, P->M, true) * sizeof(float));
-            bwd_base = std::max(bwd_base, (tile_floats_rt(P->K, P->M, false) + TILE) * sizeof(float));
-        }
-        G.fwd_cells = walk_pick_cells(fwd_base, NWARPS);
-        G.bwd_cells = walk_pick_cells(bwd_base, NWARPS);
-        for (int i : G.members) {
-            const tpcf_plan P = plans[i];
-            G.fwd_smem = std::max(G.fwd_smem, tile_floats_rt(P->K, P->M, true) * sizeof(float) +
-                                                  walk_scratch_bytes(NWARPS, G.fwd_cells));
-            G.bwd_smem = std::max(G.bwd_smem, bwd_smem_bytes(P->K, P->M, false, G.bwd_cells));
-        }
+        for (int i : G.members)
+            G.ws_floats = std::max(G.ws_floats, block_floats(plans[i]->K, plans[i]->M, G.M, true));
+        G.bwd_smem = adj_smem_bytes(G.M);
+        G.fwd_smem = block_smem_bytes(G.M);
         const int of = kBatch[G.M].fwd_occ(G.fwd_smem);
         TRY_CUDA(cudaGetLastError());
         if (of < 1) {
@@ -178,6 +167,7 @@ static tpcf_status batch_build(tpcf_batch_s* B, const tpcf_plan* plans, const fl
             }
             G.bwd_grid = ob * num_sms;
         }
+        TRY_CUDA(B->alloc(&G.ws, G.ws_floats * std::max(G.fwd_grid, G.bwd_grid)));
         for (int i : G.members) grid_of[i] = G.fwd_grid;
     }
     int max_nent = 0, max_nout = 0;
@@ -208,8 +198,8 @@ static tpcf_status batch_build(tpcf_batch_s* B, const tpcf_plan* plans, const fl
     TRY_CUDA(B->alloc(&B->d_counters, 2 * B->groups.size()));
 
     for (Group& G : B->groups) {
-        std::vector<BatchItem> items, items_b;
-        long long t0 = 0, t0_b = 0;
+        std::vector<BatchItem> items;
+        long long t0 = 0;
         for (int i : G.members) {
             const tpcf_plan P = plans[i];
             BatchItem it{};
@@ -226,24 +216,23 @@ static tpcf_status batch_build(tpcf_batch_s* B, const tpcf_plan* plans, const fl
             it.c.grad = io[i].grad;
             it.c.self_subtract = io[i].self_subtract;
             it.c.flush = P->tune_fwd.flush;
-            it.c.cells = G.fwd_cells;
-            it.c.tile_lo = 0;
-            it.c.tile_hi = P->map.nwtiles;
+            // forward: the plan's linear blocks, then its other rings' warp tiles, two to a block
+            it.c.cells = LIN_CELLS;
+            it.c.lin_list = P->map.lin_list;
+            it.c.orb_list = P->map.orb_list;
+            it.c.nlin = P->lin_off_h.back();
+            it.c.norb = P->orb_off_h.back();
+            it.c.tiles = 2;
+            it.c.parts = 1;
+            it.c.ws = G.ws;
+            it.c.ws_floats = G.ws_floats;
             it.tile0 = t0;
-            t0 += P->map.nwtiles;
+            t0 += it.c.nlin + (it.c.norb + it.c.tiles - 1) / it.c.tiles;
             items.push_back(it);
-            it.c.cells = G.bwd_cells;
-            it.c.tile_hi = P->map.ntiles;
-            it.tile0 = t0_b;
-            t0_b += P->map.ntiles;
-            items_b.push_back(it);
         }
-        G.total_wtiles = t0;
-        G.total_tiles = t0_b;
+        G.total_blocks = t0;
         TRY_CUDA(B->alloc(&G.d_items, items.size()));
         TRY_CUDA(cudaMemcpy(G.d_items, items.data(), sizeof(BatchItem) * items.size(), cudaMemcpyHostToDevice));
-        TRY_CUDA(B->alloc(&G.d_items_b, items_b.size()));
-        TRY_CUDA(cudaMemcpy(G.d_items_b, items_b.data(), sizeof(BatchItem) * items_b.size(), cudaMemcpyHostToDevice));
     }
 
     TRY_CUDA(cudaStreamCreateWithFlags(&B->cap, cudaStreamNonBlocking));

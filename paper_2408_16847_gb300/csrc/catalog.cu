@@ -429,7 +429,7 @@ tpcf_status catalog_forward_multi(tpcf_plan_s* P, const float* const* d_delta, c
     c.counter = P->counter;
     c.status = P->status;
     TRY_CUDA(kCat[M].multi(g, c, P->wdw_b, P->wdw_c, P->multi_grid, s));
-    reduce_slots_kernel<<<(nent + 127) / 128, 128, 0, s>>>(P->mslots, P->multi_grid, nent, P->msums);
+    reduce_slots_kernel<<<(nent + 31) / 32, REDUCE_THREADS, 0, s>>>(P->mslots, P->multi_grid, nent, P->msums);
     const int nout = (M + 1) * K * K;
     finalize_full_kernel<<<(nout + 127) / 128, 128, 0, s>>>(P->msums, K, M, d_zeta, d_norm, d_sums);
     P->launches += 6;  // three packs, the pair kernel, reduce, finalize
@@ -454,7 +454,7 @@ tpcf_status catalog_forward(tpcf_plan_s* P, const float* d_delta, const float* d
     c.self_subtract = (P->flags & TPCF_SELF_PAIRS_SUBTRACT) ? 1 : 0;
     c.norm = norm_of_flags(P->flags);
     TRY_CUDA(kCat[P->M].fwd(g, c, P->fwd_grid, s));
-    reduce_slots_kernel<<<(P->nent + 127) / 128, 128, 0, s>>>(P->slots, P->fwd_grid, P->nent, P->sums);
+    reduce_slots_kernel<<<(P->nent + 31) / 32, REDUCE_THREADS, 0, s>>>(P->slots, P->fwd_grid, P->nent, P->sums);
     const int nout = (P->M + 1) * P->K * P->K;
     finalize_kernel<<<(nout + 127) / 128, 128, 0, s>>>(P->sums, P->K, P->M, c.self_subtract, 1.0, d_zeta, d_norm,
                                                        d_sums);

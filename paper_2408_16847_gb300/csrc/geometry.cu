@@ -85,14 +85,15 @@ __device__ int2 ring_window(const double* th, int nrings, int i, double E) {
     return make_int2(rlo, lo);
 }
 
-// Also the class of each ring for the walk (map_walk.cuh): linear when all its neighbour
+// Also the class of each ring (map_block.cuh): linear when it is long enough, all its neighbour
 // rings have its own pixel count and the outer edge leaves part of each of them out (both
 // decided at the ends of the window: the pixel count and the sine of the colatitude rise and
 // fall once from pole to pole); reach bounds how far, in pixels, a linear tile's rows extend
 // beyond a pivot (offsets of at most T plus rounding).
 __global__ void ring_range_kernel(int nrings, int K, const double* th, const double* s, const double* E,
-                                  const int* npr, const int* shift, int2* ring_range, int2* bin_range,
-                                  int64_t* npairs, int64_t* ntiles, int64_t* nwtiles, unsigned char* lin, int* reach) {
+                                  const int* npr, int2* ring_range, int2* bin_range,
+                                  int64_t* npairs, int64_t* ntiles, int64_t* nlin, int64_t* norb, int np,
+                                  unsigned char* lin, int* reach) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= nrings) return;
     const int2 rr = ring_window(th, nrings, i, E[K]);
@@ -102,11 +103,11 @@ __global__ void ring_range_kernel(int nrings, int K, const double* th, const dou
     const int n = npr[i];
     ntiles[i] = (n + TILE - 1) / TILE;
     const double q = E[K] / (s[i] * fmin(s[rr.x], s[rr.y]));
-    const bool same = npr[rr.x] == n && npr[rr.y] == n && q <= 1.0;
+    const bool same = npr[rr.x] == n && npr[rr.y] == n && q <= 1.0 && n >= LIN_MIN;
     lin[i] = same ? 1 : 0;
     reach[i] = same ? (int)(n / M_PI * asin(sqrt(q))) + 4 : n;
-    const int norb = shift[i] ? ((n >> 2) + 1) >> 1 : (n >> 3) + 1;  // orbit_count(n, shift)
-    nwtiles[i] = same ? (n + TILE - 1) / TILE : (norb + TILE / 8 - 1) / (TILE / 8);
+    nlin[i] = same ? (n + BT * np - 1) / (BT * np) : 0;
+    norb[i] = same ? 0 : (n / np + TILE - 1) / TILE;
 }
 
 // Exclusive prefix sum of n int64 values by one block (n is at most 4 * 8192 - 1).
@@ -178,16 +179,14 @@ __global__ void pair_table_kernel(int nrings, int K, const int64_t* pair_off, in
     }
 }
 
-// lin: NULL for tiles of 32 consecutive pivots, else the walk's tiles (four orbits each on
-// rings that are not linear).
-__global__ void tile_list_kernel(int nrings, const int64_t* tile_off, const int64_t* ntiles_ring,
-                                 const unsigned char* lin, int2* tiles) {
+// tiles[o .. o + ntiles_ring[i]) of ring i: (i, 0), (i, step), (i, 2 step), ...
+__global__ void tile_list_kernel(int nrings, const int64_t* tile_off, const int64_t* ntiles_ring, int step,
+                                 int2* tiles) {
     const int i = blockIdx.x;
     if (i >= nrings) return;
     const int64_t o = tile_off[i];
     const int64_t nt = ntiles_ring[i];
-    const int per = lin == nullptr || lin[i] ? TILE : TILE / 8;
-    for (int64_t t = threadIdx.x; t < nt; t += blockDim.x) tiles[o + t] = make_int2(i, (int)(t * per));
+    for (int64_t t = threadIdx.x; t < nt; t += blockDim.x) tiles[o + t] = make_int2(i, (int)(t * step));
 }
 
 __global__ void edges_kernel(int K, const double* theta, double* E) {

@@ -61,12 +61,6 @@ __device__ __forceinline__ void red_add_f32(double* p, float x) {
     atomicAdd(p, d);  // result unused: a reduction, no wait
 }
 
-__device__ __forceinline__ long long floordiv_ll(long long a, long long b) {
-    long long q = a / b;
-    if ((a % b) != 0 && a < 0) --q;
-    return q;
-}
-
 // Position of the lane's pivot in units of ring-r pixels: c = cint + crem / den,
 // so that pixel p of ring r is at longitude offset o = p - c pixels from the pivot.
 struct LaneC {
@@ -105,6 +99,26 @@ __device__ __forceinline__ LaneC lane_c(int q, int s_i, int n_i, int s_r, int n_
     return c;
 }
 
+// The same in 32 bits, for pivots in the first half of their ring: n_r (2 q + 1) <= 16 nside^2 < 2^31.
+__device__ __forceinline__ LaneC lane_c32(int q, int s_i, int n_i, int s_r, int n_r) {
+    const int num = n_r * (2 * q + s_i) - s_r * n_i, den = 2 * n_i;
+    int ci = (int)floorf(__fdividef((float)num, (float)den));
+    int rem = num - ci * den;
+    if (rem < 0) {
+        --ci;
+        rem += den;
+    } else if (rem >= den) {
+        ++ci;
+        rem -= den;
+    }
+    LaneC c;
+    c.cint = ci;
+    c.crem = rem;
+    c.den = den;
+    c.cfrac = __fdiv_rn((float)rem, (float)den);
+    return c;
+}
+
 // Exact (FP64) quarter squared chord of pixel p of ring r about the pivot:
 // f = sin^2((theta_r - theta_i)/2) + s_i s_r sin^2(pi o / n_r).  Only evaluated for
 // the rare edge pixels whose fp32 position is ambiguous, so the context holds the
@@ -140,6 +154,35 @@ __device__ __forceinline__ int neg_edge(const LaneC& c, int2 T, double Ee, const
     if (fabsf(y - ry) > AMBIGUITY) return base + (int)floorf(y);
     const int ps = base + (int)ry;
     return (exact_f(x.th_i, x.th_r, x.s_i, x.s_r, x.n_r, c.cint, c.crem, c.den, ps) >= Ee) ? ps : ps - 1;
+}
+
+// The same with the FP64 values of the rare ambiguous edges read only when needed: whether the
+// pixel p lies at or beyond edge k + e of rings (i, r).
+struct LazyEdge {
+    const MapDev& g;
+    int i, r, k;
+    __device__ __forceinline__ bool beyond(const LaneC& c, int p, int e) const {
+        return exact_f(g.ring_th[i], g.ring_th[r], g.ring_s[i], g.ring_s[r], g.ring_n[r], c.cint, c.crem, c.den, p) >=
+               g.E[k + e];
+    }
+};
+
+__device__ __forceinline__ int pos_edge(const LaneC& c, int2 T, const LazyEdge& x, int e) {
+    const float y = c.cfrac + __int_as_float(T.y);
+    const float ry = rintf(y);
+    const int base = c.cint + T.x;
+    if (fabsf(y - ry) > AMBIGUITY) return base + (int)ceilf(y);
+    const int ps = base + (int)ry;
+    return x.beyond(c, ps, e) ? ps : ps + 1;
+}
+
+__device__ __forceinline__ int neg_edge(const LaneC& c, int2 T, const LazyEdge& x, int e) {
+    const float y = c.cfrac - __int_as_float(T.y);
+    const float ry = rintf(y);
+    const int base = c.cint - T.x;
+    if (fabsf(y - ry) > AMBIGUITY) return base + (int)floorf(y);
+    const int ps = base + (int)ry;
+    return x.beyond(c, ps, e) ? ps : ps - 1;
 }
 
 // Warp-uniform description of neighbour ring r for pivot ring i.
@@ -221,8 +264,6 @@ __device__ __forceinline__ Fold fold_angle(float cph, float sph) {
     return f;
 }
 
-__device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
-
 // acc[m] += (wc cos(m phi), ws sin(m phi)), m = 0..M, from the folded angle.
 // mr <= M: the multipoles computed (a runtime m_max below the compiled one).
 template <int M>
@@ -249,50 +290,6 @@ template <int M>
 __device__ __forceinline__ void harmonics(float2 (&acc)[M + 1], float cph, float sph, float wc, float ws,
                                           int mr = M) {
     harmonicsf<M>(acc, fold_angle(cph, sph), wc, ws, mr);
-}
-
-// The same for two pixels a and b at once (two independent chains for
-// instruction-level parallelism), from their folded angles.
-template <int M>
-__device__ __forceinline__ void harmonics2f(float2 (&acc)[M + 1], const Fold& fa, float wca, float wsa,
-                                            const Fold& fb, float wcb, float wsb, int mr = M) {
-    acc[0].x += wca + wcb;
-    if constexpr (M >= 1) {
-        if (mr < 1) return;
-        float2 Xa = make_float2(wca * fa.ac, wsa * fa.ss), Da = make_float2(0.5f * fa.lam * wca, wsa * fa.ss);
-        float2 Xb = make_float2(wcb * fb.ac, wsb * fb.ss), Db = make_float2(0.5f * fb.lam * wcb, wsb * fb.ss);
-        const float2 Sa = make_float2(fa.sg, fa.sg), Sb = make_float2(fb.sg, fb.sg);
-        const float2 La = make_float2(fa.lam, fa.lam), Lb = make_float2(fb.lam, fb.lam);
-        acc[1] = __ffma2_rn(Sb, Xb, __ffma2_rn(Sa, Xa, acc[1]));
-#pragma unroll
-        for (int m = 2; m <= M; ++m) {
-            if (m > mr) break;
-            Da = __ffma2_rn(La, Xa, Da);
-            Db = __ffma2_rn(Lb, Xb, Db);
-            Xa = __fadd2_rn(Xa, Da);
-            Xb = __fadd2_rn(Xb, Db);
-            if (m & 1)
-                acc[m] = __ffma2_rn(Sb, Xb, __ffma2_rn(Sa, Xa, acc[m]));
-            else
-                acc[m] = __fadd2_rn(acc[m], __fadd2_rn(Xa, Xb));
-        }
-    }
-}
-
-template <int M>
-__device__ __forceinline__ void harmonics2(float2 (&acc)[M + 1], float ca, float sa, float wca, float wsa, float cb,
-                                           float sb, float wcb, float wsb, int mr = M) {
-    harmonics2f<M>(acc, fold_angle(ca, sa), wca, wsa, fold_angle(cb, sb), wcb, wsb, mr);
-}
-
-// A folded angle held by lane `src`, broadcast to the warp.
-__device__ __forceinline__ Fold shfl_fold(const Fold& f, int src) {
-    Fold g;
-    g.ac = __shfl_sync(0xffffffffu, f.ac, src);
-    g.ss = __shfl_sync(0xffffffffu, f.ss, src);
-    g.sg = __shfl_sync(0xffffffffu, f.sg, src);
-    g.lam = __shfl_sync(0xffffffffu, f.lam, src);
-    return g;
 }
 
 // p mod n for -n <= p < 2n (every unwrapped index of a run lies in that range).
@@ -331,188 +328,6 @@ struct DirectLoad {
     };
     __device__ __forceinline__ Row row(long long first) const { return Row{d + first, w + first}; }
 };
-
-// Walk pixels [a, a + len) of ring R (lane-private run), accumulating into the bin.
-// Two pixels per iteration.  When no lane's run wraps around the ring, the first
-// min-length iterations run without predicates or index wrapping; the rest (and
-// wrapping runs) take the general loop.
-template <int M, bool FAST, bool SELF, class L>
-__device__ __forceinline__ void walk_run(const RingCtx& R, const L& ld, const LaneC& c, int a, int len,
-                                         float2 (&acc)[M + 1], float& W, float& Q, float& QW, int mr = M) {
-    const int maxlen = __reduce_max_sync(0xffffffffu, len);
-    if (maxlen <= 0) return;
-    const float i0 = (float)(a - c.cint);
-    const float xneg = -c.cfrac * R.step, uneg = -c.cfrac * R.inv_n;
-    int idx = wrap_idx(a, R.n);
-    const auto row = ld.row(R.first);
-    int t = 0;
-    const int minlen = __reduce_min_sync(0xffffffffu, len);
-    if (minlen >= 2 && __all_sync(0xffffffffu, idx + len <= R.n)) {
-        float ft = i0;
-        for (; t + 1 < minlen; t += 2, ft += 2.0f) {
-            const float2 v0 = row(idx + t), v1 = row(idx + t + 1);
-            float ca, sa, cb, sb;
-            pixel_dir<FAST>(ft, xneg, uneg, R, ca, sa);
-            pixel_dir<FAST>(ft + 1.0f, xneg, uneg, R, cb, sb);
-            harmonics2<M>(acc, ca, sa, v0.x, v0.x, cb, sb, v1.x, v1.x, mr);
-            W += v0.y + v1.y;
-            if (SELF) {
-                Q = fmaf(v0.x, v0.x, fmaf(v1.x, v1.x, Q));
-                QW = fmaf(v0.y, v0.y, fmaf(v1.y, v1.y, QW));
-            }
-        }
-        idx += t;
-        if (idx >= R.n) idx -= R.n;
-    }
-    for (; t < maxlen; t += 2) {
-        const bool on0 = t < len, on1 = t + 1 < len;
-        const int idx1 = idx + 1 >= R.n ? idx + 1 - R.n : idx + 1;
-        const float2 v0 = on0 ? row(idx) : make_float2(0.0f, 0.0f);
-        const float2 v1 = on1 ? row(idx1) : make_float2(0.0f, 0.0f);
-        const float oa = on0 ? i0 + (float)t : i0;
-        const float ob = on1 ? i0 + (float)(t + 1) : i0;
-        float ca, sa, cb, sb;
-        pixel_dir<FAST>(oa, xneg, uneg, R, ca, sa);
-        pixel_dir<FAST>(ob, xneg, uneg, R, cb, sb);
-        harmonics2<M>(acc, ca, sa, v0.x, v0.x, cb, sb, v1.x, v1.x, mr);
-        W += v0.y + v1.y;
-        if (SELF) {
-            Q = fmaf(v0.x, v0.x, fmaf(v1.x, v1.x, Q));
-            QW = fmaf(v0.y, v0.y, fmaf(v1.y, v1.y, QW));
-        }
-        idx = idx1 + 1 >= R.n ? idx1 + 1 - R.n : idx1 + 1;
-    }
-}
-
-// Walk the pixel pairs (p, mb - p), p in [a, a + len): mirror images about the
-// pivot's meridian (belt rings with as many pixels as the pivot ring).  Two pairs
-// (four pixels) per iteration; the same no-wrap fast loop as walk_run.
-template <int M, bool FAST, bool SELF, class L>
-__device__ __forceinline__ void walk_pairs(const RingCtx& R, const L& ld, const LaneC& c, int a, int len,
-                                           int mb, float2 (&acc)[M + 1], float& W, float& Q,
-                                           float& QW, int mr = M) {
-    const int maxlen = __reduce_max_sync(0xffffffffu, len);
-    if (maxlen <= 0) return;
-    const float i0 = (float)(a - c.cint);
-    const float xneg = -c.cfrac * R.step, uneg = -c.cfrac * R.inv_n;
-    int ip = wrap_idx(a, R.n);
-    int im_ = wrap_idx(mb - a, R.n);
-    const auto row = ld.row(R.first);
-    int t = 0;
-    const int minlen = __reduce_min_sync(0xffffffffu, len);
-    if (minlen >= 2 && __all_sync(0xffffffffu, ip + len <= R.n && im_ - len + 1 >= 0)) {
-        float ft = i0;
-        for (; t + 1 < minlen; t += 2, ft += 2.0f) {
-            const float2 p0 = row(ip + t), m0 = row(im_ - t);
-            const float2 p1 = row(ip + t + 1), m1 = row(im_ - t - 1);
-            float ca, sa, cb, sb;
-            pixel_dir<FAST>(ft, xneg, uneg, R, ca, sa);
-            pixel_dir<FAST>(ft + 1.0f, xneg, uneg, R, cb, sb);
-            harmonics2<M>(acc, ca, sa, p0.x + m0.x, p0.x - m0.x, cb, sb, p1.x + m1.x, p1.x - m1.x, mr);
-            W += (p0.y + m0.y) + (p1.y + m1.y);
-            if (SELF) {
-                Q = fmaf(p0.x, p0.x, fmaf(m0.x, m0.x, fmaf(p1.x, p1.x, fmaf(m1.x, m1.x, Q))));
-                QW = fmaf(p0.y, p0.y, fmaf(m0.y, m0.y, fmaf(p1.y, p1.y, fmaf(m1.y, m1.y, QW))));
-            }
-        }
-        ip += t;
-        if (ip >= R.n) ip -= R.n;
-        im_ -= t;
-        if (im_ < 0) im_ += R.n;
-    }
-    for (; t < maxlen; t += 2) {
-        const bool on0 = t < len, on1 = t + 1 < len;
-        const int ip1 = ip + 1 >= R.n ? ip + 1 - R.n : ip + 1;
-        const int im1 = im_ - 1 < 0 ? im_ - 1 + R.n : im_ - 1;
-        const float2 p0 = on0 ? row(ip) : make_float2(0.0f, 0.0f);
-        const float2 m0 = on0 ? row(im_) : make_float2(0.0f, 0.0f);
-        const float2 p1 = on1 ? row(ip1) : make_float2(0.0f, 0.0f);
-        const float2 m1 = on1 ? row(im1) : make_float2(0.0f, 0.0f);
-        const float oa = on0 ? i0 + (float)t : i0;
-        const float ob = on1 ? i0 + (float)(t + 1) : i0;
-        float ca, sa, cb, sb;
-        pixel_dir<FAST>(oa, xneg, uneg, R, ca, sa);
-        pixel_dir<FAST>(ob, xneg, uneg, R, cb, sb);
-        harmonics2<M>(acc, ca, sa, p0.x + m0.x, p0.x - m0.x, cb, sb, p1.x + m1.x, p1.x - m1.x, mr);
-        W += (p0.y + m0.y) + (p1.y + m1.y);
-        if (SELF) {
-            Q = fmaf(p0.x, p0.x, fmaf(m0.x, m0.x, fmaf(p1.x, p1.x, fmaf(m1.x, m1.x, Q))));
-            QW = fmaf(p0.y, p0.y, fmaf(m0.y, m0.y, fmaf(p1.y, p1.y, fmaf(m1.y, m1.y, QW))));
-        }
-        ip = ip1 + 1 >= R.n ? ip1 + 1 - R.n : ip1 + 1;
-        im_ = im1 - 1 < 0 ? im1 - 1 + R.n : im1 - 1;
-    }
-}
-
-// walk_pairs for the case of a belt ring pair (the neighbour ring has as many pixels
-// as the pivot ring): the 32 pivots of the tile then sit at the same fractional
-// position relative to ring r, so every lane's run starts at the same offset from its
-// own pivot and has the same length, and at step t all lanes see a neighbour at the
-// same offset, hence the same position angle.  Each lane computes the (folded) angle of
-// one step of a block of 32 and the warp shares them by shuffles, instead of every lane
-// computing the same angle.  Lane l's pixels are those of lane 0 shifted by l, so the
-// loads of a step stay coalesced.
-template <int M, bool SELF, class L>
-__device__ __forceinline__ void walk_pairs_shared(const RingCtx& R, const L& ld, const LaneC& c, int a, int len,
-                                                  int mb, float2 (&acc)[M + 1], float& W, float& Q, float& QW,
-                                                  int mr = M) {
-    if (len <= 0) return;
-    const int lane = threadIdx.x & 31;
-    const float i0 = (float)(a - c.cint);
-    const float xneg = -c.cfrac * R.step, uneg = -c.cfrac * R.inv_n;
-    const auto row = ld.row(R.first);
-    int ip = wrap_idx(a, R.n);
-    int im_ = wrap_idx(mb - a, R.n);
-    for (int t0 = 0; t0 < len; t0 += 32) {
-        // this lane's step: t0 + lane
-        Fold mine;
-        {
-            const float ft = i0 + (float)(t0 + lane);
-            float cph, sph;
-            if (fabsf(ft - c.cfrac) * R.step <= FAST_XMAX)
-                pixel_dir<true>(ft, xneg, uneg, R, cph, sph);
-            else
-                pixel_dir<false>(ft, xneg, uneg, R, cph, sph);
-            mine = fold_angle(cph, sph);
-        }
-        const int nstep = min(32, len - t0);
-        int tt = 0;
-        for (; tt + 1 < nstep; tt += 2) {
-            const Fold fa = shfl_fold(mine, tt), fb = shfl_fold(mine, tt + 1);
-            const int ip1 = ip + 1 >= R.n ? ip + 1 - R.n : ip + 1;
-            const int im1 = im_ - 1 < 0 ? im_ - 1 + R.n : im_ - 1;
-            const float2 p0 = row(ip), m0 = row(im_), p1 = row(ip1), m1 = row(im1);
-            harmonics2f<M>(acc, fa, p0.x + m0.x, p0.x - m0.x, fb, p1.x + m1.x, p1.x - m1.x, mr);
-            W += (p0.y + m0.y) + (p1.y + m1.y);
-            if (SELF) {
-                Q = fmaf(p0.x, p0.x, fmaf(m0.x, m0.x, fmaf(p1.x, p1.x, fmaf(m1.x, m1.x, Q))));
-                QW = fmaf(p0.y, p0.y, fmaf(m0.y, m0.y, fmaf(p1.y, p1.y, fmaf(m1.y, m1.y, QW))));
-            }
-            ip = ip1 + 1 >= R.n ? ip1 + 1 - R.n : ip1 + 1;
-            im_ = im1 - 1 < 0 ? im1 - 1 + R.n : im1 - 1;
-        }
-        if (tt < nstep) {
-            const Fold fa = shfl_fold(mine, tt);
-            const float2 p0 = row(ip), m0 = row(im_);
-            harmonicsf<M>(acc, fa, p0.x + m0.x, p0.x - m0.x, mr);
-            W += p0.y + m0.y;
-            if (SELF) {
-                Q = fmaf(p0.x, p0.x, fmaf(m0.x, m0.x, Q));
-                QW = fmaf(p0.y, p0.y, fmaf(m0.y, m0.y, QW));
-            }
-            ip = ip + 1 >= R.n ? ip + 1 - R.n : ip + 1;
-            im_ = im_ - 1 < 0 ? im_ - 1 + R.n : im_ - 1;
-        }
-    }
-}
-
-// True when every lane's run has lane 0's start offset and length (belt ring pairs).
-__device__ __forceinline__ bool runs_shared(const LaneC& c, int a, int len) {
-    const int rel = a - c.cint;
-    const int rel0 = __shfl_sync(0xffffffffu, rel, 0), len0 = __shfl_sync(0xffffffffu, len, 0);
-    const unsigned cf = __float_as_uint(c.cfrac), cf0 = __shfl_sync(0xffffffffu, cf, 0);
-    return __all_sync(0xffffffffu, rel == rel0 && len == len0 && cf == cf0);
-}
 
 // Runs of bin k on ring r for the lane's pivot.  Fills up to two runs (a, len) and,
 // in mirror mode, one pair run plus an optional centre pixel.
@@ -567,6 +382,25 @@ __device__ __forceinline__ BinRuns bin_runs(const LaneC& c, int2 Tk, int2 Tk1, d
     return b;
 }
 
+// The plain runs (two at most) of bin k, edges decided with LazyEdge.
+__device__ __forceinline__ BinRuns bin_runs(const LaneC& c, int2 Tk, int2 Tk1, const LazyEdge& x, int n_r) {
+    BinRuns b;
+    b.sym = b.centre = false;
+    b.mb = b.a1 = b.n1 = 0;
+    const int pe = Tk1.x == T_INF ? c.cint + n_r / 2 : pos_edge(c, Tk1, x, 1) - 1;
+    const int ns = Tk1.x == T_INF ? c.cint - n_r / 2 + 1 : neg_edge(c, Tk1, x, 1) + 1;
+    if (Tk.x == T_ZERO) {
+        b.a0 = ns;
+        b.n0 = max(0, pe - ns + 1);
+    } else {
+        b.a0 = pos_edge(c, Tk, x, 0);
+        b.n0 = max(0, pe - b.a0 + 1);
+        b.a1 = ns;
+        b.n1 = max(0, neg_edge(c, Tk, x, 0) - ns + 1);
+    }
+    return b;
+}
+
 // Largest |o| a run reaches, for the FAST test.
 __device__ __forceinline__ float run_omax(const LaneC& c, int a, int len) {
     if (len <= 0) return 0.0f;
@@ -583,24 +417,6 @@ struct PivotRing {
     long long pair0;
 };
 
-__device__ __forceinline__ RingCtx ring_ctx(const MapDev& g, const PivotRing& P, int r, long long pr) {
-    RingCtx R;
-    R.first = g.ring_first[r];
-    R.n = g.ring_n[r];
-    R.shift = g.ring_shift[r];
-    R.s_r = g.ring_sf[r];
-    R.s_lo = g.ring_sf_lo[r];
-    const float2 Ap = g.pair_A[pr];
-    R.A = Ap.x;
-    R.A_lo = Ap.y;
-    R.B = 2.0f * P.z_i * R.s_r;
-    R.step = g.ring_step[r];
-    R.step_lo = g.ring_step_lo[r];
-    R.inv_n = g.ring_invn[r];
-    R.invn_lo = g.ring_invn_lo[r];
-    return R;
-}
-
 __device__ __forceinline__ ExactCtx exact_ctx(const MapDev& g, const PivotRing& P, int r) {
     ExactCtx x;
     x.th_i = P.th_i;
@@ -609,54 +425,6 @@ __device__ __forceinline__ ExactCtx exact_ctx(const MapDev& g, const PivotRing& 
     x.s_r = g.ring_s[r];
     x.n_r = g.ring_n[r];
     return x;
-}
-
-// Accumulate the bin-k moments of ring r into the lane's registers.
-template <int M, bool SELF, class L>
-__device__ __forceinline__ void fwd_ring_bin(const MapDev& g, const PivotRing& P, int r, int k, int q,
-                                             const L& ld, float2 (&acc)[M + 1], float& W,
-                                             float& Q, float& QW, int mr = M) {
-    const long long pr = P.pair0 + (r - P.rlo);
-    const int2 Tk = g.pair_T[pr * (g.K + 1) + k];
-    const int2 Tk1 = g.pair_T[pr * (g.K + 1) + k + 1];
-    if (Tk.x == T_INF || Tk1.x == T_ZERO) return;  // no bin-k pixel on this ring
-    const RingCtx R = ring_ctx(g, P, r, pr);
-    const ExactCtx x = exact_ctx(g, P, r);
-    const LaneC c = lane_c(q, P.s_i, P.n_i, R.shift, R.n);
-    const bool sym = (R.n == P.n_i) && (Tk1.x != T_INF);
-    const BinRuns b = bin_runs(c, Tk, Tk1, g.E[k], g.E[k + 1], x, R.n, sym);
-    if (sym) {
-        if (b.centre) {  // the pixel straight north or south of the pivot
-            const float2 v = ld(R.first + wrap_idx(c.cint, R.n));
-            float cph, sph;
-            pixel_dir<false>(0.0f, 0.0f, -c.cfrac * R.inv_n, R, cph, sph);
-            harmonics<M>(acc, cph, sph, v.x, v.x, mr);
-            W += v.y;
-            if (SELF) {
-                Q = fmaf(v.x, v.x, Q);
-                QW = fmaf(v.y, v.y, QW);
-            }
-        }
-        if (runs_shared(c, b.a0, b.n0)) {
-            walk_pairs_shared<M, SELF>(R, ld, c, b.a0, b.n0, b.mb, acc, W, Q, QW, mr);
-            return;
-        }
-        const bool fast = __all_sync(0xffffffffu, run_omax(c, b.a0, b.n0) * R.step <= FAST_XMAX);
-        if (fast)
-            walk_pairs<M, true, SELF>(R, ld, c, b.a0, b.n0, b.mb, acc, W, Q, QW, mr);
-        else
-            walk_pairs<M, false, SELF>(R, ld, c, b.a0, b.n0, b.mb, acc, W, Q, QW, mr);
-        return;
-    }
-    const float om = fmaxf(run_omax(c, b.a0, b.n0), run_omax(c, b.a1, b.n1));
-    const bool fast = __all_sync(0xffffffffu, om * R.step <= FAST_XMAX);
-    if (fast) {
-        walk_run<M, true, SELF>(R, ld, c, b.a0, b.n0, acc, W, Q, QW, mr);
-        walk_run<M, true, SELF>(R, ld, c, b.a1, b.n1, acc, W, Q, QW, mr);
-    } else {
-        walk_run<M, false, SELF>(R, ld, c, b.a0, b.n0, acc, W, Q, QW, mr);
-        walk_run<M, false, SELF>(R, ld, c, b.a1, b.n1, acc, W, Q, QW, mr);
-    }
 }
 
 // Shared-memory layout of a tile's moments.
@@ -679,72 +447,6 @@ __device__ __forceinline__ PivotRing pivot_ring(const MapDev& g, int i) {
     P.rlo = g.ring_range[i].x;
     P.pair0 = g.pair_off[i];
     return P;
-}
-
-}  // namespace tpcf
-
-#include "map_walk.cuh"
-
-namespace tpcf {
-
-// Where the tile's moments live in shared memory.  LayKM: A[k][m][re/im][32 pivots],
-// W[k][32], Q[k][32], QW[k][32] (the FP32 contraction and the adjoint read this).
-struct LayKM {
-    float *sA, *sW, *sQ, *sQW;
-    int M1;  // m_max + 1
-    __device__ __forceinline__ float* a(int k, int m, int part, int lane) const {
-        return sA + ((size_t)(k * M1 + m) * 2 + part) * TILE + lane;
-    }
-    __device__ __forceinline__ float* w(int k, int lane) const { return sW + k * TILE + lane; }
-    __device__ __forceinline__ float* q(int k, int lane) const { return sQ + k * TILE + lane; }
-    __device__ __forceinline__ float* qw(int k, int lane) const { return sQW + k * TILE + lane; }
-};
-
-// All warps of the CTA: accumulate the moments of the tile into shared memory.
-// Smem must be zeroed beforehand; it is complete after the caller's __syncthreads().
-template <int M, bool SELF, class L, class Lay>
-__device__ __forceinline__ void tile_moments_l(const MapDev& g, const PivotRing& P, int q, const L& ld,
-                                               const Lay& lay, int flush, int mr = M) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int k = 0; k < g.K; ++k) {
-        const int2 br = g.bin_range[(long long)P.i * g.K + k];
-        if (br.x + warp > br.y) continue;
-        float2 acc[M + 1];
-#pragma unroll
-        for (int m = 0; m <= M; ++m) acc[m] = make_float2(0.0f, 0.0f);
-        float W = 0.0f, Q = 0.0f, QW = 0.0f;
-        // Blocked summation: the registers sum `flush` rings (FLUSH_RINGS unless
-        // tuned), then the block is added into shared memory, which keeps the running
-        // sums short.
-        int nr = 0;
-        for (int r = br.x + warp; r <= br.y; r += NWARPS) {
-            fwd_ring_bin<M, SELF>(g, P, r, k, q, ld, acc, W, Q, QW, mr);
-            if (++nr == flush || r + NWARPS > br.y) {
-                nr = 0;
-#pragma unroll
-                for (int m = 0; m <= M; ++m) {
-                    if (m > mr) break;
-                    atomicAdd(lay.a(k, m, 0, lane), acc[m].x);
-                    atomicAdd(lay.a(k, m, 1, lane), acc[m].y);
-                    acc[m] = make_float2(0.0f, 0.0f);
-                }
-                atomicAdd(lay.w(k, lane), W);
-                W = 0.0f;
-                if (SELF) {
-                    atomicAdd(lay.q(k, lane), Q);
-                    atomicAdd(lay.qw(k, lane), QW);
-                    Q = 0.0f;
-                    QW = 0.0f;
-                }
-            }
-        }
-    }
-}
-
-template <int M, bool SELF, class L>
-__device__ __forceinline__ void tile_moments(const MapDev& g, const PivotRing& P, int q, const L& ld, float* sA,
-                                             float* sW, float* sQ, float* sQW, int flush, int mr = M) {
-    tile_moments_l<M, SELF>(g, P, q, ld, LayKM{sA, sW, sQ, sQW, mr + 1}, flush, mr);
 }
 
 // Per-pivot normalisation of the tile's moments (Sec. 3.1): each lane's a_m^k is
@@ -891,10 +593,9 @@ __device__ __forceinline__ void tile_contract(int K, const float* sA, const floa
 // in the convention a = re - i im; D is the Gram matrix of the W^k rows with the
 // weights w.  On the 5th-generation tensor cores (kind::tf32, FP32 accumulation in
 // tensor memory), per block of rows (each m, then the W block):
-//   * the moments are accumulated straight into the layout the MMA reads (K-major,
+//   * the moments are staged from the workspace in the layout the MMA reads (K-major,
 //     no swizzle: 8-row x 16-byte core matrices, pivot-adjacent ones 128 B apart,
-//     8-row groups 1024 B apart, blocks starting on a row group); no operand copy of
-//     X exists;
+//     8-row groups 1024 B apart, blocks starting on a row group);
 //   * with Y = X diag(sqrt|w d|) and s = sign(w d), G = Y diag(s) Y^T.  Y is split into
 //     a tf32 part hi (its low 13 mantissa bits cleared, written back in place) and
 //     the fp32 remainder lo, and G = hi s hi^T + C + C^T with C = hi s lo^T (the
@@ -905,8 +606,6 @@ __device__ __forceinline__ void tile_contract(int K, const float* sA, const floa
 //   * one thread issues, an mbarrier tracks completion (bounded wait), warps 0-1 read
 //     the two accumulators back, C^T goes through shared memory, and S (or D) is added
 //     into the CTA's FP64 slot.
-// The operands cost no shared memory beyond the moments but the staging buffer, so
-// the kernel keeps the FP32 forward's 3 CTAs per SM at 20 bins and m_max 10.
 constexpr int TC_TMEM_COLS = 128;  // two accumulators of up to 64 columns
 constexpr int ST_TC_TIMEOUT = ST_TC_TIMEOUT_BIT;
 
@@ -916,8 +615,7 @@ struct TcLayout {
     int Rm, RD, NBm, NBd;  // rows per m block and of the W block; MMA N of each
     int x0, D0;            // first row of the moments; first row of the W block
     int offB, offPiv, offSc, offQ, offQW;
-    int offWalk;           // the walk's scratch (over the staging, which is used after it)
-    int total;             // floats, without the walk's scratch
+    int total;             // floats
 };
 
 __host__ __device__ inline TcLayout tc_layout(int K, int M, bool self) {
@@ -936,7 +634,6 @@ __host__ __device__ inline TcLayout tc_layout(int K, int M, bool self) {
     L.offQ = off;
     L.offQW = off + (self ? K * TILE : 0);
     if (self) off += 2 * K * TILE;
-    L.offWalk = off;
     L.offB = off;  // B hi rows, then B lo rows (NBm each); reused for the C^T staging
     off += 2 * L.NBm * TILE;
     // the MMA of the last block reads 128 rows from its start
@@ -946,10 +643,8 @@ __host__ __device__ inline TcLayout tc_layout(int K, int M, bool self) {
 }
 
 // bytes of dynamic shared memory
-__host__ __device__ inline size_t tc_smem_bytes(int K, int M, bool self, int cells) {
-    const TcLayout L = tc_layout(K, M, self);
-    const size_t a = (size_t)L.total * sizeof(float);
-    const size_t b = (size_t)L.offWalk * sizeof(float) + walk_scratch_bytes(NWARPS, cells);
+__host__ __device__ inline size_t tc_smem_bytes(int K, int M, bool self) {
+    const size_t a = (size_t)tc_layout(K, M, self).total * sizeof(float), b = block_smem_bytes(M);
     return a > b ? a : b;
 }
 
@@ -957,18 +652,6 @@ __host__ __device__ inline size_t tc_smem_bytes(int K, int M, bool self, int cel
 // matrices of 8 rows x 4 pivots (128 contiguous bytes, rows 16 B apart), the 8
 // pivot-adjacent core matrices of a row group 128 B apart, row groups 1024 B apart.
 __device__ __forceinline__ int kmaj(int r, int p) { return ((r >> 3) << 8) + ((p >> 2) << 5) + ((r & 7) << 2) + (p & 3); }
-
-struct LayTC {
-    float* sX;
-    float *sQ, *sQW;
-    int Rm, D0;
-    __device__ __forceinline__ float* a(int k, int m, int part, int lane) const {
-        return sX + kmaj(m * Rm + 2 * k + part, lane);
-    }
-    __device__ __forceinline__ float* w(int k, int lane) const { return sX + kmaj(D0 + k, lane); }
-    __device__ __forceinline__ float* q(int k, int lane) const { return sQ + k * TILE + lane; }
-    __device__ __forceinline__ float* qw(int k, int lane) const { return sQW + k * TILE + lane; }
-};
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
     return (uint32_t)__cvta_generic_to_shared(p);
@@ -1096,7 +779,7 @@ __device__ void tile_contract_tc(int K, float* base, double* slot, TcState& tc, 
         // beyond the block are zero.  e runs over the layout in memory order (row group,
         // pivot chunk, row in group, pivot in chunk); r0 is a multiple of 8, so the
         // block's element e sits at sX[r0 * 32 + e] and B's at B[e].
-        for (int e = threadIdx.x; e < N * TILE; e += NTHREADS) {
+        for (int e = threadIdx.x; e < N * TILE; e += BT) {
             const int i = ((e >> 8) << 3) + ((e >> 2) & 7);
             const int p = (((e >> 5) & 7) << 2) + (e & 3);
             float bh = 0.0f, bl = 0.0f;
@@ -1193,7 +876,7 @@ __device__ void tile_contract_tc(int K, float* base, double* slot, TcState& tc, 
         const float* wt = sPiv + TILE;
         const float* sQ = base + L.offQ;
         const float* sQW = base + L.offQW;
-        for (int k = threadIdx.x; k < K; k += NTHREADS) {
+        for (int k = threadIdx.x; k < K; k += BT) {
             float s1 = 0.0f, s2 = 0.0f;
             for (int j = 0; j < TILE; ++j) {
                 s1 = fmaf(wd[j], sQ[k * TILE + j], s1);
@@ -1205,155 +888,84 @@ __device__ void tile_contract_tc(int K, float* base, double* slot, TcState& tc, 
     }
 }
 
-// One forward tile: the moments of its 32 pivots, then their partial sums added to
-// the CTA's slot.  Called by every thread of the CTA (contains barriers).
-template <int M, bool SELF, bool DIRECT, bool GROUPED = false>
-__device__ __forceinline__ void fwd_tile(const MapDev& g, const MapCall& c, int tile, double* slot, float* smem,
-                                         int mr = M) {
-    const int K = g.K;
-    float* sA = smem;
-    float* sW = sA + (size_t)K * (mr + 1) * 2 * TILE;
-    float* sQ = sW + K * TILE;  // Q, QW with SELF only
-    float* sQW = sQ + K * TILE;
-    float* sPiv = SELF ? sQW + K * TILE : sQ;
-    char* scratch = reinterpret_cast<char*>(sPiv + 2 * TILE);
-    const int lane = threadIdx.x & 31;
-    const size_t nfl = tile_floats_rt(K, mr, SELF) - 2 * TILE;
-    constexpr bool grouped = GROUPED;  // shared neighbour lists (c.group > 1): own instantiation
-    const int2 tq = grouped ? c.gtiles[tile] : g.wtiles[tile];
-    if (tq.x < 0 || tq.x >= g.nrings) {
-        if (threadIdx.x == 0) atomicOr(c.status, ST_BAD_TILE);
-        __syncthreads();
-        return;
-    }
-    const PivotRing P = pivot_ring(g, tq.x);
-    const bool lin = g.lin[P.i] != 0;
-    float2 pv = make_float2(0.0f, 0.0f);
-    int qg, qa, qb;  // geometry of the lane's pivot, and of pivots lane & 15 and 16 + (lane & 15)
-    if (grouped) {
-        // shared neighbour lists: the lane stands for the run of c.group consecutive ring
-        // pixels gi, sits at the run's middle pixel and carries the run's summed weights
-        const int ng = (P.n_i + c.group - 1) / c.group;
-        auto middle = [&](int gi) {
-            const int s0 = min(gi, ng - 1) * c.group;
-            return s0 + (min(c.group, P.n_i - s0) - 1) / 2;
-        };
-        const int gi = tq.y + lane;
-        const int s0 = min(gi, ng - 1) * c.group, ln = min(c.group, P.n_i - s0);
-        qg = middle(gi);
-        qa = middle(tq.y + (lane & 15));
-        qb = middle(tq.y + 16 + (lane & 15));
-        if (gi < ng) {
-            const long long f = g.ring_first[P.i] + s0;
-            for (int u = 0; u < ln; ++u) {
-                const long long pix = f + u;
-                if (pix >= c.piv_lo && pix < c.piv_hi) {
-                    const float2 v = DIRECT ? DirectLoad{c.delta, c.w, g.npix}(pix) : c.wdw[pix];
-                    pv.x += v.x;
-                    pv.y += v.y;
-                }
-            }
-        }
-    } else {
-        const TileSlot tp = tile_slot(lin, P.n_i, P.s_i, tq.y, lane);
-        const long long pix = g.ring_first[P.i] + tp.q;
-        if (tp.valid && pix >= c.piv_lo && pix < c.piv_hi)
-            pv = DIRECT ? DirectLoad{c.delta, c.w, g.npix}(pix) : c.wdw[pix];
-        qg = tp.q;
-        qa = tile_slot(lin, P.n_i, P.s_i, tq.y, lane & 15).q;
-        qb = tile_slot(lin, P.n_i, P.s_i, tq.y, 16 + (lane & 15)).q;
-    }
-    if (!__syncthreads_or(pv.y != 0.0f)) return;
-    for (size_t e = threadIdx.x; e < nfl; e += NTHREADS) sA[e] = 0.0f;
-    if (threadIdx.x < TILE) {
-        sPiv[lane] = pv.x;
-        sPiv[TILE + lane] = pv.y;
-    }
-    __syncthreads();
-    auto moments = [&](const auto& ld) {
-        // runs of pixels on other rings have no common angles: one pivot per lane
-        if (grouped && !lin)
-            tile_moments<M, SELF>(g, P, qg, ld, sA, sW, sQ, sQW, c.flush, mr);
-        else
-            walk_tile<M, SELF>(g, P, lin, qa, qb, tq.y, ld, LayKM{sA, sW, sQ, sQW, mr + 1}, scratch, c.cells, c.flush,
-                               mr);
-    };
-    if constexpr (DIRECT)
-        moments(DirectLoad{c.delta, c.w, g.npix});
-    else
-        moments(PackedLoad{c.wdw});
-    __syncthreads();
-    if (c.norm != NORM_NONE) tile_normalize<M>(K, sA, sW, c.norm, mr);
-    tile_contract<M>(K, sA, sW, sQ, sQW, sPiv, slot, SELF && c.self_subtract, mr);
-    __syncthreads();
-}
+}  // namespace tpcf
 
-// One forward tile with the tensor-core contraction: the moments accumulate in the
-// tensor-core layout of tc_layout(), then tile_contract_tc.
+#include "map_block.cuh"
+#include "map_block_bwd.cuh"
+
+namespace tpcf {
+
+// One work item of the forward with the tensor-core contraction: the block's moments as in
+// fwd_block, then each live subtile is brought into the layout of tc_layout() and
+// contracted by tile_contract_tc.
 template <int M, bool SELF>
-__device__ __forceinline__ void fwd_tile_tc(const MapDev& g, const MapCall& c, int tile, double* slot, float* base,
-                                            TcState& tc) {
-    const int K = g.K;
-    const int lane = threadIdx.x & 31;
-    const int2 tq = g.wtiles[tile];
-    if (tq.x < 0 || tq.x >= g.nrings) {
-        if (threadIdx.x == 0) atomicOr(c.status, ST_BAD_TILE);
-        __syncthreads();
-        return;
-    }
-    const PivotRing P = pivot_ring(g, tq.x);
-    const bool lin = g.lin[P.i] != 0;
-    const TileSlot tp = tile_slot(lin, P.n_i, P.s_i, tq.y, lane);
-    const long long pix = g.ring_first[P.i] + tp.q;
-    const bool in = tp.valid && pix >= c.piv_lo && pix < c.piv_hi;
-    float2 pv = make_float2(0.0f, 0.0f);
-    if (in) pv = c.wdw[pix];
-    if (!__syncthreads_or(pv.y != 0.0f)) return;
-    {
-        const TcLayout L = tc_layout(K, M, SELF);
-        const int nx = (L.D0 + L.RD) * TILE;
-        for (int e = threadIdx.x; e < nx; e += NTHREADS) base[e] = 0.0f;
-        if (SELF)
-            for (int e = threadIdx.x; e < 2 * K * TILE; e += NTHREADS) base[L.offQ + e] = 0.0f;
-        if (threadIdx.x < TILE) {
-            base[L.offPiv + lane] = pv.x;
-            base[L.offPiv + TILE + lane] = pv.y;
+__device__ __forceinline__ void fwd_block_tc(const MapDev& g, const MapCall& c, long long b, int part, float* ws,
+                                             double* slot, float* base, TcState& tc) {
+    const int K = g.K, lane = threadIdx.x & 31;
+    const Block<M, false> B(g, c, b);
+    const size_t sub_floats = sub_floats_rt(K, M, SELF);
+    const PackedLoad ld{c.wdw};
+    auto value = [&](int s, int l) { return B.value(g, c, ld, s, l); };
+    const unsigned live = block_live(B.nsub, [&](int s, int l) { return value(s, l).y != 0.0f; });
+    if (live == 0u) return;
+    block_moments<M, SELF, false>(g, c, b, live, part, ld, ws, sub_floats, reinterpret_cast<char*>(base), M);
+    if (!block_complete(c, b)) return;
+    const TcLayout L = tc_layout(K, M, SELF);
+    for (int s = 0; s < B.nsub; ++s) {
+        if (!((live >> s) & 1u)) continue;
+        const float* sub = ws + (size_t)s * sub_floats;
+        const float* W = sub + (size_t)(M + 1) * K * 2 * TILE;
+        // every row of the layout: rows beyond a block's 2 K (or K) are zero
+        for (int r = threadIdx.x >> 5; r < L.D0 + L.RD; r += BW) {
+            float v = 0.0f;
+            if (r < L.D0) {
+                const int m = r / L.Rm, i = r - m * L.Rm;
+                if (i < 2 * K) v = __ldcg(sub + ((size_t)m * 2 * K + i) * TILE + lane);
+            } else if (r - L.D0 < K) {
+                v = __ldcg(W + (r - L.D0) * TILE + lane);
+            }
+            base[kmaj(r, lane)] = v;
         }
+        if (SELF)
+            for (int e = threadIdx.x; e < 2 * K * TILE; e += BT) base[L.offQ + e] = __ldcg(W + K * TILE + e);
+        if (threadIdx.x < TILE) {
+            const float2 v = value(s, lane);
+            base[L.offPiv + lane] = v.x;
+            base[L.offPiv + TILE + lane] = v.y;
+        }
+        __syncthreads();
+        tile_contract_tc<M, SELF>(K, base, slot, tc, c.status);
+        __syncthreads();
+        if (*tc.fail) return;
     }
-    __syncthreads();
-    {
-        const int Rm = (2 * K + 7) & ~7, D0 = (M + 1) * Rm;
-        const TcLayout L = tc_layout(K, M, SELF);
-        walk_tile<M, SELF>(g, P, lin, tile_slot(lin, P.n_i, P.s_i, tq.y, lane & 15).q,
-                           tile_slot(lin, P.n_i, P.s_i, tq.y, 16 + (lane & 15)).q, tq.y, PackedLoad{c.wdw},
-                           LayTC{base, base + L.offQ, base + L.offQW, Rm, D0},
-                           reinterpret_cast<char*>(base + L.offWalk), c.cells, c.flush, M);
-    }
-    __syncthreads();
-    tile_contract_tc<M, SELF>(K, base, slot, tc, c.status);
-    __syncthreads();
 }
 
-// OCC: CTAs per SM the register allocation is sized for (3: 80 registers, 2: 128);
-// the autotuner picks the variant and the grid.
-template <int M, bool SELF, bool DIRECT, int OCC = 3, bool GROUPED = false>
-__global__ void __launch_bounds__(NTHREADS, OCC) map_fwd_kernel(MapDev g, MapCall c) {
-    extern __shared__ float smem[];
+// Persistent CTAs draw work items (block, part) from a counter.
+template <int M, bool SELF, bool DIRECT, bool GROUPED = false>
+__global__ void __launch_bounds__(BT, 4) map_fwd_kernel(MapDev g, MapCall c) {
+    extern __shared__ __align__(16) float smem[];
     __shared__ int s_tile;
     double* slot = c.slots + (size_t)blockIdx.x * n_entries(g.K, M);
+    const long long nblk = c.nlin + (c.norb + c.tiles - 1) / c.tiles;
     for (;;) {
         if (threadIdx.x == 0) s_tile = atomicAdd(c.counter, 1);
         __syncthreads();
-        const long long tile = c.tile_lo + s_tile;
-        if (tile >= c.tile_hi) break;
-        fwd_tile<M, SELF, DIRECT, GROUPED>(g, c, (int)tile, slot, smem);
+        const long long item = s_tile;
+        if (item >= nblk * c.parts) break;
+        const long long b = item / c.parts;
+        float* ws = c.ws + (c.parts > 1 ? (size_t)b : (size_t)blockIdx.x) * c.ws_floats;
+        const int part = (int)(item - b * c.parts);
+        if constexpr (DIRECT)
+            fwd_block<M, SELF, GROUPED>(g, c, b, part, DirectLoad{c.delta, c.w, g.npix}, ws, slot,
+                                        reinterpret_cast<char*>(smem), M);
+        else
+            fwd_block<M, SELF, GROUPED>(g, c, b, part, PackedLoad{c.wdw}, ws, slot, reinterpret_cast<char*>(smem), M);
     }
 }
 
-// The forward with the tensor-core contraction (3 CTAs per SM where the shared
-// memory allows it; 128 accumulator columns each, so at most 4 fit an SM's TMEM).
+// The forward with the tensor-core contraction (128 accumulator columns per CTA).
 template <int M, bool SELF>
-__global__ void __launch_bounds__(NTHREADS, 2) map_fwd_tc_kernel(MapDev g, MapCall c) {
+__global__ void __launch_bounds__(BT, 4) map_fwd_tc_kernel(MapDev g, MapCall c) {
     extern __shared__ __align__(16) float smem_tc[];
     __shared__ int s_tile;
     __shared__ uint32_t s_tmem;
@@ -1365,28 +977,30 @@ __global__ void __launch_bounds__(NTHREADS, 2) map_fwd_tc_kernel(MapDev g, MapCa
     // the no-swizzle operand layout needs 16-byte alignment only
     float* base = smem_tc;
     double* slot = c.slots + (size_t)blockIdx.x * n_entries(g.K, M);
+    const long long nblk = c.nlin + (c.norb + c.tiles - 1) / c.tiles;
     for (;;) {
         if (threadIdx.x == 0) s_tile = atomicAdd(c.counter, 1);
         __syncthreads();
-        const long long tile = c.tile_lo + s_tile;
-        if (tile >= c.tile_hi || s_fail) break;
-        fwd_tile_tc<M, SELF>(g, c, (int)tile, slot, base, tc);
+        const long long item = s_tile;
+        if (item >= nblk * c.parts || s_fail) break;
+        const long long b = item / c.parts;
+        float* ws = c.ws + (c.parts > 1 ? (size_t)b : (size_t)blockIdx.x) * c.ws_floats;
+        fwd_block_tc<M, SELF>(g, c, b, (int)(item - b * c.parts), ws, slot, base, tc);
     }
     tc_teardown(s_tmem);
 }
 
 // Batched forward over all the plans of a batch, one launch: one work queue over the
-// concatenated tiles of all its plans (plan-major); each CTA adds into that plan's
+// concatenated blocks of all its plans (plan-major); each CTA adds into that plan's
 // slot number blockIdx.x.  Compiled for the largest m_max of the batch (M); each
-// plan's tiles run with its own m_max (the multipole loops stop there) and its own
-// shared-memory layout, and with its own self-pair mode.
+// plan's blocks run with its own m_max (the multipole loops stop there) and its own self-pair mode.
 template <int M>
-__global__ void __launch_bounds__(NTHREADS, 2) batch_fwd_kernel(const BatchItem* __restrict__ items, int n,
+__global__ void __launch_bounds__(BT, 4) batch_fwd_kernel(const BatchItem* __restrict__ items, int n,
                                                                long long total, unsigned long long* counter) {
-    extern __shared__ float smem[];
+    extern __shared__ __align__(16) float smem[];
     __shared__ long long s_t;
     __shared__ long long s_first[TPCF_MAX_BATCH + 1];
-    for (int i = threadIdx.x; i <= n; i += NTHREADS) s_first[i] = i < n ? items[i].tile0 : total;
+    for (int i = threadIdx.x; i <= n; i += BT) s_first[i] = i < n ? items[i].tile0 : total;
     __syncthreads();
     for (;;) {
         if (threadIdx.x == 0) s_t = (long long)atomicAdd(counter, 1ull);
@@ -1398,21 +1012,24 @@ __global__ void __launch_bounds__(NTHREADS, 2) batch_fwd_kernel(const BatchItem*
             const int mid = (lo + hi + 1) / 2;
             if (s_first[mid] <= t) lo = mid; else hi = mid - 1;
         }
-        const BatchItem& it = items[lo];
-        double* slot = it.c.slots + (size_t)blockIdx.x * n_entries(it.g.K, it.g.M);
-        fwd_tile<M, true, false>(it.g, it.c, (int)(t - s_first[lo]), slot, smem, it.g.M);
+        const MapDev& g = items[lo].g;
+        const MapCall& c = items[lo].c;
+        double* slot = c.slots + (size_t)blockIdx.x * n_entries(g.K, g.M);
+        fwd_block<M, true, false>(g, c, t - s_first[lo], 0, PackedLoad{c.wdw}, c.ws + (size_t)blockIdx.x * c.ws_floats,
+                                  slot, reinterpret_cast<char*>(smem), g.M);
     }
 }
 
 // ------------------------------------------------------------ multi-field
-// Three fields A, B, C on the same pixels (end of Sec. 2, after eq. ubEstimator): a
-// tile accumulates the moments a^k(i; F), W^k(i; F) of every field F in its own block
-// of shared memory (three passes of the single-field walk), then adds, over the
+// Three fields A, B, C on the same pixels (end of Sec. 2, after eq. ubEstimator): the moments
+// a^k(i; F), W^k(i; F) of every field F (three walks of the single-field kind), then, over the
 // cyclic permutations (P, X, Y) of (A, B, C),
 //     S_m(k1,k2) += sum_i w^P_i P_i a_m^{k1}(i; X) conj(a_m^{k2}(i; Y)),
 //     D(k1,k2)   += sum_i w^P_i W^{k1}(i; X) W^{k2}(i; Y),
 // into the CTA's FP64 slot.  These sums are not Hermitian: the slot holds the full
 // K x K matrices, for m, for (k1, k2): (Re S, Im S); then D for (k1, k2).
+// multi_field_floats, multi_tile_floats, tile_contract_multi: the catalogue's form, whose tile
+// keeps the three fields' moments in shared memory.
 __host__ __device__ inline size_t multi_field_floats(int K, int M) { return (size_t)K * (M + 1) * 2 * TILE + (size_t)K * TILE; }
 __host__ __device__ inline size_t multi_tile_floats(int K, int M) { return 3 * multi_field_floats(K, M) + 6 * TILE; }
 
@@ -1462,66 +1079,41 @@ __device__ __forceinline__ void tile_contract_multi(int K, const float* sF, cons
 }
 
 // The multi-field forward: c.wdw holds (w d, w) of field A, wdwB and wdwC those of
-// B and C.  One tile at a time, as map_fwd_kernel.
+// B and C; the block's workspace holds the three fields' in turn.
 template <int M>
-__global__ void __launch_bounds__(NTHREADS, 2) map_fwd_multi_kernel(MapDev g, MapCall c,
+__global__ void __launch_bounds__(BT, 4) map_fwd_multi_kernel(MapDev g, MapCall c,
                                                                     const float2* __restrict__ wdwB,
                                                                     const float2* __restrict__ wdwC) {
-    extern __shared__ float smem[];
+    extern __shared__ __align__(16) float smem[];
     __shared__ int s_tile;
     const int K = g.K;
-    const size_t fsz = multi_field_floats(K, M);
-    float* sF = smem;
-    float* sPiv = smem + 3 * fsz;  // [field][w d, w][32]
+    const size_t sub_floats = sub_floats_rt(K, M, false), field_ws = c.ws_floats / 3;
     double* slot = c.slots + (size_t)blockIdx.x * n_entries_multi(K, M);
-    const int lane = threadIdx.x & 31;
-    const float2* arr[3] = {c.wdw, wdwB, wdwC};
+    const long long nblk = c.nlin + (c.norb + c.tiles - 1) / c.tiles;
     for (;;) {
         if (threadIdx.x == 0) s_tile = atomicAdd(c.counter, 1);
         __syncthreads();
-        const long long tile = c.tile_lo + s_tile;
-        if (tile >= c.tile_hi) break;
-        const int2 tq = g.wtiles[tile];
-        if (tq.x < 0 || tq.x >= g.nrings) {
-            if (threadIdx.x == 0) atomicOr(c.status, ST_BAD_TILE);
+        const long long item = s_tile;
+        if (item >= nblk * c.parts) break;
+        const long long b = item / c.parts;
+        const int part = (int)(item - b * c.parts);
+        float* ws = c.ws + (c.parts > 1 ? (size_t)b : (size_t)blockIdx.x) * c.ws_floats;
+        const Block<M, false> B(g, c, b);
+        auto value = [&](int f, int s, int l) {
+            return B.value(g, c, PackedLoad{f == 0 ? c.wdw : (f == 1 ? wdwB : wdwC)}, s, l);
+        };
+        const unsigned live = block_live(B.nsub, [&](int s, int l) {
+            return value(0, s, l).y != 0.0f || value(1, s, l).y != 0.0f || value(2, s, l).y != 0.0f;
+        });
+        if (live == 0u) continue;
+#pragma unroll 1
+        for (int f = 0; f < 3; ++f) {
+            block_moments<M, false, false>(g, c, b, live, part, PackedLoad{f == 0 ? c.wdw : (f == 1 ? wdwB : wdwC)},
+                                           ws + f * field_ws, sub_floats, reinterpret_cast<char*>(smem), M);
             __syncthreads();
-            continue;
         }
-        const PivotRing P = pivot_ring(g, tq.x);
-        const bool lin = g.lin[P.i] != 0;
-        const TileSlot tp = tile_slot(lin, P.n_i, P.s_i, tq.y, lane);
-        const long long pix = g.ring_first[P.i] + tp.q;
-        const bool in = tp.valid && pix >= c.piv_lo && pix < c.piv_hi;
-        float2 pv[3];
-        bool live = false;
-#pragma unroll
-        for (int f = 0; f < 3; ++f) {
-            pv[f] = in ? arr[f][pix] : make_float2(0.0f, 0.0f);
-            live = live || pv[f].y != 0.0f;
-        }
-        const int qa = tile_slot(lin, P.n_i, P.s_i, tq.y, lane & 15).q;
-        const int qb = tile_slot(lin, P.n_i, P.s_i, tq.y, 16 + (lane & 15)).q;
-        if (!__syncthreads_or(live)) continue;
-        for (size_t e = threadIdx.x; e < 3 * fsz; e += NTHREADS) sF[e] = 0.0f;
-        if (threadIdx.x < TILE) {
-#pragma unroll
-            for (int f = 0; f < 3; ++f) {
-                sPiv[f * 2 * TILE + lane] = pv[f].x;
-                sPiv[f * 2 * TILE + TILE + lane] = pv[f].y;
-            }
-        }
-        __syncthreads();
-        for (int f = 0; f < 3; ++f) {
-            float* sA = sF + f * fsz;
-            float* sW = sA + (size_t)K * (M + 1) * 2 * TILE;
-            if (c.cells > 0)
-                walk_tile<M, false>(g, P, lin, qa, qb, tq.y, PackedLoad{arr[f]}, LayKM{sA, sW, nullptr, nullptr, M + 1},
-                                    reinterpret_cast<char*>(sPiv + 6 * TILE), c.cells, c.flush, M);
-            else  // the walk's scratch does not fit beside three fields' moments
-                tile_moments<M, false>(g, P, tp.q, PackedLoad{arr[f]}, sA, sW, nullptr, nullptr, c.flush, M);
-        }
-        __syncthreads();
-        tile_contract_multi<M>(K, sF, sPiv, slot);
+        if (!block_complete(c, b)) continue;
+        block_contract_multi(K, M, ws, field_ws, sub_floats, B.nsub, live, value, reinterpret_cast<char*>(smem), slot);
         __syncthreads();
     }
 }
@@ -1575,18 +1167,6 @@ __global__ void __launch_bounds__(NTHREADS) map_count_kernel(MapDev g, const flo
 }
 #endif
 
-// ------------------------------------------------------------------ adjoint
-//
-// dL/d d_p for L(zeta), with C_m = (dL/dRe zeta + i dL/dIm zeta) / D and
-// H_m(k,k') = conj(C_m(k,k')) + C_m(k',k) (prepared by the host side):
-//   primary term      w_p * (1/2) sum_{k,m} Re[a_m^k(p) h_m^k(p)]
-//   neighbour legs    w_p * sum_{i: p in nbr(i)} w_i d_i sum_m Re[e^{-i m phi_ip} h_m^{k(ip)}(i)]
-//   with h_m^k(i) = sum_{k'} H_m(k,k') conj(a_m^{k'}(i)).
-// A tile recomputes its a (as the forward), turns it into h in place, then sweeps its
-// neighbour rings again; each warp gathers its ring's contributions in a shared-memory
-// row buffer and flushes the row to the gradient with one atomic add per pixel.
-
-
 // val = sum_m (cos(m phi) hr_m + sin(m phi) hi_m): X the cosine part, Y the sine part.
 // h[m] = (hr_m, hi_m); the (cos, sin) chains run packed, in the folded frame psi, by
 // the recurrence of harmonics(); even and odd multipoles are summed apart and the odd
@@ -1629,407 +1209,31 @@ __device__ __forceinline__ void adj_harmonics(const float2 (&h)[M + 1], float cp
     adj_harmonicsf<M>(h, fold_angle(cph, sph), X, Y, mr);
 }
 
-// Where the contribution to pixel p (unwrapped index on ring R) goes.
-struct RowSink {
-    float* buf;     // warp row buffer, or NULL for direct global adds
-    int lo;         // buffer index = p - lo (window mode) ...
-    bool whole;     // ... or = wrap(p) (whole-ring mode)
-    float* grad;    // gradient row base (grad + first of ring)
-    int n;
-};
-
-__device__ __forceinline__ void sink_add(const RowSink& s, int p_unwrapped, int p_wrapped, float v) {
-    if (s.buf) {
-        atomicAdd(s.buf + (s.whole ? p_wrapped : p_unwrapped - s.lo), v);
-    } else {
-        atomicAdd(s.grad + p_wrapped, v);
-    }
-}
-
-template <int M>
-__device__ __forceinline__ void adj_harmonics2f(const float2 (&h)[M + 1], const Fold& fa, const Fold& fb, float& Xa,
-                                                float& Ya, float& Xb, float& Yb, int mr = M) {
-    float2 eva = make_float2(h[0].x, 0.0f), evb = eva;
-    float2 oda = make_float2(0.0f, 0.0f), odb = oda;
-    float sga = 1.0f, sgb = 1.0f;
-    if constexpr (M >= 1) {
-        if (mr < 1) {
-            Xa = Xb = eva.x;
-            Ya = Yb = eva.y;
-            return;
-        }
-        sga = fa.sg;
-        sgb = fb.sg;
-        float2 Ta = make_float2(fa.ac, fa.ss), Da = make_float2(0.5f * fa.lam, fa.ss);
-        float2 Tb = make_float2(fb.ac, fb.ss), Db = make_float2(0.5f * fb.lam, fb.ss);
-        const float2 La = make_float2(fa.lam, fa.lam), Lb = make_float2(fb.lam, fb.lam);
-        oda = __ffma2_rn(Ta, h[1], oda);
-        odb = __ffma2_rn(Tb, h[1], odb);
-#pragma unroll
-        for (int m = 2; m <= M; ++m) {
-            if (m > mr) break;
-            Da = __ffma2_rn(La, Ta, Da);
-            Db = __ffma2_rn(Lb, Tb, Db);
-            Ta = __fadd2_rn(Ta, Da);
-            Tb = __fadd2_rn(Tb, Db);
-            if (m & 1) {
-                oda = __ffma2_rn(Ta, h[m], oda);
-                odb = __ffma2_rn(Tb, h[m], odb);
-            } else {
-                eva = __ffma2_rn(Ta, h[m], eva);
-                evb = __ffma2_rn(Tb, h[m], evb);
-            }
-        }
-    }
-    Xa = fmaf(sga, oda.x, eva.x);
-    Ya = fmaf(sga, oda.y, eva.y);
-    Xb = fmaf(sgb, odb.x, evb.x);
-    Yb = fmaf(sgb, odb.y, evb.y);
-}
-
-template <int M>
-__device__ __forceinline__ void adj_harmonics2(const float2 (&h)[M + 1], float ca, float sa, float cb, float sb,
-                                               float& Xa, float& Ya, float& Xb, float& Yb, int mr = M) {
-    adj_harmonics2f<M>(h, fold_angle(ca, sa), fold_angle(cb, sb), Xa, Ya, Xb, Yb, mr);
-}
-
-template <int M, bool FAST, bool SELF = false>
-__device__ __forceinline__ void adj_run(const RingCtx& R, const float2* __restrict__ wdw, const LaneC& c,
-                                        int a, int len, const float2 (&h)[M + 1], float wdi, const RowSink& s,
-                                        float ck = 0.0f, int mr = M) {
-    const int maxlen = __reduce_max_sync(0xffffffffu, len);
-    const float i0 = (float)(a - c.cint);
-    const float xneg = -c.cfrac * R.step, uneg = -c.cfrac * R.inv_n;
-    int idx = wrap_idx(a, R.n);
-    const float2* row = wdw + R.first;
-    for (int t = 0; t < maxlen; t += 2) {
-        const bool on0 = t < len, on1 = t + 1 < len;
-        const int idx1 = idx + 1 >= R.n ? idx + 1 - R.n : idx + 1;
-        const float2 v0 = on0 ? __ldg(row + idx) : make_float2(0.0f, 0.0f);
-        const float2 v1 = on1 ? __ldg(row + idx1) : make_float2(0.0f, 0.0f);
-        const float oa = on0 ? i0 + (float)t : i0;
-        const float ob = on1 ? i0 + (float)(t + 1) : i0;
-        float ca, sa, cb, sb, Xa, Ya, Xb, Yb;
-        pixel_dir<FAST>(oa, xneg, uneg, R, ca, sa);
-        pixel_dir<FAST>(ob, xneg, uneg, R, cb, sb);
-        adj_harmonics2<M>(h, ca, sa, cb, sb, Xa, Ya, Xb, Yb, mr);
-        if (SELF) {  // self-pair subtraction: -2 cdiag_k (w_p d_p) per neighbour p
-            Xa = fmaf(ck, v0.x, Xa);
-            Xb = fmaf(ck, v1.x, Xb);
-        }
-        if (on0) sink_add(s, a + t, idx, wdi * v0.y * (Xa + Ya));
-        if (on1) sink_add(s, a + t + 1, idx1, wdi * v1.y * (Xb + Yb));
-        idx = idx1 + 1 >= R.n ? idx1 + 1 - R.n : idx1 + 1;
-    }
-}
-
-template <int M, bool FAST, bool SELF = false>
-__device__ __forceinline__ void adj_pairs(const RingCtx& R, const float2* __restrict__ wdw, const LaneC& c,
-                                          int a, int len, int mb, const float2 (&h)[M + 1], float wdi,
-                                          const RowSink& s, float ck = 0.0f, int mr = M) {
-    const int maxlen = __reduce_max_sync(0xffffffffu, len);
-    const float i0 = (float)(a - c.cint);
-    const float xneg = -c.cfrac * R.step, uneg = -c.cfrac * R.inv_n;
-    int ip = wrap_idx(a, R.n);
-    int im_ = wrap_idx(mb - a, R.n);
-    const float2* row = wdw + R.first;
-    for (int t = 0; t < maxlen; t += 2) {
-        const bool on0 = t < len, on1 = t + 1 < len;
-        const int ip1 = ip + 1 >= R.n ? ip + 1 - R.n : ip + 1;
-        const int im1 = im_ - 1 < 0 ? im_ - 1 + R.n : im_ - 1;
-        const float2 p0 = on0 ? __ldg(row + ip) : make_float2(0.0f, 0.0f);
-        const float2 m0 = on0 ? __ldg(row + im_) : make_float2(0.0f, 0.0f);
-        const float2 p1 = on1 ? __ldg(row + ip1) : make_float2(0.0f, 0.0f);
-        const float2 m1 = on1 ? __ldg(row + im1) : make_float2(0.0f, 0.0f);
-        const float oa = on0 ? i0 + (float)t : i0;
-        const float ob = on1 ? i0 + (float)(t + 1) : i0;
-        float ca, sa, cb, sb, Xa, Ya, Xb, Yb;
-        pixel_dir<FAST>(oa, xneg, uneg, R, ca, sa);
-        pixel_dir<FAST>(ob, xneg, uneg, R, cb, sb);
-        adj_harmonics2<M>(h, ca, sa, cb, sb, Xa, Ya, Xb, Yb, mr);
-        if (on0) {
-            sink_add(s, a + t, ip, wdi * p0.y * (Xa + Ya + (SELF ? ck * p0.x : 0.0f)));
-            sink_add(s, mb - a - t, im_, wdi * m0.y * (Xa - Ya + (SELF ? ck * m0.x : 0.0f)));
-        }
-        if (on1) {
-            sink_add(s, a + t + 1, ip1, wdi * p1.y * (Xb + Yb + (SELF ? ck * p1.x : 0.0f)));
-            sink_add(s, mb - a - t - 1, im1, wdi * m1.y * (Xb - Yb + (SELF ? ck * m1.x : 0.0f)));
-        }
-        ip = ip1 + 1 >= R.n ? ip1 + 1 - R.n : ip1 + 1;
-        im_ = im1 - 1 < 0 ? im1 - 1 + R.n : im1 - 1;
-    }
-}
-
-// adj_pairs for a belt ring pair, with the position angles shared across the warp
-// (see walk_pairs_shared).
-template <int M, bool SELF = false>
-__device__ __forceinline__ void adj_pairs_shared(const RingCtx& R, const float2* __restrict__ wdw, const LaneC& c,
-                                                 int a, int len, int mb, const float2 (&h)[M + 1], float wdi,
-                                                 const RowSink& s, float ck = 0.0f, int mr = M) {
-    if (len <= 0) return;
-    const int lane = threadIdx.x & 31;
-    const float i0 = (float)(a - c.cint);
-    const float xneg = -c.cfrac * R.step, uneg = -c.cfrac * R.inv_n;
-    int ip = wrap_idx(a, R.n);
-    int im_ = wrap_idx(mb - a, R.n);
-    const float2* row = wdw + R.first;
-    for (int t0 = 0; t0 < len; t0 += 32) {
-        Fold mine;
-        {
-            const float ft = i0 + (float)(t0 + lane);
-            float cph, sph;
-            if (fabsf(ft - c.cfrac) * R.step <= FAST_XMAX)
-                pixel_dir<true>(ft, xneg, uneg, R, cph, sph);
-            else
-                pixel_dir<false>(ft, xneg, uneg, R, cph, sph);
-            mine = fold_angle(cph, sph);
-        }
-        const int nstep = min(32, len - t0);
-        for (int tt = 0; tt < nstep; tt += 2) {
-            const int t = t0 + tt;
-            const bool two = tt + 1 < nstep;
-            const Fold fa = shfl_fold(mine, tt), fb = shfl_fold(mine, two ? tt + 1 : tt);
-            const int ip1 = ip + 1 >= R.n ? ip + 1 - R.n : ip + 1;
-            const int im1 = im_ - 1 < 0 ? im_ - 1 + R.n : im_ - 1;
-            const float2 p0 = __ldg(row + ip), m0 = __ldg(row + im_);
-            const float2 p1 = two ? __ldg(row + ip1) : make_float2(0.0f, 0.0f);
-            const float2 m1 = two ? __ldg(row + im1) : make_float2(0.0f, 0.0f);
-            float Xa, Ya, Xb, Yb;
-            adj_harmonics2f<M>(h, fa, fb, Xa, Ya, Xb, Yb, mr);
-            sink_add(s, a + t, ip, wdi * p0.y * (Xa + Ya + (SELF ? ck * p0.x : 0.0f)));
-            sink_add(s, mb - a - t, im_, wdi * m0.y * (Xa - Ya + (SELF ? ck * m0.x : 0.0f)));
-            if (two) {
-                sink_add(s, a + t + 1, ip1, wdi * p1.y * (Xb + Yb + (SELF ? ck * p1.x : 0.0f)));
-                sink_add(s, mb - a - t - 1, im1, wdi * m1.y * (Xb - Yb + (SELF ? ck * m1.x : 0.0f)));
-            }
-            ip = ip1 + 1 >= R.n ? ip1 + 1 - R.n : ip1 + 1;
-            im_ = im1 - 1 < 0 ? im1 - 1 + R.n : im1 - 1;
-        }
-    }
-}
-
-// Neighbour legs of one ring r for the warp's lanes (all bins of r).
-template <int M, bool SELF = false>
-__device__ __forceinline__ void adj_ring(const MapDev& g, const PivotRing& P, int r, int q, float wdi,
-                                         const float2* __restrict__ wdw, const float* sH, float* rowbuf,
-                                         float* grad, int* status,
-                                         const float* cdiag = nullptr, int mr = M) {
-    const int lane = threadIdx.x & 31;
-    const long long pr = P.pair0 + (r - P.rlo);
-    const int2 TK = g.pair_T[pr * (g.K + 1) + g.K];
-    if (TK.x == T_ZERO) return;
-    const RingCtx R = ring_ctx(g, P, r, pr);
-    const ExactCtx x = exact_ctx(g, P, r);
-    const LaneC c = lane_c(q, P.s_i, P.n_i, R.shift, R.n);
-    // row window: every pixel of r within the outer edge of some lane's pivot
-    RowSink s;
-    s.grad = grad + R.first;
-    s.n = R.n;
-    s.whole = false;
-    s.lo = 0;
-    s.buf = rowbuf;
-    int width;
-    {
-        const int clo = __shfl_sync(0xffffffffu, c.cint, 0);
-        const int chi = __shfl_sync(0xffffffffu, c.cint, 31);
-        if (TK.x != T_INF) {
-            s.lo = clo - TK.x - 2;
-            width = chi + TK.x + 3 - s.lo + 1;
-        } else {
-            width = ROW + 1;
-        }
-        if (width > ROW || width >= R.n) {
-            if (R.n <= ROW) {
-                s.whole = true;
-                width = R.n;
-            } else {
-                s.buf = nullptr;
-                width = 0;
-                if (lane == 0) atomicOr(status, ST_ROW_OVERFLOW);
-            }
-        }
-    }
-    for (int e = lane; e < width; e += 32) rowbuf[e] = 0.0f;
-    __syncwarp();
-    for (int k = 0; k < g.K; ++k) {
-        const int2 br = g.bin_range[(long long)P.i * g.K + k];
-        if (r < br.x || r > br.y) continue;
-        const int2 Tk = g.pair_T[pr * (g.K + 1) + k];
-        const int2 Tk1 = g.pair_T[pr * (g.K + 1) + k + 1];
-        if (Tk.x == T_INF || Tk1.x == T_ZERO) continue;
-        float2 h[M + 1];
-        const float* hk = sH + (size_t)k * (mr + 1) * 2 * TILE;
-#pragma unroll
-        for (int m = 0; m <= M; ++m) {
-            h[m] = m <= mr ? make_float2(hk[(2 * m) * TILE + lane], hk[(2 * m + 1) * TILE + lane])
-                           : make_float2(0.0f, 0.0f);
-        }
-        const bool sym = (R.n == P.n_i) && (Tk1.x != T_INF);
-        const BinRuns b = bin_runs(c, Tk, Tk1, g.E[k], g.E[k + 1], x, R.n, sym);
-        const float ck = SELF ? -2.0f * cdiag[k] : 0.0f;
-        if (sym) {
-            if (b.centre) {
-                const int p = c.cint;
-                const int pw = wrap_idx(p, R.n);
-                const float2 v = __ldg(wdw + R.first + pw);
-                float cph, sph, X, Y;
-                pixel_dir<false>(0.0f, 0.0f, -c.cfrac * R.inv_n, R, cph, sph);
-                adj_harmonics<M>(h, cph, sph, X, Y, mr);
-                if (SELF) X = fmaf(ck, v.x, X);
-                sink_add(s, p, pw, wdi * v.y * (X + Y));
-            }
-            if (runs_shared(c, b.a0, b.n0)) {
-                adj_pairs_shared<M, SELF>(R, wdw, c, b.a0, b.n0, b.mb, h, wdi, s, ck, mr);
-            } else {
-                const bool fast = __all_sync(0xffffffffu, run_omax(c, b.a0, b.n0) * R.step <= FAST_XMAX);
-                if (fast)
-                    adj_pairs<M, true, SELF>(R, wdw, c, b.a0, b.n0, b.mb, h, wdi, s, ck, mr);
-                else
-                    adj_pairs<M, false, SELF>(R, wdw, c, b.a0, b.n0, b.mb, h, wdi, s, ck, mr);
-            }
-        } else {
-            const float om = fmaxf(run_omax(c, b.a0, b.n0), run_omax(c, b.a1, b.n1));
-            const bool fast = __all_sync(0xffffffffu, om * R.step <= FAST_XMAX);
-            if (fast) {
-                adj_run<M, true, SELF>(R, wdw, c, b.a0, b.n0, h, wdi, s, ck, mr);
-                adj_run<M, true, SELF>(R, wdw, c, b.a1, b.n1, h, wdi, s, ck, mr);
-            } else {
-                adj_run<M, false, SELF>(R, wdw, c, b.a0, b.n0, h, wdi, s, ck, mr);
-                adj_run<M, false, SELF>(R, wdw, c, b.a1, b.n1, h, wdi, s, ck, mr);
-            }
-        }
-    }
-    __syncwarp();
-    if (s.buf) {
-        for (int e = lane; e < width; e += 32) {
-            const float v = rowbuf[e];
-            if (v != 0.0f) {
-                const int pw = s.whole ? e : wrap_idx(s.lo + e, R.n);
-                atomicAdd(s.grad + pw, v);
-            }
-        }
-        __syncwarp();
-    }
-}
-
-// One adjoint tile (all three phases).  Called by every thread of the CTA.  With
-// SELF (self-pair subtraction) the subtracted diagonal adds, per bin k with
-// cdiag_k = sum_m Re C_m(k,k), -w_p Q^k(p) cdiag_k to a pivot and
-// -2 w_p^2 d_p w_i d_i cdiag_k to each neighbour p of pivot i.
-template <int M, bool SELF = false>
-__device__ __forceinline__ void bwd_tile(const MapDev& g, const MapCall& c, int tile, float* smem, int mr = M) {
-    const int K = g.K;
-    float* sA = smem;
-    float* sW = sA + (size_t)K * (mr + 1) * 2 * TILE;
-    float* sQ = sW + K * TILE;
-    float* sQW = sQ + K * TILE;
-    float* sPiv = SELF ? sQW + K * TILE : sQ;
-    float* sPrim = sPiv + 2 * TILE;
-    char* scratch = reinterpret_cast<char*>(sPrim + TILE);
-    float* sHm = reinterpret_cast<float*>(scratch);   // phase 2: [K][K][2], one m at a time
-    float* sRow = reinterpret_cast<float*>(scratch);  // phase 3: [NWARPS][ROW]
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const size_t nfl = tile_floats_rt(K, mr, SELF) - 2 * TILE;
-
-    const int2 tq = g.tiles[tile];
-    if (tq.x < 0 || tq.x >= g.nrings) {
-        if (threadIdx.x == 0) atomicOr(c.status, ST_BAD_TILE);
-        __syncthreads();
-        return;
-    }
-    const PivotRing P = pivot_ring(g, tq.x);
-    const int q = tq.y + lane;
-    const long long pix = g.ring_first[P.i] + q;
-    const bool in = (q < P.n_i) && pix >= c.piv_lo && pix < c.piv_hi;
-    const float2 pv = in ? c.wdw[pix] : make_float2(0.0f, 0.0f);
-    const int qg = min(q, P.n_i - 1);  // see map_fwd_kernel
-    if (!__syncthreads_or(pv.y != 0.0f)) return;  // no pivot with w != 0: no term
-    for (size_t e = threadIdx.x; e < nfl; e += NTHREADS) sA[e] = 0.0f;
-    if (threadIdx.x < TILE) {
-        sPiv[lane] = pv.x;
-        sPiv[TILE + lane] = pv.y;
-        sPrim[lane] = 0.0f;
-    }
-    __syncthreads();
-    // phase 1: the tile's moments, exactly as in the forward
-    if (g.lin[P.i])
-        walk_tile<M, SELF>(g, P, true, tile_slot(true, P.n_i, P.s_i, tq.y, lane & 15).q,
-                           tile_slot(true, P.n_i, P.s_i, tq.y, 16 + (lane & 15)).q, tq.y, PackedLoad{c.wdw},
-                           LayKM{sA, sW, sQ, sQW, mr + 1}, scratch, c.cells, c.flush, mr);
-    else
-        tile_moments<M, SELF>(g, P, qg, PackedLoad{c.wdw}, sA, sW, sQ, sQW, c.flush, mr);
-    __syncthreads();
-    // phase 2: h = H conj(a) per m, in place; primary term (1/2) sum Re[a h]
-    for (int m = 0; m <= mr; ++m) {
-        for (int e = threadIdx.x; e < K * K * 2; e += NTHREADS)
-            sHm[e] = c.H[(size_t)m * K * K * 2 + e];
-        __syncthreads();
-        float hrv[(TPCF_MAX_BINS * TILE + NTHREADS - 1) / NTHREADS];
-        float hiv[(TPCF_MAX_BINS * TILE + NTHREADS - 1) / NTHREADS];
-        int nmine = 0;
-        for (int e = threadIdx.x; e < K * TILE; e += NTHREADS, ++nmine) {
-            const int k = e / TILE, l = e - k * TILE;
-            float hr = 0.0f, hi = 0.0f;
-            for (int kp = 0; kp < K; ++kp) {
-                const float Hr = sHm[(k * K + kp) * 2], Hi = sHm[(k * K + kp) * 2 + 1];
-                const float* ap = sA + ((size_t)kp * (mr + 1) + m) * 2 * TILE;
-                const float tr = ap[l], ti = ap[TILE + l];
-                hr = fmaf(Hr, tr, fmaf(-Hi, ti, hr));
-                hi = fmaf(Hr, ti, fmaf(Hi, tr, hi));
-            }
-            const float* ak = sA + ((size_t)k * (mr + 1) + m) * 2 * TILE;
-            atomicAdd(sPrim + l, fmaf(ak[l], hr, ak[TILE + l] * hi));
-            hrv[nmine] = hr;
-            hiv[nmine] = hi;
-        }
-        __syncthreads();
-        nmine = 0;
-        for (int e = threadIdx.x; e < K * TILE; e += NTHREADS, ++nmine) {
-            const int k = e / TILE, l = e - k * TILE;
-            float* ak = sA + ((size_t)k * (mr + 1) + m) * 2 * TILE;
-            ak[l] = hrv[nmine];
-            ak[TILE + l] = hiv[nmine];
-        }
-        __syncthreads();
-    }
-    const float* cdiag = SELF ? c.H + (size_t)(mr + 1) * K * K * 2 : nullptr;
-    if (threadIdx.x < TILE && in) {
-        float gp = 0.5f * pv.y * sPrim[lane];
-        if (SELF) {
-            float t = 0.0f;
-            for (int k = 0; k < K; ++k) t = fmaf(cdiag[k], sQ[k * TILE + lane], t);
-            gp = fmaf(-pv.y, t, gp);
-        }
-        if (gp != 0.0f) atomicAdd(c.grad + pix, gp);
-    }
-    __syncthreads();  // the row buffers of phase 3 overlay sPrim and the rest
-    // phase 3: neighbour legs, warps split the neighbour rings
-    const int2 rr = g.ring_range[P.i];
-    for (int r = rr.x + warp; r <= rr.y; r += NWARPS)
-        adj_ring<M, SELF>(g, P, r, qg, pv.x, c.wdw, sA, sRow + (size_t)warp * ROW, c.grad, c.status, cdiag, mr);
-    __syncthreads();
-}
-
-template <int M, bool SELF, int OCC = 3>
-__global__ void __launch_bounds__(NTHREADS, OCC) map_bwd_kernel(MapDev g, MapCall c) {
-    extern __shared__ float smem[];
+// Adjoint: persistent CTAs draw work items (block, part); c.step: see bwd_block.
+template <int M, bool SELF>
+__global__ void __launch_bounds__(BT, 4) map_bwd_kernel(MapDev g, MapCall c) {
+    extern __shared__ __align__(16) float smem[];
     __shared__ int s_tile;
+    const long long nblk = c.nlin + (c.norb + c.tiles - 1) / c.tiles;
     for (;;) {
         if (threadIdx.x == 0) s_tile = atomicAdd(c.counter, 1);
         __syncthreads();
-        const long long tile = c.tile_lo + s_tile;
-        if (tile >= c.tile_hi) break;
-        bwd_tile<M, SELF>(g, c, (int)tile, smem);
+        const long long item = s_tile;
+        if (item >= nblk * c.parts) break;
+        const long long b = item / c.parts;
+        float* ws = c.ws + (c.step != 0 ? (size_t)b : (size_t)blockIdx.x) * c.ws_floats;
+        bwd_block<M, SELF>(g, c, b, (int)(item - b * c.parts), c.step, ws, reinterpret_cast<char*>(smem), M);
     }
 }
 
+// The adjoint of all the plans of a batch, one launch (the work queue of batch_fwd_kernel).
 template <int M>
-__global__ void __launch_bounds__(NTHREADS, 2) batch_bwd_kernel(const BatchItem* __restrict__ items, int n,
+__global__ void __launch_bounds__(BT, 4) batch_bwd_kernel(const BatchItem* __restrict__ items, int n,
                                                                long long total, unsigned long long* counter) {
-    extern __shared__ float smem[];
+    extern __shared__ __align__(16) float smem[];
     __shared__ long long s_t;
     __shared__ long long s_first[TPCF_MAX_BATCH + 1];
-    for (int i = threadIdx.x; i <= n; i += NTHREADS) s_first[i] = i < n ? items[i].tile0 : total;
+    for (int i = threadIdx.x; i <= n; i += BT) s_first[i] = i < n ? items[i].tile0 : total;
     __syncthreads();
     for (;;) {
         if (threadIdx.x == 0) s_t = (long long)atomicAdd(counter, 1ull);
@@ -2041,7 +1245,10 @@ __global__ void __launch_bounds__(NTHREADS, 2) batch_bwd_kernel(const BatchItem*
             const int mid = (lo + hi + 1) / 2;
             if (s_first[mid] <= t) lo = mid; else hi = mid - 1;
         }
-        bwd_tile<M>(items[lo].g, items[lo].c, (int)(t - s_first[lo]), smem, items[lo].g.M);
+        const MapDev& g = items[lo].g;
+        const MapCall& c = items[lo].c;
+        bwd_block<M, false>(g, c, t - s_first[lo], 0, 0, c.ws + (size_t)blockIdx.x * c.ws_floats,
+                            reinterpret_cast<char*>(smem), g.M);
     }
 }
 

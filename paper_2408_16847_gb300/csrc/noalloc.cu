@@ -5,8 +5,8 @@
 // the pool), programs whose hot loop must not enter the CUDA allocator because
 // cudaMalloc/cudaFree can synchronise the device, and embedders that account for
 // every byte of device memory.  They create the plan once, during set-up, and then
-// call this entry point, which uses only the caller's buffers, the plan's
-// read-only tables and the fixed scratch array below.
+// call this entry point, which uses only the caller's buffers, the plan's tables and
+// workspace (allocated with the plan) and the fixed scratch array below.
 //
 // The scratch lives in a file-scope __device__ array.  This file is its own CUDA
 // module, and CUDA loads modules lazily, so the array is placed on a device when its
@@ -19,6 +19,7 @@
 #include <cuda_runtime.h>
 #include <string.h>
 
+#include <algorithm>
 #include <mutex>
 
 #include "geometry.cuh"
@@ -121,7 +122,7 @@ extern "C" tpcf_status tpcf_forward_noalloc(tpcf_plan plan, const float* d_delta
     double* sums = (double*)(base + NOALLOC_HEADER);
     double* slots = (double*)(base + NOALLOC_HEADER + sums_bytes);
     const size_t room = (NOALLOC_SCRATCH_BYTES - NOALLOC_HEADER - sums_bytes) / slot_bytes;
-    const int grid = (int)std::min<size_t>((size_t)plan->fwd_grid, room);
+    const int grid = (int)std::min<size_t>((size_t)std::min(plan->fwd_grid, plan->ws_slots), room);
     cudaStream_t s = (cudaStream_t)stream;
     plan->last_stream = s;
     TRY_CUDA(cudaMemsetAsync(counter, 0, sizeof(int), s));
@@ -137,10 +138,18 @@ extern "C" tpcf_status tpcf_forward_noalloc(tpcf_plan plan, const float* d_delta
     c.self_subtract = 0;
     c.norm = norm_of_flags(plan->flags);
     c.flush = plan->tune_fwd.flush;
-    c.tile_lo = 0;  // every tile; those without a pivot in range return at once
-    c.tile_hi = plan->map.nwtiles;
+    // every block; those without a pivot in range return at once
+    c.lin_list = plan->map.lin_list;
+    c.orb_list = plan->map.orb_list;
+    c.nlin = plan->lin_off_h.back();
+    c.norb = plan->orb_off_h.back();
+    c.tiles = 2;
+    c.parts = 1;
+    c.ws = plan->ws;
+    c.ws_floats = plan->ws_floats;
+    c.cells = LIN_CELLS;
     TRY_CUDA(kDirect[plan->M](plan->map, c, grid, s));
-    reduce_slots_kernel<<<(plan->nent + 127) / 128, 128, 0, s>>>(slots, grid, plan->nent, sums);
+    reduce_slots_kernel<<<(plan->nent + 31) / 32, REDUCE_THREADS, 0, s>>>(slots, grid, plan->nent, sums);
     const int nout = (plan->M + 1) * plan->K * plan->K;
     finalize_kernel<<<(nout + 127) / 128, 128, 0, s>>>(sums, plan->K, plan->M, 0, 1.0, d_zeta, d_norm, nullptr);
     TRY_CUDA(cudaGetLastError());

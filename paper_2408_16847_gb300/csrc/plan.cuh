@@ -40,15 +40,20 @@ struct tpcf_plan_s {
     MapDev map{};
     tpcf::CatDev cat{};
     std::vector<int64_t> tile_off_h;   // map plans: first tile of each ring (host copy)
-    std::vector<int64_t> wtile_off_h;  // map plans: first walk tile of each ring
-    std::vector<unsigned char> lin_h;  // map plans: ring has linear walk tiles
-    // launch configuration of the map pair kernels (defaults, or picked by the autotuner):
-    // register variant (CTAs per SM the registers are sized for), CTAs per SM launched,
-    // rings summed in registers per shared-memory flush
+    // map plans: first linear block and first warp tile of each ring (and the totals), whether the
+    // ring has linear blocks (map_block.cuh)
+    std::vector<int64_t> lin_off_h, orb_off_h;
+    std::vector<unsigned char> lin_h;
+    float* ws = nullptr;  // workspace of the block kernels: ws_slots blocks of ws_floats
+    int ws_slots = 0;
+    size_t ws_floats = 0;
+    // launch configuration of the map pair kernels (defaults, or picked by the autotuner): pairs of
+    // CTAs per SM launched, and the entries summed in registers before they are added to the
+    // workspace, in units of 32; the register variant (3 or 2, one kernel serves both)
     // and, for the forward, a tile-layout choice that is kept for callers that store configurations
-    // (the layout follows from the ring, map_walk.cuh)
+    // (the layout follows from the ring, map_block.cuh)
     struct Tune {
-        int variant = 3, ctas = 0, flush = 8, quad = 0;
+        int variant = 2, ctas = 0, flush = 8, quad = 0;
     } tune_fwd, tune_bwd;
     bool tuned = false;
     // per-call scratch
@@ -63,12 +68,13 @@ struct tpcf_plan_s {
     // multi-field forward (allocated on its first call): packed fields B and C, slots
     float2* wdw_b = nullptr;
     float2* wdw_c = nullptr;
+    float* ws3 = nullptr;  // workspace: three fields per block
     double* mslots = nullptr;
     double* msums = nullptr;
     int multi_grid = 0;
     // shared-neighbour-list forward: tile list of the last group size used
-    int2* gtiles = nullptr;
-    int64_t ngtiles = 0, gtiles_cap = 0;
+    int2* gtiles = nullptr;  // linear blocks, then warp tiles
+    int64_t nglin = 0, ngorb = 0, gtiles_cap = 0;
     int ggroup = 0;
     // staging for tpcf_run_host
     float* st_delta = nullptr;

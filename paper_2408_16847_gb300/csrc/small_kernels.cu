@@ -16,19 +16,51 @@ __global__ void pack_kernel(const float* __restrict__ delta, const float* __rest
     if (blockIdx.x == 0 && threadIdx.x == 0) wdw[n] = make_float2(0.0f, 0.0f);
 }
 
+// Everything a map forward needs before its pair kernel, in one launch: the packed map, zeroed CTA
+// slots (nz doubles) and counters (nc ints).  Apart they were three small launches, which
+// small maps spend more time on than on the sums.
+__global__ void fwd_prep_kernel(const float* __restrict__ delta, const float* __restrict__ w, float2* wdw, int64_t n,
+                                double* slots, int64_t nz, int* counters, int nc) {
+    const int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, step = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t i = t0; i < n; i += step) {
+        const float wi = w[i];
+        wdw[i] = make_float2(wi * delta[i], wi);
+    }
+    if (t0 == 0) wdw[n] = make_float2(0.0f, 0.0f);
+    for (int64_t i = t0; i < nz; i += step) slots[i] = 0.0;
+    for (int64_t i = t0; i < nc; i += step) counters[i] = 0;
+}
+
 __global__ void zero_f32_kernel(float* p, int64_t n) {
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
          i += (int64_t)gridDim.x * blockDim.x)
         p[i] = 0.0f;
 }
 
-// sums[e] = sum over CTA slots of slots[s * nent + e], in FP64.
-__global__ void reduce_slots_kernel(const double* __restrict__ slots, int nslots, int nent, double* sums) {
-    const int e = blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= nent) return;
+// sums[e] = sum over CTA slots of slots[s * nent + e], in FP64.  A block takes 32 entries, a warp
+// of it every 32nd slot: with one thread per entry going over all slots the chain of loads took
+// longer than a small map's pair kernel.
+__device__ __forceinline__ void reduce_slots_block(const double* __restrict__ slots, int nslots, int nent, double* sums) {
+    __shared__ double part[32][33];
+    const int lane = threadIdx.x & 31, row = threadIdx.x >> 5;
+    const int e = blockIdx.x * 32 + lane;
     double acc = 0.0;
-    for (int s = 0; s < nslots; ++s) acc += slots[(size_t)s * nent + e];
-    sums[e] = acc;
+    if (e < nent) {
+#pragma unroll 4
+        for (int s = row; s < nslots; s += 32) acc += slots[(size_t)s * nent + e];
+    }
+    part[row][lane] = acc;
+    __syncthreads();
+    if (row == 0 && e < nent) {
+        acc = 0.0;
+        for (int r = 0; r < 32; ++r) acc += part[r][lane];
+        sums[e] = acc;
+    }
+}
+
+__global__ void __launch_bounds__(REDUCE_THREADS) reduce_slots_kernel(const double* __restrict__ slots, int nslots,
+                                                                      int nent, double* sums) {
+    reduce_slots_block(slots, nslots, nent, sums);
 }
 
 // zeta_m(k1,k2) = S_m(k1,k2) / (scale * D(k1,k2)), Hermitian fill of the lower triangle,
@@ -117,18 +149,38 @@ __device__ __forceinline__ void adjoint_prep_one(const double* __restrict__ dL, 
 
 // With self-pair subtraction H is followed by cdiag_k = sum_m Re dL_m(k,k) / D(k,k)
 // (the subtracted diagonal enters every m with the same real weight).
+__device__ __forceinline__ void adjoint_diag_one(const double* __restrict__ dL, const double* __restrict__ norm, int K,
+                                                 int M, float* H, int k) {
+    const double d = norm[k * K + k];
+    double t = 0.0;
+    if (d != 0.0)
+        for (int m = 0; m <= M; ++m) t += dL[2 * ((size_t)m * K * K + (size_t)k * K + k)] / d;
+    H[(size_t)(M + 1) * K * K * 2 + k] = (float)t;
+}
+
 __global__ void adjoint_prep_kernel(const double* __restrict__ dL, const double* __restrict__ norm, int K,
                                     int M, float* H, int with_diag) {
     const int idx = blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= (M + 1) * K * K) return;
     adjoint_prep_one(dL, norm, K, H, idx);
-    if (with_diag && idx < K) {
-        const double d = norm[idx * K + idx];
-        double t = 0.0;
-        if (d != 0.0)
-            for (int m = 0; m <= M; ++m) t += dL[2 * ((size_t)m * K * K + (size_t)idx * K + idx)] / d;
-        H[(size_t)(M + 1) * K * K * 2 + idx] = (float)t;
+    if (with_diag && idx < K) adjoint_diag_one(dL, norm, K, M, H, idx);
+}
+
+// The same for an adjoint: the packed map, the zeroed gradient, H (and cdiag) and the counters.
+__global__ void bwd_prep_kernel(const float* __restrict__ delta, const float* __restrict__ w, float2* wdw, float* grad,
+                                int64_t n, const double* __restrict__ dL, const double* __restrict__ norm, int K, int M,
+                                float* H, int with_diag, int* counters, int nc) {
+    const int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, step = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t i = t0; i < n; i += step) {
+        const float wi = w[i];
+        wdw[i] = make_float2(wi * delta[i], wi);
+        grad[i] = 0.0f;
     }
+    if (t0 == 0) wdw[n] = make_float2(0.0f, 0.0f);
+    for (int64_t i = t0; i < (M + 1) * K * K; i += step) adjoint_prep_one(dL, norm, K, H, (int)i);
+    if (with_diag)
+        for (int64_t i = t0; i < K; i += step) adjoint_diag_one(dL, norm, K, M, H, (int)i);
+    for (int64_t i = t0; i < nc; i += step) counters[i] = 0;
 }
 
 // ------------------------------------------------------------------ batches
@@ -158,13 +210,9 @@ __global__ void batch_zero_kernel(const BatchIO* __restrict__ io, int with_grad)
             b.grad[i] = 0.0f;
 }
 
-__global__ void batch_reduce_kernel(const BatchIO* __restrict__ io) {
+__global__ void __launch_bounds__(REDUCE_THREADS) batch_reduce_kernel(const BatchIO* __restrict__ io) {
     const BatchIO& b = io[blockIdx.y];
-    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < b.nent; e += gridDim.x * blockDim.x) {
-        double acc = 0.0;
-        for (int s = 0; s < b.nslots; ++s) acc += b.slots[(size_t)s * b.nent + e];
-        b.sums[e] = acc;
-    }
+    reduce_slots_block(b.slots, b.nslots, b.nent, b.sums);
 }
 
 __global__ void batch_finalize_kernel(const BatchIO* __restrict__ io) {

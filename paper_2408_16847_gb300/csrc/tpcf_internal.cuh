@@ -12,6 +12,8 @@ namespace tpcf {
 constexpr int TILE = 32;     // pivots per tile: one pivot per lane
 constexpr int NWARPS = 8;    // warps per CTA; they split the neighbour rings of a tile
 constexpr int NTHREADS = TILE * NWARPS;
+constexpr int BW = 4;        // warps per CTA of the block kernels (map_block.cuh), four CTAs per SM
+constexpr int BT = TILE * BW;
 
 // Threshold encoding of pair_T entries (see geometry.cu).
 constexpr int T_ZERO = -1;          // every pixel of ring r is at or beyond the edge
@@ -40,8 +42,8 @@ struct MapDev {
     const int2* pair_T;         // [npairs * (K+1)] edge offsets T_e in ring-r pixels
     const int2* tiles;          // [ntiles] (ring, first pivot index in ring): 32 consecutive pivots
     int64_t ntiles;
-    const int2* wtiles;         // [nwtiles] (ring, first pivot or orbit): the walk's tiles (map_walk.cuh)
-    int64_t nwtiles;
+    const int2* lin_list;       // linear blocks (ring, first pivot): BT walk_np consecutive pivots (map_block.cuh)
+    const int2* orb_list;       // warp tiles (ring, first position) of the other rings: 32 positions and their turned images
     const unsigned char* lin;   // [nrings] 1: linear walk tiles (every neighbour ring has n_i pixels)
     const int* ring_reach;      // [nrings] pixels that a linear tile's rows reach beyond a pivot
     const float4* rc;           // [2 * nrings] (s, s_lo, step, step_lo), (1/n, its lo, 2 n + shift, first)
@@ -87,7 +89,16 @@ struct MapCall {
     int flush;              // rings summed in registers before a shared-memory flush (tuned)
     int64_t tile_lo, tile_hi;  // tiles that can hold a pivot of [piv_lo, piv_hi)
     int norm;               // NORM_*: per-pivot normalisation of the moments before the contraction
-    int cells;              // cell table of the walk (map_walk.cuh); 0: the per-lane path
+    // blocks of the call (map_block.cuh): nlin of lin_list from lin_lo, then norb warp tiles of
+    // orb_list from orb_lo, `tiles` to a block; each block in `parts` by bins
+    const int2 *lin_list, *orb_list;
+    long long lin_lo, nlin, orb_lo, norb;
+    int tiles, parts;
+    int* done;              // parts > 1: [blocks] finished parts (zeroed before launch)
+    int step;               // adjoint: phases of this launch (bwd_block)
+    float* ws;              // workspace: per block (parts > 1) or per CTA
+    size_t ws_floats;       // floats of a block's workspace
+    int cells;              // cells listed at a time on linear rings
     int group;              // > 1: shared neighbour lists, one lane per run of `group` ring pixels
     const int2* gtiles;     // group > 1: tiles (ring, first run of the tile)
 };
@@ -120,7 +131,47 @@ inline __host__ __device__ int n_entries(int K, int M) {
 // Entries of the multi-field partial sums: full K x K matrices, S (complex) per m, then D.
 inline __host__ __device__ int n_entries_multi(int K, int M) { return 2 * (M + 1) * K * K + K * K; }
 
-constexpr int ROW = 512;  // floats per warp row buffer of the adjoint (wider rows: whole-ring or global adds)
+// Pivots per lane of the block kernels (map_block.cuh): 2 bins' sums of M + 1 multipoles each
+// take 4 (M + 1) registers.
+__host__ __device__ constexpr int walk_np(int M) { return 2; }
+// Floats of 32 pivots' moments in the workspace: A[m][k][re/im][32], W[k][32], and Q, QW with
+// self-pair subtraction; and of a block's.
+__host__ __device__ inline size_t sub_floats_rt(int K, int mr, bool self) {
+    return (size_t)K * (mr + 1) * 2 * TILE + (self ? 3 : 1) * (size_t)K * TILE;
+}
+inline size_t block_floats(int K, int mr, int M, bool self) { return (size_t)BW * walk_np(M) * sub_floats_rt(K, mr, self); }
+constexpr int LIN_MIN = 256;  // smallest ring that is worth a linear block
+constexpr int LIN_CELLS = 1024;       // (bin, ring) cells listed at a time (6 bytes each)
+constexpr int LIN_CHUNK = BT;         // entries staged at a time, one per thread
+constexpr int LIN_HEAD = 512;         // small tables
+constexpr int CON_STAGE = 35 * 1024;  // bytes of moments staged by the contraction
+// Bytes of a staged entry of the linear walk: two pixel offsets and a weight, then 8 bytes per
+// multipole; an odd number of 16-byte words against bank conflicts of the staging stores.
+__host__ __device__ constexpr int lin_stride(int M) { return 16 * (((M + 1) / 2 + 1) | 1); }
+constexpr int ORB_STRIDE = 80;        // bytes of a staged ring of the other rings' walk (64, odd in 16-byte words)
+// Shared memory (bytes) of a block kernel: the linear walk's tables and two chunks, or each warp's
+// staged rings, or the contraction's stage with the pivots' values of up to three fields.
+__host__ __device__ constexpr size_t block_smem_bytes(int M) {
+    const size_t a = LIN_HEAD + (size_t)2 * LIN_CHUNK * lin_stride(M) + (LIN_CELLS + 4) * 4 + LIN_CELLS * 2;
+    const size_t b = CON_STAGE + 6 * TILE * 4, c = (size_t)BW * 32 * ORB_STRIDE;
+    return a > b ? (a > c ? a : c) : (b > c ? b : c);
+}
+
+// The adjoint's phase 3 on linear rings (map_block_bwd.cuh): two chunks of staged entries and the
+// cell table, then each warp's rows; phase 2's stage is smaller.
+constexpr int ADJ_CHUNK = 64;          // entries staged at a time
+constexpr int ADJ_CELLS = 1024;        // cells listed at a time
+constexpr int ADJ_ROW_FLOATS = 2048;   // words of a warp's rows
+__host__ __device__ constexpr size_t adj_head_bytes(int M) {
+    return LIN_HEAD + (size_t)2 * ADJ_CHUNK * lin_stride(M) + (ADJ_CELLS + 4) * 4 + ADJ_CELLS * 2;
+}
+__host__ __device__ constexpr size_t adj_smem_bytes(int M) {
+    const size_t a = adj_head_bytes(M) + (size_t)BW * ADJ_ROW_FLOATS * 4;
+    const size_t b = (size_t)4 * TPCF_MAX_BINS * 2 * TILE * 4 + (size_t)TPCF_MAX_BINS * TPCF_MAX_BINS * 8 + 3 * 4 * TILE * 4;
+    const size_t c = LIN_HEAD + (size_t)2 * LIN_CHUNK * lin_stride(M) + (LIN_CELLS + 4) * 4 + LIN_CELLS * 2;
+    const size_t d = a > b ? a : b;
+    return d > c ? d : c;
+}
 
 // Shared memory (floats) of a map forward tile with runtime m_max mr: moments
 // A[k][m][re/im][32], W, Q, QW [k][32], the pivots' (w d, w).
@@ -129,43 +180,8 @@ __host__ __device__ inline size_t tile_floats_rt(int K, int mr, bool self) {
     return (size_t)K * (mr + 1) * 2 * TILE + (self ? 3 : 1) * (size_t)K * TILE + 2 * TILE;
 }
 
-// The shared-angle walk (map_walk.cuh).
-constexpr int WALK_CELLS = 4096;      // largest cell table (shared memory: 10 bytes per cell)
-constexpr int WALK_HEAD = 640;        // bytes of the small tables in front of it
-
-// Bytes between staged entries: up to eight pixel indices and the angle; an odd number of
-// 16-byte words, so that eight different entries fall in different banks.
-constexpr int WALK_STRIDE = 48;
-
-__host__ __device__ inline size_t walk_scratch_bytes(int nwarps, int cells) {
-    return WALK_HEAD + (size_t)cells * 10 + 16 + (size_t)nwarps * 32 * WALK_STRIDE;
-}
-
-// Cell table of the walk for a kernel with `base` other bytes of dynamic shared memory: the
-// largest that leaves room for two CTAs per SM (228 KB, 1 KB reserved per CTA and about 1 KB of
-// static tables), else the largest that fits one; 0 if none fits.
-inline int walk_pick_cells(size_t base, int nwarps) {
-    const size_t limit[2] = {114000, 231000};
-    for (int i = 0; i < 2; ++i)
-        for (int cells = WALK_CELLS; cells >= 256; cells /= 2)
-            if (base + walk_scratch_bytes(nwarps, cells) <= limit[i]) return cells;
-    return 0;
-}
-
-// Shared memory (bytes) of an adjoint tile with runtime m_max mr: the moments (then h), W,
-// Q and QW, the pivots' values, the primary-term sums, and one region used in turn by the
-// walk, by one m of H and by the warps' row buffers.
-__host__ __device__ inline size_t bwd_smem_bytes(int K, int mr, bool self, int cells) {
-    const size_t a = walk_scratch_bytes(NWARPS, cells), b = (size_t)K * K * 2 * sizeof(float),
-                 c = (size_t)NWARPS * ROW * sizeof(float);
-    size_t u = a > b ? a : b;
-    u = u > c ? u : c;
-    return (tile_floats_rt(K, mr, self) + TILE) * sizeof(float) + u;
-}
-
 // Device status bits.
 constexpr int ST_BAD_TILE = 1;
-constexpr int ST_ROW_OVERFLOW = 2;   // informational: a row wider than the warp buffer used direct global adds
 constexpr int ST_TC_TIMEOUT_BIT = 4;  // a tensor-core completion wait gave up
 
 }  // namespace tpcf

@@ -24,8 +24,8 @@
 using namespace tpcf;
 
 namespace tpcf {
-int map_fwd_occupancy(int M, int K, int self, int variant);
-int map_bwd_occupancy(int M, int K, int variant);
+int map_fwd_occupancy(int M);
+int map_bwd_occupancy(int M);
 
 static std::string tune_key(const tpcf_plan_s* P) {
     cudaDeviceProp prop;
@@ -84,9 +84,8 @@ static void cache_store(const std::string& key, const tpcf_plan_s::Tune& f, cons
 static bool valid(const tpcf_plan_s* P, const tpcf_plan_s::Tune& t, bool bwd) {
     if (t.variant != 2 && t.variant != 3) return false;
     if (t.flush < 1 || t.flush > 64 || t.ctas < 1 || t.quad < 0 || t.quad > 1) return false;
-    const int self = (P->flags & TPCF_SELF_PAIRS_SUBTRACT) ? 1 : 0;
-    const int occ = bwd ? map_bwd_occupancy(P->M, P->K, t.variant) : map_fwd_occupancy(P->M, P->K, self, t.variant);
-    return t.ctas <= occ;
+    const int occ = bwd ? map_bwd_occupancy(P->M) : map_fwd_occupancy(P->M);
+    return t.ctas <= (occ + 1) / 2;
 }
 
 // Applies a cached configuration to a new map plan (called at plan creation).
@@ -172,7 +171,6 @@ extern "C" tpcf_status tpcf_plan_autotune(tpcf_plan plan, const float* d_delta, 
     // the adjoint candidates take the normalisation D of the first sample slice
     if (st == TPCF_OK && (passes & 2))
         st = tpcf_forward(P, d_delta, d_w, sample[0].first, sample[0].second, zeta, norm, nullptr, s);
-    const int self = (P->flags & TPCF_SELF_PAIRS_SUBTRACT) ? 1 : 0;
     for (int pass = 0; pass < 2 && st == TPCF_OK; ++pass) {
         if (!(passes & (1 << pass))) continue;
         const bool bwd = pass == 1;
@@ -204,22 +202,14 @@ extern "C" tpcf_status tpcf_plan_autotune(tpcf_plan plan, const float* d_delta, 
                 best = T;
             }
         };
-        for (int variant = 3; variant >= 2 && st == TPCF_OK; --variant) {
-            const int occ = bwd ? map_bwd_occupancy(M, K, variant) : map_fwd_occupancy(M, K, self, variant);
-            for (int ctas = occ; ctas >= std::max(1, occ - 1) && st == TPCF_OK; --ctas) {
-                const int flushes[4] = {4, 8, 16, 32};
-                for (int fi = 0; fi < 4 && st == TPCF_OK; ++fi) {
-                    T.variant = variant;
-                    T.ctas = ctas;
-                    T.flush = flushes[fi];
-                    try_config();
-                }
+        const int occ = ((bwd ? map_bwd_occupancy(M) : map_fwd_occupancy(M)) + 1) / 2;  // pairs
+        for (int ctas = occ; ctas >= std::max(1, occ - 1) && st == TPCF_OK; --ctas) {
+            const int flushes[4] = {4, 8, 16, 32};
+            for (int fi = 0; fi < 4 && st == TPCF_OK; ++fi) {
+                T.ctas = ctas;
+                T.flush = flushes[fi];
+                try_config();
             }
-        }
-        if (!bwd && st == TPCF_OK) {  // the forward's tile layout, at the best shape
-            T = best;
-            T.quad = 1 - best.quad;
-            try_config();
         }
         T = st == TPCF_OK ? best : keep;
     }
