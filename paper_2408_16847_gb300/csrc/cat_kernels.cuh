@@ -1,18 +1,22 @@
-// Catalogue forward kernel: the estimator of Sec. 3.1 (eqs. Xm.binned, zetamEst)
-// for points at arbitrary positions, found through the plan's sphere grid.
+// Catalogue kernels: the estimator of Sec. 3.1 (eqs. Xm.binned, zetamEst) for points at
+// arbitrary positions, found through the plan's sphere grid.
 //
 // A tile is 32 consecutive points of the grid order (spatially compact), one pivot
 // per lane.  Warp 0 bounds the tile's live pivots by a cap (centre, radius R); every
 // point within R + theta_max of the centre lies in the cells the cap overlaps, which
-// are a handful of contiguous index ranges per colatitude band.  Every warp walks the
-// bands in reach and takes every 8th chunk of 32 candidates (so the warps finish
-// together), stages the chunk in shared memory and lets each lane pair its pivot with
-// all 32.  Per pair: the chord from fp32 hi/lo positions,
-// the bin from a log-scale lookup table (FP64 check within CAT_AMB of an edge), the
-// position angle from the pivot's local north/east basis, the harmonics by the
-// stable three-term recurrence of map_kernels.cuh (harmonics()).  The per-lane
-// register sums follow one bin at a time and are added into the tile's shared-memory moments when the bin changes; the tile
-// contraction and the cross-CTA reduction are those of the map path.
+// are a handful of contiguous index ranges per colatitude band.  The CTA stages those of these
+// candidates that are close enough to the centre, up to 512 at a time, as fp32 hi/lo offsets
+// from it, and makes two passes:
+//   1. a warp takes 32 candidates (a word) and bins each for its 32 pivots, from one broadcast
+//      read and a table over the bits of chord^2.  Bin k of pivot `lane` is one bit in the word's
+//      mask [k][lane];
+//   2. a warp takes a bin: each lane goes through the candidates in its own masks of that bin, so
+//      every lane's sums stay in registers for the whole batch and go to the CTA's workspace in
+//      global memory once per bin and batch, without atomics.
+// Pass 2 has no bin decision and pass 1 no angle; neither diverges but for the lanes' different
+// numbers of candidates in a bin.  Candidates whose chord^2 is too close to an edge for the table
+// go a slower way (cat_near_edge), down to FP64 within CAT_AMB of the edge.  The contraction of a
+// tile is that of the map blocks (block_contract).
 #pragma once
 
 #include "map_kernels.cuh"
@@ -21,62 +25,36 @@ namespace tpcf {
 
 constexpr float CAT_AMB = 2.0e-6f;  // relative margin of fp32 chord^2 to an edge (error ~3e-7)
 constexpr float CAT_MARGIN = 8.0e-6f;  // angular margin of the fp32 cell query (rad)
+constexpr float CAT_FAR = 1.0e3f;      // where lanes and slots that are not in use are placed
 
 // Bin of chord^2 in fp64 over the edges (ties to the upper bin) for sorted points j
-// (candidate) and si (pivot; si < 0: the placeholder pivot (0, 0, 1) of a padding
-// lane): -1 below the first edge, K at or beyond the last.
+// (candidate) and si (pivot): -1 below the first edge, K at or beyond the last.
 static __device__ __noinline__ int cat_exact_bin(const double* __restrict__ Ed2, int K, const double* __restrict__ xyz,
                                           int64_t j, int64_t si) {
-    const double px = si >= 0 ? xyz[3 * si] : 0.0, py = si >= 0 ? xyz[3 * si + 1] : 0.0,
-                 pz = si >= 0 ? xyz[3 * si + 2] : 1.0;
-    const double dx = xyz[3 * j] - px, dy = xyz[3 * j + 1] - py, dz = xyz[3 * j + 2] - pz;
+    const double dx = xyz[3 * j] - xyz[3 * si], dy = xyz[3 * j + 1] - xyz[3 * si + 1],
+                 dz = xyz[3 * j + 2] - xyz[3 * si + 2];
     const double c2 = dx * dx + dy * dy + dz * dz;
     int k = -1;
     while (k < K && c2 >= Ed2[k + 1]) ++k;
     return k;
 }
 
-// fp32 bin of c2 from the lookup table, corrected against the fp32 edges.
-__device__ __forceinline__ int cat_bin(float c2, const float* sE2, const unsigned char* slut, float l0, float linv,
-                                       int K) {
-    const float x = (__log2f(c2) - l0) * linv;
-    int k = x < 0.0f ? -1 : (x >= (float)CAT_LUT ? K : (int)slut[(int)x]);
-    while (k < K && c2 >= sE2[k + 1]) ++k;
-    while (k >= 0 && c2 < sE2[k]) --k;
-    return k;
-}
-
-template <int M, bool SELF>
-__device__ __forceinline__ void cat_flush(float* sA, float* sW, float* sQ, float* sQW, int k, int lane,
-                                          float2 (&acc)[M + 1], float& W, float& Q, float& QW) {
-    float* a = sA + (size_t)k * (M + 1) * 2 * TILE;
-    atomicAdd(a + lane, acc[0].x);
-    acc[0] = make_float2(0.0f, 0.0f);
-#pragma unroll
-    for (int m = 1; m <= M; ++m) {
-        atomicAdd(a + (2 * m) * TILE + lane, acc[m].x);
-        atomicAdd(a + (2 * m + 1) * TILE + lane, acc[m].y);
-        acc[m] = make_float2(0.0f, 0.0f);
+// The bin of a candidate near an edge, or where the table's cells hold several edges: from
+// chord^2 to full fp32 precision (c2), in FP64 within CAT_AMB of an edge.
+static __device__ __noinline__ int cat_near_edge(const CatDev& g, float c2, int64_t j, int64_t si) {
+    int k = -1;
+    bool near = false;
+    for (int e = 0; e <= g.K; ++e) {
+        const float E = __ldg(g.E2 + e);
+        k += c2 >= E ? 1 : 0;
+        near = near || fabsf(c2 - E) <= CAT_AMB * E;
     }
-    atomicAdd(sW + k * TILE + lane, W);
-    W = 0.0f;
-    if (SELF) {
-        atomicAdd(sQ + k * TILE + lane, Q);
-        atomicAdd(sQW + k * TILE + lane, QW);
-        Q = 0.0f;
-        QW = 0.0f;
-    }
+    return near && si >= 0 ? cat_exact_bin(g.Ed2, g.K, g.xyz, j, si) : k;
 }
 
-// Shared memory of the catalogue forward beyond the tile's moments: per-warp
-// staging of 32 candidates (hi, lo positions and (w d, w)).
-template <int M>
-__host__ __device__ inline size_t cat_tile_bytes(int K) {
-    return tile_floats<M>(K) * sizeof(float) + (size_t)NWARPS * TILE * (2 * sizeof(float4) + sizeof(float2));
-}
-
-// The lane's pivot: fp32 hi/lo position, local north / east basis and its sorted
-// index (the FP64 position is read only for the rare exact bin decisions).
+// The lane's pivot: fp32 hi/lo position (of the unit vector; cat_place moves it to the cap's
+// centre), local north / east basis and its sorted index (the FP64 position is read only for
+// the rare exact bin decisions).
 struct CatPivot {
     float hx, hy, hz, lx, ly, lz;
     float nx, ny, nz, ex, ey;
@@ -120,7 +98,8 @@ __device__ __forceinline__ CatPivot cat_pivot(const CatDev& g, int64_t si) {
 
 // Warp 0: a cap holding every live pivot of the tile together with its neighbours
 // (radius theta_max), as a range of cell bands and a longitude half-width about the
-// cap's centre: s_cap = (phi_c, dphi, first band, last band, full).  All in fp32:
+// cap's centre: s_cap = (phi_c, dphi, first band, last band, full, centre x, y, z, largest
+// chord from the centre to a live pivot).  All in fp32:
 // CAT_MARGIN (rad) exceeds every rounding of the centre, radius, colatitude and band
 // division (each below ~1e-6 rad), and the sine ratio is rounded up, so the cells are
 // a superset of the exact cap; bins are then decided per candidate.  The caller
@@ -142,14 +121,18 @@ __device__ __forceinline__ void cat_tile_cap(const CatDev& g, bool live, const C
         nrm = 1.0f;
     }
     const float cx = sx / nrm, cy = sy / nrm, cz = sz / nrm;
-    float r = 0.0f;
+    float r = 0.0f, rho = 0.0f;
     if (live) {
         const float dx = px - cx, dy = py - cy, dz = pz - cz;
         const float ch = sqrtf(fmaf(dx, dx, fmaf(dy, dy, dz * dz)));
         r = 2.0f * asinf(fminf(1.0f, 0.5f * ch));
+        rho = ch;
     }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) r = fmaxf(r, __shfl_xor_sync(0xffffffffu, r, o));
+    for (int o = 16; o > 0; o >>= 1) {
+        r = fmaxf(r, __shfl_xor_sync(0xffffffffu, r, o));
+        rho = fmaxf(rho, __shfl_xor_sync(0xffffffffu, rho, o));
+    }
     if ((threadIdx.x & 31) == 0) {
         const float PI_F = 3.14159265f;
         const float Q = r + (float)g.theta_max + CAT_MARGIN;
@@ -178,622 +161,563 @@ __device__ __forceinline__ void cat_tile_cap(const CatDev& g, bool live, const C
         s_cap[2] = (float)b0;
         s_cap[3] = (float)b1;
         s_cap[4] = full;
+        s_cap[5] = cx;
+        s_cap[6] = cy;
+        s_cap[7] = cz;
+        s_cap[8] = rho;
     }
 }
 
-// Every candidate of the cap for this warp, with its bin k (-1 below the first edge,
-// K beyond the last), the chord vector from the lane's pivot, its (w d, w) and its
-// sorted index: f(k, dx, dy, dz, v, j).  Calls are warp-uniform (every lane sees the
-// same candidate at the same time).  Candidates are staged 32 at a
-// time in the warp's shared buffers wh / wl / wv.
+// Coordinate h + l relative to c, again as hi/lo (Knuth's two-sum: no digit of the pair is lost).
+__device__ __forceinline__ void cat_rel(float h, float l, float c, float& H, float& L) {
+    const float s = h - c, b = s - h;
+    const float t = ((h - (s - b)) + (-c - b)) + l;
+    H = s + t;
+    L = t - (H - s);
+}
+
+// Shared memory of a catalogue CTA.  The union is the candidates and their masks, the
+// contraction's stage, or the adjoint's phase 2.
+struct CatShared {
+    unsigned char* lut;  // [CAT_LUT] next edge above a cell of chord^2 (see cat_edges_kernel)
+    float2* edge;        // [K + 3] chord^2 of the edge, margin below which cat_near_edge decides
+    float* cap;          // [9] (cat_tile_cap)
+    int* item;           // next bin of the batch
+    int* cnt;            // [BW] candidates staged by a warp
+    int* wsum;           // [BW]
+    int* pre;            // [2 BT + 1] candidates before a cell range of the band group
+    int* start;          // [2 BT] first candidate of the range
+    char* stage;         // the union
+    int words;           // words of 32 candidates a warp stages at a time; BW words of them in all
+    float4 *hi, *lo;     // [32 BW words] offset from the cap's centre and w d; its remainder and w
+    int* idx;            // [32 BW words] sorted index
+    unsigned* mask;      // [K + 1][BW words][32]; row K takes the candidates outside the bins
+    float* leg;          // [32 BW words] adjoint only: sums of the legs to a candidate
+};
+
+constexpr size_t CAT_HEAD = CAT_LUT + 8 * 40 + 4 * 16 + 4 * 16 + 4 * (4 * BT + 16);
+
+// Words a warp stages at a time: as many as leave room for four CTAs on an SM (57,000 bytes each), at
+// most 4.  More candidates to a batch mean fewer trips of the sums to the workspace and lanes
+// with more equal numbers of candidates in a bin.
+__host__ __device__ inline size_t cat_word_bytes(int K, bool legs) {
+    return BW * (32 * (2 * sizeof(float4) + (legs ? 2 : 1) * sizeof(int)) + (size_t)(K + 1) * TILE * 4);
+}
+__host__ __device__ inline int cat_words(int K, bool legs) {
+    const int w = (int)((57000 - CAT_HEAD) / cat_word_bytes(K, legs));
+    return w > 4 ? 4 : w;
+}
+__host__ __device__ inline size_t cat_smem_bytes(int K, bool legs, size_t other) {
+    const size_t b = cat_words(K, legs) * cat_word_bytes(K, legs);
+    return CAT_HEAD + (b > other ? b : other);
+}
+// forward (6 TILE floats of pivot values, as for three fields), adjoint
+template <int M>
+__host__ __device__ inline size_t cat_fwd_bytes(int K) {
+    return cat_smem_bytes(K, false, CON_STAGE + 6 * TILE * sizeof(float));
+}
+template <int M>
+__host__ __device__ inline size_t cat_bwd_bytes(int K) { return cat_smem_bytes(K, true, adj_smem_bytes(M)); }
+
+__device__ __forceinline__ CatShared cat_shared(char* smem, int K, bool legs) {
+    CatShared S;
+    S.lut = reinterpret_cast<unsigned char*>(smem);
+    S.edge = reinterpret_cast<float2*>(smem + CAT_LUT);
+    S.cap = reinterpret_cast<float*>(S.edge + 40);
+    S.item = reinterpret_cast<int*>(S.cap + 16);
+    S.cnt = S.item + 4;
+    S.wsum = S.item + 8;
+    S.pre = S.item + 16;
+    S.start = S.pre + 2 * BT + 16;
+    S.stage = smem + CAT_HEAD;
+    S.words = cat_words(K, legs);
+    const int n = BW * 32 * S.words;
+    S.hi = reinterpret_cast<float4*>(S.stage);
+    S.lo = S.hi + n;
+    S.idx = reinterpret_cast<int*>(S.lo + n);
+    S.mask = reinterpret_cast<unsigned*>(S.idx + n);
+    S.leg = reinterpret_cast<float*>(S.mask + (K + 1) * n);
+    return S;
+}
+
+__device__ __forceinline__ void cat_load_lut(const CatDev& g, const CatShared& S) {
+    for (int e = threadIdx.x; e < CAT_LUT / 4; e += BT)
+        reinterpret_cast<unsigned*>(S.lut)[e] = __ldg(reinterpret_cast<const unsigned*>(g.lut) + e);
+}
+
+// (w d, w) of pivot `lane` of a tile; zero outside the call's pivot range and where w = 0.
+__device__ __forceinline__ float2 cat_value(const CatDev& g, const float2* __restrict__ wdw, int64_t lo, int64_t hi,
+                                            int64_t tile, int lane) {
+    const int64_t si = tile * TILE + lane;
+    float2 v = make_float2(0.0f, 0.0f);
+    if (si < g.n) {
+        const int64_t o = g.orig[si];
+        if (o >= lo && o < hi) v = wdw[si];
+    }
+    return v.y != 0.0f ? v : make_float2(0.0f, 0.0f);
+}
+
+// Prepares a tile: its cap, the margins of the edges and the lane's pivot relative to the cap's
+// centre; lanes that are not live are moved away from every candidate.  Called by every thread.
+//
+// Pass 1 uses the offsets' fp32 high parts alone.  With p, q the offsets of pivot and candidate,
+// each rounded to 2^-24 of itself, and d = q - p, |q| <= |d| + |p|: chord^2 is off by at most
+// 2^-24 (7 d^2 + 8 |d| |p|), a quarter of the margin 2e-6 (E + rho sqrt(E)) at an edge.  A
+// table cell only knows the one edge within a cell's width, so margins stay below that width (2^(shift - 24)
+// of E at least); a tile too wide for that decides every candidate in cat_near_edge.
+__device__ __forceinline__ CatPivot cat_place(const CatDev& g, const CatShared& S, int64_t tile, bool live) {
+    const int lane = threadIdx.x & 31;
+    const int64_t si = tile * TILE + lane;
+    CatPivot P = cat_pivot(g, si < g.n ? si : -1);
+    if ((threadIdx.x >> 5) == 0) {
+        cat_tile_cap(g, live, P, S.cap);
+        __syncwarp();
+        const float rho = S.cap[8];
+        const float cell = exp2f((float)(g.lut_shift - 24)) * 0.99f;
+        bool wide = false;
+        for (int e = lane; e < g.K + 3; e += 32) {
+            const float E = e <= g.K ? g.E2[e] : 0.0f;
+            const float amb = 2.0e-6f * fmaf(rho, sqrtf(E), E);
+            wide = wide || amb > cell * E;
+            S.edge[e] = e <= g.K ? make_float2(E, amb)
+                                 : (e == g.K + 1 ? make_float2(INFINITY, 0.0f) : make_float2(0.0f, INFINITY));
+        }
+        if (__any_sync(0xffffffffu, wide))
+            for (int e = lane; e < g.K + 2; e += 32) S.edge[e].y = INFINITY;
+    }
+    __syncthreads();
+    cat_rel(P.hx, P.lx, S.cap[5], P.hx, P.lx);
+    cat_rel(P.hy, P.ly, S.cap[6], P.hy, P.ly);
+    cat_rel(P.hz, P.lz, S.cap[7], P.hz, P.lz);
+    if (!live) {
+        P.hx = CAT_FAR;
+        P.si = -1;
+    }
+    return P;
+}
+
+// The candidates of the cap, staged a batch at a time: batch(first) for each, between barriers; at
+// least once.  A candidate is kept if it can be in a bin of a live pivot, all of which are within
+// rho of the centre.  Each warp fills words of its own (the order of a sum stays the same from run
+// to run), the rest of its last word with points far away; S.cnt says how many.  Called by every thread.
 template <class F>
-__device__ __forceinline__ void cat_walk(const CatDev& g, const float2* __restrict__ wdw, const float* s_cap,
-                                         const CatPivot& P, const float* sE2, const unsigned char* slut,
-                                         float4* wh, float4* wl, float2* wv, F&& f) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int K = g.K;
+__device__ __forceinline__ void cat_batches(const CatDev& g, const float2* __restrict__ wdw, const CatShared& S,
+                                            F&& batch) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     // sector bounds in fp32: the extra 4e-6 rad covers its rounding (phi < 2 pi), so the
     // cell ranges stay a superset of the cap
-    const float phc = s_cap[0], dphi = s_cap[1] + 4.0e-6f;
-    const int b0 = (int)s_cap[2], b1 = (int)s_cap[3];
-    const bool full = s_cap[4] != 0.0f;
-    // every warp walks every band and takes every NWARPS-th chunk of 32 candidates
-    int chunk = 0;
-    for (int b = b0; b <= b1; ++b) {
-        const int64_t ns = g.band_ns[b];
-        const int64_t cf = g.band_first[b];
-        // at most two cell ranges (the sector range may wrap around phi = 0)
-        int64_t ca0 = cf, ca1 = cf + ns, cb0 = 0, cb1 = 0;
-        if (!full) {
-            const float scale = (float)ns * (float)(0.5 / M_PI);
-            const int64_t sa = (int64_t)floorf((phc - dphi) * scale);
-            const int64_t sb = (int64_t)floorf((phc + dphi) * scale);
-            const int64_t len = sb - sa + 1;
-            if (len < ns) {
-                int64_t s0 = sa % ns;
-                if (s0 < 0) s0 += ns;
-                ca0 = cf + s0;
-                if (s0 + len <= ns) {
-                    ca1 = cf + s0 + len;
-                } else {
-                    ca1 = cf + ns;
-                    cb0 = cf;
-                    cb1 = cf + (s0 + len - ns);
+    const float phc = S.cap[0], dphi = S.cap[1] + 4.0e-6f;
+    const int b0 = (int)S.cap[2], b1 = (int)S.cap[3];
+    const bool full = S.cap[4] != 0.0f;
+    const float rho = S.cap[8], rlo = sqrtf(__ldg(g.E2)), rhi = sqrtf(__ldg(g.E2 + g.K));
+    const float far = (rhi + rho) * (1.0f + 1.0e-5f), nearby = fmaxf(rlo - rho - 1.0e-5f * (rlo + rho), 0.0f);
+    const float far2 = far * far, near2 = nearby * nearby;
+    bool first = true;
+    int c = 0;  // candidates staged by this warp
+    const int w0 = 32 * S.words * warp, cap = 32 * S.words;
+    for (int bg = b0; bg <= b1; bg += BT) {
+        // a band per thread: at most two cell ranges (the sector range may wrap around phi = 0)
+        int64_t pa0 = 0, pa1 = 0, pb0 = 0, pb1 = 0;
+        if (bg + tid <= b1) {
+            const int64_t ns = g.band_ns[bg + tid], cf = g.band_first[bg + tid];
+            int64_t ca0 = cf, ca1 = cf + ns, cb1 = cf;
+            if (!full) {
+                const float scale = (float)ns * (float)(0.5 / M_PI);
+                const int64_t sa = (int64_t)floorf((phc - dphi) * scale);
+                const int64_t sb = (int64_t)floorf((phc + dphi) * scale);
+                const int64_t len = sb - sa + 1;
+                if (len < ns) {
+                    int64_t s0 = sa % ns;
+                    if (s0 < 0) s0 += ns;
+                    ca0 = cf + s0;
+                    if (s0 + len <= ns) {
+                        ca1 = ca0 + len;
+                    } else {
+                        cb1 = cf + (s0 + len - ns);
+                    }
                 }
+            }
+            pa0 = g.cell_start[ca0];
+            pa1 = g.cell_start[ca1];
+            if (cb1 > cf) {
+                pb0 = g.cell_start[cf];
+                pb1 = g.cell_start[cb1];
             }
         }
-#pragma unroll 1
-        for (int sg = 0; sg < 2; ++sg) {
-            const int64_t cl0 = sg == 0 ? ca0 : cb0, cl1 = sg == 0 ? ca1 : cb1;
-            if (cl1 <= cl0) continue;
-            const int64_t p0 = g.cell_start[cl0], p1 = g.cell_start[cl1];
-            for (int64_t base = p0; base < p1; base += TILE, ++chunk) {
-                if ((chunk % NWARPS) != warp) continue;
-                const int64_t j = base + lane;
-                __syncwarp();
-                if (j < p1) {
-                    wh[lane] = g.p_hi[j];
-                    wl[lane] = g.p_lo[j];
-                    wv[lane] = wdw[j];
+        const int na = (int)(pa1 - pa0), s = na + (int)(pb1 - pb0);
+        int inc = s;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const int v = __shfl_up_sync(0xffffffffu, inc, d);
+            if (lane >= d) inc += v;
+        }
+        if (lane == 31) S.wsum[warp] = inc;
+        __syncthreads();
+        int base = inc - s;
+        for (int w = 0; w < warp; ++w) base += S.wsum[w];
+        S.pre[2 * tid] = base;
+        S.pre[2 * tid + 1] = base + na;
+        S.start[2 * tid] = (int)pa0;
+        S.start[2 * tid + 1] = (int)pb0;
+        if (tid == BT - 1) S.pre[2 * BT] = base + s;
+        __syncthreads();
+        const int total = S.pre[2 * BT];
+        const bool last = bg + BT > b1;
+        for (int x = 32 * warp;;) {
+            for (; x < total && c <= cap - 32; x += BT) {
+                const int e = x + lane;
+                bool keep = false;
+                float4 H, L;
+                int j = 0;
+                if (e < total) {
+                    int lo = 0, hi = 2 * BT - 1;  // the last range that starts at or before e
+                    while (lo < hi) {
+                        const int mid = (lo + hi + 1) >> 1;
+                        if (S.pre[mid] <= e) lo = mid; else hi = mid - 1;
+                    }
+                    j = S.start[lo] + (e - S.pre[lo]);
+                    const float4 h = g.p_hi[j], l = g.p_lo[j];
+                    const float2 v = wdw[j];
+                    cat_rel(h.x, l.x, S.cap[5], H.x, L.x);
+                    cat_rel(h.y, l.y, S.cap[6], H.y, L.y);
+                    cat_rel(h.z, l.z, S.cap[7], H.z, L.z);
+                    H.w = v.x;
+                    L.w = v.y;
+                    const float d2 = fmaf(H.x, H.x, fmaf(H.y, H.y, H.z * H.z));
+                    keep = d2 <= far2 && d2 >= near2;
                 }
-                __syncwarp();
-                const int cnt = (int)min((int64_t)TILE, p1 - base);
-                for (int u = 0; u < cnt; ++u) {
-                    const float4 qh = wh[u], ql = wl[u];
-                    const float dx = (qh.x - P.hx) + (ql.x - P.lx);
-                    const float dy = (qh.y - P.hy) + (ql.y - P.ly);
-                    const float dz = (qh.z - P.hz) + (ql.z - P.lz);
-                    const float c2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-                    int k = cat_bin(c2, sE2, slut, g.lut_l0, g.lut_inv, K);
-                    const int e1 = max(k, 0), e2 = min(k + 1, K);
-                    if (fabsf(c2 - sE2[e1]) <= CAT_AMB * sE2[e1] || fabsf(c2 - sE2[e2]) <= CAT_AMB * sE2[e2])
-                        k = cat_exact_bin(g.Ed2, K, g.xyz, (int64_t)__float_as_int(ql.w), P.si);
-                    f(k, dx, dy, dz, wv[u], __float_as_int(ql.w));
+                const unsigned kept = __ballot_sync(0xffffffffu, keep);
+                if (keep) {
+                    const int at = w0 + c + __popc(kept & ((1u << lane) - 1u));
+                    S.hi[at] = H;
+                    S.lo[at] = L;
+                    S.idx[at] = j;
                 }
+                c += __popc(kept);
             }
+            const bool more = __syncthreads_or(x < total) != 0;
+            if (!more && !last) break;  // the next group of bands fills up
+            if (lane < ((32 - c) & 31)) {
+                S.hi[w0 + c + lane] = make_float4(-CAT_FAR, 0.0f, 0.0f, 0.0f);
+                S.lo[w0 + c + lane] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            }
+            if (lane == 0) S.cnt[warp] = c;
+            if (tid == 0) *S.item = 0;
+            __syncwarp();
+            batch(first);
+            __syncthreads();
+            first = false;
+            c = 0;
+            if (!more) break;
         }
     }
 }
 
-// The candidates of the cap grouped by bin, chunk by chunk.  For each staged chunk of
-// 32 candidates, pass A bins every candidate for the lane's pivot and records, per
-// lane, one bit mask per bin kb + j (j = 0..GROUPS-1, kb = the first in-range bin seen
-// in the chunk minus three; a tile's pivots lie close together, so the candidates of a
-// chunk cover few bins for every lane) plus a mask of the rare in-range candidates
-// beyond that window; out-of-range candidates are dropped there.  With 8 bins in the
-// window about 6% of the in-range candidates of the 2e6-point catalogue fall outside
-// it (30% with 4), each of which costs a flush of the register sums.  Pass B then runs,
-// for each j in lockstep, every lane over the candidates of its own bin kb + j:
-//     pair(active, k, dx, dy, dz, v, u)   for each candidate (u its slot in the chunk;
-//                                         active false on padding iterations, where k
-//                                         may be out of range and must not be used)
-//     group_end(k, nonempty)              once per j, warp-uniform
-// and the candidates beyond the window one by one: single(k, dx, dy, dz, v, u).
-// chunk_end(base, cnt) closes each chunk (uniform).  This replaces per-candidate bin
-// changes (a divergent flush whenever one lane's bin changed) by a uniform flush per
-// bin and chunk.
-constexpr int CAT_GROUPS = 8;
+// Pass 1 for J of the warp's words at once, from word w on: a candidate of each, so that their chains of
+// loads and the updates of their masks, which are in different words, overlap.
+template <int J>
+__device__ __forceinline__ void cat_bin_words(const CatDev& g, const CatShared& S, const CatPivot& P, int w) {
+    const int lane = threadIdx.x & 31;
+    const int base = g.lut_base, shift = g.lut_shift, row = BW * S.words * TILE;
+    unsigned* mw = S.mask + w * TILE + lane;
+    const float4* q = S.hi + w * 32;
+#pragma unroll 1
+    for (int u = 0; u < 32; ++u) {
+        float3 d[J];
+        float c2[J], x[J], amb[J];
+        int k[J];
+        bool near = false;
+#pragma unroll
+        for (int j = 0; j < J; ++j) {
+            const float4 qh = q[j * 32 + u];
+            d[j] = make_float3(qh.x - P.hx, qh.y - P.hy, qh.z - P.hz);
+            c2[j] = fmaf(d[j].x, d[j].x, fmaf(d[j].y, d[j].y, d[j].z * d[j].z));
+            k[j] = S.lut[min((max(__float_as_int(c2[j]), base) - base) >> shift, CAT_LUT - 1)];
+        }
+#pragma unroll
+        for (int j = 0; j < J; ++j) {
+            const float2 e = S.edge[k[j]];
+            x[j] = c2[j] - e.x;
+            amb[j] = e.y;
+            if (x[j] < 0.0f) --k[j];
+            near = near || fabsf(x[j]) <= amb[j];
+        }
+        if (near) {
+#pragma unroll
+            for (int j = 0; j < J; ++j)
+                if (fabsf(x[j]) <= amb[j]) {
+                    const int at = (w + j) * 32 + u;
+                    const float4 ql = S.lo[at];
+                    const float ex = d[j].x + (ql.x - P.lx), ey = d[j].y + (ql.y - P.ly), ez = d[j].z + (ql.z - P.lz);
+                    k[j] = cat_near_edge(g, fmaf(ex, ex, fmaf(ey, ey, ez * ez)), S.idx[at], P.si);
+                }
+        }
+        unsigned m[J];
+#pragma unroll
+        for (int j = 0; j < J; ++j) {
+            k[j] = (int)min((unsigned)k[j], (unsigned)g.K) * row + j * TILE;
+            m[j] = mw[k[j]];
+        }
+#pragma unroll
+        for (int j = 0; j < J; ++j) mw[k[j]] = m[j] | (1u << u);
+    }
+}
 
-template <class FP, class FE, class FS, class FC>
-__device__ __forceinline__ void cat_walk_grouped(const CatDev& g, const float2* __restrict__ wdw,
-                                                 const float* s_cap, const CatPivot& P, const float* sE2,
-                                                 const unsigned char* slut, float4* wh, float4* wl, float2* wv,
-                                                 FP&& pair, FE&& group_end, FS&& single, FC&& chunk_end) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+// Pass 1 of a batch: the masks of the warp's own candidates.  The masks are zero on entry.
+__device__ __forceinline__ void cat_bins(const CatDev& g, const CatShared& S, const CatPivot& P) {
+    const int warp = threadIdx.x >> 5;
+    int w = S.words * warp;
+    const int we = w + ((S.cnt[warp] + 31) >> 5);
+    for (; w + 3 < we; w += 4) cat_bin_words<4>(g, S, P, w);
+    for (; w + 1 < we; w += 2) cat_bin_words<2>(g, S, P, w);
+    if (w < we) cat_bin_words<1>(g, S, P, w);
+}
+
+// Position angle of a candidate: the lane's pivot sees the offset (hi, lo) under this folded angle.
+__device__ __forceinline__ Fold cat_angle(const CatPivot& P, const float4& qh, const float4& ql) {
+    const float dx = (qh.x - P.hx) + (ql.x - P.lx);
+    const float dy = (qh.y - P.hy) + (ql.y - P.ly);
+    const float dz = (qh.z - P.hz) + (ql.z - P.lz);
+    const float N = fmaf(dx, P.nx, fmaf(dy, P.ny, dz * P.nz));
+    const float E = fmaf(dx, P.ex, dy * P.ey);
+    const float rinv = rsqrtf(fmaxf(fmaf(N, N, E * E), 1e-30f));
+    return fold_angle(N * rinv, E * rinv);
+}
+
+// Pass 2 over bin k of a batch: f(on, u, hi, lo) for each candidate u of the lane (on false
+// where other lanes have more), two at a time.  Leaves the bin's masks zero.
+template <class FB, class F>
+__device__ __forceinline__ void cat_bin_pairs(const CatShared& S, int k, FB&& begin, F&& f) {
+    const int lane = threadIdx.x & 31;
+    unsigned* mk = S.mask + (size_t)k * BW * S.words * TILE + lane;
+    unsigned words = 0u;
+    int cnt = 0;
+#pragma unroll 4
+    for (int w = 0; w < BW * S.words; ++w) {  // (words that were not filled are zero)
+        const unsigned m = mk[w * TILE];
+        cnt += __popc(m);
+        words |= (m != 0u ? 1u : 0u) << w;
+    }
+    const int most = __reduce_max_sync(0xffffffffu, cnt);
+    if (!begin(most)) return;
+    unsigned m = 0u;
+    int base = 0;
+    auto next = [&]() {  // the lane's next candidate, or some candidate
+        if (m == 0u && words != 0u) {
+            const int w = __ffs(words) - 1;
+            words &= words - 1u;
+            m = mk[w * TILE];
+            mk[w * TILE] = 0u;
+            base = w * 32;
+        }
+        const int u = base + max(__ffs(m) - 1, 0);
+        m &= m - 1u;
+        return u;
+    };
+#pragma unroll 1
+    for (int i = 0; i < most; i += 2) {
+        const int u0 = next(), u1 = next();
+        const float4 h0 = S.hi[u0], l0 = S.lo[u0], h1 = S.hi[u1], l1 = S.lo[u1];
+        f(i < cnt, u0, h0, l0);
+        f(i + 1 < cnt, u1, h1, l1);
+    }
+}
+
+__device__ __forceinline__ int cat_next_bin(const CatShared& S) {
+    int k = 0;
+    if ((threadIdx.x & 31) == 0) k = atomicAdd(S.item, 1);
+    return __shfl_sync(0xffffffffu, k, 0);
+}
+
+__device__ __forceinline__ void cat_zero_masks(const CatShared& S, int K) {
+    for (int e = threadIdx.x; e < K * BW * S.words * TILE; e += BT) S.mask[e] = 0u;
+}
+
+// The moments of a tile with the neighbour values `wdw`, into its subtile of the workspace.
+// Called by every thread; complete after the caller's barrier.
+template <int M, bool SELF>
+__device__ __forceinline__ void cat_tile_moments(const CatDev& g, const float2* __restrict__ wdw, const CatShared& S,
+                                                 const CatPivot& P, float* ws, size_t sub_floats) {
     const int K = g.K;
-    const float phc = s_cap[0], dphi = s_cap[1] + 4.0e-6f;
-    const int b0 = (int)s_cap[2], b1 = (int)s_cap[3];
-    const bool full = s_cap[4] != 0.0f;
-    int chunk = 0;
-    for (int b = b0; b <= b1; ++b) {
-        const int64_t ns = g.band_ns[b];
-        const int64_t cf = g.band_first[b];
-        int64_t ca0 = cf, ca1 = cf + ns, cb0 = 0, cb1 = 0;
-        if (!full) {
-            const float scale = (float)ns * (float)(0.5 / M_PI);
-            const int64_t sa = (int64_t)floorf((phc - dphi) * scale);
-            const int64_t sb = (int64_t)floorf((phc + dphi) * scale);
-            const int64_t len = sb - sa + 1;
-            if (len < ns) {
-                int64_t s0 = sa % ns;
-                if (s0 < 0) s0 += ns;
-                ca0 = cf + s0;
-                if (s0 + len <= ns) {
-                    ca1 = cf + s0 + len;
-                } else {
-                    ca1 = cf + ns;
-                    cb0 = cf;
-                    cb1 = cf + (s0 + len - ns);
-                }
-            }
+    cat_zero_masks(S, K);  // the union held other things
+    cat_batches(g, wdw, S, [&](bool first) {
+        cat_bins(g, S, P);
+        __syncthreads();
+        BinAcc<M, 1, SELF> A;
+        A.zero();
+        for (int k = cat_next_bin(S); k < K; k = cat_next_bin(S)) {
+            bool any = false;
+            cat_bin_pairs(
+                S, k,
+                [&](int most) {
+                    any = most > 0;
+                    return any;
+                },
+                [&](bool on, int, const float4& qh, const float4& ql) {
+                    const float wd = on ? qh.w : 0.0f, w = on ? ql.w : 0.0f;
+                    harmonicsf<M>(A.a[0], cat_angle(P, qh, ql), wd, wd);
+                    A.a[0][0].y += w;
+                    if (SELF) A.q[0] = __ffma2_rn(make_float2(wd, w), make_float2(wd, w), A.q[0]);
+                });
+            if (any || first) A.flush(ws, sub_floats, K, k, first, M);
         }
-#pragma unroll 1
-        for (int sg = 0; sg < 2; ++sg) {
-            const int64_t cl0 = sg == 0 ? ca0 : cb0, cl1 = sg == 0 ? ca1 : cb1;
-            if (cl1 <= cl0) continue;
-            const int64_t p0 = g.cell_start[cl0], p1 = g.cell_start[cl1];
-            for (int64_t base = p0; base < p1; base += TILE, ++chunk) {
-                if ((chunk % NWARPS) != warp) continue;
-                const int64_t j = base + lane;
-                __syncwarp();
-                if (j < p1) {
-                    wh[lane] = g.p_hi[j];
-                    wl[lane] = g.p_lo[j];
-                    wv[lane] = wdw[j];
-                }
-                __syncwarp();
-                const int cnt = (int)min((int64_t)TILE, p1 - base);
-                // pass A: bins, per-lane masks
-                unsigned mk[CAT_GROUPS];
-#pragma unroll
-                for (int q = 0; q < CAT_GROUPS; ++q) mk[q] = 0u;
-                unsigned mo = 0u;
-                int kb = -1000;
-                for (int u = 0; u < cnt; ++u) {
-                    const float4 qh = wh[u], ql = wl[u];
-                    const float dx = (qh.x - P.hx) + (ql.x - P.lx);
-                    const float dy = (qh.y - P.hy) + (ql.y - P.ly);
-                    const float dz = (qh.z - P.hz) + (ql.z - P.lz);
-                    const float c2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-                    int k = cat_bin(c2, sE2, slut, g.lut_l0, g.lut_inv, K);
-                    const int e1 = max(k, 0), e2 = min(k + 1, K);
-                    if (fabsf(c2 - sE2[e1]) <= CAT_AMB * sE2[e1] || fabsf(c2 - sE2[e2]) <= CAT_AMB * sE2[e2])
-                        k = cat_exact_bin(g.Ed2, K, g.xyz, (int64_t)__float_as_int(ql.w), P.si);
-                    if (k < 0 || k >= K) continue;
-                    if (kb == -1000) kb = max(k - 3, 0);
-                    const int q = k - kb;
-                    const unsigned bit = 1u << u;
-#pragma unroll
-                    for (int r = 0; r < CAT_GROUPS; ++r)
-                        if (q == r) mk[r] |= bit;
-                    if (q < 0 || q >= CAT_GROUPS) mo |= bit;
-                }
-                // pass B: per bin of the window, in lockstep
-#pragma unroll 1
-                for (int r = 0; r < CAT_GROUPS; ++r) {
-                    unsigned msk = 0u;
-#pragma unroll
-                    for (int q = 0; q < CAT_GROUPS; ++q)
-                        if (q == r) msk = mk[q];
-                    const bool had = msk != 0u;
-                    if (!__any_sync(0xffffffffu, had)) continue;
-                    while (__any_sync(0xffffffffu, msk != 0u)) {
-                        const bool active = msk != 0u;
-                        const int u = active ? __ffs(msk) - 1 : 0;
-                        msk &= msk - 1u;
-                        const float4 qh = wh[u], ql = wl[u];
-                        const float dx = (qh.x - P.hx) + (ql.x - P.lx);
-                        const float dy = (qh.y - P.hy) + (ql.y - P.ly);
-                        const float dz = (qh.z - P.hz) + (ql.z - P.lz);
-                        pair(active, kb + r, dx, dy, dz, wv[u], u);
-                    }
-                    group_end(kb + r, had);
-                }
-                // the rare in-range candidates outside the window, one by one
-                while (__any_sync(0xffffffffu, mo != 0u)) {
-                    const bool active = mo != 0u;
-                    const int u = active ? __ffs(mo) - 1 : 0;
-                    mo &= mo - 1u;
-                    if (active) {
-                        const float4 qh = wh[u], ql = wl[u];
-                        const float dx = (qh.x - P.hx) + (ql.x - P.lx);
-                        const float dy = (qh.y - P.hy) + (ql.y - P.ly);
-                        const float dz = (qh.z - P.hz) + (ql.z - P.lz);
-                        const float c2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-                        int k = cat_bin(c2, sE2, slut, g.lut_l0, g.lut_inv, K);
-                        const int e1 = max(k, 0), e2 = min(k + 1, K);
-                        if (fabsf(c2 - sE2[e1]) <= CAT_AMB * sE2[e1] || fabsf(c2 - sE2[e2]) <= CAT_AMB * sE2[e2])
-                            k = cat_exact_bin(g.Ed2, K, g.xyz, (int64_t)__float_as_int(ql.w), P.si);
-                        single(k, dx, dy, dz, wv[u], u);
-                    }
-                }
-                chunk_end(base, cnt);
-            }
-        }
-    }
+    });
 }
 
-// The tile's moments over the catalogue walk (the body of the forward): every warp
-// walks its share of the cap's candidates for the lane's pivot P with the neighbour
-// values `wdw` and adds its register sums into the tile's shared moments once per bin
-// and chunk.  The caller zeroes the moments before and synchronises after.
+// Forward: persistent CTAs draw tiles.
 template <int M, bool SELF>
-__device__ __forceinline__ void cat_tile_moments(const CatDev& g, const float2* __restrict__ wdw,
-                                                 const float* s_cap, const CatPivot& P, const float* sE2,
-                                                 const unsigned char* slut, float4* sCh, float4* sCl, float2* sCv,
-                                                 float* sA, float* sW, float* sQ, float* sQW) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    float2 acc[M + 1];
-#pragma unroll
-    for (int m = 0; m <= M; ++m) acc[m] = make_float2(0.0f, 0.0f);
-    float W = 0.0f, Qs = 0.0f, QW = 0.0f;
-    cat_walk_grouped(
-        g, wdw, s_cap, P, sE2, slut, sCh + warp * TILE, sCl + warp * TILE, sCv + warp * TILE,
-        [&](bool active, int, float dx, float dy, float dz, float2 v, int) {
-            const float N = fmaf(dx, P.nx, fmaf(dy, P.ny, dz * P.nz));
-            const float E = fmaf(dx, P.ex, dy * P.ey);
-            const float rinv = rsqrtf(fmaxf(fmaf(N, N, E * E), 1e-30f));
-            const float wd = active ? v.x : 0.0f;
-            const float ww = active ? v.y : 0.0f;
-            harmonics<M>(acc, N * rinv, E * rinv, wd, wd);
-            W += ww;
-            if (SELF) {
-                Qs = fmaf(wd, wd, Qs);
-                QW = fmaf(ww, ww, QW);
-            }
-        },
-        [&](int k, bool had) {
-            if (had) {
-                cat_flush<M, SELF>(sA, sW, sQ, sQW, k, lane, acc, W, Qs, QW);
-            }
-        },
-        [&](int k, float dx, float dy, float dz, float2 v, int) {
-            // every group is flushed by now, so the register sums are free
-            const float N = fmaf(dx, P.nx, fmaf(dy, P.ny, dz * P.nz));
-            const float E = fmaf(dx, P.ex, dy * P.ey);
-            const float rinv = rsqrtf(fmaxf(fmaf(N, N, E * E), 1e-30f));
-            harmonics<M>(acc, N * rinv, E * rinv, v.x, v.x);
-            W = v.y;
-            if (SELF) {
-                Qs = v.x * v.x;
-                QW = v.y * v.y;
-            }
-            cat_flush<M, SELF>(sA, sW, sQ, sQW, k, lane, acc, W, Qs, QW);
-        },
-        [&](int64_t, int) {});
-}
-
-template <int M, bool SELF>
-__global__ void __launch_bounds__(NTHREADS, 3) cat_fwd_kernel(CatDev g, MapCall c) {
+__global__ void __launch_bounds__(BT, 4) cat_fwd_kernel(CatDev g, MapCall c) {
     extern __shared__ __align__(16) float smem[];
     __shared__ int s_tile;
-    __shared__ float s_cap[5];  // cap query: phi_c, dphi, first band, last band, full
-    __shared__ float sE2[TPCF_MAX_BINS + 1];
-    __shared__ unsigned char slut[CAT_LUT];
-    const int K = g.K;
-    float* sA = smem;
-    float* sW = sA + (size_t)K * (M + 1) * 2 * TILE;
-    float* sQ = sW + K * TILE;
-    float* sQW = sQ + K * TILE;
-    float* sPiv = sQW + K * TILE;
-    float4* sCh = reinterpret_cast<float4*>(smem + tile_floats<M>(K));
-    float4* sCl = sCh + NWARPS * TILE;
-    float2* sCv = reinterpret_cast<float2*>(sCl + NWARPS * TILE);
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const size_t nfl = tile_floats<M>(K) - 2 * TILE;
-    for (int e = threadIdx.x; e <= K; e += NTHREADS) sE2[e] = g.E2[e];
-    for (int e = threadIdx.x; e < CAT_LUT; e += NTHREADS) slut[e] = g.lut[e];
-    double* slot = c.slots + (size_t)blockIdx.x * n_entries(K, M);
-
+    const CatShared S = cat_shared(reinterpret_cast<char*>(smem), g.K, false);
+    const int lane = threadIdx.x & 31;
+    const size_t sub_floats = sub_floats_rt(g.K, M, SELF);
+    float* ws = c.ws + (size_t)blockIdx.x * c.ws_floats;
+    double* slot = c.slots + (size_t)blockIdx.x * n_entries(g.K, M);
+    cat_load_lut(g, S);
     for (;;) {
         if (threadIdx.x == 0) s_tile = atomicAdd(c.counter, 1);
         __syncthreads();
-        const int tile = s_tile;
-        if ((long long)tile >= g.ntiles) break;
-        const int64_t si = (int64_t)tile * TILE + lane;
-        bool live = false;
-        float2 pv = make_float2(0.0f, 0.0f);
-        if (si < g.n) {
-            const int64_t o = g.orig[si];
-            if (o >= c.piv_lo && o < c.piv_hi) {
-                pv = c.wdw[si];
-                live = pv.y != 0.0f;
-                if (!live) pv = make_float2(0.0f, 0.0f);
-            }
-        }
+        const int64_t tile = s_tile;
+        if (tile >= g.ntiles) break;
+        const bool live = cat_value(g, c.wdw, c.piv_lo, c.piv_hi, tile, lane).y != 0.0f;
         if (!__syncthreads_or(live)) continue;
-        for (size_t e = threadIdx.x; e < nfl; e += NTHREADS) sA[e] = 0.0f;
-        if (threadIdx.x < TILE) {
-            sPiv[lane] = pv.x;
-            sPiv[TILE + lane] = pv.y;
-        }
-        const CatPivot P = cat_pivot(g, si < g.n ? si : -1);
-        if (warp == 0) cat_tile_cap(g, live, P, s_cap);
-        __syncthreads();
-
-        cat_tile_moments<M, SELF>(g, c.wdw, s_cap, P, sE2, slut, sCh, sCl, sCv, sA, sW, sQ, sQW);
-        __syncthreads();
-        if (c.norm != NORM_NONE) tile_normalize<M>(K, sA, sW, c.norm);
-        tile_contract<M>(K, sA, sW, sQ, sQW, sPiv, slot, SELF);
+        const CatPivot P = cat_place(g, S, tile, live);
+        cat_tile_moments<M, SELF>(g, c.wdw, S, P, ws, sub_floats);
+        block_contract<SELF>(
+            g.K, M, ws, sub_floats, 1, 1u,
+            [&](int, int l) { return cat_value(g, c.wdw, c.piv_lo, c.piv_hi, tile, l); }, S.stage, slot, SELF, c.norm);
         __syncthreads();
     }
 }
 
 // Multi-field forward on a catalogue (tpcf_forward_multi): three fields on the same
-// points, each with its own weights.  The tile's cap is walked once per field (the
-// moments of the neighbour fields A, B, C), and tile_contract_multi forms the cyclic
-// sum over the pivot field.  Shared memory: the three fields' moments, the pivots'
-// three (w d, w), and the per-warp candidate staging.
+// points, each with its own weights.  The tile's candidates are gone through once per field (the
+// moments of the neighbour fields A, B, C), and block_contract_multi forms the cyclic
+// sum over the pivot field.
 template <int M>
-__host__ __device__ inline size_t cat_multi_bytes(int K) {
-    return multi_tile_floats(K, M) * sizeof(float) + (size_t)NWARPS * TILE * (2 * sizeof(float4) + sizeof(float2));
-}
-
-template <int M>
-__global__ void __launch_bounds__(NTHREADS, 1) cat_fwd_multi_kernel(CatDev g, MapCall c,
-                                                                    const float2* __restrict__ wdwB,
-                                                                    const float2* __restrict__ wdwC) {
+__global__ void __launch_bounds__(BT, 4) cat_fwd_multi_kernel(CatDev g, MapCall c, const float2* __restrict__ wdwB,
+                                                              const float2* __restrict__ wdwC) {
     extern __shared__ __align__(16) float smem[];
     __shared__ int s_tile;
-    __shared__ float s_cap[5];
-    __shared__ float sE2[TPCF_MAX_BINS + 1];
-    __shared__ unsigned char slut[CAT_LUT];
-    const int K = g.K;
-    const size_t fsz = multi_field_floats(K, M);
-    float* sF = smem;
-    float* sPiv = smem + 3 * fsz;  // [field][w d, w][32]
-    float4* sCh = reinterpret_cast<float4*>(smem + multi_tile_floats(K, M));
-    float4* sCl = sCh + NWARPS * TILE;
-    float2* sCv = reinterpret_cast<float2*>(sCl + NWARPS * TILE);
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int e = threadIdx.x; e <= K; e += NTHREADS) sE2[e] = g.E2[e];
-    for (int e = threadIdx.x; e < CAT_LUT; e += NTHREADS) slut[e] = g.lut[e];
-    double* slot = c.slots + (size_t)blockIdx.x * n_entries_multi(K, M);
+    const CatShared S = cat_shared(reinterpret_cast<char*>(smem), g.K, false);
+    const int lane = threadIdx.x & 31;
+    const size_t sub_floats = sub_floats_rt(g.K, M, false);
+    float* ws = c.ws + (size_t)blockIdx.x * c.ws_floats;
+    double* slot = c.slots + (size_t)blockIdx.x * n_entries_multi(g.K, M);
     const float2* arr[3] = {c.wdw, wdwB, wdwC};
+    cat_load_lut(g, S);
     for (;;) {
         if (threadIdx.x == 0) s_tile = atomicAdd(c.counter, 1);
         __syncthreads();
-        const int tile = s_tile;
-        if ((long long)tile >= g.ntiles) break;
-        const int64_t si = (int64_t)tile * TILE + lane;
-        float2 pv[3] = {make_float2(0.0f, 0.0f), make_float2(0.0f, 0.0f), make_float2(0.0f, 0.0f)};
+        const int64_t tile = s_tile;
+        if (tile >= g.ntiles) break;
         bool live = false;
-        if (si < g.n) {
-            const int64_t o = g.orig[si];
-            if (o >= c.piv_lo && o < c.piv_hi) {
 #pragma unroll
-                for (int f = 0; f < 3; ++f) {
-                    pv[f] = arr[f][si];
-                    live = live || pv[f].y != 0.0f;
-                }
-            }
-        }
+        for (int f = 0; f < 3; ++f)
+            live = live || cat_value(g, arr[f], c.piv_lo, c.piv_hi, tile, lane).y != 0.0f;
         if (!__syncthreads_or(live)) continue;
-        for (size_t e = threadIdx.x; e < 3 * fsz; e += NTHREADS) sF[e] = 0.0f;
-        if (threadIdx.x < TILE) {
-#pragma unroll
-            for (int f = 0; f < 3; ++f) {
-                sPiv[f * 2 * TILE + lane] = pv[f].x;
-                sPiv[f * 2 * TILE + TILE + lane] = pv[f].y;
-            }
-        }
-        const CatPivot P = cat_pivot(g, si < g.n ? si : -1);
-        if (warp == 0) cat_tile_cap(g, live, P, s_cap);
-        __syncthreads();
+        const CatPivot P = cat_place(g, S, tile, live);
 #pragma unroll 1
-        for (int f = 0; f < 3; ++f) {
-            float* sA = sF + f * fsz;
-            cat_tile_moments<M, false>(g, arr[f], s_cap, P, sE2, slut, sCh, sCl, sCv, sA,
-                                       sA + (size_t)K * (M + 1) * 2 * TILE, nullptr, nullptr);
-        }
-        __syncthreads();
-        tile_contract_multi<M>(K, sF, sPiv, slot);
+        for (int f = 0; f < 3; ++f) cat_tile_moments<M, false>(g, arr[f], S, P, ws + f * sub_floats, sub_floats);
+        block_contract_multi(
+            g.K, M, ws, sub_floats, sub_floats, 1, 1u,
+            [&](int f, int, int l) { return cat_value(g, arr[f], c.piv_lo, c.piv_hi, tile, l); }, S.stage, slot);
         __syncthreads();
     }
 }
 
-// Shared memory of the catalogue adjoint: the forward's, plus one m of H and the
-// primary-term sums.
-template <int M>
-__host__ __device__ inline size_t cat_bwd_bytes(int K) {
-    return cat_tile_bytes<M>(K) + ((size_t)K * K * 2 + TILE + NWARPS * TILE) * sizeof(float);
-}
-
 // Catalogue adjoint, dL/d(delta_p) (the map adjoint's three phases on the catalogue
-// walk): phase 1 recomputes the tile's moments, phase 2 forms h = H conj(a) in place
-// and the primary term, phase 3 walks the candidates again and adds
+// walk): phase 1 recomputes the tile's moments, phase 2 (block_h) forms w d H conj(a) in place
+// and the primary term, phase 3 goes through the batches again and adds
 // w_j w_i d_i sum_m (cos(m phi) Re h_m^k + sin(m phi) Im h_m^k) for every in-bin pair;
-// the 32 pivots' contributions to one candidate are summed across the warp before one
+// the 32 pivots' contributions to a candidate are summed in shared memory before one
 // atomic add to its gradient.
 template <int M>
-__global__ void __launch_bounds__(NTHREADS, 2) cat_bwd_kernel(CatDev g, MapCall c) {
+__global__ void __launch_bounds__(BT, 4) cat_bwd_kernel(CatDev g, MapCall c) {
     extern __shared__ __align__(16) float smem[];
     __shared__ int s_tile;
-    __shared__ float s_cap[5];
-    __shared__ float sE2[TPCF_MAX_BINS + 1];
-    __shared__ unsigned char slut[CAT_LUT];
     const int K = g.K;
-    float* sA = smem;
-    float* sW = sA + (size_t)K * (M + 1) * 2 * TILE;
-    float* sQ = sW + K * TILE;
-    float* sQW = sQ + K * TILE;
-    float* sPiv = sQW + K * TILE;
-    float4* sCh = reinterpret_cast<float4*>(smem + tile_floats<M>(K));
-    float4* sCl = sCh + NWARPS * TILE;
-    float2* sCv = reinterpret_cast<float2*>(sCl + NWARPS * TILE);
-    float* sHm = reinterpret_cast<float*>(sCv + NWARPS * TILE);  // [K][K][2], one m at a time
-    float* sPrim = sHm + (size_t)K * K * 2;                       // [TILE], then sG [NWARPS][TILE]
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const size_t nfl = tile_floats<M>(K) - 2 * TILE;
-    for (int e = threadIdx.x; e <= K; e += NTHREADS) sE2[e] = g.E2[e];
-    for (int e = threadIdx.x; e < CAT_LUT; e += NTHREADS) slut[e] = g.lut[e];
-
+    const CatShared S = cat_shared(reinterpret_cast<char*>(smem), K, true);
+    const int lane = threadIdx.x & 31;
+    const size_t sub_floats = sub_floats_rt(K, M, false);
+    float* ws = c.ws + (size_t)blockIdx.x * c.ws_floats;
+    cat_load_lut(g, S);
     for (;;) {
         if (threadIdx.x == 0) s_tile = atomicAdd(c.counter, 1);
         __syncthreads();
-        const int tile = s_tile;
-        if ((long long)tile >= g.ntiles) break;
-        const int64_t si = (int64_t)tile * TILE + lane;
-        bool live = false;
-        float2 pv = make_float2(0.0f, 0.0f);
-        int64_t oi = -1;
-        if (si < g.n) {
-            oi = g.orig[si];
-            if (oi >= c.piv_lo && oi < c.piv_hi) {
-                pv = c.wdw[si];
-                live = pv.y != 0.0f;
-                if (!live) pv = make_float2(0.0f, 0.0f);
-            }
-        }
+        const int64_t tile = s_tile;
+        if (tile >= g.ntiles) break;
+        const bool live = cat_value(g, c.wdw, c.piv_lo, c.piv_hi, tile, lane).y != 0.0f;
         if (!__syncthreads_or(live)) continue;
-        for (size_t e = threadIdx.x; e < nfl; e += NTHREADS) sA[e] = 0.0f;
-        if (threadIdx.x < TILE) {
-            sPiv[lane] = pv.x;
-            sPiv[TILE + lane] = pv.y;
-            sPrim[lane] = 0.0f;
-        }
-        const CatPivot P = cat_pivot(g, si < g.n ? si : -1);
-        if (warp == 0) cat_tile_cap(g, live, P, s_cap);
+        const CatPivot P = cat_place(g, S, tile, live);
+        cat_tile_moments<M, false>(g, c.wdw, S, P, ws, sub_floats);
+        block_h<M, false>(
+            c, K, M, ws, sub_floats, 1, 1u,
+            [&](int s, int l) {
+                return s == 0 ? cat_value(g, c.wdw, c.piv_lo, c.piv_hi, tile, l) : make_float2(0.0f, 0.0f);
+            },
+            [&](int, int l) { return g.orig[tile * TILE + l]; }, S.stage);
         __syncthreads();
-
-        // phase 1: the moments, as in the forward
-        {
-            float2 acc[M + 1];
-#pragma unroll
-            for (int m = 0; m <= M; ++m) acc[m] = make_float2(0.0f, 0.0f);
-            float W = 0.0f, Qs = 0.0f, QW = 0.0f;
-            cat_walk_grouped(
-                g, c.wdw, s_cap, P, sE2, slut, sCh + warp * TILE, sCl + warp * TILE, sCv + warp * TILE,
-                [&](bool active, int, float dx, float dy, float dz, float2 v, int) {
-                    const float N = fmaf(dx, P.nx, fmaf(dy, P.ny, dz * P.nz));
-                    const float E = fmaf(dx, P.ex, dy * P.ey);
-                    const float rinv = rsqrtf(fmaxf(fmaf(N, N, E * E), 1e-30f));
-                    const float wd = active ? v.x : 0.0f;
-                    harmonics<M>(acc, N * rinv, E * rinv, wd, wd);
-                    W += active ? v.y : 0.0f;
-                },
-                [&](int k, bool had) {
-                    if (had) cat_flush<M, false>(sA, sW, sQ, sQW, k, lane, acc, W, Qs, QW);
-                },
-                [&](int k, float dx, float dy, float dz, float2 v, int) {
-                    const float N = fmaf(dx, P.nx, fmaf(dy, P.ny, dz * P.nz));
-                    const float E = fmaf(dx, P.ex, dy * P.ey);
-                    const float rinv = rsqrtf(fmaxf(fmaf(N, N, E * E), 1e-30f));
-                    harmonics<M>(acc, N * rinv, E * rinv, v.x, v.x);
-                    W = v.y;
-                    cat_flush<M, false>(sA, sW, sQ, sQW, k, lane, acc, W, Qs, QW);
-                },
-                [&](int64_t, int) {});
-        }
-        __syncthreads();
-        // phase 2: h = H conj(a) per m, in place; primary term (1/2) sum Re[a h]
-        for (int m = 0; m <= M; ++m) {
-            for (int e = threadIdx.x; e < K * K * 2; e += NTHREADS) sHm[e] = c.H[(size_t)m * K * K * 2 + e];
+        cat_zero_masks(S, K);
+        for (int e = threadIdx.x; e < 32 * BW * S.words; e += BT) S.leg[e] = 0.0f;
+        cat_batches(g, c.wdw, S, [&](bool) {
+            cat_bins(g, S, P);
             __syncthreads();
-            float hrv[(TPCF_MAX_BINS * TILE + NTHREADS - 1) / NTHREADS];
-            float hiv[(TPCF_MAX_BINS * TILE + NTHREADS - 1) / NTHREADS];
-            int nmine = 0;
-            for (int e = threadIdx.x; e < K * TILE; e += NTHREADS, ++nmine) {
-                const int k = e / TILE, l = e - k * TILE;
-                float hr = 0.0f, hi = 0.0f;
-                for (int kp = 0; kp < K; ++kp) {
-                    const float Hr = sHm[(k * K + kp) * 2], Hi = sHm[(k * K + kp) * 2 + 1];
-                    const float* ap = sA + ((size_t)kp * (M + 1) + m) * 2 * TILE;
-                    const float tr = ap[l], ti = ap[TILE + l];
-                    hr = fmaf(Hr, tr, fmaf(-Hi, ti, hr));
-                    hi = fmaf(Hr, ti, fmaf(Hi, tr, hi));
-                }
-                const float* ak = sA + ((size_t)k * (M + 1) + m) * 2 * TILE;
-                atomicAdd(sPrim + l, fmaf(ak[l], hr, ak[TILE + l] * hi));
-                hrv[nmine] = hr;
-                hiv[nmine] = hi;
+            for (int k = cat_next_bin(S); k < K; k = cat_next_bin(S)) {
+                float2 h[1][M + 1];
+                cat_bin_pairs(
+                    S, k,
+                    [&](int most) {
+                        if (most > 0) load_h<M, 1>(h, ws, sub_floats, K, k, 1u, M);
+                        return most > 0;
+                    },
+                    [&](bool on, int u, const float4& qh, const float4& ql) {
+                        float X, Y;
+                        adj_harmonicsf<M>(h[0], cat_angle(P, qh, ql), X, Y);
+                        if (on) atomicAdd(S.leg + u, X + Y);
+                    });
             }
             __syncthreads();
-            nmine = 0;
-            for (int e = threadIdx.x; e < K * TILE; e += NTHREADS, ++nmine) {
-                const int k = e / TILE, l = e - k * TILE;
-                float* ak = sA + ((size_t)k * (M + 1) + m) * 2 * TILE;
-                ak[l] = hrv[nmine];
-                ak[TILE + l] = hiv[nmine];
+            for (int e = threadIdx.x; e < 32 * BW * S.words; e += BT) {
+                if (e % (32 * S.words) >= S.cnt[e / (32 * S.words)]) continue;
+                const float v = S.lo[e].w * S.leg[e];
+                S.leg[e] = 0.0f;
+                if (v != 0.0f) atomicAdd(c.grad + g.orig[S.idx[e]], v);
             }
-            __syncthreads();
-        }
-        if (threadIdx.x < TILE && live) {
-            const float gp = 0.5f * pv.y * sPrim[lane];
-            if (gp != 0.0f) atomicAdd(c.grad + oi, gp);
-        }
-        // phase 3: the neighbour legs; each candidate's contributions from the warp's
-        // 32 pivots are summed in the warp's shared buffer sG, then added once to its
-        // gradient entry at the end of the chunk
-        {
-            float2 h[M + 1];
-            int kh = -1;
-            const float wdi = pv.x;
-            float* sG = sPrim + TILE + warp * TILE;
-            sG[lane] = 0.0f;
-            __syncwarp();
-            auto load_h = [&](int k) {
-                const float* hk = sA + (size_t)k * (M + 1) * 2 * TILE;
-#pragma unroll
-                for (int m = 0; m <= M; ++m)
-                    h[m] = make_float2(hk[(2 * m) * TILE + lane], hk[(2 * m + 1) * TILE + lane]);
-                kh = k;
-            };
-            auto leg = [&](float dx, float dy, float dz, float2 v) {
-                const float N = fmaf(dx, P.nx, fmaf(dy, P.ny, dz * P.nz));
-                const float E = fmaf(dx, P.ex, dy * P.ey);
-                const float rinv = rsqrtf(fmaxf(fmaf(N, N, E * E), 1e-30f));
-                float X, Y;
-                adj_harmonics<M>(h, N * rinv, E * rinv, X, Y);
-                return wdi * v.y * (X + Y);
-            };
-            cat_walk_grouped(
-                g, c.wdw, s_cap, P, sE2, slut, sCh + warp * TILE, sCl + warp * TILE, sCv + warp * TILE,
-                [&](bool active, int k, float dx, float dy, float dz, float2 v, int u) {
-                    // an inactive lane may have no valid bin in this chunk (k is then
-                    // out of range): it neither loads h nor adds anything
-                    if (active) {
-                        if (k != kh) load_h(k);
-                        const float val = leg(dx, dy, dz, v);
-                        if (val != 0.0f) atomicAdd(sG + u, val);
-                    }
-                },
-                [&](int, bool) {},
-                [&](int k, float dx, float dy, float dz, float2 v, int u) {
-                    load_h(k);
-                    const float val = leg(dx, dy, dz, v);
-                    if (val != 0.0f) atomicAdd(sG + u, val);
-                },
-                [&](int64_t base, int cnt) {
-                    __syncwarp();
-                    if (lane < cnt) {
-                        const float val = sG[lane];
-                        if (val != 0.0f) atomicAdd(c.grad + g.orig[base + lane], val);
-                        sG[lane] = 0.0f;
-                    }
-                    __syncwarp();
-                });
-        }
+        });
         __syncthreads();
     }
 }
 
 #if defined(TPCF_M) && TPCF_M == 0  // one definition, in the M = 0 object
 // Exact number of in-bin ordered pairs (i, j) with w_i != 0 and caller index of i in
-// [lo, hi): counts[0] += total.  Same tiles and candidate walk as the forward.
-__global__ void __launch_bounds__(NTHREADS) cat_count_kernel(CatDev g, const float2* __restrict__ wdw, long long lo,
-                                                             long long hi, int* counter,
-                                                             unsigned long long* counts) {
+// [lo, hi): counts[0] += total.  Same tiles and candidates as the forward.
+__global__ void __launch_bounds__(BT) cat_count_kernel(CatDev g, const float2* __restrict__ wdw, long long lo,
+                                                       long long hi, int* counter, unsigned long long* counts) {
+    extern __shared__ __align__(16) float smem[];
     __shared__ int s_tile;
-    __shared__ float s_cap[5];
-    __shared__ float sE2[TPCF_MAX_BINS + 1];
-    __shared__ unsigned char slut[CAT_LUT];
-    __shared__ __align__(16) float4 sCh[NWARPS * TILE];
-    __shared__ __align__(16) float4 sCl[NWARPS * TILE];
-    __shared__ __align__(16) float2 sCv[NWARPS * TILE];
-    const int K = g.K;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int e = threadIdx.x; e <= K; e += NTHREADS) sE2[e] = g.E2[e];
-    for (int e = threadIdx.x; e < CAT_LUT; e += NTHREADS) slut[e] = g.lut[e];
+    const CatShared S = cat_shared(reinterpret_cast<char*>(smem), g.K, false);
+    const int lane = threadIdx.x & 31;
+    cat_load_lut(g, S);
+    cat_zero_masks(S, g.K);
     for (;;) {
         if (threadIdx.x == 0) s_tile = atomicAdd(counter, 1);
         __syncthreads();
-        const int tile = s_tile;
-        if ((long long)tile >= g.ntiles) break;
-        const int64_t si = (int64_t)tile * TILE + lane;
-        bool live = false;
-        if (si < g.n) {
-            const int64_t o = g.orig[si];
-            live = o >= lo && o < hi && wdw[si].y != 0.0f;
-        }
+        const int64_t tile = s_tile;
+        if (tile >= g.ntiles) break;
+        const bool live = cat_value(g, wdw, lo, hi, tile, lane).y != 0.0f;
         if (!__syncthreads_or(live)) continue;
-        const CatPivot P = cat_pivot(g, si < g.n ? si : -1);
-        if (warp == 0) cat_tile_cap(g, live, P, s_cap);
-        __syncthreads();
+        const CatPivot P = cat_place(g, S, tile, live);
         unsigned long long cnt = 0;
-        cat_walk(g, wdw, s_cap, P, sE2, slut, sCh + warp * TILE, sCl + warp * TILE, sCv + warp * TILE,
-                 [&](int k, float, float, float, float2, int) { cnt += (k >= 0 && k < K) ? 1ull : 0ull; });
-        cnt = live ? cnt : 0ull;
+        cat_batches(g, wdw, S, [&](bool) {
+            cat_bins(g, S, P);
+            __syncthreads();
+            for (int e = threadIdx.x; e < g.K * BW * S.words * TILE; e += BT) {
+                cnt += __popc(S.mask[e]);  // lanes that are not live are in no bin
+                S.mask[e] = 0u;
+            }
+        });
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
         if (lane == 0 && cnt) atomicAdd(counts, cnt);

@@ -101,10 +101,14 @@ __global__ void cat_scatter_kernel(int64_t n, const double* __restrict__ xyz, co
     }
 }
 
-// Edge tables: chord^2 = 4 sin^2(theta / 2) in fp64 and fp32, the lookup table over
-// log2(chord^2) and its origin / scale (lut_par[0], lut_par[1]).
+// Edge tables: chord^2 = 4 sin^2(theta / 2) in fp64 and fp32, and the lookup table over the bits
+// of fp32 chord^2 (a positive float's bits rise with it): cell i holds the bits
+// [base + (i << shift), base + ((i + 1) << shift)), the first and the last cell also all below and
+// above.  The cells span the edges, at most 16 octaves of them, as finely as the
+// table allows.  Entry: the number of edges more than a cell's width below the cell; at
+// most one further edge lies within a cell's width of it, else K + 2 (decided without the table).
 __global__ void cat_edges_kernel(int K, const double* theta, double* Ed2, float* E2, unsigned char* lut,
-                                 float* lut_par) {
+                                 int* lut_par) {
     __shared__ float e2[TPCF_MAX_BINS + 1];
     for (int e = threadIdx.x; e <= K; e += blockDim.x) {
         const double h = 2.0 * sin(0.5 * theta[e]);
@@ -113,18 +117,23 @@ __global__ void cat_edges_kernel(int K, const double* theta, double* Ed2, float*
         e2[e] = (float)(h * h);
     }
     __syncthreads();
-    const float l0 = log2f(e2[0]);
-    const float span = log2f(e2[K]) - l0;
-    const float linv = (float)CAT_LUT / fmaxf(span, 1e-6f);
+    const int lo = __float_as_int(fmaxf(e2[0], e2[K] * 0x1p-16f)), hi = __float_as_int(e2[K]);
+    int shift = 8;
+    while ((hi >> shift) - (lo >> shift) + 6 > CAT_LUT) ++shift;
+    const int base = ((lo >> shift) - 2) << shift;
     for (int t = threadIdx.x; t < CAT_LUT; t += blockDim.x) {
-        const float c2 = exp2f(l0 + (float)t / linv);
-        int k = 0;
-        while (k + 1 < K && c2 >= e2[k + 1]) ++k;
-        lut[t] = (unsigned char)k;
+        const float L = t == 0 ? -1.0f : __int_as_float(base + ((t - 1) << shift));
+        const float H = t == CAT_LUT - 1 ? INFINITY : __int_as_float(base + ((t + 2) << shift));
+        int below = 0, in = 0;
+        for (int e = 0; e <= K; ++e) {
+            below += e2[e] < L ? 1 : 0;
+            in += e2[e] >= L && e2[e] <= H ? 1 : 0;
+        }
+        lut[t] = (unsigned char)(in > 1 ? K + 2 : below);
     }
     if (threadIdx.x == 0) {
-        lut_par[0] = l0;
-        lut_par[1] = linv;
+        lut_par[0] = base;
+        lut_par[1] = shift;
     }
 }
 
@@ -254,7 +263,8 @@ tpcf_status build_catalog(tpcf_plan_s* P, const double* d_xyz, int64_t n, cudaSt
     g.hband = M_PI / nb;
     int64_t *band_ns, *band_first, *cell, *cell_start, *orig;
     double *theta, *Ed2, *xyz_s;
-    float *E2, *lut_par;
+    float* E2;
+    int* lut_par;
     unsigned char* lut;
     float4 *p_hi, *p_lo;
     TRY_CUDA(P->alloc(&band_ns, nb));
@@ -270,12 +280,12 @@ tpcf_status build_catalog(tpcf_plan_s* P, const double* d_xyz, int64_t n, cudaSt
     exclusive_scan_kernel<<<1, 1024, 0, s>>>(band_ns, band_first, nb, band_first + nb);
     TRY_CUDA(cudaGetLastError());
     int64_t ncells = 0;
-    float lp[2];
+    int lp[2];
     TRY_CUDA(cudaMemcpyAsync(&ncells, band_first + nb, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
     TRY_CUDA(cudaMemcpyAsync(lp, lut_par, sizeof(lp), cudaMemcpyDeviceToHost, s));
     TRY_CUDA(cudaStreamSynchronize(s));
-    g.lut_l0 = lp[0];
-    g.lut_inv = lp[1];
+    g.lut_base = lp[0];
+    g.lut_shift = lp[1];
 
     // count, scan, scatter (the cell index and cursor arrays are temporary)
     TRY_CUDA(P->alloc(&cell_start, ncells + 1));
@@ -331,6 +341,9 @@ tpcf_status build_catalog(tpcf_plan_s* P, const double* d_xyz, int64_t n, cudaSt
     TRY_CUDA(cudaGetLastError());
     P->bwd_grid = occ_b < 1 ? 0 : (int)std::max<int64_t>(1, std::min<int64_t>(g.ntiles, (int64_t)P->num_sms * occ_b));
     TRY_CUDA(P->alloc(&P->H, (size_t)(P->M + 1) * K * K * 2 + K));
+    P->ws_floats = sub_floats_rt(K, P->M, self != 0);
+    P->ws_slots = std::max(P->fwd_grid, P->bwd_grid);
+    TRY_CUDA(P->alloc(&P->ws, P->ws_floats * P->ws_slots));
     P->nent = n_entries(K, P->M);
     TRY_CUDA(P->alloc(&P->wdw, n));
     TRY_CUDA(P->alloc(&P->slots, (size_t)P->fwd_grid * P->nent));
@@ -384,6 +397,8 @@ tpcf_status catalog_backward(tpcf_plan_s* P, const float* d_delta, const float* 
     c.status = P->status;
     c.H = P->H;
     c.grad = d_grad;
+    c.ws = P->ws;
+    c.ws_floats = P->ws_floats;
     TRY_CUDA(kCat[P->M].bwd(g, c, P->bwd_grid, s));
     return TPCF_OK;
 }
@@ -395,8 +410,9 @@ tpcf_status catalog_forward_multi(tpcf_plan_s* P, const float* const* d_delta, c
     const int K = P->K, M = P->M;
     const int nent = n_entries_multi(K, M);
     if (!P->wdw_b) {  // the second and third fields' packed values and the slots, on the first call
+        // the three fields' moments of one tile have to fit an SM's shared memory (the map's limit)
         const int occ = kCat[M].multi_occ(K);
-        if (occ < 1) {
+        if (((size_t)3 * (K * (M + 1) * 2 + K) * TILE + 6 * TILE) * sizeof(float) + 20480 > 232448 || occ < 1) {
             char msg[160];
             snprintf(msg, sizeof(msg),
                      "tpcf_forward_multi: three fields' moments (K=%d, m_max=%d) do not fit in shared memory", K, M);
@@ -410,6 +426,9 @@ tpcf_status catalog_forward_multi(tpcf_plan_s* P, const float* const* d_delta, c
         TRY_CUDA(P->alloc(&c, g.n));
         TRY_CUDA(P->alloc(&sl, (size_t)grid * nent));
         TRY_CUDA(P->alloc(&su, (size_t)nent));
+        float* w3;
+        TRY_CUDA(P->alloc(&w3, 3 * sub_floats_rt(K, M, false) * grid));
+        P->ws3 = w3;
         P->wdw_c = c;
         P->mslots = sl;
         P->msums = su;
@@ -428,6 +447,8 @@ tpcf_status catalog_forward_multi(tpcf_plan_s* P, const float* const* d_delta, c
     c.slots = P->mslots;
     c.counter = P->counter;
     c.status = P->status;
+    c.ws = P->ws3;
+    c.ws_floats = 3 * sub_floats_rt(K, M, false);
     TRY_CUDA(kCat[M].multi(g, c, P->wdw_b, P->wdw_c, P->multi_grid, s));
     reduce_slots_kernel<<<(nent + 31) / 32, REDUCE_THREADS, 0, s>>>(P->mslots, P->multi_grid, nent, P->msums);
     const int nout = (M + 1) * K * K;
@@ -453,6 +474,8 @@ tpcf_status catalog_forward(tpcf_plan_s* P, const float* d_delta, const float* d
     c.status = P->status;
     c.self_subtract = (P->flags & TPCF_SELF_PAIRS_SUBTRACT) ? 1 : 0;
     c.norm = norm_of_flags(P->flags);
+    c.ws = P->ws;
+    c.ws_floats = P->ws_floats;
     TRY_CUDA(kCat[P->M].fwd(g, c, P->fwd_grid, s));
     reduce_slots_kernel<<<(P->nent + 31) / 32, REDUCE_THREADS, 0, s>>>(P->slots, P->fwd_grid, P->nent, P->sums);
     const int nout = (P->M + 1) * P->K * P->K;

@@ -674,6 +674,10 @@ __device__ __forceinline__ void orbit_bin(const MapDev& g, const PivotRing& P, i
 // shared-memory words feed 64 multiply-adds.  fp32 sums run over four subtiles
 // (128 pivots), then go through shared memory to the slot, in order.
 constexpr int CON_RUN = 4;            // subtiles summed in fp32
+// Pivots summed at a time before they are added to the run's sum: the two multiply-adds of a pivot
+// both round at the size of the sum, and short first sums keep that below one rounding per pivot of a
+// single chain, for 3% more instructions.
+constexpr int CON_FOLD = 16;
 
 // Multipoles staged at once: the groups are of equal size, fit the stage and leave threads for D.
 __host__ __device__ inline int con_group(int K, int mr, int slices) {
@@ -757,12 +761,12 @@ __device__ __forceinline__ void block_contract(int K, int mr, const float* ws, s
             o1[i] = isD ? nm * K * 2 * TILE + k1 * TILE : (ml * K + k1) * 2 * TILE;
             o2[i] = isD ? nm * K * 2 * TILE + k2 * TILE : (ml * K + k2) * 2 * TILE;
         }
-        float2 acc[CB][CB];
+        float2 tot[CB][CB], acc[CB][CB];
         float q1 = 0.0f, q2 = 0.0f;  // self-pair diagonals of bin tid
 #pragma unroll
         for (int i = 0; i < CB; ++i)
 #pragma unroll
-            for (int j = 0; j < CB; ++j) acc[i][j] = make_float2(0.0f, 0.0f);
+            for (int j = 0; j < CB; ++j) tot[i][j] = make_float2(0.0f, 0.0f);
         int run = 0;
         for (int s = 0; s < nsub; ++s) {
             if ((live >> s) & 1u) {
@@ -777,36 +781,47 @@ __device__ __forceinline__ void block_contract(int K, int mr, const float* ws, s
                 stage_wait();
                 __syncthreads();
                 if (norm != NORM_NONE) stage_normalize(K, nm, sA, sW, norm);
-                if (isS) {
+#pragma unroll 1
+                for (int t0 = 0; t0 < TILE; t0 += CON_FOLD) {
+#pragma unroll
+                    for (int i = 0; i < CB; ++i)
+#pragma unroll
+                        for (int j = 0; j < CB; ++j) acc[i][j] = make_float2(0.0f, 0.0f);
+                    if (isS) {
 #pragma unroll 2
-                    for (int t = 0; t < TILE; ++t) {
-                        const int l = (t + lane) & (TILE - 1);  // a warp's 32 reads of a word hit 32 banks
-                        const float w = sPiv[l];
-                        float2 x[CB], y[CB];
+                        for (int t = t0; t < t0 + CON_FOLD; ++t) {
+                            const int l = (t + lane) & (TILE - 1);  // a warp's 32 reads of a word hit 32 banks
+                            const float w = sPiv[l];
+                            float2 x[CB], y[CB];
 #pragma unroll
-                        for (int i = 0; i < CB; ++i) {
-                            x[i] = make_float2(w * sA[o1[i] + l], w * sA[o1[i] + TILE + l]);
-                            y[i] = make_float2(sA[o2[i] + l], sA[o2[i] + TILE + l]);
+                            for (int i = 0; i < CB; ++i) {
+                                x[i] = make_float2(w * sA[o1[i] + l], w * sA[o1[i] + TILE + l]);
+                                y[i] = make_float2(sA[o2[i] + l], sA[o2[i] + TILE + l]);
+                            }
+#pragma unroll
+                            for (int j = 0; j < CB; ++j) {
+                                const float2 z = make_float2(y[j].y, -y[j].x);
+#pragma unroll
+                                for (int i = 0; i < CB; ++i)  // (a c + b d, a d - b c)
+                                    acc[i][j] = __ffma2_rn(make_float2(x[i].x, x[i].x), y[j],
+                                                           __ffma2_rn(make_float2(x[i].y, x[i].y), z, acc[i][j]));
+                            }
                         }
+                    } else if (isD) {
+                        for (int t = t0; t < t0 + CON_FOLD; ++t) {
+                            const int l = (t + lane) & (TILE - 1);
+                            const float w = sPiv[TILE + l];
 #pragma unroll
-                        for (int j = 0; j < CB; ++j) {
-                            const float2 z = make_float2(y[j].y, -y[j].x);
+                            for (int i = 0; i < CB; ++i)
 #pragma unroll
-                            for (int i = 0; i < CB; ++i)  // (a c + b d, a d - b c)
-                                acc[i][j] = __ffma2_rn(make_float2(x[i].x, x[i].x), y[j],
-                                                       __ffma2_rn(make_float2(x[i].y, x[i].y), z, acc[i][j]));
+                                for (int j = 0; j < CB; ++j)
+                                    acc[i][j].x = fmaf(w, sA[o1[i] + l] * sA[o2[j] + l], acc[i][j].x);
                         }
                     }
-                } else if (isD) {
-                    for (int t = 0; t < TILE; ++t) {
-                        const int l = (t + lane) & (TILE - 1);
-                        const float w = sPiv[TILE + l];
 #pragma unroll
-                        for (int i = 0; i < CB; ++i)
+                    for (int i = 0; i < CB; ++i)
 #pragma unroll
-                            for (int j = 0; j < CB; ++j)
-                                acc[i][j].x = fmaf(w, sA[o1[i] + l] * sA[o2[j] + l], acc[i][j].x);
-                    }
+                        for (int j = 0; j < CB; ++j) tot[i][j] = __fadd2_rn(tot[i][j], acc[i][j]);
                 }
                 if (SELF && self && m0 == 0 && tid < K) {
                     const float* Q = sW + (K + tid) * TILE;
@@ -832,13 +847,13 @@ __device__ __forceinline__ void block_contract(int K, int mr, const float* ws, s
                             const int k1 = CB * b1 + i, k2 = CB * b2 + j, pi = k2 * (k2 + 1) / 2 + k1;
                             if (k1 <= k2 && k2 < K) {
                                 if (isD) {
-                                    out[base + pi] = acc[i][j].x;
+                                    out[base + pi] = tot[i][j].x;
                                 } else {
-                                    out[base + 2 * pi] = acc[i][j].x;
-                                    out[base + 2 * pi + 1] = acc[i][j].y;
+                                    out[base + 2 * pi] = tot[i][j].x;
+                                    out[base + 2 * pi + 1] = tot[i][j].y;
                                 }
                             }
-                            acc[i][j] = make_float2(0.0f, 0.0f);
+                            tot[i][j] = make_float2(0.0f, 0.0f);
                         }
                 }
                 if (SELF && self && m0 == 0 && tid < K) {
@@ -891,11 +906,11 @@ __device__ __forceinline__ void block_contract_multi(int K, int mr, const float*
             o1[i] = isD ? nm * K * 2 * TILE + k1 * TILE : (ml * K + k1) * 2 * TILE;
             o2[i] = isD ? nm * K * 2 * TILE + k2 * TILE : (ml * K + k2) * 2 * TILE;
         }
-        float2 acc[CB][CB];
+        float2 tot[CB][CB], acc[CB][CB];
 #pragma unroll
         for (int i = 0; i < CB; ++i)
 #pragma unroll
-            for (int j = 0; j < CB; ++j) acc[i][j] = make_float2(0.0f, 0.0f);
+            for (int j = 0; j < CB; ++j) tot[i][j] = make_float2(0.0f, 0.0f);
         int run = 0;
         for (int s = 0; s < nsub; ++s) {
             if ((live >> s) & 1u) {
@@ -916,35 +931,46 @@ __device__ __forceinline__ void block_contract_multi(int K, int mr, const float*
                     const float* X = sA + ((cyc + 1) % 3) * fstr;
                     const float* Y = sA + ((cyc + 2) % 3) * fstr;
                     const float* pv = sPiv + cyc * 2 * TILE + (isD ? TILE : 0);
-                    if (isS) {
+#pragma unroll 1
+                    for (int t0 = 0; t0 < TILE; t0 += CON_FOLD) {
+#pragma unroll
+                        for (int i = 0; i < CB; ++i)
+#pragma unroll
+                            for (int j = 0; j < CB; ++j) acc[i][j] = make_float2(0.0f, 0.0f);
+                        if (isS) {
 #pragma unroll 2
-                        for (int t = 0; t < TILE; ++t) {
-                            const int l = (t + lane) & (TILE - 1);
-                            const float w = pv[l];
-                            float2 x[CB], y[CB];
+                            for (int t = t0; t < t0 + CON_FOLD; ++t) {
+                                const int l = (t + lane) & (TILE - 1);
+                                const float w = pv[l];
+                                float2 x[CB], y[CB];
 #pragma unroll
-                            for (int i = 0; i < CB; ++i) {
-                                x[i] = make_float2(w * X[o1[i] + l], w * X[o1[i] + TILE + l]);
-                                y[i] = make_float2(Y[o2[i] + l], Y[o2[i] + TILE + l]);
+                                for (int i = 0; i < CB; ++i) {
+                                    x[i] = make_float2(w * X[o1[i] + l], w * X[o1[i] + TILE + l]);
+                                    y[i] = make_float2(Y[o2[i] + l], Y[o2[i] + TILE + l]);
+                                }
+#pragma unroll
+                                for (int j = 0; j < CB; ++j) {
+                                    const float2 z = make_float2(y[j].y, -y[j].x);
+#pragma unroll
+                                    for (int i = 0; i < CB; ++i)
+                                        acc[i][j] = __ffma2_rn(make_float2(x[i].x, x[i].x), y[j],
+                                                               __ffma2_rn(make_float2(x[i].y, x[i].y), z, acc[i][j]));
+                                }
                             }
-#pragma unroll
-                            for (int j = 0; j < CB; ++j) {
-                                const float2 z = make_float2(y[j].y, -y[j].x);
+                        } else if (isD) {
+                            for (int t = t0; t < t0 + CON_FOLD; ++t) {
+                                const int l = (t + lane) & (TILE - 1);
 #pragma unroll
                                 for (int i = 0; i < CB; ++i)
-                                    acc[i][j] = __ffma2_rn(make_float2(x[i].x, x[i].x), y[j],
-                                                           __ffma2_rn(make_float2(x[i].y, x[i].y), z, acc[i][j]));
+#pragma unroll
+                                    for (int j = 0; j < CB; ++j)
+                                        acc[i][j].x = fmaf(pv[l], X[o1[i] + l] * Y[o2[j] + l], acc[i][j].x);
                             }
                         }
-                    } else if (isD) {
-                        for (int t = 0; t < TILE; ++t) {
-                            const int l = (t + lane) & (TILE - 1);
 #pragma unroll
-                            for (int i = 0; i < CB; ++i)
+                        for (int i = 0; i < CB; ++i)
 #pragma unroll
-                                for (int j = 0; j < CB; ++j)
-                                    acc[i][j].x = fmaf(pv[l], X[o1[i] + l] * Y[o2[j] + l], acc[i][j].x);
-                        }
+                            for (int j = 0; j < CB; ++j) tot[i][j] = __fadd2_rn(tot[i][j], acc[i][j]);
                     }
                 }
                 ++run;
@@ -961,13 +987,13 @@ __device__ __forceinline__ void block_contract_multi(int K, int mr, const float*
                             const int k1 = CB * b1 + i, k2 = CB * b2 + j;
                             if (k1 < K && k2 < K) {
                                 if (isD) {
-                                    out[2 * nm * KK + k1 * K + k2] = acc[i][j].x;
+                                    out[2 * nm * KK + k1 * K + k2] = tot[i][j].x;
                                 } else {
-                                    out[2 * (ml * KK + k1 * K + k2)] = acc[i][j].x;
-                                    out[2 * (ml * KK + k1 * K + k2) + 1] = acc[i][j].y;
+                                    out[2 * (ml * KK + k1 * K + k2)] = tot[i][j].x;
+                                    out[2 * (ml * KK + k1 * K + k2) + 1] = tot[i][j].y;
                                 }
                             }
-                            acc[i][j] = make_float2(0.0f, 0.0f);
+                            tot[i][j] = make_float2(0.0f, 0.0f);
                         }
                 }
                 __syncthreads();

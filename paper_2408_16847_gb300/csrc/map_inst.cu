@@ -137,16 +137,16 @@ int TPCF_CAT(map_fwd_multi_occupancy_m, TPCF_M)() {
 // Multi-field forward on a catalogue.
 cudaError_t TPCF_CAT(cat_fwd_multi_launch_m, TPCF_M)(const CatDev& g, const MapCall& c, const float2* wdwB,
                                                      const float2* wdwC, int grid, cudaStream_t s) {
-    const size_t smem = cat_multi_bytes<TPCF_M>(g.K);
+    const size_t smem = cat_fwd_bytes<TPCF_M>(g.K);
     auto* k = cat_fwd_multi_kernel<TPCF_M>;
-    cudaError_t e = prefer_shared(k, smem);
+    cudaError_t e = prefer_shared(k, smem, BT);
     if (e != cudaSuccess) return e;
-    k<<<grid, NTHREADS, smem, s>>>(g, c, wdwB, wdwC);
+    k<<<grid, BT, smem, s>>>(g, c, wdwB, wdwC);
     return cudaGetLastError();
 }
 
 int TPCF_CAT(cat_fwd_multi_occupancy_m, TPCF_M)(int K) {
-    return occupancy(cat_fwd_multi_kernel<TPCF_M>, cat_multi_bytes<TPCF_M>(K));
+    return occupancy(cat_fwd_multi_kernel<TPCF_M>, cat_fwd_bytes<TPCF_M>(K), BT);
 }
 
 // Forward that reads the caller's delta and w directly (no packed copy).
@@ -187,48 +187,48 @@ int TPCF_CAT(batch_bwd_occupancy_m, TPCF_M)(size_t smem) { return occupancy(batc
 
 // Catalogue forward.
 cudaError_t TPCF_CAT(cat_fwd_launch_m, TPCF_M)(const CatDev& g, const MapCall& c, int grid, cudaStream_t s) {
-    const size_t smem = cat_tile_bytes<TPCF_M>(g.K);
+    const size_t smem = cat_fwd_bytes<TPCF_M>(g.K);
     if (c.self_subtract) {
         auto* k = cat_fwd_kernel<TPCF_M, true>;
-        cudaError_t e = prefer_shared(k, smem);
+        cudaError_t e = prefer_shared(k, smem, BT);
         if (e != cudaSuccess) return e;
-        k<<<grid, NTHREADS, smem, s>>>(g, c);
+        k<<<grid, BT, smem, s>>>(g, c);
     } else {
         auto* k = cat_fwd_kernel<TPCF_M, false>;
-        cudaError_t e = prefer_shared(k, smem);
+        cudaError_t e = prefer_shared(k, smem, BT);
         if (e != cudaSuccess) return e;
-        k<<<grid, NTHREADS, smem, s>>>(g, c);
+        k<<<grid, BT, smem, s>>>(g, c);
     }
     return cudaGetLastError();
 }
 
 int TPCF_CAT(cat_fwd_occupancy_m, TPCF_M)(int K, int self_subtract) {
-    const size_t smem = cat_tile_bytes<TPCF_M>(K);
-    return self_subtract ? occupancy(cat_fwd_kernel<TPCF_M, true>, smem) : occupancy(cat_fwd_kernel<TPCF_M, false>, smem);
+    const size_t smem = cat_fwd_bytes<TPCF_M>(K);
+    return self_subtract ? occupancy(cat_fwd_kernel<TPCF_M, true>, smem, BT) : occupancy(cat_fwd_kernel<TPCF_M, false>, smem, BT);
 }
 
 // Catalogue adjoint.
 cudaError_t TPCF_CAT(cat_bwd_launch_m, TPCF_M)(const CatDev& g, const MapCall& c, int grid, cudaStream_t s) {
     const size_t smem = cat_bwd_bytes<TPCF_M>(g.K);
     auto* k = cat_bwd_kernel<TPCF_M>;
-    cudaError_t e = prefer_shared(k, smem);
+    cudaError_t e = prefer_shared(k, smem, BT);
     if (e != cudaSuccess) return e;
-    k<<<grid, NTHREADS, smem, s>>>(g, c);
+    k<<<grid, BT, smem, s>>>(g, c);
     return cudaGetLastError();
 }
 
 int TPCF_CAT(cat_bwd_occupancy_m, TPCF_M)(int K) {
     const size_t smem = cat_bwd_bytes<TPCF_M>(K);
-    int nb = 0;
-    prefer_shared(cat_bwd_kernel<TPCF_M>, smem);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, cat_bwd_kernel<TPCF_M>, NTHREADS, smem);
-    return nb;
+    return occupancy(cat_bwd_kernel<TPCF_M>, smem, BT);
 }
 
 #if TPCF_M == 0
 cudaError_t cat_count_launch(const CatDev& g, const float2* wdw, long long lo, long long hi, int* counter,
                              unsigned long long* counts, int grid, cudaStream_t s) {
-    cat_count_kernel<<<grid, NTHREADS, 0, s>>>(g, wdw, lo, hi, counter, counts);
+    const size_t smem = cat_smem_bytes(g.K, false, 0);
+    cudaError_t e = prefer_shared(cat_count_kernel, smem, BT);
+    if (e != cudaSuccess) return e;
+    cat_count_kernel<<<grid, BT, smem, s>>>(g, wdw, lo, hi, counter, counts);
     return cudaGetLastError();
 }
 

@@ -37,7 +37,6 @@ namespace tpcf {
 
 constexpr float AMBIGUITY = 1.0e-6f;  // > worst fp32 error of the edge position (~1.5e-7 px)
 constexpr float FAST_XMAX = 0.25f;    // |half longitude offset| covered by the polynomial
-constexpr int FLUSH_RINGS = 8;        // default rings summed in registers before a shared-memory flush
 
 // Fire-and-forget FP64 reduction of an fp32 partial sum into a CTA slot.  The float
 // is widened by moving its IEEE 754 fields (exponent re-biased by 1023 - 127 = 896,
@@ -286,12 +285,6 @@ __device__ __forceinline__ void harmonicsf(float2 (&acc)[M + 1], const Fold& f, 
     }
 }
 
-template <int M>
-__device__ __forceinline__ void harmonics(float2 (&acc)[M + 1], float cph, float sph, float wc, float ws,
-                                          int mr = M) {
-    harmonicsf<M>(acc, fold_angle(cph, sph), wc, ws, mr);
-}
-
 // p mod n for -n <= p < 2n (every unwrapped index of a run lies in that range).
 __device__ __forceinline__ int wrap_idx(int p, int n) {
     return p < 0 ? p + n : (p >= n ? p - n : p);
@@ -427,14 +420,6 @@ __device__ __forceinline__ ExactCtx exact_ctx(const MapDev& g, const PivotRing& 
     return x;
 }
 
-// Shared-memory layout of a tile's moments.
-//   A[k][m][2][32] : sum w d cos(m phi), sum w d sin(m phi)   (a = re - i im)
-//   W[k][32], Q[k][32], QW[k][32], piv[2][32] (w d, w of the pivots)
-template <int M>
-__host__ __device__ inline size_t tile_floats(int K, bool self = true) {
-    return tile_floats_rt(K, M, self);
-}
-
 // Load the tile's pivot description; returns false if no lane has w != 0.
 __device__ __forceinline__ PivotRing pivot_ring(const MapDev& g, int i) {
     PivotRing P;
@@ -449,44 +434,6 @@ __device__ __forceinline__ PivotRing pivot_ring(const MapDev& g, int i) {
     return P;
 }
 
-// Per-pivot normalisation of the tile's moments (Sec. 3.1): each lane's a_m^k is
-// divided by its bin weight W^k (NORM_BIN_MEAN) or by its total sum_k W^k
-// (NORM_PIVOT_TOTAL), 0 where that weight is 0; W^k is then set to 1, so that the
-// contraction's D entries become the tile's sum of pivot weights.  Layout of
-// tile_moments (m-major within each bin, TILE lanes innermost).  Called by every
-// thread of the CTA after the moments are complete (contains barriers).
-template <int M>
-__device__ __forceinline__ void tile_normalize(int K, float* sA, float* sW, int norm, int mr = M) {
-    constexpr int PER = (TPCF_MAX_BINS * TILE + NTHREADS - 1) / NTHREADS;
-    float inv[PER];
-#pragma unroll
-    for (int u = 0; u < PER; ++u) {
-        const int e = threadIdx.x + u * NTHREADS;
-        float W = 0.0f;
-        if (e < K * TILE) {
-            if (norm == NORM_BIN_MEAN) {
-                W = sW[e];
-            } else {
-                const int l = e & (TILE - 1);
-                for (int k = 0; k < K; ++k) W += sW[k * TILE + l];
-            }
-        }
-        inv[u] = W > 0.0f ? 1.0f / W : 0.0f;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int u = 0; u < PER; ++u) {
-        const int e = threadIdx.x + u * NTHREADS;
-        if (e < K * TILE) {
-            const int k = e / TILE, l = e & (TILE - 1);
-            float* a = sA + (size_t)k * (mr + 1) * 2 * TILE + l;
-            for (int j = 0; j < 2 * (mr + 1); ++j) a[j * TILE] *= inv[u];
-            sW[e] = 1.0f;
-        }
-    }
-    __syncthreads();
-}
-
 // Block (b1 <= b2) number i of the CB x CB blocks of a triangle, columns first.
 __device__ __forceinline__ void tri_block(int i, int& b1, int& b2) {
     b2 = (int)((sqrtf(8.0f * i + 1.0f) - 1.0f) * 0.5f);
@@ -495,96 +442,7 @@ __device__ __forceinline__ void tri_block(int i, int& b1, int& b2) {
     b1 = i - b2 * (b2 + 1) / 2;
 }
 
-// Per-tile partial sums into the CTA's FP64 slot (eq. zetamEst2 summed over the
-// tile's pivots).  Slot layout: for m, for pair (k1 <= k2): (Re S, Im S); then D for
-// pairs; then sum_i w_i d_i Q^k(i) and sum_i w_i QW^k(i) for k.
-//
-// A thread takes a 4 x 4 block of bin pairs of one multipole over half of the tile's pivots:
-// 17 shared-memory words feed 64 multiply-adds (one bin pair per thread needed 5 words for 8,
-// and the loads bounded it).  Neighbouring lanes hold the two halves; they add them, and
-// one of them adds the real part to the slot, the other the imaginary part.
-constexpr int CB = 4;  // bins on a side of a block
-
-template <int M>
-__device__ __forceinline__ void tile_contract(int K, const float* sA, const float* sW, const float* sQ,
-                                              const float* sQW, const float* sPiv, double* slot,
-                                              bool self, int mr = M) {
-    const int P = n_pairs_tri(K);
-    const int nS = (mr + 1) * P;
-    const float* wd = sPiv;
-    const float* wt = sPiv + TILE;
-    const int nb = (K + CB - 1) / CB, nbp = nb * (nb + 1) / 2;
-    const int half = threadIdx.x & 1, l0 = threadIdx.x >> 1;
-    const size_t kstr = (size_t)(mr + 1) * 2 * TILE;
-    // both lanes of a pair take the same number of turns (2 (mr + 1) nbp is even)
-    for (int e = threadIdx.x; e < 2 * (mr + 1) * nbp; e += NTHREADS) {
-        const int m = (e >> 1) / nbp;
-        int b1, b2;
-        tri_block((e >> 1) - m * nbp, b1, b2);
-        const float *r1[CB], *r2[CB];
-#pragma unroll
-        for (int i = 0; i < CB; ++i) {  // bins past the last one repeat it and are not written
-            r1[i] = sA + min(CB * b1 + i, K - 1) * kstr + m * 2 * TILE + half * (TILE / 2);
-            r2[i] = sA + min(CB * b2 + i, K - 1) * kstr + m * 2 * TILE + half * (TILE / 2);
-        }
-        float2 acc[CB][CB];
-#pragma unroll
-        for (int i = 0; i < CB; ++i)
-#pragma unroll
-            for (int j = 0; j < CB; ++j) acc[i][j] = make_float2(0.0f, 0.0f);
-#pragma unroll 2
-        for (int t = 0; t < TILE / 2; ++t) {
-            const int l = (t + l0) & (TILE / 2 - 1);  // a warp's 32 reads of a word hit 32 banks
-            const float w = wd[half * (TILE / 2) + l];
-            float2 x[CB], y[CB], z[CB];
-#pragma unroll
-            for (int i = 0; i < CB; ++i) {
-                x[i] = make_float2(w * r1[i][l], w * r1[i][TILE + l]);
-                y[i] = make_float2(r2[i][l], r2[i][TILE + l]);
-                z[i] = make_float2(y[i].y, -y[i].x);
-            }
-#pragma unroll
-            for (int i = 0; i < CB; ++i)
-#pragma unroll
-                for (int j = 0; j < CB; ++j)  // (a c + b d, a d - b c)
-                    acc[i][j] = __ffma2_rn(make_float2(x[i].x, x[i].x), y[j],
-                                           __ffma2_rn(make_float2(x[i].y, x[i].y), z[j], acc[i][j]));
-        }
-        const unsigned pair = 3u << (threadIdx.x & 30);
-#pragma unroll
-        for (int i = 0; i < CB; ++i)
-#pragma unroll
-            for (int j = 0; j < CB; ++j) {
-                const float2 v = acc[i][j];
-                const float s = (half ? v.y : v.x) + __shfl_xor_sync(pair, half ? v.x : v.y, 1);
-                const int k1 = CB * b1 + i, k2 = CB * b2 + j;
-                if (k1 <= k2 && k2 < K) red_add_f32(slot + 2 * (m * P + k2 * (k2 + 1) / 2 + k1) + half, s);
-            }
-    }
-    for (int e = threadIdx.x; e < P + (self ? K : 0); e += NTHREADS) {
-        if (e < P) {
-            int k1, k2;
-            tri_block(e, k1, k2);
-            float s = 0.0f;
-#pragma unroll 8
-            for (int j = 0; j < TILE; ++j) {
-                const int l = (j + threadIdx.x) & (TILE - 1);
-                s = fmaf(wt[l], sW[k1 * TILE + l] * sW[k2 * TILE + l], s);
-            }
-            red_add_f32(slot + 2 * nS + e, s);
-        } else {
-            const int k = e - P;
-            float s1 = 0.0f, s2 = 0.0f;
-            for (int j = 0; j < TILE; ++j) {
-                const int l = (j + threadIdx.x) & (TILE - 1);
-                s1 = fmaf(wd[l], sQ[k * TILE + l], s1);
-                s2 = fmaf(wt[l], sQW[k * TILE + l], s2);
-            }
-            red_add_f32(slot + 2 * nS + P + k, s1);
-            red_add_f32(slot + 2 * nS + P + K + k, s2);
-        }
-    }
-}
+constexpr int CB = 4;  // bins on a side of a block of the contraction
 
 // ------------------------------------------------- tensor-core contraction (TF32x3)
 // The contraction of eq. zetamEst2 over a tile's 32 pivots is, for each m, the Gram
@@ -1028,56 +886,6 @@ __global__ void __launch_bounds__(BT, 4) batch_fwd_kernel(const BatchItem* __res
 //     D(k1,k2)   += sum_i w^P_i W^{k1}(i; X) W^{k2}(i; Y),
 // into the CTA's FP64 slot.  These sums are not Hermitian: the slot holds the full
 // K x K matrices, for m, for (k1, k2): (Re S, Im S); then D for (k1, k2).
-// multi_field_floats, multi_tile_floats, tile_contract_multi: the catalogue's form, whose tile
-// keeps the three fields' moments in shared memory.
-__host__ __device__ inline size_t multi_field_floats(int K, int M) { return (size_t)K * (M + 1) * 2 * TILE + (size_t)K * TILE; }
-__host__ __device__ inline size_t multi_tile_floats(int K, int M) { return 3 * multi_field_floats(K, M) + 6 * TILE; }
-
-template <int M>
-__device__ __forceinline__ void tile_contract_multi(int K, const float* sF, const float* sPiv, double* slot) {
-    const size_t fsz = multi_field_floats(K, M);
-    const int KK = K * K;
-    const int nS = (M + 1) * KK;
-    const int cyc[3][3] = {{0, 1, 2}, {1, 2, 0}, {2, 0, 1}};
-    for (int e = threadIdx.x; e < nS + KK; e += NTHREADS) {
-        if (e < nS) {
-            const int m = e / KK, r = e - m * KK, k1 = r / K, k2 = r - k1 * K;
-            float sr = 0.0f, si = 0.0f;
-#pragma unroll
-            for (int t = 0; t < 3; ++t) {
-                const float* wd = sPiv + cyc[t][0] * 2 * TILE;
-                const float* r1 = sF + cyc[t][1] * fsz + ((size_t)k1 * (M + 1) + m) * 2 * TILE;
-                const float* i1 = r1 + TILE;
-                const float* r2 = sF + cyc[t][2] * fsz + ((size_t)k2 * (M + 1) + m) * 2 * TILE;
-                const float* i2 = r2 + TILE;
-#pragma unroll 8
-                for (int j = 0; j < TILE; ++j) {
-                    const int l = (j + threadIdx.x) & (TILE - 1);
-                    const float a = r1[l], b = i1[l], cc = r2[l], d = i2[l];
-                    sr = fmaf(wd[l], fmaf(a, cc, b * d), sr);
-                    si = fmaf(wd[l], fmaf(a, d, -b * cc), si);
-                }
-            }
-            red_add_f32(slot + 2 * e, sr);
-            red_add_f32(slot + 2 * e + 1, si);
-        } else {
-            const int idx = e - nS, k1 = idx / K, k2 = idx - k1 * K;
-            float sd = 0.0f;
-#pragma unroll
-            for (int t = 0; t < 3; ++t) {
-                const float* wt = sPiv + cyc[t][0] * 2 * TILE + TILE;
-                const float* W1 = sF + cyc[t][1] * fsz + (size_t)K * (M + 1) * 2 * TILE + k1 * TILE;
-                const float* W2 = sF + cyc[t][2] * fsz + (size_t)K * (M + 1) * 2 * TILE + k2 * TILE;
-                for (int j = 0; j < TILE; ++j) {
-                    const int l = (j + threadIdx.x) & (TILE - 1);
-                    sd = fmaf(wt[l], W1[l] * W2[l], sd);
-                }
-            }
-            red_add_f32(slot + 2 * nS + idx, sd);
-        }
-    }
-}
-
 // The multi-field forward: c.wdw holds (w d, w) of field A, wdwB and wdwC those of
 // B and C; the block's workspace holds the three fields' in turn.
 template <int M>
@@ -1201,12 +1009,6 @@ __device__ __forceinline__ void adj_harmonicsf(const float2 (&h)[M + 1], const F
     }
     X = fmaf(sg, od.x, ev.x);
     Y = fmaf(sg, od.y, ev.y);
-}
-
-template <int M>
-__device__ __forceinline__ void adj_harmonics(const float2 (&h)[M + 1], float cph, float sph, float& X, float& Y,
-                                              int mr = M) {
-    adj_harmonicsf<M>(h, fold_angle(cph, sph), X, Y, mr);
 }
 
 // Adjoint: persistent CTAs draw work items (block, part); c.step: see bwd_block.

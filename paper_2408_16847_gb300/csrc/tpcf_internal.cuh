@@ -53,7 +53,7 @@ struct MapDev {
 // Read-only device view of a catalogue plan: the points sorted into a sphere grid
 // of colatitude bands, each cut into equal longitude sectors (cells).  Points of a
 // cell are contiguous, cells are ordered band by band, sectors by longitude.
-constexpr int CAT_LUT = 512;  // entries of the bin lookup table (uniform in log2 chord^2)
+constexpr int CAT_LUT = 1024;  // entries of the bin lookup table (uniform in the bits of fp32 chord^2)
 struct CatDev {
     int64_t n;
     int K, M;
@@ -69,8 +69,8 @@ struct CatDev {
     double theta_max;            // outer bin edge (rad)
     const float* E2;             // [K+1] chord^2 of the edges, fp32
     const double* Ed2;           // [K+1] chord^2 of the edges, fp64
-    const unsigned char* lut;    // [CAT_LUT] bin at the lower end of each table cell
-    float lut_l0, lut_inv;       // table origin log2(E2[0]) and entries per unit of log2
+    const unsigned char* lut;    // [CAT_LUT] first edge above each table cell's lower end (cat_edges_kernel)
+    int lut_base, lut_shift;     // bits of the table's origin, and their right shift to a cell
     int64_t ntiles;              // ceil(n / TILE)
 };
 
@@ -171,13 +171,6 @@ __host__ __device__ constexpr size_t adj_smem_bytes(int M) {
     const size_t c = LIN_HEAD + (size_t)2 * LIN_CHUNK * lin_stride(M) + (LIN_CELLS + 4) * 4 + LIN_CELLS * 2;
     const size_t d = a > b ? a : b;
     return d > c ? d : c;
-}
-
-// Shared memory (floats) of a map forward tile with runtime m_max mr: moments
-// A[k][m][re/im][32], W, Q, QW [k][32], the pivots' (w d, w).
-// (Q, QW: self-pair subtraction only.)
-__host__ __device__ inline size_t tile_floats_rt(int K, int mr, bool self) {
-    return (size_t)K * (mr + 1) * 2 * TILE + (self ? 3 : 1) * (size_t)K * TILE + 2 * TILE;
 }
 
 // Device status bits.
