@@ -189,35 +189,37 @@ static tpcf_status build_map(tpcf_plan_s* P, int64_t nside, cudaStream_t s) {
     unsigned char* lin;  // ring classes (map_block.cuh)
     int* reach;
     float4* rc;
-    TRY_CUDA(P->alloc(&first, nrings));
-    TRY_CUDA(P->alloc(&npr, nrings));
-    TRY_CUDA(P->alloc(&shift, nrings));
-    TRY_CUDA(P->alloc(&z, nrings));
-    TRY_CUDA(P->alloc(&sd, nrings));
-    TRY_CUDA(P->alloc(&th, nrings));
-    TRY_CUDA(P->alloc(&zf, nrings));
-    TRY_CUDA(P->alloc(&sf, nrings));
-    TRY_CUDA(P->alloc(&rstep, nrings));
-    TRY_CUDA(P->alloc(&rinvn, nrings));
-    TRY_CUDA(P->alloc(&sf_lo, nrings));
-    TRY_CUDA(P->alloc(&rstep_lo, nrings));
-    TRY_CUDA(P->alloc(&rinvn_lo, nrings));
-    TRY_CUDA(P->alloc(&ring_range, nrings));
-    TRY_CUDA(P->alloc(&bin_range, (size_t)nrings * K));
-    TRY_CUDA(P->alloc(&pair_off, nrings));
-    TRY_CUDA(P->alloc(&tile_off, nrings));
-    TRY_CUDA(P->alloc(&npairs_r, nrings));
-    TRY_CUDA(P->alloc(&ntiles_r, nrings));
-    TRY_CUDA(P->alloc(&lin_off, nrings));
-    TRY_CUDA(P->alloc(&orb_off, nrings));
-    TRY_CUDA(P->alloc(&nlin_r, nrings));
-    TRY_CUDA(P->alloc(&norb_r, nrings));
-    TRY_CUDA(P->alloc(&lin, nrings));
-    TRY_CUDA(P->alloc(&reach, nrings));
-    TRY_CUDA(P->alloc(&rc, 2 * (size_t)nrings));
-    TRY_CUDA(P->alloc(&tot, 4));
-    TRY_CUDA(P->alloc(&E, K + 1));
-    TRY_CUDA(P->alloc(&theta, K + 1));
+    tpcf_plan_s::Arrays rings, pairs, scratch;
+    rings.add(&first, nrings);
+    rings.add(&npr, nrings);
+    rings.add(&shift, nrings);
+    rings.add(&z, nrings);
+    rings.add(&sd, nrings);
+    rings.add(&th, nrings);
+    rings.add(&zf, nrings);
+    rings.add(&sf, nrings);
+    rings.add(&rstep, nrings);
+    rings.add(&rinvn, nrings);
+    rings.add(&sf_lo, nrings);
+    rings.add(&rstep_lo, nrings);
+    rings.add(&rinvn_lo, nrings);
+    rings.add(&ring_range, nrings);
+    rings.add(&bin_range, (size_t)nrings * K);
+    rings.add(&pair_off, nrings);
+    rings.add(&tile_off, nrings);
+    rings.add(&npairs_r, nrings);
+    rings.add(&ntiles_r, nrings);
+    rings.add(&lin_off, nrings);
+    rings.add(&orb_off, nrings);
+    rings.add(&nlin_r, nrings);
+    rings.add(&norb_r, nrings);
+    rings.add(&lin, nrings);
+    rings.add(&reach, nrings);
+    rings.add(&rc, 2 * (size_t)nrings);
+    rings.add(&tot, 4);
+    rings.add(&E, K + 1);
+    rings.add(&theta, K + 1);
+    TRY_CUDA(rings.take(P));
     TRY_CUDA(cudaMemcpyAsync(theta, P->edges.data(), sizeof(double) * (K + 1), cudaMemcpyHostToDevice, s));
     edges_kernel<<<1, 64, 0, s>>>(K, theta, E);
     ring_table_kernel<<<n_blocks(nrings, 128), 128, 0, s>>>((int)nside, nrings, first, npr, shift, z, sd, th,
@@ -238,19 +240,20 @@ static tpcf_status build_map(tpcf_plan_s* P, int64_t nside, cudaStream_t s) {
     P->lin_off_h.resize(nrings + 1);
     P->orb_off_h.resize(nrings + 1);
     P->lin_h.resize(nrings);
-    TRY_CUDA(cudaMemcpy(P->tile_off_h.data(), tile_off, sizeof(int64_t) * nrings, cudaMemcpyDeviceToHost));
-    TRY_CUDA(cudaMemcpy(P->lin_off_h.data(), lin_off, sizeof(int64_t) * nrings, cudaMemcpyDeviceToHost));
-    TRY_CUDA(cudaMemcpy(P->orb_off_h.data(), orb_off, sizeof(int64_t) * nrings, cudaMemcpyDeviceToHost));
+    TRY_CUDA(cudaMemcpyAsync(P->tile_off_h.data(), tile_off, sizeof(int64_t) * nrings, cudaMemcpyDeviceToHost, s));
+    TRY_CUDA(cudaMemcpyAsync(P->lin_off_h.data(), lin_off, sizeof(int64_t) * nrings, cudaMemcpyDeviceToHost, s));
+    TRY_CUDA(cudaMemcpyAsync(P->orb_off_h.data(), orb_off, sizeof(int64_t) * nrings, cudaMemcpyDeviceToHost, s));
     P->lin_off_h[nrings] = nlin;
     P->orb_off_h[nrings] = norb;
-    TRY_CUDA(cudaMemcpy(P->lin_h.data(), lin, nrings, cudaMemcpyDeviceToHost));
+    TRY_CUDA(cudaMemcpyAsync(P->lin_h.data(), lin, nrings, cudaMemcpyDeviceToHost, s));
     float2* pair_A;
     int2 *pair_T, *tiles, *lin_list, *orb_list;
-    TRY_CUDA(P->alloc(&pair_A, npairs));
-    TRY_CUDA(P->alloc(&pair_T, (size_t)npairs * (K + 1)));
-    TRY_CUDA(P->alloc(&tiles, ntiles));
-    TRY_CUDA(P->alloc(&lin_list, nlin));
-    TRY_CUDA(P->alloc(&orb_list, norb));
+    pairs.add(&pair_A, npairs);
+    pairs.add(&pair_T, (size_t)npairs * (K + 1));
+    pairs.add(&tiles, ntiles);
+    pairs.add(&lin_list, nlin);
+    pairs.add(&orb_list, norb);
+    TRY_CUDA(pairs.take(P));
     pair_table_kernel<<<n_blocks(npairs, 128), 128, 0, s>>>(nrings, K, pair_off, npairs, ring_range, th, sd,
                                                             npr, E, pair_A, pair_T);
     tile_list_kernel<<<nrings, 128, 0, s>>>(nrings, tile_off, ntiles_r, TILE, tiles);
@@ -306,10 +309,11 @@ static tpcf_status build_map(tpcf_plan_s* P, int64_t nside, cudaStream_t s) {
     P->nent = n_entries(K, P->M);
     TRY_CUDA(P->alloc(&P->wdw, g.npix + 1));  // and a zero after the last pixel
     TRY_CUDA(P->alloc(&P->slots, (size_t)P->fwd_grid * P->nent));
-    TRY_CUDA(P->alloc(&P->sums, P->nent));
-    TRY_CUDA(P->alloc(&P->counter, 4 + P->ws_slots));  // work counter (4 words), then finished parts per block
-    TRY_CUDA(P->alloc(&P->status, 4));
-    TRY_CUDA(P->alloc(&P->H, (size_t)(P->M + 1) * K * K * 2 + K));  // H, then cdiag (self-pair mode)
+    scratch.add(&P->sums, P->nent);
+    scratch.add(&P->counter, 4 + P->ws_slots);  // work counter (4 words), then finished parts per block
+    scratch.add(&P->status, 4);
+    scratch.add(&P->H, (size_t)(P->M + 1) * K * K * 2 + K);  // H, then cdiag (self-pair mode)
+    TRY_CUDA(scratch.take(P));
     TRY_CUDA(cudaMemsetAsync(P->status, 0, sizeof(int) * 4, s));
     TRY_CUDA(cudaStreamSynchronize(s));
     return TPCF_OK;

@@ -95,6 +95,24 @@ struct tpcf_plan_s {
         *p = (T*)q;
         return cudaSuccess;
     }
+    // Several arrays from one allocation (each cudaMalloc and cudaFree costs tens of us): add()
+    // each, then take().
+    struct Arrays {
+        std::vector<std::pair<void**, size_t>> parts;  // pointer to set, offset
+        size_t bytes = 0;
+        template <typename T>
+        void add(T** p, size_t count) {
+            parts.push_back({(void**)p, bytes});
+            bytes += (count * sizeof(T) + 255) / 256 * 256;
+        }
+        cudaError_t take(tpcf_plan_s* P) {
+            char* q = nullptr;
+            cudaError_t e = P->alloc(&q, bytes);
+            if (e == cudaSuccess)
+                for (auto& t : parts) *t.first = q + t.second;
+            return e;
+        }
+    };
     ~tpcf_plan_s() {
         for (void* p : allocs) tpcf::dev_free(p);
     }
