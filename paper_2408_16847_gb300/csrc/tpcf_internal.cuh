@@ -144,7 +144,10 @@ constexpr int LIN_MIN = 256;  // smallest ring that is worth a linear block
 constexpr int LIN_CELLS = 1024;       // (bin, ring) cells listed at a time (6 bytes each)
 constexpr int LIN_CHUNK = BT;         // entries staged at a time, one per thread
 constexpr int LIN_HEAD = 512;         // small tables
-constexpr int CON_STAGE = 35 * 1024;  // bytes of moments staged by the contraction
+// Bytes of moments staged by the contraction: three fields at the most bins, one multipole and W, need
+// 3 x 3 x 32 x 32 words.
+constexpr int CON_STAGE = 36 * 1024;
+static_assert(CON_STAGE >= 3 * 3 * TPCF_MAX_BINS * TILE * 4, "three fields' stage");
 // Bytes of a staged entry of the linear walk: two pixel offsets and a weight, then 8 bytes per
 // multipole; an odd number of 16-byte words against bank conflicts of the staging stores.
 __host__ __device__ constexpr int lin_stride(int M) { return 16 * (((M + 1) / 2 + 1) | 1); }
