@@ -397,7 +397,9 @@ __device__ __forceinline__ void cat_batches(const CatDev& g, const float2* __res
             }
             const bool more = __syncthreads_or(x < total) != 0;
             if (!more && !last) break;  // the next group of bands fills up
-            if (lane < ((32 - c) & 31)) {
+            // (a warp without a candidate fills its first word: lanes of pass 2 that have none read slot 0,
+            // which must hold numbers)
+            if (lane < (c ? (32 - c) & 31 : 32)) {
                 S.hi[w0 + c + lane] = make_float4(-CAT_FAR, 0.0f, 0.0f, 0.0f);
                 S.lo[w0 + c + lane] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
             }
