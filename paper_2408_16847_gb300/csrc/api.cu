@@ -301,7 +301,7 @@ static tpcf_status build_map(tpcf_plan_s* P, int64_t nside, cudaStream_t s) {
     P->tune_fwd.variant = P->tune_bwd.variant = 2;
     P->tune_fwd.ctas = (occ_f + 1) / 2;
     P->tune_bwd.ctas = (occ_b + 1) / 2;
-    // workspace: a block per CTA, or (calls with few blocks) one per block, see block_call
+    // workspace: a block per CTA, or (calls with few blocks) one per block, see block_shape
     P->ws_slots = (int)std::max<int64_t>(1, std::min<int64_t>(2 * std::max(P->fwd_grid, P->bwd_grid), nlin + (norb + 1) / 2));
     P->fwd_grid = (int)std::min<int64_t>(P->fwd_grid, 8 * (int64_t)P->ws_slots);
     P->ws_floats = block_floats(K, P->M, P->M, self != 0);
@@ -437,7 +437,7 @@ static void tile_range(const tpcf_plan_s* P, int64_t lo, int64_t hi, int64_t* tl
 // per warp), or two if that leaves fewer than four blocks per CTA of a full grid; a call with
 // fewer than three blocks per CTA splits each by bins, if the workspace has a slot for each block.
 static int block_shape(const tpcf_plan_s* P, const tpcf_plan_s::Tune& t, int cap, MapCall* c) {
-    const int64_t full = (int64_t)P->num_sms * 2 * t.ctas;
+    const int64_t full = (int64_t)P->num_sms * std::min(2 * t.ctas, 4);  // (four CTAs of BT threads fit an SM)
     auto blocks = [&](int tiles) { return c->nlin + (c->norb + tiles - 1) / tiles; };
     c->tiles = BW;
     while (c->tiles > 2 && blocks(c->tiles) < 4 * full) c->tiles /= 2;

@@ -1,10 +1,11 @@
 // Launch-configuration autotuner of the map pair kernels.
 //
 // The search space, per pass (forward, adjoint):
-//   * register variant: the kernel compiled for 3 resident CTAs per SM (80 registers
-//     per thread, a few spills at large m_max) or for 2 (128 registers, none);
-//   * CTAs per SM actually launched: the variant's occupancy or one fewer;
-//   * rings summed in registers before a shared-memory flush: 4, 8 or 16.
+//   * pairs of CTAs per SM launched: what the kernel's occupancy gives, or one fewer;
+//   * entries summed in registers before they are added to the workspace, in units of 32:
+//     4, 8, 16 or 32.
+// A stored configuration also names a register variant and a tile layout; one kernel
+// serves every value of both (map_block.cuh).
 // Each candidate runs the pass on a sample of pivots (slices at three latitudes, about
 // 0.5% of a large map, the whole map when it is small), once to warm up and then twice
 // timed with CUDA events; the fastest is kept in the plan.  Results are cached in the
@@ -43,7 +44,7 @@ static std::string tune_key(const tpcf_plan_s* P) {
     std::string name(prop.name);
     for (char& c : name)
         if (c == ' ') c = '_';
-    snprintf(buf, sizeof(buf), "v2 dev=%s sms=%d map nside=%d K=%d M=%d flags=%u edges=%016llx", name.c_str(),
+    snprintf(buf, sizeof(buf), "v3 dev=%s sms=%d map nside=%d K=%d M=%d flags=%u edges=%016llx", name.c_str(),
              P->num_sms, P->map.nside, P->K, P->M, P->flags, h);
     return buf;
 }
@@ -84,8 +85,10 @@ static void cache_store(const std::string& key, const tpcf_plan_s::Tune& f, cons
 static bool valid(const tpcf_plan_s* P, const tpcf_plan_s::Tune& t, bool bwd) {
     if (t.variant != 2 && t.variant != 3) return false;
     if (t.flush < 1 || t.flush > 64 || t.ctas < 1 || t.quad < 0 || t.quad > 1) return false;
+    // callers may name as many CTAs per SM as their variant stands for; the launch is cut to what
+    // fits (block_shape)
     const int occ = bwd ? map_bwd_occupancy(P->M) : map_fwd_occupancy(P->M);
-    return t.ctas <= (occ + 1) / 2;
+    return t.ctas <= std::max(t.variant, (occ + 1) / 2);
 }
 
 // Applies a cached configuration to a new map plan (called at plan creation).
