@@ -341,7 +341,7 @@ tpcf_status build_catalog(tpcf_plan_s* P, const double* d_xyz, int64_t n, cudaSt
     TRY_CUDA(cudaGetLastError());
     P->bwd_grid = occ_b < 1 ? 0 : (int)std::max<int64_t>(1, std::min<int64_t>(g.ntiles, (int64_t)P->num_sms * occ_b));
     TRY_CUDA(P->alloc(&P->H, (size_t)(P->M + 1) * K * K * 2 + K));
-    P->ws_floats = sub_floats_rt(K, P->M, self != 0);
+    P->ws_floats = cat_slices(K) * sub_floats_rt(K, P->M, self != 0);
     P->ws_slots = std::max(P->fwd_grid, P->bwd_grid);
     TRY_CUDA(P->alloc(&P->ws, P->ws_floats * P->ws_slots));
     P->nent = n_entries(K, P->M);
@@ -427,7 +427,7 @@ tpcf_status catalog_forward_multi(tpcf_plan_s* P, const float* const* d_delta, c
         TRY_CUDA(P->alloc(&sl, (size_t)grid * nent));
         TRY_CUDA(P->alloc(&su, (size_t)nent));
         float* w3;
-        TRY_CUDA(P->alloc(&w3, 3 * sub_floats_rt(K, M, false) * grid));
+        TRY_CUDA(P->alloc(&w3, 3 * P->ws_floats * grid));
         P->ws3 = w3;
         P->wdw_c = c;
         P->mslots = sl;
@@ -448,7 +448,7 @@ tpcf_status catalog_forward_multi(tpcf_plan_s* P, const float* const* d_delta, c
     c.counter = P->counter;
     c.status = P->status;
     c.ws = P->ws3;
-    c.ws_floats = 3 * sub_floats_rt(K, M, false);
+    c.ws_floats = 3 * P->ws_floats;
     TRY_CUDA(kCat[M].multi(g, c, P->wdw_b, P->wdw_c, P->multi_grid, s));
     reduce_slots_kernel<<<(nent + 31) / 32, REDUCE_THREADS, 0, s>>>(P->mslots, P->multi_grid, nent, P->msums);
     const int nout = (M + 1) * K * K;

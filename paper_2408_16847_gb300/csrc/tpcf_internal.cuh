@@ -94,6 +94,7 @@ struct MapCall {
     const int2 *lin_list, *orb_list;
     long long lin_lo, nlin, orb_lo, norb;
     int tiles, parts;
+    int slices;             // 1, or (tiles = 1) slices of the rings of a bin that go to warps of their own
     int* done;              // parts > 1: [blocks] finished parts (zeroed before launch)
     int step;               // adjoint: phases of this launch (bwd_block)
     float* ws;              // workspace: per block (parts > 1) or per CTA
@@ -140,6 +141,16 @@ __host__ __device__ inline size_t sub_floats_rt(int K, int mr, bool self) {
     return (size_t)K * (mr + 1) * 2 * TILE + (self ? 3 : 1) * (size_t)K * TILE;
 }
 inline size_t block_floats(int K, int mr, int M, bool self) { return (size_t)BW * walk_np(M) * sub_floats_rt(K, mr, self); }
+// Slices of a batch's words that go to warps of their own in pass 2 where there are few bins for the four
+// warps; each has a subtile of its own, which cat_tile_moments adds up.  (A bin per warp leaves three of four warps idle at
+// one bin.  3,000 points: 131 us at 1 bin, 156 us at 12, against 236 and 334 with 8 warps and atomics.)
+__host__ __device__ inline int cat_slices(int K) { return K >= 8 ? 1 : (K >= 4 ? 2 : 4); }
+// Calls whose (warp tile, bin) items would leave most warps of the GPU without two: tiles then go one
+// to a block and a bin's rings to four warps.  (Nside 24, 8 bins: 137 us.  One bin at Nside 24 is
+// still a long chain per warp: 147 us, against 94 with the earlier eight warps per tile.)
+__host__ __device__ inline bool few_tiles(long long norb, int K, int num_sms) {
+    return norb * K < (long long)2 * 4 * BW * num_sms;
+}
 constexpr int LIN_MIN = 256;  // smallest ring that is worth a linear block
 constexpr int LIN_CELLS = 1024;       // (bin, ring) cells listed at a time (6 bytes each)
 constexpr int LIN_CHUNK = BT;         // entries staged at a time, one per thread
