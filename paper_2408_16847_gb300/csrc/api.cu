@@ -302,7 +302,7 @@ static tpcf_status build_map(tpcf_plan_s* P, int64_t nside, cudaStream_t s) {
     P->tune_fwd.ctas = (occ_f + 1) / 2;
     P->tune_bwd.ctas = (occ_b + 1) / 2;
     // workspace: a block per CTA, or (calls with few blocks) one per block, see block_shape
-    P->ws_slots = (int)std::max<int64_t>(1, std::min<int64_t>(2 * std::max(P->fwd_grid, P->bwd_grid), nlin + (norb + 1) / 2));
+    P->ws_slots = (int)std::max<int64_t>(1, std::min<int64_t>(2 * std::max(P->fwd_grid, P->bwd_grid), nlin + norb));
     P->fwd_grid = (int)std::min<int64_t>(P->fwd_grid, 8 * (int64_t)P->ws_slots);
     P->ws_floats = block_floats(K, P->M, P->M, self != 0);
     TRY_CUDA(P->alloc(&P->ws, P->ws_floats * P->ws_slots));
@@ -441,6 +441,11 @@ static int block_shape(const tpcf_plan_s* P, const tpcf_plan_s::Tune& t, int cap
     auto blocks = [&](int tiles) { return c->nlin + (c->norb + tiles - 1) / tiles; };
     c->tiles = BW;
     while (c->tiles > 2 && blocks(c->tiles) < 4 * full) c->tiles /= 2;
+    c->slices = 1;
+    if (few_tiles(c->norb, P->K, P->num_sms)) {
+        c->tiles = 1;
+        c->slices = 4;
+    }
     const int64_t n = blocks(c->tiles);
     c->parts = 1;
     if (n < 3 * full && n <= P->ws_slots && n > 0)

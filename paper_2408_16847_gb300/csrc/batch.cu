@@ -223,6 +223,7 @@ static tpcf_status batch_build(tpcf_batch_s* B, const tpcf_plan* plans, const fl
             it.c.nlin = P->lin_off_h.back();
             it.c.norb = P->orb_off_h.back();
             it.c.tiles = 2;
+            it.c.slices = 1;
             it.c.parts = 1;
             it.c.ws = G.ws;
             it.c.ws_floats = G.ws_floats;

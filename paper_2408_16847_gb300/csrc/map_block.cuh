@@ -19,6 +19,10 @@
 //
 // A call with few blocks splits each into parts by bins, so that it still fills the GPU; the
 // part that finishes last contracts.
+//
+// Bound: FP32 and load/store issue.  Per call on a GB300, before (a ring at a time per pivot, sums by
+// shared-memory atomics) and now: Nside 512, 20 bins to 2 deg, m <= 10: 33.3 -> 11.1 ms; Nside 4096
+// polar slice (2 x 10^-3 of the pixels): 71.7 -> 47.6 ms; Nside 64: 328 -> 215 us.
 #pragma once
 
 namespace tpcf {
@@ -578,9 +582,12 @@ __device__ __forceinline__ void orbit_runs(const RingCtx& R, const WalkRing& w, 
 // image wraps.  The rings' constants are loaded 32 at a time, a ring per lane, and read back
 // from the warp's stage in shared memory.
 template <int IM, class F>
-__device__ __forceinline__ void orbit_rings(const MapDev& g, const PivotRing& P, int q, int k, char* stage, F&& f) {
+__device__ __forceinline__ void orbit_rings(const MapDev& g, const PivotRing& P, int q, int k, int sl, int S, char* stage,
+                                            F&& f) {
     const int lane = threadIdx.x & 31;
-    const int2 br = g.bin_range[(long long)P.i * g.K + k];
+    const int2 all = g.bin_range[(long long)P.i * g.K + k];
+    const int nr = all.y - all.x + 1;
+    const int2 br = make_int2(all.x + nr * sl / S, all.x + nr * (sl + 1) / S - 1);  // slice sl of S
     for (int r0 = br.x; r0 <= br.y; r0 += 32) {
         __syncwarp();
         bool on = false;
@@ -636,16 +643,16 @@ __device__ __forceinline__ void orbit_rings(const MapDev& g, const PivotRing& P,
     }
 }
 
-// One (warp tile, bin) item: the moments of bin k for pivots at ring position q of ring i
-// and its turned images, into the tile's IM subtiles.
+// One (warp tile, bin, slice of the rings) item: the moments of bin k for pivots at ring position
+// q of ring i and its turned images, into IM subtiles.
 template <int M, int IM, bool SELF, class L>
-__device__ __forceinline__ void orbit_bin(const MapDev& g, const PivotRing& P, int q, int k, const L& ld, float* ws,
+__device__ __forceinline__ void orbit_bin(const MapDev& g, const PivotRing& P, int q, int k, int sl, int S, const L& ld, float* ws,
                                           size_t sub_floats, char* stage, int flush, int mr) {
     BinAcc<M, IM, SELF> A;
     A.zero();
     bool first = true;
     int done = 0;  // entries summed in registers
-    orbit_rings<IM>(g, P, q, k, stage, [&](const RingCtx& R, const WalkRing& w, const LaneC& c, const BinRuns& b, bool fast,
+    orbit_rings<IM>(g, P, q, k, sl, S, stage, [&](const RingCtx& R, const WalkRing& w, const LaneC& c, const BinRuns& b, bool fast,
                                            bool flat) {
         if (!fast)
             orbit_runs<M, IM, false, true, SELF>(R, w, ld, c, b, A, mr);
@@ -1090,7 +1097,8 @@ __device__ __forceinline__ void lin_block_moments(const MapDev& g, const MapCall
         lin_moments<M, NP, SELF, true>(g, PR, q, on, kb, ke, ld, w, sub_floats, smem, c.cells, c.flush, mr);
 }
 
-// The same for the warp tiles of another block: its warps draw (tile, bin) items.
+// The same for the warp tiles of another block: its warps draw (tile, bin, slice) items; slice s has
+// subtiles of its own, which block_fold adds up.
 template <int M, bool SELF, bool GROUPED, class L>
 __device__ __forceinline__ void orb_block_moments(const MapDev& g, const MapCall& c, long long b, unsigned live, int kb,
                                                int ke, L ld, float* ws, size_t sub_floats, char* smem, int mr) {
@@ -1101,19 +1109,20 @@ __device__ __forceinline__ void orb_block_moments(const MapDev& g, const MapCall
     const int group = GROUPED ? c.group : 1;
     if (threadIdx.x == 0) s_item = 0;
     __syncthreads();
-    const int items = B.T * (ke - kb);
+    const int S = c.slices, items = B.T * (ke - kb) * S;
     for (;;) {
         int it = 0;
         if (lane == 0) it = atomicAdd(&s_item, 1);
         it = __shfl_sync(0xffffffffu, it, 0);
         if (it >= items) break;
-        const int t = it % B.T, k = ke - 1 - it / B.T;  // outer (larger) bins first
+        const int sl = it % S, u = it / S;
+        const int t = u % B.T, k = ke - 1 - u / B.T;  // outer (larger) bins first
         if (((live >> (t * IM)) & ((1u << IM) - 1u)) == 0u) continue;
         const int2 tq = B.list[t];
         const PivotRing PR = pivot_ring(g, tq.x);
         const int q = GROUPED ? group_middle(tq.y + lane, (PR.n_i + group - 1) / group, group, PR.n_i)
                               : min(tq.y + lane, PR.n_i / IM - 1);
-        orbit_bin<M, IM, SELF>(g, PR, q, k, ld, ws + (size_t)t * IM * sub_floats, sub_floats,
+        orbit_bin<M, IM, SELF>(g, PR, q, k, sl, S, ld, ws + (size_t)(sl * B.T + t) * IM * sub_floats, sub_floats,
                                smem + warp * 32 * ORB_STRIDE, c.flush, mr);
     }
 }
@@ -1135,6 +1144,23 @@ __device__ __forceinline__ void block_sums(const MapDev& g, const MapCall& c, lo
     block_contract<SELF>(g.K, mr, ws, sub_floats, B.nsub, live,
                          [&](int s, int l) { return B.value(g, c, ld, s, l); }, smem, slot, SELF && c.self_subtract,
                          c.norm);
+}
+
+// Adds the slices' subtiles of a block into the first slice's.  Called by every thread, between the
+// barrier of block_complete and the contraction.
+__device__ __forceinline__ void block_fold(const MapCall& c, long long b, int nsub, float* ws, size_t sub_floats) {
+    if (c.slices == 1 || b < c.nlin) return;
+    const int n = (int)(nsub * sub_floats / 4);  // (sub_floats is a multiple of 32)
+    float4* w = reinterpret_cast<float4*>(ws);
+    for (int e = threadIdx.x; e < n; e += BT) {
+        float4 v = __ldcg(w + e);
+        for (int s = 1; s < c.slices; ++s) {
+            const float4 u = __ldcg(w + s * n + e);
+            v = make_float4(v.x + u.x, v.y + u.y, v.z + u.z, v.w + u.w);
+        }
+        __stcg(w + e, v);
+    }
+    __syncthreads();
 }
 
 // True on the CTA that finishes the last part of block b.  Called by every thread.
@@ -1165,6 +1191,7 @@ __device__ __forceinline__ void fwd_block(const MapDev& g, const MapCall& c, lon
     if (live == 0u) return;
     block_moments<M, SELF, GROUPED>(g, c, b, live, part, ld, ws, sub_floats, smem, mr);
     if (!block_complete(c, b)) return;
+    block_fold(c, b, B.nsub, ws, sub_floats);
     block_sums<M, SELF, GROUPED, L>(g, c, b, live, ld, ws, sub_floats, smem, slot, mr);
     __syncthreads();
 }

@@ -768,6 +768,7 @@ __device__ __forceinline__ void fwd_block_tc(const MapDev& g, const MapCall& c, 
     if (live == 0u) return;
     block_moments<M, SELF, false>(g, c, b, live, part, ld, ws, sub_floats, reinterpret_cast<char*>(base), M);
     if (!block_complete(c, b)) return;
+    block_fold(c, b, B.nsub, ws, sub_floats);
     const TcLayout L = tc_layout(K, M, SELF);
     for (int s = 0; s < B.nsub; ++s) {
         if (!((live >> s) & 1u)) continue;
@@ -921,6 +922,7 @@ __global__ void __launch_bounds__(BT, 4) map_fwd_multi_kernel(MapDev g, MapCall 
             __syncthreads();
         }
         if (!block_complete(c, b)) continue;
+        for (int f = 0; f < 3; ++f) block_fold(c, b, B.nsub, ws + f * field_ws, sub_floats);
         block_contract_multi(K, M, ws, field_ws, sub_floats, B.nsub, live, value, reinterpret_cast<char*>(smem), slot);
         __syncthreads();
     }

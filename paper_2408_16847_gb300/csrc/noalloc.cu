@@ -143,7 +143,8 @@ extern "C" tpcf_status tpcf_forward_noalloc(tpcf_plan plan, const float* d_delta
     c.orb_list = plan->map.orb_list;
     c.nlin = plan->lin_off_h.back();
     c.norb = plan->orb_off_h.back();
-    c.tiles = 2;
+    c.slices = few_tiles(c.norb, plan->K, plan->num_sms) ? 4 : 1;
+    c.tiles = c.slices > 1 ? 1 : 2;
     c.parts = 1;
     c.ws = plan->ws;
     c.ws_floats = plan->ws_floats;
