@@ -22,7 +22,7 @@
 //
 // Bound: FP32 and load/store issue.  Per call on a GB300, before (a ring at a time per pivot, sums by
 // shared-memory atomics) and now: Nside 512, 20 bins to 2 deg, m <= 10: 33.3 -> 11.1 ms; Nside 4096
-// polar slice (2 x 10^-3 of the pixels): 71.7 -> 47.6 ms; Nside 64: 328 -> 215 us.
+// polar slice (2 x 10^-3 of the pixels): 71.7 -> 47.6 ms; Nside 64: 328 -> 210 us.
 #pragma once
 
 namespace tpcf {
