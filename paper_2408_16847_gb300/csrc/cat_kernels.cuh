@@ -100,8 +100,7 @@ __device__ __forceinline__ CatPivot cat_pivot(const CatDev& g, int64_t si) {
 
 // Warp 0: a cap holding every live pivot of the tile together with its neighbours
 // (radius theta_max), as a range of cell bands and a longitude half-width about the
-// cap's centre: s_cap = (phi_c, dphi, first band, last band, full, centre x, y, z, largest
-// chord from the centre to a live pivot).  All in fp32:
+// cap's centre: s_cap = (phi_c, dphi, first band, last band, full, centre x, y, z).  All in fp32:
 // CAT_MARGIN (rad) exceeds every rounding of the centre, radius, colatitude and band
 // division (each below ~1e-6 rad), and the sine ratio is rounded up, so the cells are
 // a superset of the exact cap; bins are then decided per candidate.  The caller
@@ -123,18 +122,14 @@ __device__ __forceinline__ void cat_tile_cap(const CatDev& g, bool live, const C
         nrm = 1.0f;
     }
     const float cx = sx / nrm, cy = sy / nrm, cz = sz / nrm;
-    float r = 0.0f, rho = 0.0f;
+    float r = 0.0f;
     if (live) {
         const float dx = px - cx, dy = py - cy, dz = pz - cz;
         const float ch = sqrtf(fmaf(dx, dx, fmaf(dy, dy, dz * dz)));
         r = 2.0f * asinf(fminf(1.0f, 0.5f * ch));
-        rho = ch;
     }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        r = fmaxf(r, __shfl_xor_sync(0xffffffffu, r, o));
-        rho = fmaxf(rho, __shfl_xor_sync(0xffffffffu, rho, o));
-    }
+    for (int o = 16; o > 0; o >>= 1) r = fmaxf(r, __shfl_xor_sync(0xffffffffu, r, o));
     if ((threadIdx.x & 31) == 0) {
         const float PI_F = 3.14159265f;
         const float Q = r + (float)g.theta_max + CAT_MARGIN;
@@ -166,7 +161,6 @@ __device__ __forceinline__ void cat_tile_cap(const CatDev& g, bool live, const C
         s_cap[5] = cx;
         s_cap[6] = cy;
         s_cap[7] = cz;
-        s_cap[8] = rho;
     }
 }
 
@@ -183,7 +177,7 @@ __device__ __forceinline__ void cat_rel(float h, float l, float c, float& H, flo
 struct CatShared {
     unsigned char* lut;  // [CAT_LUT] next edge above a cell of chord^2 (see cat_edges_kernel)
     float2* edge;        // [K + 3] chord^2 of the edge, margin below which cat_near_edge decides
-    float* cap;          // [9] (cat_tile_cap)
+    float* cap;          // [9]: cat_tile_cap, then the largest chord from the cap's centre to a live pivot
     int* item;           // next bin of the batch
     int* cnt;            // [BW] candidates staged by a warp
     int* wsum;           // [BW]
@@ -271,10 +265,19 @@ __device__ __forceinline__ CatPivot cat_place(const CatDev& g, const CatShared& 
     const int lane = threadIdx.x & 31;
     const int64_t si = tile * TILE + lane;
     CatPivot P = cat_pivot(g, si < g.n ? si : -1);
+    if ((threadIdx.x >> 5) == 0) cat_tile_cap(g, live, P, S.cap);
+    __syncthreads();
+    cat_rel(P.hx, P.lx, S.cap[5], P.hx, P.lx);
+    cat_rel(P.hy, P.ly, S.cap[6], P.hy, P.ly);
+    cat_rel(P.hz, P.lz, S.cap[7], P.hz, P.lz);
     if ((threadIdx.x >> 5) == 0) {
-        cat_tile_cap(g, live, P, S.cap);
-        __syncwarp();
-        const float rho = S.cap[8];
+        // from the offsets, which are good to 2^-24 of themselves: the unit vectors' fp32 parts
+        // are off by 6e-8, which is more than the relative margins of cat_batches where theta_max is small
+        float d2 = live ? fmaf(P.hx, P.hx, fmaf(P.hy, P.hy, P.hz * P.hz)) : 0.0f;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) d2 = fmaxf(d2, __shfl_xor_sync(0xffffffffu, d2, o));
+        const float rho = sqrtf(d2) * (1.0f + 1.0e-6f);
+        if (lane == 0) S.cap[8] = rho;
         const float cell = exp2f((float)(g.lut_shift - 24)) * 0.99f;
         bool wide = false;
         for (int e = lane; e < g.K + 3; e += 32) {
@@ -288,9 +291,6 @@ __device__ __forceinline__ CatPivot cat_place(const CatDev& g, const CatShared& 
             for (int e = lane; e < g.K + 2; e += 32) S.edge[e].y = INFINITY;
     }
     __syncthreads();
-    cat_rel(P.hx, P.lx, S.cap[5], P.hx, P.lx);
-    cat_rel(P.hy, P.ly, S.cap[6], P.hy, P.ly);
-    cat_rel(P.hz, P.lz, S.cap[7], P.hz, P.lz);
     if (!live) {
         P.hx = CAT_FAR;
         P.si = -1;
