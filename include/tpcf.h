@@ -369,10 +369,13 @@ tpcf_status tpcf_probe_fp32_peak(double* tflops, void* stream);
  * now on fails as if the device were out of memory (the calls above then return
  * TPCF_ERR_OOM); n <= 0 disarms.  tpcf_test_live_allocations(): the number of device
  * allocations the library holds (plans, batches, staging), so that a test can check
- * that a failed call leaked nothing.
+ * that a failed call leaked nothing.  tpcf_test_route(plan, r): the map plan's calls take the
+ * kernels that the library picks by size (r = 0), those for small calls (1), those for large
+ * ones (2); results agree to rounding.
  */
 void tpcf_test_fail_allocation(int64_t n);
 int64_t tpcf_test_live_allocations(void);
+tpcf_status tpcf_test_route(tpcf_plan plan, int32_t route);
 
 #ifdef __cplusplus
 }

@@ -25,7 +25,7 @@ MAX_M = 16
 EXPORTS = ["tpcf_status_string", "tpcf_last_error", "tpcf_plan_create_map", "tpcf_plan_create_catalog",
            "tpcf_plan_npoints", "tpcf_plan_kernel_launches", "tpcf_forward", "tpcf_forward_noalloc", "tpcf_backward", "tpcf_count_pairs", "tpcf_run_host", "tpcf_batch_create",
            "tpcf_batch_launch", "tpcf_batch_kernel_launches", "tpcf_batch_destroy", "tpcf_forward_batched", "tpcf_plan_sync", "tpcf_normalize",
-           "tpcf_plan_destroy", "tpcf_test_fail_allocation", "tpcf_test_live_allocations",
+           "tpcf_plan_destroy", "tpcf_test_fail_allocation", "tpcf_test_live_allocations", "tpcf_test_route",
            "tpcf_plan_halo", "tpcf_plan_autotune", "tpcf_plan_launch_config", "tpcf_plan_set_launch_config",
            "tpcf_probe_fp32_peak", "tpcf_forward_multi", "tpcf_edge_correct", "tpcf_forward_grouped"]
 
@@ -115,6 +115,8 @@ def lib() -> ctypes.CDLL:
     L.tpcf_test_fail_allocation.argtypes = [_i64]
     L.tpcf_test_live_allocations.restype = _i64
     L.tpcf_test_live_allocations.argtypes = []
+    L.tpcf_test_route.restype = ctypes.c_int
+    L.tpcf_test_route.argtypes = [_vp, ctypes.c_int32]
     _lib = L
     return L
 

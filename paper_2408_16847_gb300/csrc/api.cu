@@ -20,33 +20,38 @@ namespace tpcf {
 #define TPCF_DECL_MULTI(m)                                                                                    \
     cudaError_t map_fwd_multi_launch_m##m(const MapDev&, const MapCall&, const float2*, const float2*, int, \
                                           cudaStream_t);                                                  \
-    int map_fwd_multi_occupancy_m##m();
+    int map_fwd_multi_occupancy_m##m();                                                                   \
+    cudaError_t map_tile_multi_launch_m##m(const MapDev&, const MapCall&, const float2*, const float2*, int, \
+                                           cudaStream_t);                                                 \
+    int map_tile_multi_occupancy_m##m(int);
 TPCF_DECL_MULTI(0) TPCF_DECL_MULTI(1) TPCF_DECL_MULTI(2) TPCF_DECL_MULTI(3) TPCF_DECL_MULTI(4) TPCF_DECL_MULTI(5)
 TPCF_DECL_MULTI(6) TPCF_DECL_MULTI(7) TPCF_DECL_MULTI(8) TPCF_DECL_MULTI(9) TPCF_DECL_MULTI(10)
 TPCF_DECL_MULTI(11) TPCF_DECL_MULTI(12) TPCF_DECL_MULTI(13) TPCF_DECL_MULTI(14) TPCF_DECL_MULTI(15)
 TPCF_DECL_MULTI(16)
 #undef TPCF_DECL_MULTI
-typedef cudaError_t (*multi_fn)(const MapDev&, const MapCall&, const float2*, const float2*, int, cudaStream_t);
-static const multi_fn kMulti[TPCF_MAX_M + 1] = {
-    map_fwd_multi_launch_m0,  map_fwd_multi_launch_m1,  map_fwd_multi_launch_m2,  map_fwd_multi_launch_m3,
-    map_fwd_multi_launch_m4,  map_fwd_multi_launch_m5,  map_fwd_multi_launch_m6,  map_fwd_multi_launch_m7,
-    map_fwd_multi_launch_m8,  map_fwd_multi_launch_m9,  map_fwd_multi_launch_m10, map_fwd_multi_launch_m11,
-    map_fwd_multi_launch_m12, map_fwd_multi_launch_m13, map_fwd_multi_launch_m14, map_fwd_multi_launch_m15,
-    map_fwd_multi_launch_m16};
-static int (*const kMultiOcc[TPCF_MAX_M + 1])() = {
-    map_fwd_multi_occupancy_m0,  map_fwd_multi_occupancy_m1,  map_fwd_multi_occupancy_m2,
-    map_fwd_multi_occupancy_m3,  map_fwd_multi_occupancy_m4,  map_fwd_multi_occupancy_m5,
-    map_fwd_multi_occupancy_m6,  map_fwd_multi_occupancy_m7,  map_fwd_multi_occupancy_m8,
-    map_fwd_multi_occupancy_m9,  map_fwd_multi_occupancy_m10, map_fwd_multi_occupancy_m11,
-    map_fwd_multi_occupancy_m12, map_fwd_multi_occupancy_m13, map_fwd_multi_occupancy_m14,
-    map_fwd_multi_occupancy_m15, map_fwd_multi_occupancy_m16};
+struct MultiLaunch {
+    cudaError_t (*blocks)(const MapDev&, const MapCall&, const float2*, const float2*, int, cudaStream_t);
+    int (*blocks_occ)();
+    cudaError_t (*tiles)(const MapDev&, const MapCall&, const float2*, const float2*, int, cudaStream_t);
+    int (*tiles_occ)(int);
+};
+#define TPCF_ROW_MULTI(m) \
+    {map_fwd_multi_launch_m##m, map_fwd_multi_occupancy_m##m, map_tile_multi_launch_m##m, map_tile_multi_occupancy_m##m}
+static const MultiLaunch kMulti[TPCF_MAX_M + 1] = {
+    TPCF_ROW_MULTI(0),  TPCF_ROW_MULTI(1),  TPCF_ROW_MULTI(2),  TPCF_ROW_MULTI(3),  TPCF_ROW_MULTI(4),
+    TPCF_ROW_MULTI(5),  TPCF_ROW_MULTI(6),  TPCF_ROW_MULTI(7),  TPCF_ROW_MULTI(8),  TPCF_ROW_MULTI(9),
+    TPCF_ROW_MULTI(10), TPCF_ROW_MULTI(11), TPCF_ROW_MULTI(12), TPCF_ROW_MULTI(13), TPCF_ROW_MULTI(14),
+    TPCF_ROW_MULTI(15), TPCF_ROW_MULTI(16)};
+#undef TPCF_ROW_MULTI
 #define TPCF_DECL_M(m)                                                                         \
     cudaError_t map_fwd_launch_m##m(const MapDev&, const MapCall&, int, cudaStream_t);         \
     cudaError_t map_fwd_tc_launch_m##m(const MapDev&, const MapCall&, int, cudaStream_t);      \
     int map_fwd_tc_occupancy_m##m(int, int);                                                  \
     cudaError_t map_bwd_launch_m##m(const MapDev&, const MapCall&, int, cudaStream_t);         \
     int map_fwd_occupancy_m##m();                                                             \
-    int map_bwd_occupancy_m##m();
+    int map_bwd_occupancy_m##m();                                                             \
+    cudaError_t map_tile_launch_m##m(const MapDev&, const MapCall&, int, int, cudaStream_t);   \
+    int map_tile_occupancy_m##m(int, int, int);
 TPCF_DECL_M(0) TPCF_DECL_M(1) TPCF_DECL_M(2) TPCF_DECL_M(3) TPCF_DECL_M(4) TPCF_DECL_M(5)
 TPCF_DECL_M(6) TPCF_DECL_M(7) TPCF_DECL_M(8) TPCF_DECL_M(9) TPCF_DECL_M(10) TPCF_DECL_M(11)
 TPCF_DECL_M(12) TPCF_DECL_M(13) TPCF_DECL_M(14) TPCF_DECL_M(15) TPCF_DECL_M(16)
@@ -73,9 +78,12 @@ struct MLaunch {
     cudaError_t (*bwd)(const MapDev&, const MapCall&, int, cudaStream_t);
     int (*fwd_occ)();
     int (*bwd_occ)();
+    cudaError_t (*tile)(const MapDev&, const MapCall&, int, int, cudaStream_t);  // TileKernel, grid
+    int (*tile_occ)(int, int, int);                                            // TileKernel, K, self
 };
 #define TPCF_ROW_M(m) \
-    {map_fwd_launch_m##m, map_fwd_tc_launch_m##m, map_fwd_tc_occupancy_m##m, map_bwd_launch_m##m, map_fwd_occupancy_m##m, map_bwd_occupancy_m##m}
+    {map_fwd_launch_m##m,    map_fwd_tc_launch_m##m,  map_fwd_tc_occupancy_m##m, map_bwd_launch_m##m, \
+     map_fwd_occupancy_m##m, map_bwd_occupancy_m##m, map_tile_launch_m##m,      map_tile_occupancy_m##m}
 static const MLaunch kLaunch[TPCF_MAX_M + 1] = {
     TPCF_ROW_M(0),  TPCF_ROW_M(1),  TPCF_ROW_M(2),  TPCF_ROW_M(3),  TPCF_ROW_M(4),  TPCF_ROW_M(5),
     TPCF_ROW_M(6),  TPCF_ROW_M(7),  TPCF_ROW_M(8),  TPCF_ROW_M(9),  TPCF_ROW_M(10), TPCF_ROW_M(11),
@@ -122,6 +130,12 @@ void dev_free(void* p) {
 extern "C" void tpcf_test_fail_allocation(int64_t n) { g_fail_countdown.store(n > 0 ? n : 0); }
 
 extern "C" int64_t tpcf_test_live_allocations(void) { return g_live_allocs.load(); }
+
+extern "C" tpcf_status tpcf_test_route(tpcf_plan plan, int32_t route) {
+    if (!plan || route < 0 || route > 2) return TPCF_ERR_INVALID_ARG;
+    plan->route = route;
+    return TPCF_OK;
+}
 
 namespace tpcf {
 tpcf_status cuda_fail(cudaError_t e, const char* where) {
@@ -306,9 +320,17 @@ static tpcf_status build_map(tpcf_plan_s* P, int64_t nside, cudaStream_t s) {
     P->fwd_grid = (int)std::min<int64_t>(P->fwd_grid, 8 * (int64_t)P->ws_slots);
     P->ws_floats = block_floats(K, P->M, P->M, self != 0);
     TRY_CUDA(P->alloc(&P->ws, P->ws_floats * P->ws_slots));
+    for (int t = TILE_FWD; t <= TILE_BWD; ++t)
+        if (t != (tc ? TILE_FWD : TILE_TC)) P->tile_ctas[t] = L.tile_occ(t, K, self);
+    cudaGetLastError();  // (a kernel that does not fit leaves its calls to the blocks)
+    P->nslots = (int)std::max<int64_t>(
+        P->fwd_grid, std::min<int64_t>(ntiles, (int64_t)P->num_sms * P->tile_ctas[tc ? TILE_TC : TILE_FWD]));
+    P->bin_share = 0.0;
+    auto area = [&](int e) { return pow(sin(0.5 * P->edges[e]), 2); };
+    for (int k = 0; k < K; ++k) P->bin_share = std::max(P->bin_share, (area(k + 1) - area(k)) / (area(K) - area(0)));
     P->nent = n_entries(K, P->M);
     TRY_CUDA(P->alloc(&P->wdw, g.npix + 1));  // and a zero after the last pixel
-    TRY_CUDA(P->alloc(&P->slots, (size_t)P->fwd_grid * P->nent));
+    TRY_CUDA(P->alloc(&P->slots, (size_t)P->nslots * P->nent));
     scratch.add(&P->sums, P->nent);
     scratch.add(&P->counter, 4 + P->ws_slots);  // work counter (4 words), then finished parts per block
     scratch.add(&P->status, 4);
@@ -420,14 +442,20 @@ static int64_t ring_first_pixel(int64_t nside, int64_t ri) {  // 0-based ring
     return 12 * nside * nside - 2 * rr * (rr + 1);
 }
 
-// Tiles [*tlo, *thi) of 32 consecutive pivots that hold the pivots [lo, hi).
-static void tile_range(const tpcf_plan_s* P, int64_t lo, int64_t hi, int64_t* tlo, int64_t* thi) {
+// Tiles [*tlo, *thi) of 32 pivots that can hold one of [lo, hi): those of the range's pixels, in the
+// quarter-turn layout those of its rings (a ring's pivots are spread over all of its tiles).
+static void tile_range(const tpcf_plan_s* P, int64_t lo, int64_t hi, int64_t* tlo, int64_t* thi, bool quad = false) {
     if (hi <= lo) {
         *tlo = *thi = 0;
         return;
     }
     const int64_t nside = P->map.nside;
     const int64_t ra = ring_of_pixel(nside, lo), rb = ring_of_pixel(nside, hi - 1);
+    if (quad) {
+        *tlo = P->tile_off_h[ra];
+        *thi = rb + 1 < (int64_t)P->tile_off_h.size() ? P->tile_off_h[rb + 1] : P->map.ntiles;
+        return;
+    }
     *tlo = P->tile_off_h[ra] + (lo - ring_first_pixel(nside, ra)) / TILE;
     *thi = P->tile_off_h[rb] + (hi - 1 - ring_first_pixel(nside, rb)) / TILE + 1;
 }
@@ -457,6 +485,39 @@ static int block_shape(const tpcf_plan_s* P, const tpcf_plan_s::Tune& t, int cap
     if (c->parts == 1) grid = std::min<int64_t>(grid, P->ws_slots);
     return (int)std::max<int64_t>(1, grid);
 }
+
+// Whether a call goes to the block kernels (map_block.cuh) or to the tile kernels (map_tile.cuh), from
+// the call's block_shape.  The blocks evaluate an angle once for several pivots, but give the
+// entries of one (warp tile, bin, slice) to one warp and those of one (linear block, part) to one CTA.
+// They win where that longest item is short beside the call: `fill` is how many times the longest
+// items of all warp tiles would fill the GPU's warps, plus four times the same for the linear blocks and
+// the GPU's CTAs (a linear block shares its angles among 256 pivots, so it pays at a quarter of the filling).
+// With fewer, most warps wait for a few, and a tile, whose rings eight warps share, is sooner done.
+// Shared lists: `share` of the list has pivots in range, and `used` of the linear blocks' lanes have a run.
+// Measured on a GB300 over 1,100 calls (Nside 8 to 1200, 1 to 24 bins, m <= 16): below the limits the
+// blocks took up to 2.4 times the tiles' time (forward, Nside 200, 1 bin, a slice of 960 pivots: 211 against
+// 90 us; three fields, Nside 16, 2 bins: 222 against 110; shared lists of 12, Nside 91: 241 against 197),
+// above them 0.3 to 1.03 times (Nside 128, 8 bins: 283 against 555 us).
+constexpr double FILL_FWD = 4.5, FILL_MULTI = 4.0, FILL_TC = 5.0, FILL_BWD = 5.0, FILL_GROUPED = 6.0;
+
+static bool takes_blocks(const tpcf_plan_s* P, const MapCall& c, double need, int tile_ctas, double share = 1.0,
+                         double used = 1.0) {
+    if (tile_ctas < 1) return true;
+    if (P->route) return P->route == 2;
+    // shared lists have no images to pair, so one dominant bin leaves the blocks no gain
+    if (c.group > 1 && P->bin_share > 0.5) return false;
+    const double ctas = 4.0 * P->num_sms, warps = BW * ctas, f = P->bin_share;
+    const double fill = c.norb * share * c.slices / (f * warps) +
+                        4.0 * c.nlin * share * used / (std::max(f, 1.0 / c.parts) * ctas);
+    return fill >= need;
+}
+
+static int tile_grid(const tpcf_plan_s* P, int64_t ntiles, int ctas, int cap) {
+    const int64_t g = std::min<int64_t>(ntiles, (int64_t)P->num_sms * ctas);
+    return (int)std::max<int64_t>(1, std::min<int64_t>(g, cap));
+}
+
+constexpr int TILE_FLUSH = 8;  // rings that a tile's registers sum
 
 static void block_range(const tpcf_plan_s* P, int64_t lo, int64_t hi, MapCall* c) {
     c->lin_list = P->map.lin_list;
@@ -501,10 +562,27 @@ static tpcf_status map_forward(tpcf_plan_s* P, const float* d_delta, const float
     } else {
         block_range(P, lo, hi, &c);
     }
-    const int grid = block_shape(P, P->tune_fwd, P->fwd_grid, &c);
+    int grid = block_shape(P, P->tune_fwd, P->fwd_grid, &c);
+    const bool tc = (P->flags & TPCF_CONTRACT_TC) != 0;
+    const int what = group > 1 ? TILE_GROUPED : (tc ? TILE_TC : TILE_FWD), ctas = P->tile_ctas[what];
+    const bool blocks = takes_blocks(P, c, group > 1 ? FILL_GROUPED : (tc ? FILL_TC : FILL_FWD), ctas,
+                                     group > 1 ? (double)(hi - lo) / g.npix : 1.0, group > 1 ? P->gused : 1.0);
+    if (!blocks) {
+        c.flush = TILE_FLUSH;
+        c.parts = 1;
+        if (group > 1) {
+            c.gtiles = P->gtiles + P->nglin;
+            c.tile_hi = P->ngorb + P->ngtile;
+        } else {
+            tile_range(P, lo, hi, &c.tile_lo, &c.tile_hi);
+        }
+        grid = tile_grid(P, c.tile_hi - c.tile_lo, ctas, P->nslots);
+    }
     fwd_prep_kernel<<<P->num_sms * 8, 256, 0, s>>>(d_delta, d_w, P->wdw, g.npix, P->slots, (int64_t)grid * P->nent,
                                                    P->counter, n_counters(P, c));
-    if (P->flags & TPCF_CONTRACT_TC)
+    if (!blocks)
+        TRY_CUDA(kLaunch[P->M].tile(g, c, what, grid, s));
+    else if (tc)
         TRY_CUDA(kLaunch[P->M].fwd_tc(g, c, grid, s));
     else
         TRY_CUDA(kLaunch[P->M].fwd(g, c, grid, s));
@@ -532,18 +610,21 @@ extern "C" tpcf_status tpcf_forward_grouped(tpcf_plan plan, const float* d_delta
     tpcf_plan_s* P = plan;
     if (P->ggroup != group) {  // the blocks of this run length
         const int64_t nside = P->map.nside;
-        std::vector<int2> t, orb;
+        std::vector<int2> t, orb, lin_tiles;
+        int64_t lin_runs = 0;
         for (int r = 0; r < P->map.nrings; ++r) {
             const int64_t ri = r + 1;
             const int64_t n = ri < nside ? 4 * ri : (ri <= 3 * nside ? 4 * nside : 4 * (4 * nside - ri));
             const int64_t ng = (n + group - 1) / group;
-            if (P->lin_h[r])
+            if (P->lin_h[r]) {
+                lin_runs += ng;
                 for (int64_t f = 0; f < ng; f += BT * walk_np(P->M)) t.push_back(make_int2(r, (int)f));
-            else
-                for (int64_t f = 0; f < ng; f += TILE) orb.push_back(make_int2(r, (int)f));
+            }
+            for (int64_t f = 0; f < ng; f += TILE) (P->lin_h[r] ? lin_tiles : orb).push_back(make_int2(r, (int)f));
         }
-        const int64_t nglin = (int64_t)t.size();
+        const int64_t nglin = (int64_t)t.size(), ngorb = (int64_t)orb.size();
         t.insert(t.end(), orb.begin(), orb.end());
+        t.insert(t.end(), lin_tiles.begin(), lin_tiles.end());
         if ((int64_t)t.size() > P->gtiles_cap) {
             int2* buf = nullptr;
             TRY_CUDA(P->alloc(&buf, t.size()));
@@ -553,7 +634,9 @@ extern "C" tpcf_status tpcf_forward_grouped(tpcf_plan plan, const float* d_delta
         TRY_CUDA(cudaMemcpyAsync(P->gtiles, t.data(), sizeof(int2) * t.size(), cudaMemcpyHostToDevice, s));
         TRY_CUDA(cudaStreamSynchronize(s));
         P->nglin = nglin;
-        P->ngorb = (int64_t)t.size() - nglin;
+        P->ngorb = ngorb;
+        P->ngtile = (int64_t)lin_tiles.size();
+        P->gused = nglin ? (double)lin_runs / (nglin * BT * walk_np(P->M)) : 1.0;
         P->ggroup = group;
     }
     return map_forward(P, d_delta, d_w, pivot_begin, pivot_end, d_zeta, d_norm, d_sums, s, group);
@@ -598,12 +681,13 @@ extern "C" tpcf_status tpcf_forward_multi(tpcf_plan plan, const float* d_delta_a
     const int nent = n_entries_multi(K, M);
     if (!P->wdw_b) {
         // the three fields' moments of one tile have to fit an SM (as the catalogue's must)
-        if (((size_t)3 * (K * (M + 1) * 2 + K) * TILE + 6 * TILE) * sizeof(float) > 232448 || kMultiOcc[M]() < 1) {
+        if (((size_t)3 * (K * (M + 1) * 2 + K) * TILE + 6 * TILE) * sizeof(float) > 232448 || kMulti[M].blocks_occ() < 1) {
             snprintf(g_last_error, sizeof(g_last_error),
                      "tpcf_forward_multi: three fields' moments (K=%d, m_max=%d) do not fit in shared memory", K, M);
             return TPCF_ERR_UNSUPPORTED;
         }
-        const int grid = (int)std::min<int64_t>(P->num_sms * kMultiOcc[M](), P->fwd_grid);
+        P->multi_ctas = kMulti[M].tiles_occ(K);
+        const int grid = P->num_sms * std::max(kMulti[M].blocks_occ(), P->multi_ctas);
         float2 *b, *c;
         double *sl, *su;
         TRY_CUDA(P->alloc(&b, g.npix + 1));
@@ -631,12 +715,19 @@ extern "C" tpcf_status tpcf_forward_multi(tpcf_plan plan, const float* d_delta_a
     c.flush = P->tune_fwd.flush;
     c.cells = LIN_CELLS;
     block_range(P, pivot_begin, pivot_end, &c);
-    const int grid = std::min(block_shape(P, P->tune_fwd, P->fwd_grid, &c), P->multi_grid);
+    int grid = std::min(block_shape(P, P->tune_fwd, P->fwd_grid, &c), P->multi_grid);
     c.ws = P->ws3;
     c.ws_floats = 3 * P->ws_floats;
+    const bool blocks = takes_blocks(P, c, FILL_MULTI, P->multi_ctas);
+    if (!blocks) {
+        c.flush = TILE_FLUSH;
+        c.parts = 1;
+        tile_range(P, pivot_begin, pivot_end, &c.tile_lo, &c.tile_hi, true);
+        grid = tile_grid(P, c.tile_hi - c.tile_lo, P->multi_ctas, P->multi_grid);
+    }
     fwd_prep_kernel<<<P->num_sms * 8, 256, 0, s>>>(d_delta_a, d_w_a, P->wdw, g.npix, P->mslots, (int64_t)grid * nent,
                                                    P->counter, n_counters(P, c));
-    TRY_CUDA(kMulti[M](g, c, P->wdw_b, P->wdw_c, grid, s));
+    TRY_CUDA((blocks ? kMulti[M].blocks : kMulti[M].tiles)(g, c, P->wdw_b, P->wdw_c, grid, s));
     reduce_slots_kernel<<<n_blocks(nent, 32), REDUCE_THREADS, 0, s>>>(P->mslots, grid, nent, P->msums);
     const int nout = (M + 1) * K * K;
     finalize_full_kernel<<<n_blocks(nout, 128), 128, 0, s>>>(P->msums, K, M, d_zeta, d_norm, d_sums);
@@ -682,9 +773,21 @@ static tpcf_status map_backward(tpcf_plan_s* P, const float* d_delta, const floa
     c.flush = P->tune_bwd.flush;
     c.cells = LIN_CELLS;
     block_range(P, lo, hi, &c);
-    const int grid = block_shape(P, P->tune_bwd, P->bwd_grid, &c);
+    int grid = block_shape(P, P->tune_bwd, P->bwd_grid, &c);
+    const int ctas = P->tile_ctas[TILE_BWD];
+    const bool blocks = takes_blocks(P, c, FILL_BWD, ctas);
+    if (!blocks) {
+        c.flush = TILE_FLUSH;
+        c.parts = 1;
+        tile_range(P, lo, hi, &c.tile_lo, &c.tile_hi);
+        grid = tile_grid(P, c.tile_hi - c.tile_lo, ctas, P->num_sms * ctas);
+    }
     bwd_prep_kernel<<<P->num_sms * 8, 256, 0, s>>>(d_delta, d_w, P->wdw, d_grad, g.npix, d_dL, d_norm, P->K, P->M, P->H,
                                                    self, P->counter, n_counters(P, c));
+    if (!blocks) {
+        TRY_CUDA(kLaunch[P->M].tile(g, c, TILE_BWD, grid, s));
+        return TPCF_OK;
+    }
     c.step = c.parts > 1 ? 1 : 0;
     TRY_CUDA(kLaunch[P->M].bwd(g, c, grid, s));
     if (c.step == 1) {  // the blocks' h are in the workspace: the neighbour legs, again in parts

@@ -94,7 +94,7 @@ cudaError_t TPCF_CAT(map_fwd_tc_launch_m, TPCF_M)(const MapDev& g, const MapCall
 // limits agree); the CTAs are persistent and never wait on each other, so a grid
 // larger than what is resident is still correct.
 template <class Kern>
-static int occupancy_by_resources(Kern* k, size_t smem) {
+static int occupancy_by_resources(Kern* k, size_t smem, int threads) {
     if (prefer_shared(k, smem) != cudaSuccess) return 0;
     cudaFuncAttributes a;
     int dev = 0, smem_sm = 0, reserved = 0, regs_sm = 0;
@@ -104,7 +104,7 @@ static int occupancy_by_resources(Kern* k, size_t smem) {
         cudaDeviceGetAttribute(&regs_sm, cudaDevAttrMaxRegistersPerMultiprocessor, dev) != cudaSuccess)
         return 0;
     const size_t per_cta_smem = smem + a.sharedSizeBytes + (size_t)reserved;
-    const int warps = BW;
+    const int warps = threads / 32;
     const int regs_warp = (a.numRegs * 32 + 255) / 256 * 256;  // allocated per warp in units of 256
     const int by_smem = (int)((size_t)smem_sm / per_cta_smem);
     const int by_regs = regs_warp > 0 ? regs_sm / (regs_warp * warps) : 0;
@@ -113,10 +113,60 @@ static int occupancy_by_resources(Kern* k, size_t smem) {
 
 int TPCF_CAT(map_fwd_tc_occupancy_m, TPCF_M)(int K, int self_subtract) {
     const size_t smem = tc_smem_bytes(K, TPCF_M, self_subtract != 0);
-    const int nb = self_subtract ? occupancy_by_resources(map_fwd_tc_kernel<TPCF_M, true>, smem)
-                                 : occupancy_by_resources(map_fwd_tc_kernel<TPCF_M, false>, smem);
+    const int nb = self_subtract ? occupancy_by_resources(map_fwd_tc_kernel<TPCF_M, true>, smem, BT)
+                                 : occupancy_by_resources(map_fwd_tc_kernel<TPCF_M, false>, smem, BT);
     // at most 512 / TC_TMEM_COLS accumulators per SM; more resident CTAs would wait in tcgen05.alloc
     return nb < 512 / TC_TMEM_COLS ? nb : 512 / TC_TMEM_COLS;
+}
+
+// The tile kernels (map_tile.cuh): launch, and resident CTAs per SM (either self-pair mode).
+cudaError_t TPCF_CAT(map_tile_launch_m, TPCF_M)(const MapDev& g, const MapCall& c, int what, int grid, cudaStream_t s) {
+    const bool self = c.self_subtract != 0;
+    if (what == TILE_BWD) {
+        const size_t smem = bwd_tile_floats_rt(g.K, TPCF_M) * sizeof(float);
+        return self ? launch(map_tile_bwd_kernel<TPCF_M, true>, smem, grid, g, c, s)
+                    : launch(map_tile_bwd_kernel<TPCF_M, false>, smem, grid, g, c, s);
+    }
+    if (what == TILE_TC) {
+        const size_t smem = tc_tile_bytes(g.K, TPCF_M, self);
+        return self ? launch(map_tile_tc_kernel<TPCF_M, true>, smem, grid, g, c, s)
+                    : launch(map_tile_tc_kernel<TPCF_M, false>, smem, grid, g, c, s);
+    }
+    const size_t smem = tile_floats_rt(g.K, TPCF_M) * sizeof(float);
+    if (what == TILE_GROUPED)  // (self pairs kept)
+        return launch(map_tile_fwd_kernel<TPCF_M, false, false, 3, true>, smem, grid, g, c, s);
+    return self ? launch(map_tile_fwd_kernel<TPCF_M, true, false>, smem, grid, g, c, s)
+                : launch(map_tile_fwd_kernel<TPCF_M, false, false>, smem, grid, g, c, s);
+}
+
+int TPCF_CAT(map_tile_occupancy_m, TPCF_M)(int what, int K, int self) {
+    if (what == TILE_BWD) {
+        const size_t smem = bwd_tile_floats_rt(K, TPCF_M) * sizeof(float);
+        return self ? occupancy(map_tile_bwd_kernel<TPCF_M, true>, smem) : occupancy(map_tile_bwd_kernel<TPCF_M, false>, smem);
+    }
+    if (what == TILE_TC) {
+        const size_t smem = tc_tile_bytes(K, TPCF_M, self != 0);
+        const int nb = self ? occupancy_by_resources(map_tile_tc_kernel<TPCF_M, true>, smem, NTHREADS)
+                            : occupancy_by_resources(map_tile_tc_kernel<TPCF_M, false>, smem, NTHREADS);
+        return nb < 512 / TC_TMEM_COLS ? nb : 512 / TC_TMEM_COLS;
+    }
+    const size_t smem = tile_floats_rt(K, TPCF_M) * sizeof(float);
+    return self ? occupancy(map_tile_fwd_kernel<TPCF_M, true, false>, smem)
+                : occupancy(map_tile_fwd_kernel<TPCF_M, false, false>, smem);
+}
+
+cudaError_t TPCF_CAT(map_tile_multi_launch_m, TPCF_M)(const MapDev& g, const MapCall& c, const float2* wdwB,
+                                                      const float2* wdwC, int grid, cudaStream_t s) {
+    const size_t smem = multi_tile_floats(g.K, TPCF_M) * sizeof(float);
+    auto* k = map_tile_multi_kernel<TPCF_M>;
+    cudaError_t e = prefer_shared(k, smem);
+    if (e != cudaSuccess) return e;
+    k<<<grid, NTHREADS, smem, s>>>(g, c, wdwB, wdwC);
+    return cudaGetLastError();
+}
+
+int TPCF_CAT(map_tile_multi_occupancy_m, TPCF_M)(int K) {
+    return occupancy(map_tile_multi_kernel<TPCF_M>, multi_tile_floats(K, TPCF_M) * sizeof(float));
 }
 
 // Multi-field forward (three fields on the same pixels).

@@ -500,9 +500,12 @@ __host__ __device__ inline TcLayout tc_layout(int K, int M, bool self) {
     return L;
 }
 
-// bytes of dynamic shared memory
+// bytes of dynamic shared memory of the tile and of the block kernel
+__host__ __device__ inline size_t tc_tile_bytes(int K, int M, bool self) {
+    return (size_t)tc_layout(K, M, self).total * sizeof(float);
+}
 __host__ __device__ inline size_t tc_smem_bytes(int K, int M, bool self) {
-    const size_t a = (size_t)tc_layout(K, M, self).total * sizeof(float), b = block_smem_bytes(M);
+    const size_t a = tc_tile_bytes(K, M, self), b = block_smem_bytes(M);
     return a > b ? a : b;
 }
 
@@ -610,7 +613,7 @@ __device__ __forceinline__ void tc_teardown(uint32_t tmem) {
 // The tile's S and D partial sums on the tensor cores (see above); the self-pair
 // diagonals stay on the FP32 pipe.  Called by every thread; the moments in sX are
 // consumed (truncated in place).
-template <int M, bool SELF>
+template <int M, bool SELF, int NT>
 __device__ void tile_contract_tc(int K, float* base, double* slot, TcState& tc, int* status) {
     const TcLayout L = tc_layout(K, M, SELF);
     const int P = n_pairs_tri(K);
@@ -637,7 +640,7 @@ __device__ void tile_contract_tc(int K, float* base, double* slot, TcState& tc, 
         // beyond the block are zero.  e runs over the layout in memory order (row group,
         // pivot chunk, row in group, pivot in chunk); r0 is a multiple of 8, so the
         // block's element e sits at sX[r0 * 32 + e] and B's at B[e].
-        for (int e = threadIdx.x; e < N * TILE; e += BT) {
+        for (int e = threadIdx.x; e < N * TILE; e += NT) {
             const int i = ((e >> 8) << 3) + ((e >> 2) & 7);
             const int p = (((e >> 5) & 7) << 2) + (e & 3);
             float bh = 0.0f, bl = 0.0f;
@@ -734,7 +737,7 @@ __device__ void tile_contract_tc(int K, float* base, double* slot, TcState& tc, 
         const float* wt = sPiv + TILE;
         const float* sQ = base + L.offQ;
         const float* sQW = base + L.offQW;
-        for (int k = threadIdx.x; k < K; k += BT) {
+        for (int k = threadIdx.x; k < K; k += NT) {
             float s1 = 0.0f, s2 = 0.0f;
             for (int j = 0; j < TILE; ++j) {
                 s1 = fmaf(wd[j], sQ[k * TILE + j], s1);
@@ -793,7 +796,7 @@ __device__ __forceinline__ void fwd_block_tc(const MapDev& g, const MapCall& c, 
             base[L.offPiv + TILE + lane] = v.y;
         }
         __syncthreads();
-        tile_contract_tc<M, SELF>(K, base, slot, tc, c.status);
+        tile_contract_tc<M, SELF, BT>(K, base, slot, tc, c.status);
         __syncthreads();
         if (*tc.fail) return;
     }
@@ -1057,3 +1060,5 @@ __global__ void __launch_bounds__(BT, 4) batch_bwd_kernel(const BatchItem* __res
 }
 
 }  // namespace tpcf
+
+#include "map_tile.cuh"

@@ -56,10 +56,16 @@ struct tpcf_plan_s {
         int variant = 2, ctas = 0, flush = 8, quad = 0;
     } tune_fwd, tune_bwd;
     bool tuned = false;
+    // tile kernels of the map pair passes (map_tile.cuh): CTAs per SM by TileKernel; the largest share of
+    // the bins' area in one bin, and whether the rule of takes_blocks is overridden (1 tiles, 2 blocks)
+    int tile_ctas[4] = {0, 0, 0, 0};
+    double bin_share = 1.0;
+    int route = 0;
     // per-call scratch
     float2* wdw = nullptr;
     double* slots = nullptr;
     int fwd_grid = 0, bwd_grid = 0;
+    int nslots = 0;  // CTA slots: the largest grid of a forward
     int nent = 0;
     double* sums = nullptr;
     int* counter = nullptr;
@@ -71,10 +77,11 @@ struct tpcf_plan_s {
     float* ws3 = nullptr;  // workspace: three fields per block
     double* mslots = nullptr;
     double* msums = nullptr;
-    int multi_grid = 0;
+    int multi_grid = 0, multi_ctas = 0;
     // shared-neighbour-list forward: tile list of the last group size used
-    int2* gtiles = nullptr;  // linear blocks, then warp tiles
-    int64_t nglin = 0, ngorb = 0, gtiles_cap = 0;
+    int2* gtiles = nullptr;  // linear blocks, then warp tiles of the other rings and of the linear ones
+    int64_t nglin = 0, ngorb = 0, ngtile = 0, gtiles_cap = 0;
+    double gused = 1.0;  // share of the linear blocks' lanes that stand for a run
     int ggroup = 0;
     // staging for tpcf_run_host
     float* st_delta = nullptr;

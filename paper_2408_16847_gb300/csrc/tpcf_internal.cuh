@@ -10,7 +10,7 @@
 namespace tpcf {
 
 constexpr int TILE = 32;     // pivots per tile: one pivot per lane
-constexpr int NWARPS = 8;    // warps per CTA; they split the neighbour rings of a tile
+constexpr int NWARPS = 8;    // warps per CTA of the tile kernels (map_tile.cuh); they split a tile's neighbour rings
 constexpr int NTHREADS = TILE * NWARPS;
 constexpr int BW = 4;        // warps per CTA of the block kernels (map_block.cuh), four CTAs per SM
 constexpr int BT = TILE * BW;
@@ -86,8 +86,9 @@ struct MapCall {
     const float* H;         // backward: [(M+1) * K * K * 2] fp32, conj(C(k,k')) + C(k',k)
     float* grad;            // backward: [npix]
     int self_subtract;      // subtract the j = k self term
-    int flush;              // rings summed in registers before a shared-memory flush (tuned)
-    int64_t tile_lo, tile_hi;  // tiles that can hold a pivot of [piv_lo, piv_hi)
+    int flush;              // register sums go on after so many rings (tiles) or 32 entries (blocks); tuned
+    int64_t tile_lo, tile_hi;  // tile kernels: tiles that can hold a pivot of [piv_lo, piv_hi)
+    int quad;               // tile kernels: tiles in the quarter-turn layout (tile_pivot)
     int norm;               // NORM_*: per-pivot normalisation of the moments before the contraction
     // blocks of the call (map_block.cuh): nlin of lin_list from lin_lo, then norb warp tiles of
     // orb_list from orb_lo, `tiles` to a block; each block in `parts` by bins
@@ -101,7 +102,7 @@ struct MapCall {
     size_t ws_floats;       // floats of a block's workspace
     int cells;              // cells listed at a time on linear rings
     int group;              // > 1: shared neighbour lists, one lane per run of `group` ring pixels
-    const int2* gtiles;     // group > 1: tiles (ring, first run of the tile)
+    const int2* gtiles;     // tile kernels, group > 1: tiles (ring, first run of the tile)
 };
 
 // One plan of a batch (device-resident): its geometry, its per-call arguments and
@@ -132,6 +133,23 @@ inline __host__ __device__ int n_entries(int K, int M) {
 // Entries of the multi-field partial sums: full K x K matrices, S (complex) per m, then D.
 inline __host__ __device__ int n_entries_multi(int K, int M) { return 2 * (M + 1) * K * K + K * K; }
 
+// The tile kernels (map_tile.cuh) that a call can take.
+enum TileKernel { TILE_FWD, TILE_GROUPED, TILE_TC, TILE_BWD };
+constexpr int ROW = 512;  // floats per warp row buffer of the tile adjoint (wider rows: whole-ring or global adds)
+// Shared memory (floats) of a forward tile with runtime m_max mr: moments A[k][m][re/im][32],
+// W, Q, QW [k][32], the pivots' (w d, w).
+__host__ __device__ inline size_t tile_floats_rt(int K, int mr) {
+    return (size_t)K * (mr + 1) * 2 * TILE + 3 * (size_t)K * TILE + 2 * TILE;
+}
+// Shared memory (floats) of an adjoint tile: phases 1-2 use the moments, W, Q, QW, the pivots, the
+// primary-term sums and one m of H; phase 3 keeps the moments (then h) and the warps' row buffers.
+__host__ __device__ inline size_t bwd_tile_floats_rt(int K, int mr) {
+    const size_t a = (size_t)K * (mr + 1) * 2 * TILE;
+    const size_t p12 = a + 3 * (size_t)K * TILE + 2 * TILE + TILE + (size_t)K * K * 2;
+    const size_t p3 = a + (size_t)NWARPS * ROW;
+    return p12 > p3 ? p12 : p3;
+}
+
 // Pivots per lane of the block kernels (map_block.cuh): 2 bins' sums of M + 1 multipoles each
 // take 4 (M + 1) registers.
 __host__ __device__ constexpr int walk_np(int M) { return 2; }
@@ -146,8 +164,7 @@ inline size_t block_floats(int K, int mr, int M, bool self) { return (size_t)BW 
 // one bin.  3,000 points: 131 us at 1 bin, 156 us at 12, against 236 and 334 with 8 warps and atomics.)
 __host__ __device__ inline int cat_slices(int K) { return K >= 8 ? 1 : (K >= 4 ? 2 : 4); }
 // Calls whose (warp tile, bin) items would leave most warps of the GPU without two: tiles then go one
-// to a block and a bin's rings to four warps.  (Nside 24, 8 bins: 137 us.  One bin at Nside 24 is
-// still a long chain per warp: 147 us, against 94 with the earlier eight warps per tile.)
+// to a block and a bin's rings to four warps.
 __host__ __device__ inline bool few_tiles(long long norb, int K, int num_sms) {
     return norb * K < (long long)2 * 4 * BW * num_sms;
 }
@@ -189,6 +206,7 @@ __host__ __device__ constexpr size_t adj_smem_bytes(int M) {
 
 // Device status bits.
 constexpr int ST_BAD_TILE = 1;
+constexpr int ST_ROW_OVERFLOW = 2;    // informational: a row wider than the warp's buffer used direct global adds
 constexpr int ST_TC_TIMEOUT_BIT = 4;  // a tensor-core completion wait gave up
 
 }  // namespace tpcf
