@@ -230,8 +230,9 @@ tpcf_status tpcf_forward_multi(tpcf_plan plan, const float* d_delta_a, const flo
  * it; such a first call should come before any stream capture.  The largest plan the
  * ABI allows (32 bins, m_max 16) needs 148 KB per CTA slot; the call runs as many
  * CTAs as there are slots in the array.  All calls share the array and each call
- * clears what must start at zero; calls whose GPU work overlaps (other streams,
- * host threads or plans at the same time) race on it and must be serialised.
+ * clears what must start at zero; calls of this function whose GPU work overlaps (other
+ * streams, host threads or plans at the same time) race on it and must be serialised.  It uses
+ * none of the plan's own scratch, so it may overlap the plan's other calls.
  * Map plans without self-pair subtraction only (else TPCF_ERR_UNSUPPORTED); a plan
  * whose per-CTA partial sums (2 (m_max+1) K(K+1)/2 + K(K+1)/2 + 2K doubles) do not
  * fit is rejected with TPCF_ERR_INVALID_ARG and a message in tpcf_last_error().

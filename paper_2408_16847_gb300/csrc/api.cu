@@ -517,8 +517,6 @@ static int tile_grid(const tpcf_plan_s* P, int64_t ntiles, int ctas, int cap) {
     return (int)std::max<int64_t>(1, std::min<int64_t>(g, cap));
 }
 
-constexpr int TILE_FLUSH = 8;  // rings that a tile's registers sum
-
 static void block_range(const tpcf_plan_s* P, int64_t lo, int64_t hi, MapCall* c) {
     c->lin_list = P->map.lin_list;
     c->orb_list = P->map.orb_list;

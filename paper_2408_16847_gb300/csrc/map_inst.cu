@@ -46,9 +46,9 @@ static int occupancy(Kern* k, size_t smem, int threads = NTHREADS) {
 cudaError_t TPCF_CAT(map_fwd_launch_m, TPCF_M)(const MapDev& g, const MapCall& c, int grid, cudaStream_t s) {
     const size_t smem = block_smem_bytes(TPCF_M);
     if (c.group > 1)  // shared neighbour lists (self pairs kept)
-        return launch(map_fwd_kernel<TPCF_M, false, false, true>, smem, grid, g, c, s, BT);
-    return c.self_subtract ? launch(map_fwd_kernel<TPCF_M, true, false>, smem, grid, g, c, s, BT)
-                           : launch(map_fwd_kernel<TPCF_M, false, false>, smem, grid, g, c, s, BT);
+        return launch(map_fwd_kernel<TPCF_M, false, true>, smem, grid, g, c, s, BT);
+    return c.self_subtract ? launch(map_fwd_kernel<TPCF_M, true>, smem, grid, g, c, s, BT)
+                           : launch(map_fwd_kernel<TPCF_M, false>, smem, grid, g, c, s, BT);
 }
 
 cudaError_t TPCF_CAT(map_bwd_launch_m, TPCF_M)(const MapDev& g, const MapCall& c, int grid, cudaStream_t s) {
@@ -59,8 +59,8 @@ cudaError_t TPCF_CAT(map_bwd_launch_m, TPCF_M)(const MapDev& g, const MapCall& c
 
 // Resident CTAs per SM of the forward (either self-pair mode).
 int TPCF_CAT(map_fwd_occupancy_m, TPCF_M)() {
-    const int a = occupancy(map_fwd_kernel<TPCF_M, false, false>, block_smem_bytes(TPCF_M), BT);
-    const int b = occupancy(map_fwd_kernel<TPCF_M, true, false>, block_smem_bytes(TPCF_M), BT);
+    const int a = occupancy(map_fwd_kernel<TPCF_M, false>, block_smem_bytes(TPCF_M), BT);
+    const int b = occupancy(map_fwd_kernel<TPCF_M, true>, block_smem_bytes(TPCF_M), BT);
     return a < b ? a : b;
 }
 
@@ -135,6 +135,8 @@ cudaError_t TPCF_CAT(map_tile_launch_m, TPCF_M)(const MapDev& g, const MapCall& 
     const size_t smem = tile_floats_rt(g.K, TPCF_M) * sizeof(float);
     if (what == TILE_GROUPED)  // (self pairs kept)
         return launch(map_tile_fwd_kernel<TPCF_M, false, false, 3, true>, smem, grid, g, c, s);
+    if (what == TILE_DIRECT)  // the caller's delta and w, no packed copy
+        return launch(map_tile_fwd_kernel<TPCF_M, false, true>, smem, grid, g, c, s);
     return self ? launch(map_tile_fwd_kernel<TPCF_M, true, false>, smem, grid, g, c, s)
                 : launch(map_tile_fwd_kernel<TPCF_M, false, false>, smem, grid, g, c, s);
 }
@@ -197,17 +199,6 @@ cudaError_t TPCF_CAT(cat_fwd_multi_launch_m, TPCF_M)(const CatDev& g, const MapC
 
 int TPCF_CAT(cat_fwd_multi_occupancy_m, TPCF_M)(int K) {
     return occupancy(cat_fwd_multi_kernel<TPCF_M>, cat_fwd_bytes<TPCF_M>(K), BT);
-}
-
-// Forward that reads the caller's delta and w directly (no packed copy).
-cudaError_t TPCF_CAT(map_fwd_direct_launch_m, TPCF_M)(const MapDev& g, const MapCall& c, int grid,
-                                                      cudaStream_t s) {
-    const size_t smem = block_smem_bytes(TPCF_M);
-    auto* k = map_fwd_kernel<TPCF_M, false, true>;
-    cudaError_t e = prefer_shared(k, smem, BT);
-    if (e != cudaSuccess) return e;
-    k<<<grid, BT, smem, s>>>(g, c);
-    return cudaGetLastError();
 }
 
 // Batched forward / adjoint over all the plans of a batch whose largest m_max is this

@@ -305,9 +305,7 @@ struct PackedLoad {
 struct DirectLoad {
     const float* __restrict__ d;
     const float* __restrict__ w;
-    long long n;  // pixels: entry n reads as zero, as in the packed array
     __device__ __forceinline__ float2 operator()(long long i) const {
-        if (i >= n) return make_float2(0.0f, 0.0f);
         const float wi = __ldg(w + i);
         return make_float2(wi * __ldg(d + i), wi);
     }
@@ -803,7 +801,7 @@ __device__ __forceinline__ void fwd_block_tc(const MapDev& g, const MapCall& c, 
 }
 
 // Persistent CTAs draw work items (block, part) from a counter.
-template <int M, bool SELF, bool DIRECT, bool GROUPED = false>
+template <int M, bool SELF, bool GROUPED = false>
 __global__ void __launch_bounds__(BT, 4) map_fwd_kernel(MapDev g, MapCall c) {
     extern __shared__ __align__(16) float smem[];
     __shared__ int s_tile;
@@ -817,11 +815,7 @@ __global__ void __launch_bounds__(BT, 4) map_fwd_kernel(MapDev g, MapCall c) {
         const long long b = item / c.parts;
         float* ws = c.ws + (c.parts > 1 ? (size_t)b : (size_t)blockIdx.x) * c.ws_floats;
         const int part = (int)(item - b * c.parts);
-        if constexpr (DIRECT)
-            fwd_block<M, SELF, GROUPED>(g, c, b, part, DirectLoad{c.delta, c.w, g.npix}, ws, slot,
-                                        reinterpret_cast<char*>(smem), M);
-        else
-            fwd_block<M, SELF, GROUPED>(g, c, b, part, PackedLoad{c.wdw}, ws, slot, reinterpret_cast<char*>(smem), M);
+        fwd_block<M, SELF, GROUPED>(g, c, b, part, PackedLoad{c.wdw}, ws, slot, reinterpret_cast<char*>(smem), M);
     }
 }
 

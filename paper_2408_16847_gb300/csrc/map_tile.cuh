@@ -623,7 +623,7 @@ __device__ __forceinline__ void fwd_tile(const MapDev& g, const MapCall& c, int 
             for (int u = 0; u < ln; ++u) {
                 const long long pix = f + u;
                 if (pix >= c.piv_lo && pix < c.piv_hi) {
-                    const float2 v = DIRECT ? DirectLoad{c.delta, c.w, g.npix}(pix) : c.wdw[pix];
+                    const float2 v = DIRECT ? DirectLoad{c.delta, c.w}(pix) : c.wdw[pix];
                     pv.x += v.x;
                     pv.y += v.y;
                 }
@@ -633,7 +633,7 @@ __device__ __forceinline__ void fwd_tile(const MapDev& g, const MapCall& c, int 
         const TilePivot tp = tile_pivot(tq.y, P.n_i, c.quad != 0);
         const long long pix = g.ring_first[P.i] + tp.q;
         if (tp.valid && pix >= c.piv_lo && pix < c.piv_hi)
-            pv = DIRECT ? DirectLoad{c.delta, c.w, g.npix}(pix) : c.wdw[pix];
+            pv = DIRECT ? DirectLoad{c.delta, c.w}(pix) : c.wdw[pix];
         qg = tp.qg;
     }
     if (!__syncthreads_or(pv.y != 0.0f)) return;
@@ -644,7 +644,7 @@ __device__ __forceinline__ void fwd_tile(const MapDev& g, const MapCall& c, int 
     }
     __syncthreads();
     if (DIRECT)
-        tile_moments<M, SELF>(g, P, qg, DirectLoad{c.delta, c.w, g.npix}, sA, sW, sQ, sQW, c.flush, mr,
+        tile_moments<M, SELF>(g, P, qg, DirectLoad{c.delta, c.w}, sA, sW, sQ, sQW, c.flush, mr,
                               !grouped && c.quad);
     else
         tile_moments<M, SELF>(g, P, qg, PackedLoad{c.wdw}, sA, sW, sQ, sQW, c.flush, mr, !grouped && c.quad);

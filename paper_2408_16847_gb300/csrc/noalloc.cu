@@ -5,8 +5,10 @@
 // the pool), programs whose hot loop must not enter the CUDA allocator because
 // cudaMalloc/cudaFree can synchronise the device, and embedders that account for
 // every byte of device memory.  They create the plan once, during set-up, and then
-// call this entry point, which uses only the caller's buffers, the plan's tables and
-// workspace (allocated with the plan) and the fixed scratch array below.
+// call this entry point, which uses only the caller's buffers, the plan's
+// read-only tables and the fixed scratch array below (so that it may also overlap the plan's
+// other calls).  It takes the tile kernel at every size: the block kernels' workspace, up to 0.7 GB,
+// has no place here.
 //
 // The scratch lives in a file-scope __device__ array.  This file is its own CUDA
 // module, and CUDA loads modules lazily, so the array is placed on a device when its
@@ -27,21 +29,18 @@
 
 namespace tpcf {
 
-#define TPCF_DECL_DIRECT(m) \
-    cudaError_t map_fwd_direct_launch_m##m(const MapDev&, const MapCall&, int, cudaStream_t);
-TPCF_DECL_DIRECT(0) TPCF_DECL_DIRECT(1) TPCF_DECL_DIRECT(2) TPCF_DECL_DIRECT(3) TPCF_DECL_DIRECT(4)
-TPCF_DECL_DIRECT(5) TPCF_DECL_DIRECT(6) TPCF_DECL_DIRECT(7) TPCF_DECL_DIRECT(8) TPCF_DECL_DIRECT(9)
-TPCF_DECL_DIRECT(10) TPCF_DECL_DIRECT(11) TPCF_DECL_DIRECT(12) TPCF_DECL_DIRECT(13) TPCF_DECL_DIRECT(14)
-TPCF_DECL_DIRECT(15) TPCF_DECL_DIRECT(16)
-#undef TPCF_DECL_DIRECT
+#define TPCF_DECL_TILE(m) cudaError_t map_tile_launch_m##m(const MapDev&, const MapCall&, int, int, cudaStream_t);
+TPCF_DECL_TILE(0) TPCF_DECL_TILE(1) TPCF_DECL_TILE(2) TPCF_DECL_TILE(3) TPCF_DECL_TILE(4) TPCF_DECL_TILE(5)
+TPCF_DECL_TILE(6) TPCF_DECL_TILE(7) TPCF_DECL_TILE(8) TPCF_DECL_TILE(9) TPCF_DECL_TILE(10) TPCF_DECL_TILE(11)
+TPCF_DECL_TILE(12) TPCF_DECL_TILE(13) TPCF_DECL_TILE(14) TPCF_DECL_TILE(15) TPCF_DECL_TILE(16)
+#undef TPCF_DECL_TILE
 
-typedef cudaError_t (*direct_fn)(const MapDev&, const MapCall&, int, cudaStream_t);
-static const direct_fn kDirect[TPCF_MAX_M + 1] = {
-    map_fwd_direct_launch_m0,  map_fwd_direct_launch_m1,  map_fwd_direct_launch_m2,  map_fwd_direct_launch_m3,
-    map_fwd_direct_launch_m4,  map_fwd_direct_launch_m5,  map_fwd_direct_launch_m6,  map_fwd_direct_launch_m7,
-    map_fwd_direct_launch_m8,  map_fwd_direct_launch_m9,  map_fwd_direct_launch_m10, map_fwd_direct_launch_m11,
-    map_fwd_direct_launch_m12, map_fwd_direct_launch_m13, map_fwd_direct_launch_m14, map_fwd_direct_launch_m15,
-    map_fwd_direct_launch_m16};
+typedef cudaError_t (*tile_fn)(const MapDev&, const MapCall&, int, int, cudaStream_t);
+static const tile_fn kTile[TPCF_MAX_M + 1] = {
+    map_tile_launch_m0,  map_tile_launch_m1,  map_tile_launch_m2,  map_tile_launch_m3,  map_tile_launch_m4,
+    map_tile_launch_m5,  map_tile_launch_m6,  map_tile_launch_m7,  map_tile_launch_m8,  map_tile_launch_m9,
+    map_tile_launch_m10, map_tile_launch_m11, map_tile_launch_m12, map_tile_launch_m13, map_tile_launch_m14,
+    map_tile_launch_m15, map_tile_launch_m16};
 
 // Scratch layout: [0, 256) work counter; [256, 256 + 8 nent) reduced sums;
 // then one slot of nent doubles per CTA.
@@ -122,7 +121,8 @@ extern "C" tpcf_status tpcf_forward_noalloc(tpcf_plan plan, const float* d_delta
     double* sums = (double*)(base + NOALLOC_HEADER);
     double* slots = (double*)(base + NOALLOC_HEADER + sums_bytes);
     const size_t room = (NOALLOC_SCRATCH_BYTES - NOALLOC_HEADER - sums_bytes) / slot_bytes;
-    const int grid = (int)std::min<size_t>((size_t)std::min(plan->fwd_grid, plan->ws_slots), room);
+    const int64_t ctas = std::min<int64_t>(plan->map.ntiles, (int64_t)plan->num_sms * std::max(1, plan->tile_ctas[TILE_FWD]));
+    const int grid = (int)std::min<size_t>((size_t)ctas, room);
     cudaStream_t s = (cudaStream_t)stream;
     plan->last_stream = s;
     TRY_CUDA(cudaMemsetAsync(counter, 0, sizeof(int), s));
@@ -137,19 +137,10 @@ extern "C" tpcf_status tpcf_forward_noalloc(tpcf_plan plan, const float* d_delta
     c.status = plan->status;
     c.self_subtract = 0;
     c.norm = norm_of_flags(plan->flags);
-    c.flush = plan->tune_fwd.flush;
-    // every block; those without a pivot in range return at once
-    c.lin_list = plan->map.lin_list;
-    c.orb_list = plan->map.orb_list;
-    c.nlin = plan->lin_off_h.back();
-    c.norb = plan->orb_off_h.back();
-    c.slices = few_tiles(c.norb, plan->K, plan->num_sms) ? 4 : 1;
-    c.tiles = c.slices > 1 ? 1 : 2;
-    c.parts = 1;
-    c.ws = plan->ws;
-    c.ws_floats = plan->ws_floats;
-    c.cells = LIN_CELLS;
-    TRY_CUDA(kDirect[plan->M](plan->map, c, grid, s));
+    c.flush = TILE_FLUSH;
+    c.tile_lo = 0;  // every tile; those without a pivot in range return at once
+    c.tile_hi = plan->map.ntiles;
+    TRY_CUDA(kTile[plan->M](plan->map, c, TILE_DIRECT, grid, s));
     reduce_slots_kernel<<<(plan->nent + 31) / 32, REDUCE_THREADS, 0, s>>>(slots, grid, plan->nent, sums);
     const int nout = (plan->M + 1) * plan->K * plan->K;
     finalize_kernel<<<(nout + 127) / 128, 128, 0, s>>>(sums, plan->K, plan->M, 0, 1.0, d_zeta, d_norm, nullptr);
