@@ -4,8 +4,8 @@
 // bins, m_max and self-pair mode) with a fixed, short launch sequence whose length
 // does not grow with n: the small per-entry kernels take the plan as blockIdx.y, and
 // one persistent forward and one persistent adjoint launch, compiled for the batch's
-// largest m_max, pull the tiles of every plan from one concatenated work queue (each
-// plan's tiles run with its own m_max, bins and self-pair mode).  The sequence is
+// largest m_max, pull the blocks (small batches: tiles) of every plan from one concatenated work
+// queue (each runs with its plan's m_max, bins and self-pair mode).  The sequence is
 // captured into a graph at creation; every launch replays it.
 #include <cuda_runtime.h>
 #include <stdio.h>
@@ -23,12 +23,12 @@ using namespace tpcf;
 
 namespace tpcf {
 #define TPCF_DECL_BATCH_M(m)                                                                                  \
-    cudaError_t batch_fwd_launch_m##m(const BatchItem*, int, long long, unsigned long long*, size_t, int,      \
+    cudaError_t batch_fwd_launch_m##m(const BatchItem*, int, long long, unsigned long long*, size_t, int, bool, \
                                       cudaStream_t);                                                          \
-    cudaError_t batch_bwd_launch_m##m(const BatchItem*, int, long long, unsigned long long*, size_t, int,      \
+    cudaError_t batch_bwd_launch_m##m(const BatchItem*, int, long long, unsigned long long*, size_t, int, bool, \
                                       cudaStream_t);                                                          \
-    int batch_fwd_occupancy_m##m(size_t);                                                                     \
-    int batch_bwd_occupancy_m##m(size_t);
+    int batch_fwd_occupancy_m##m(size_t, bool);                                                               \
+    int batch_bwd_occupancy_m##m(size_t, bool);
 TPCF_DECL_BATCH_M(0) TPCF_DECL_BATCH_M(1) TPCF_DECL_BATCH_M(2) TPCF_DECL_BATCH_M(3) TPCF_DECL_BATCH_M(4)
 TPCF_DECL_BATCH_M(5) TPCF_DECL_BATCH_M(6) TPCF_DECL_BATCH_M(7) TPCF_DECL_BATCH_M(8) TPCF_DECL_BATCH_M(9)
 TPCF_DECL_BATCH_M(10) TPCF_DECL_BATCH_M(11) TPCF_DECL_BATCH_M(12) TPCF_DECL_BATCH_M(13) TPCF_DECL_BATCH_M(14)
@@ -36,10 +36,10 @@ TPCF_DECL_BATCH_M(15) TPCF_DECL_BATCH_M(16)
 #undef TPCF_DECL_BATCH_M
 
 struct BLaunch {
-    cudaError_t (*fwd)(const BatchItem*, int, long long, unsigned long long*, size_t, int, cudaStream_t);
-    cudaError_t (*bwd)(const BatchItem*, int, long long, unsigned long long*, size_t, int, cudaStream_t);
-    int (*fwd_occ)(size_t);
-    int (*bwd_occ)(size_t);
+    cudaError_t (*fwd)(const BatchItem*, int, long long, unsigned long long*, size_t, int, bool, cudaStream_t);
+    cudaError_t (*bwd)(const BatchItem*, int, long long, unsigned long long*, size_t, int, bool, cudaStream_t);
+    int (*fwd_occ)(size_t, bool);
+    int (*bwd_occ)(size_t, bool);
 };
 #define TPCF_BROW(m) {batch_fwd_launch_m##m, batch_bwd_launch_m##m, batch_fwd_occupancy_m##m, batch_bwd_occupancy_m##m}
 static const BLaunch kBatch[TPCF_MAX_M + 1] = {
@@ -57,8 +57,9 @@ struct Group {
     std::vector<int> members;  // indices into the batch's plan list
     BatchItem* d_items = nullptr;
     size_t fwd_smem = 0, bwd_smem = 0;
-    long long total_blocks = 0;  // work items of a pass
-    float* ws = nullptr;         // workspace: one block per CTA
+    bool tiles = false;          // tile kernels (map_tile.cuh), else blocks (map_block.cuh)
+    long long total = 0;         // work items of a pass
+    float* ws = nullptr;         // blocks: workspace, one block per CTA
     size_t ws_floats = 0;
     int fwd_grid = 0, bwd_grid = 0;
 };
@@ -107,8 +108,8 @@ static tpcf_status record(tpcf_batch_s* B, int num_sms, int max_nent, int max_no
     TRY_CUDA(cudaMemsetAsync(B->d_counters, 0, sizeof(unsigned long long) * 2 * B->groups.size(), s));
     for (size_t gi = 0; gi < B->groups.size(); ++gi) {
         const Group& G = B->groups[gi];
-        TRY_CUDA(kBatch[G.M].fwd(G.d_items, (int)G.members.size(), G.total_blocks, B->d_counters + 2 * gi,
-                                 G.fwd_smem, G.fwd_grid, s));
+        TRY_CUDA(kBatch[G.M].fwd(G.d_items, (int)G.members.size(), G.total, B->d_counters + 2 * gi, G.fwd_smem,
+                                 G.fwd_grid, G.tiles, s));
         B->kernels += 1;
     }
     batch_reduce_kernel<<<dim3(n_blocks(max_nent, 32), n), REDUCE_THREADS, 0, s>>>(B->d_io);
@@ -119,14 +120,20 @@ static tpcf_status record(tpcf_batch_s* B, int num_sms, int max_nent, int max_no
         B->kernels += 1;
         for (size_t gi = 0; gi < B->groups.size(); ++gi) {
             const Group& G = B->groups[gi];
-            TRY_CUDA(kBatch[G.M].bwd(G.d_items, (int)G.members.size(), G.total_blocks, B->d_counters + 2 * gi + 1,
-                                     G.bwd_smem, G.bwd_grid, s));
+            TRY_CUDA(kBatch[G.M].bwd(G.d_items, (int)G.members.size(), G.total, B->d_counters + 2 * gi + 1,
+                                     G.bwd_smem, G.bwd_grid, G.tiles, s));
             B->kernels += 1;
         }
     }
     TRY_CUDA(cudaGetLastError());
     return TPCF_OK;
 }
+
+// Batches of fewer blocks per SM than this go to the tile kernels: a block's pivots share their angles,
+// but its whole work is one CTA's, and a batch does not split blocks.  Measured on a GB300 (152 SMs),
+// forward and adjoint, tiles against blocks: 2 maps at Nside 16, 16 bins (126 blocks in all) 229 against
+// 397 us; 4 at Nside 24, 2 bins (316 blocks) 231 against 219 us; 8 at Nside 24, 8 bins 593 against 419 us.
+constexpr long long BATCH_BLOCKS = 2;
 
 static tpcf_status batch_build(tpcf_batch_s* B, const tpcf_plan* plans, const float* const* d_delta,
                                const float* const* d_w, double* const* d_zeta, double* const* d_norm,
@@ -147,11 +154,21 @@ static tpcf_status batch_build(tpcf_batch_s* B, const tpcf_plan* plans, const fl
     std::vector<BatchIO> io(n);
     std::vector<int> grid_of(n, 0);
     for (Group& G : B->groups) {
-        for (int i : G.members)
-            G.ws_floats = std::max(G.ws_floats, block_floats(plans[i]->K, plans[i]->M, G.M, true));
-        G.bwd_smem = adj_smem_bytes(G.M);
-        G.fwd_smem = block_smem_bytes(G.M);
-        const int of = kBatch[G.M].fwd_occ(G.fwd_smem);
+        long long blocks = 0;
+        for (int i : G.members) blocks += plans[i]->lin_off_h.back() + (plans[i]->orb_off_h.back() + 1) / 2;
+        G.tiles = blocks < BATCH_BLOCKS * num_sms;
+        G.bwd_smem = G.tiles ? 0 : adj_smem_bytes(G.M);
+        G.fwd_smem = G.tiles ? 0 : block_smem_bytes(G.M);
+        for (int i : G.members) {
+            const tpcf_plan P = plans[i];
+            if (G.tiles) {
+                G.fwd_smem = std::max(G.fwd_smem, tile_floats_rt(P->K, P->M) * sizeof(float));
+                G.bwd_smem = std::max(G.bwd_smem, bwd_tile_floats_rt(P->K, P->M) * sizeof(float));
+            } else {
+                G.ws_floats = std::max(G.ws_floats, block_floats(P->K, P->M, G.M, true));
+            }
+        }
+        const int of = kBatch[G.M].fwd_occ(G.fwd_smem, G.tiles);
         TRY_CUDA(cudaGetLastError());
         if (of < 1) {
             set_error("batch forward kernel does not fit on an SM");
@@ -159,7 +176,7 @@ static tpcf_status batch_build(tpcf_batch_s* B, const tpcf_plan* plans, const fl
         }
         G.fwd_grid = of * num_sms;
         if (B->with_bwd) {
-            const int ob = kBatch[G.M].bwd_occ(G.bwd_smem);
+            const int ob = kBatch[G.M].bwd_occ(G.bwd_smem, G.tiles);
             TRY_CUDA(cudaGetLastError());
             if (ob < 1) {
                 set_error("batch adjoint kernel does not fit on an SM");
@@ -167,7 +184,7 @@ static tpcf_status batch_build(tpcf_batch_s* B, const tpcf_plan* plans, const fl
             }
             G.bwd_grid = ob * num_sms;
         }
-        TRY_CUDA(B->alloc(&G.ws, G.ws_floats * std::max(G.fwd_grid, G.bwd_grid)));
+        if (!G.tiles) TRY_CUDA(B->alloc(&G.ws, G.ws_floats * std::max(G.fwd_grid, G.bwd_grid)));
         for (int i : G.members) grid_of[i] = G.fwd_grid;
     }
     int max_nent = 0, max_nout = 0;
@@ -215,8 +232,15 @@ static tpcf_status batch_build(tpcf_batch_s* B, const tpcf_plan* plans, const fl
             it.c.H = P->H;
             it.c.grad = io[i].grad;
             it.c.self_subtract = io[i].self_subtract;
+            it.tile0 = t0;
+            if (G.tiles) {
+                it.c.flush = TILE_FLUSH;
+                t0 += P->map.ntiles;
+                items.push_back(it);
+                continue;
+            }
             it.c.flush = P->tune_fwd.flush;
-            // forward: the plan's linear blocks, then its other rings' warp tiles, two to a block
+            // the plan's linear blocks, then its other rings' warp tiles, two to a block
             it.c.cells = LIN_CELLS;
             it.c.lin_list = P->map.lin_list;
             it.c.orb_list = P->map.orb_list;
@@ -227,11 +251,10 @@ static tpcf_status batch_build(tpcf_batch_s* B, const tpcf_plan* plans, const fl
             it.c.parts = 1;
             it.c.ws = G.ws;
             it.c.ws_floats = G.ws_floats;
-            it.tile0 = t0;
             t0 += it.c.nlin + (it.c.norb + it.c.tiles - 1) / it.c.tiles;
             items.push_back(it);
         }
-        G.total_blocks = t0;
+        G.total = t0;
         TRY_CUDA(B->alloc(&G.d_items, items.size()));
         TRY_CUDA(cudaMemcpy(G.d_items, items.data(), sizeof(BatchItem) * items.size(), cudaMemcpyHostToDevice));
     }

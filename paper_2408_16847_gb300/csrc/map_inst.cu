@@ -202,29 +202,37 @@ int TPCF_CAT(cat_fwd_multi_occupancy_m, TPCF_M)(int K) {
 }
 
 // Batched forward / adjoint over all the plans of a batch whose largest m_max is this
-// M (the dynamic shared memory is the largest any of them needs).
-cudaError_t TPCF_CAT(batch_fwd_launch_m, TPCF_M)(const BatchItem* items, int n, long long total,
-                                                 unsigned long long* counter, size_t smem, int grid, cudaStream_t s) {
-    auto* k = batch_fwd_kernel<TPCF_M>;
-    cudaError_t e = prefer_shared(k, smem, BT);
+// M, by tiles or by blocks (the dynamic shared memory is the largest any of them needs).
+template <class Kern>
+static cudaError_t launch_batch(Kern* k, const BatchItem* items, int n, long long total, unsigned long long* counter,
+                                size_t smem, int grid, int threads, cudaStream_t s) {
+    cudaError_t e = prefer_shared(k, smem, threads);
     if (e != cudaSuccess) return e;
-    k<<<grid, BT, smem, s>>>(items, n, total, counter);
+    k<<<grid, threads, smem, s>>>(items, n, total, counter);
     return cudaGetLastError();
+}
+
+cudaError_t TPCF_CAT(batch_fwd_launch_m, TPCF_M)(const BatchItem* items, int n, long long total,
+                                                 unsigned long long* counter, size_t smem, int grid, bool tiles,
+                                                 cudaStream_t s) {
+    return tiles ? launch_batch(batch_tile_fwd_kernel<TPCF_M>, items, n, total, counter, smem, grid, NTHREADS, s)
+                 : launch_batch(batch_fwd_kernel<TPCF_M>, items, n, total, counter, smem, grid, BT, s);
 }
 
 cudaError_t TPCF_CAT(batch_bwd_launch_m, TPCF_M)(const BatchItem* items, int n, long long total,
-                                                 unsigned long long* counter, size_t smem, int grid,
+                                                 unsigned long long* counter, size_t smem, int grid, bool tiles,
                                                  cudaStream_t s) {
-    auto* k = batch_bwd_kernel<TPCF_M>;
-    cudaError_t e = prefer_shared(k, smem, BT);
-    if (e != cudaSuccess) return e;
-    k<<<grid, BT, smem, s>>>(items, n, total, counter);
-    return cudaGetLastError();
+    return tiles ? launch_batch(batch_tile_bwd_kernel<TPCF_M>, items, n, total, counter, smem, grid, NTHREADS, s)
+                 : launch_batch(batch_bwd_kernel<TPCF_M>, items, n, total, counter, smem, grid, BT, s);
 }
 
-int TPCF_CAT(batch_fwd_occupancy_m, TPCF_M)(size_t smem) { return occupancy(batch_fwd_kernel<TPCF_M>, smem, BT); }
+int TPCF_CAT(batch_fwd_occupancy_m, TPCF_M)(size_t smem, bool tiles) {
+    return tiles ? occupancy(batch_tile_fwd_kernel<TPCF_M>, smem) : occupancy(batch_fwd_kernel<TPCF_M>, smem, BT);
+}
 
-int TPCF_CAT(batch_bwd_occupancy_m, TPCF_M)(size_t smem) { return occupancy(batch_bwd_kernel<TPCF_M>, smem, BT); }
+int TPCF_CAT(batch_bwd_occupancy_m, TPCF_M)(size_t smem, bool tiles) {
+    return tiles ? occupancy(batch_tile_bwd_kernel<TPCF_M>, smem) : occupancy(batch_bwd_kernel<TPCF_M>, smem, BT);
+}
 
 // Catalogue forward.
 cudaError_t TPCF_CAT(cat_fwd_launch_m, TPCF_M)(const CatDev& g, const MapCall& c, int grid, cudaStream_t s) {

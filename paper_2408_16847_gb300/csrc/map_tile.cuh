@@ -739,6 +739,32 @@ __global__ void __launch_bounds__(NTHREADS, 3) map_tile_tc_kernel(MapDev g, MapC
     tc_teardown(s_tmem);
 }
 
+// batch_fwd_kernel by tiles: the same queue over the members' tiles; a tile runs with its plan's
+// shared-memory layout.
+template <int M>
+__global__ void __launch_bounds__(NTHREADS, 2) batch_tile_fwd_kernel(const BatchItem* __restrict__ items, int n,
+                                                               long long total, unsigned long long* counter) {
+    extern __shared__ __align__(16) float smem[];
+    __shared__ long long s_t;
+    __shared__ long long s_first[TPCF_MAX_BATCH + 1];
+    for (int i = threadIdx.x; i <= n; i += NTHREADS) s_first[i] = i < n ? items[i].tile0 : total;
+    __syncthreads();
+    for (;;) {
+        if (threadIdx.x == 0) s_t = (long long)atomicAdd(counter, 1ull);
+        __syncthreads();
+        const long long t = s_t;
+        if (t >= total) break;
+        int lo = 0, hi = n - 1;
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) / 2;
+            if (s_first[mid] <= t) lo = mid; else hi = mid - 1;
+        }
+        const BatchItem& it = items[lo];
+        double* slot = it.c.slots + (size_t)blockIdx.x * n_entries(it.g.K, it.g.M);
+        fwd_tile<M, true, false>(it.g, it.c, (int)(t - s_first[lo]), slot, smem, it.g.M);
+    }
+}
+
 // ------------------------------------------------------------ multi-field
 // Three fields A, B, C on the same pixels (end of Sec. 2, after eq. ubEstimator): a
 // tile accumulates the moments a^k(i; F), W^k(i; F) of every field F in its own block
@@ -1264,5 +1290,26 @@ __global__ void __launch_bounds__(NTHREADS, OCC) map_tile_bwd_kernel(MapDev g, M
     }
 }
 
+template <int M>
+__global__ void __launch_bounds__(NTHREADS, 2) batch_tile_bwd_kernel(const BatchItem* __restrict__ items, int n,
+                                                               long long total, unsigned long long* counter) {
+    extern __shared__ __align__(16) float smem[];
+    __shared__ long long s_t;
+    __shared__ long long s_first[TPCF_MAX_BATCH + 1];
+    for (int i = threadIdx.x; i <= n; i += NTHREADS) s_first[i] = i < n ? items[i].tile0 : total;
+    __syncthreads();
+    for (;;) {
+        if (threadIdx.x == 0) s_t = (long long)atomicAdd(counter, 1ull);
+        __syncthreads();
+        const long long t = s_t;
+        if (t >= total) break;
+        int lo = 0, hi = n - 1;
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) / 2;
+            if (s_first[mid] <= t) lo = mid; else hi = mid - 1;
+        }
+        bwd_tile<M>(items[lo].g, items[lo].c, (int)(t - s_first[lo]), smem, items[lo].g.M);
+    }
+}
 
 }  // namespace tpcf
