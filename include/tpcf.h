@@ -266,16 +266,20 @@ tpcf_status tpcf_count_pairs(tpcf_plan plan, const float* d_w, int64_t pivot_beg
 
 /*
  * Autotuner of the map pair kernels' launch configuration (the paper has no GPU
- * design; this picks the tile-processing shape on the device at hand).  Times the
- * forward (passes bit 0) and/or the adjoint (bit 1) of the plan on a sample of pivots
- * of the caller's field for every candidate -- register variant sized for 3 or 2
+ * design; this picks the shape on the device at hand).  Times the forward (passes bit 0)
+ * and/or the adjoint (bit 1) of the plan on a sample of pivots of the caller's field for
+ * every candidate of the kernels that a pass over the whole map takes, and keeps the
+ * fastest in the plan.  Kernels for small calls: register variant sized for 3 or 2
  * resident CTAs per SM, CTAs per SM launched, rings summed in registers between
- * shared-memory flushes, and for the forward the tile layout (32 consecutive pivots,
- * or four runs of 8 a quarter turn apart whose lanes share the position angles on
- * rings with another pixel count) -- and keeps the fastest in the plan.  With both passes and
+ * shared-memory flushes, and for the forward the tile layout (32 consecutive pivots, or
+ * four runs of 8 a quarter turn apart whose lanes share the position angles on rings
+ * with another pixel count).  Kernels for large calls: the share of their CTAs that is
+ * launched (the CTA count beside what fits) and the flush, in units of 32 neighbours;
+ * they take no register variant and no layout.  With both passes and
  * the environment variable TPCF_AUTOTUNE_CACHE naming a file, the result is appended
  * there, keyed by device, nside, bins and flags; a later autotune call or
- * tpcf_plan_create_map with the same key takes it from the file without measuring.
+ * tpcf_plan_create_map with the same key takes it from the file without measuring
+ * (plans whose passes take the kernels for small calls read files of earlier versions).
  * Results do not depend on the configuration beyond summation order.  Allocates and
  * frees temporaries (a gradient buffer of npoints floats for the adjoint);
  * synchronises `stream`.  Map plans without TPCF_CONTRACT_TC only (else
@@ -285,7 +289,8 @@ tpcf_status tpcf_plan_autotune(tpcf_plan plan, const float* d_delta, const float
                                void* stream);
 /* The plan's launch configuration: host int32[7] = forward (variant, CTAs per SM,
  * flush rings, tile layout: 0 consecutive pivots, 1 quarter-turn runs), adjoint
- * (variant, CTAs per SM, flush rings). */
+ * (variant, CTAs per SM, flush rings), in the terms of the kernels for small calls;
+ * see above for what the others take of it. */
 tpcf_status tpcf_plan_launch_config(tpcf_plan plan, int32_t* config7);
 /* Sets it (same layout); TPCF_ERR_INVALID_ARG for a configuration that does not fit. */
 tpcf_status tpcf_plan_set_launch_config(tpcf_plan plan, const int32_t* config7);

@@ -50,8 +50,8 @@ static const MultiLaunch kMulti[TPCF_MAX_M + 1] = {
     cudaError_t map_bwd_launch_m##m(const MapDev&, const MapCall&, int, cudaStream_t);         \
     int map_fwd_occupancy_m##m();                                                             \
     int map_bwd_occupancy_m##m();                                                             \
-    cudaError_t map_tile_launch_m##m(const MapDev&, const MapCall&, int, int, cudaStream_t);   \
-    int map_tile_occupancy_m##m(int, int, int);
+    cudaError_t map_tile_launch_m##m(const MapDev&, const MapCall&, int, int, int, cudaStream_t); \
+    int map_tile_occupancy_m##m(int, int, int, int);
 TPCF_DECL_M(0) TPCF_DECL_M(1) TPCF_DECL_M(2) TPCF_DECL_M(3) TPCF_DECL_M(4) TPCF_DECL_M(5)
 TPCF_DECL_M(6) TPCF_DECL_M(7) TPCF_DECL_M(8) TPCF_DECL_M(9) TPCF_DECL_M(10) TPCF_DECL_M(11)
 TPCF_DECL_M(12) TPCF_DECL_M(13) TPCF_DECL_M(14) TPCF_DECL_M(15) TPCF_DECL_M(16)
@@ -78,8 +78,8 @@ struct MLaunch {
     cudaError_t (*bwd)(const MapDev&, const MapCall&, int, cudaStream_t);
     int (*fwd_occ)();
     int (*bwd_occ)();
-    cudaError_t (*tile)(const MapDev&, const MapCall&, int, int, cudaStream_t);  // TileKernel, grid
-    int (*tile_occ)(int, int, int);                                            // TileKernel, K, self
+    cudaError_t (*tile)(const MapDev&, const MapCall&, int, int, int, cudaStream_t);  // TileKernel, variant, grid
+    int (*tile_occ)(int, int, int, int);                                            // TileKernel, variant, K, self
 };
 #define TPCF_ROW_M(m) \
     {map_fwd_launch_m##m,    map_fwd_tc_launch_m##m,  map_fwd_tc_occupancy_m##m, map_bwd_launch_m##m, \
@@ -90,9 +90,6 @@ static const MLaunch kLaunch[TPCF_MAX_M + 1] = {
     TPCF_ROW_M(12), TPCF_ROW_M(13), TPCF_ROW_M(14), TPCF_ROW_M(15), TPCF_ROW_M(16)};
 #undef TPCF_ROW_M
 
-// resident CTAs per SM (used by the autotuner, tune.cu)
-int map_fwd_occupancy(int M) { return kLaunch[M].fwd_occ(); }
-int map_bwd_occupancy(int M) { return kLaunch[M].bwd_occ(); }
 // applies a configuration cached by the autotuner (tune.cu)
 void tune_from_cache(tpcf_plan_s* P);
 }  // namespace tpcf
@@ -312,19 +309,24 @@ static tpcf_status build_map(tpcf_plan_s* P, int64_t nside, cudaStream_t s) {
     // slots for the largest grid any configuration launches
     P->fwd_grid = P->num_sms * ((occ_f + 1) / 2 * 2);
     P->bwd_grid = P->num_sms * ((occ_b + 1) / 2 * 2);
-    P->tune_fwd.variant = P->tune_bwd.variant = 2;
-    P->tune_fwd.ctas = (occ_f + 1) / 2;
-    P->tune_bwd.ctas = (occ_b + 1) / 2;
     // workspace: a block per CTA, or (calls with few blocks) one per block, see block_shape
     P->ws_slots = (int)std::max<int64_t>(1, std::min<int64_t>(2 * std::max(P->fwd_grid, P->bwd_grid), nlin + norb));
     P->fwd_grid = (int)std::min<int64_t>(P->fwd_grid, 8 * (int64_t)P->ws_slots);
     P->ws_floats = block_floats(K, P->M, P->M, self != 0);
     TRY_CUDA(P->alloc(&P->ws, P->ws_floats * P->ws_slots));
     for (int t = TILE_FWD; t <= TILE_BWD; ++t)
-        if (t != (tc ? TILE_FWD : TILE_TC)) P->tile_ctas[t] = L.tile_occ(t, K, self);
+        for (int v = 2; v <= 3; ++v)
+            if (t != TILE_GROUPED && t != (tc ? TILE_FWD : TILE_TC)) P->tile_occ[t][v - 2] = L.tile_occ(t, v, K, self);
     cudaGetLastError();  // (a kernel that does not fit leaves its calls to the blocks)
+    const int fwd = tc ? TILE_TC : TILE_FWD;
+    auto widest = [&](tpcf_plan_s::Tune& t, int what) {
+        t.variant = P->occ(what, 3) > 0 ? 3 : 2;
+        t.ctas = std::max(1, P->occ(what, t.variant));
+    };
+    widest(P->tune_fwd, fwd);
+    widest(P->tune_bwd, TILE_BWD);
     P->nslots = (int)std::max<int64_t>(
-        P->fwd_grid, std::min<int64_t>(ntiles, (int64_t)P->num_sms * P->tile_ctas[tc ? TILE_TC : TILE_FWD]));
+        P->fwd_grid, std::min<int64_t>(ntiles, (int64_t)P->num_sms * std::max(P->occ(fwd, 2), P->occ(fwd, 3))));
     P->bin_share = 0.0;
     auto area = [&](int e) { return pow(sin(0.5 * P->edges[e]), 2); };
     for (int k = 0; k < K; ++k) P->bin_share = std::max(P->bin_share, (area(k + 1) - area(k)) / (area(K) - area(0)));
@@ -464,8 +466,9 @@ static void tile_range(const tpcf_plan_s* P, int64_t lo, int64_t hi, int64_t* tl
 // [orb_lo, orb_lo + norb) (map_block.cuh); returns the grid.  Warp tiles go four to a block (one
 // per warp), or two if that leaves fewer than four blocks per CTA of a full grid; a call with
 // fewer than three blocks per CTA splits each by bins, if the workspace has a slot for each block.
-static int block_shape(const tpcf_plan_s* P, const tpcf_plan_s::Tune& t, int cap, MapCall* c) {
-    const int64_t full = (int64_t)P->num_sms * std::min(2 * t.ctas, 4);  // (four CTAs of BT threads fit an SM)
+static int block_shape(const tpcf_plan_s* P, const tpcf_plan_s::Tune& t, int occ, int cap, MapCall* c) {
+    // four CTAs of BT threads fit an SM; of `occ` tiles the configuration launches t.ctas
+    const int64_t full = (int64_t)P->num_sms * std::max(1, std::min(4, (4 * t.ctas + occ - 1) / std::max(1, occ)));
     auto blocks = [&](int tiles) { return c->nlin + (c->norb + tiles - 1) / tiles; };
     c->tiles = BW;
     while (c->tiles > 2 && blocks(c->tiles) < 4 * full) c->tiles /= 2;
@@ -500,9 +503,9 @@ static int block_shape(const tpcf_plan_s* P, const tpcf_plan_s::Tune& t, int cap
 // above them 0.3 to 1.03 times (Nside 128, 8 bins: 283 against 555 us).
 constexpr double FILL_FWD = 4.5, FILL_MULTI = 4.0, FILL_TC = 5.0, FILL_BWD = 5.0, FILL_GROUPED = 6.0;
 
-static bool takes_blocks(const tpcf_plan_s* P, const MapCall& c, double need, int tile_ctas, double share = 1.0,
+static bool takes_blocks(const tpcf_plan_s* P, const MapCall& c, double need, int tile_occ, double share = 1.0,
                          double used = 1.0) {
-    if (tile_ctas < 1) return true;
+    if (tile_occ < 1) return true;
     if (P->route) return P->route == 2;
     // shared lists have no images to pair, so one dominant bin leaves the blocks no gain
     if (c.group > 1 && P->bin_share > 0.5) return false;
@@ -535,6 +538,18 @@ static void block_range(const tpcf_plan_s* P, int64_t lo, int64_t hi, MapCall* c
 // Ints of P->counter a launch needs zeroed: the work counter, and the blocks' finished parts.
 static int n_counters(const tpcf_plan_s* P, const MapCall& c) { return 4 + (c.parts > 1 ? P->ws_slots : 0); }
 
+namespace tpcf {
+// The kernels that a pass over the whole map takes (1 tiles, 2 blocks), for the autotuner (tune.cu).
+int map_route(const tpcf_plan_s* P, bool bwd) {
+    const int occ = P->occ(bwd ? TILE_BWD : TILE_FWD, 3);
+    const tpcf_plan_s::Tune t{3, occ, 8, 0};  // (not the plan's, which tuning changes)
+    MapCall c{};
+    block_range(P, 0, P->npoints, &c);
+    block_shape(P, t, occ, bwd ? P->bwd_grid : P->fwd_grid, &c);
+    return takes_blocks(P, c, bwd ? FILL_BWD : FILL_FWD, occ) ? 2 : 1;
+}
+}  // namespace tpcf
+
 // group > 1: shared neighbour lists over P->gtiles (tpcf_forward_grouped).
 static tpcf_status map_forward(tpcf_plan_s* P, const float* d_delta, const float* d_w, int64_t lo, int64_t hi,
                                double* d_zeta, double* d_norm, double* d_sums, cudaStream_t s, int group = 1) {
@@ -560,26 +575,27 @@ static tpcf_status map_forward(tpcf_plan_s* P, const float* d_delta, const float
     } else {
         block_range(P, lo, hi, &c);
     }
-    int grid = block_shape(P, P->tune_fwd, P->fwd_grid, &c);
+    const tpcf_plan_s::Tune& t = P->tune_fwd;
     const bool tc = (P->flags & TPCF_CONTRACT_TC) != 0;
-    const int what = group > 1 ? TILE_GROUPED : (tc ? TILE_TC : TILE_FWD), ctas = P->tile_ctas[what];
-    const bool blocks = takes_blocks(P, c, group > 1 ? FILL_GROUPED : (tc ? FILL_TC : FILL_FWD), ctas,
+    const int what = group > 1 ? TILE_GROUPED : (tc ? TILE_TC : TILE_FWD), occ = P->occ(tc ? TILE_TC : TILE_FWD, t.variant);
+    int grid = block_shape(P, t, occ, P->fwd_grid, &c);
+    const bool blocks = takes_blocks(P, c, group > 1 ? FILL_GROUPED : (tc ? FILL_TC : FILL_FWD), occ,
                                      group > 1 ? (double)(hi - lo) / g.npix : 1.0, group > 1 ? P->gused : 1.0);
     if (!blocks) {
-        c.flush = TILE_FLUSH;
         c.parts = 1;
         if (group > 1) {
             c.gtiles = P->gtiles + P->nglin;
             c.tile_hi = P->ngorb + P->ngtile;
         } else {
-            tile_range(P, lo, hi, &c.tile_lo, &c.tile_hi);
+            c.quad = t.quad;
+            tile_range(P, lo, hi, &c.tile_lo, &c.tile_hi, c.quad != 0);
         }
-        grid = tile_grid(P, c.tile_hi - c.tile_lo, ctas, P->nslots);
+        grid = tile_grid(P, c.tile_hi - c.tile_lo, t.ctas, P->nslots);
     }
     fwd_prep_kernel<<<P->num_sms * 8, 256, 0, s>>>(d_delta, d_w, P->wdw, g.npix, P->slots, (int64_t)grid * P->nent,
                                                    P->counter, n_counters(P, c));
     if (!blocks)
-        TRY_CUDA(kLaunch[P->M].tile(g, c, what, grid, s));
+        TRY_CUDA(kLaunch[P->M].tile(g, c, what, t.variant, grid, s));
     else if (tc)
         TRY_CUDA(kLaunch[P->M].fwd_tc(g, c, grid, s));
     else
@@ -713,12 +729,11 @@ extern "C" tpcf_status tpcf_forward_multi(tpcf_plan plan, const float* d_delta_a
     c.flush = P->tune_fwd.flush;
     c.cells = LIN_CELLS;
     block_range(P, pivot_begin, pivot_end, &c);
-    int grid = std::min(block_shape(P, P->tune_fwd, P->fwd_grid, &c), P->multi_grid);
+    int grid = std::min(block_shape(P, P->tune_fwd, P->occ(TILE_FWD, P->tune_fwd.variant), P->fwd_grid, &c), P->multi_grid);
     c.ws = P->ws3;
     c.ws_floats = 3 * P->ws_floats;
     const bool blocks = takes_blocks(P, c, FILL_MULTI, P->multi_ctas);
     if (!blocks) {
-        c.flush = TILE_FLUSH;
         c.parts = 1;
         tile_range(P, pivot_begin, pivot_end, &c.tile_lo, &c.tile_hi, true);
         grid = tile_grid(P, c.tile_hi - c.tile_lo, P->multi_ctas, P->multi_grid);
@@ -771,19 +786,19 @@ static tpcf_status map_backward(tpcf_plan_s* P, const float* d_delta, const floa
     c.flush = P->tune_bwd.flush;
     c.cells = LIN_CELLS;
     block_range(P, lo, hi, &c);
-    int grid = block_shape(P, P->tune_bwd, P->bwd_grid, &c);
-    const int ctas = P->tile_ctas[TILE_BWD];
-    const bool blocks = takes_blocks(P, c, FILL_BWD, ctas);
+    const tpcf_plan_s::Tune& t = P->tune_bwd;
+    const int occ = P->occ(TILE_BWD, t.variant);
+    int grid = block_shape(P, t, occ, P->bwd_grid, &c);
+    const bool blocks = takes_blocks(P, c, FILL_BWD, occ);
     if (!blocks) {
-        c.flush = TILE_FLUSH;
         c.parts = 1;
         tile_range(P, lo, hi, &c.tile_lo, &c.tile_hi);
-        grid = tile_grid(P, c.tile_hi - c.tile_lo, ctas, P->num_sms * ctas);
+        grid = tile_grid(P, c.tile_hi - c.tile_lo, t.ctas, P->num_sms * t.ctas);
     }
     bwd_prep_kernel<<<P->num_sms * 8, 256, 0, s>>>(d_delta, d_w, P->wdw, d_grad, g.npix, d_dL, d_norm, P->K, P->M, P->H,
                                                    self, P->counter, n_counters(P, c));
     if (!blocks) {
-        TRY_CUDA(kLaunch[P->M].tile(g, c, TILE_BWD, grid, s));
+        TRY_CUDA(kLaunch[P->M].tile(g, c, TILE_BWD, t.variant, grid, s));
         return TPCF_OK;
     }
     c.step = c.parts > 1 ? 1 : 0;

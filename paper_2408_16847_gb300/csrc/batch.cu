@@ -232,14 +232,14 @@ static tpcf_status batch_build(tpcf_batch_s* B, const tpcf_plan* plans, const fl
             it.c.H = P->H;
             it.c.grad = io[i].grad;
             it.c.self_subtract = io[i].self_subtract;
+            it.c.flush = P->tune_fwd.flush;
             it.tile0 = t0;
             if (G.tiles) {
-                it.c.flush = TILE_FLUSH;
+                it.c.quad = P->tune_fwd.quad;
                 t0 += P->map.ntiles;
                 items.push_back(it);
                 continue;
             }
-            it.c.flush = P->tune_fwd.flush;
             // the plan's linear blocks, then its other rings' warp tiles, two to a block
             it.c.cells = LIN_CELLS;
             it.c.lin_list = P->map.lin_list;

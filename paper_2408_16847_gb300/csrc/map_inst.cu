@@ -119,42 +119,57 @@ int TPCF_CAT(map_fwd_tc_occupancy_m, TPCF_M)(int K, int self_subtract) {
     return nb < 512 / TC_TMEM_COLS ? nb : 512 / TC_TMEM_COLS;
 }
 
-// The tile kernels (map_tile.cuh): launch, and resident CTAs per SM (either self-pair mode).
-cudaError_t TPCF_CAT(map_tile_launch_m, TPCF_M)(const MapDev& g, const MapCall& c, int what, int grid, cudaStream_t s) {
+// The tile kernels (map_tile.cuh): launch, and resident CTAs per SM; variant 3 or 2 = CTAs per SM
+// that the registers are sized for.
+template <int OCC>
+static cudaError_t tile_launch(const MapDev& g, const MapCall& c, int what, int grid, cudaStream_t s) {
     const bool self = c.self_subtract != 0;
     if (what == TILE_BWD) {
         const size_t smem = bwd_tile_floats_rt(g.K, TPCF_M) * sizeof(float);
-        return self ? launch(map_tile_bwd_kernel<TPCF_M, true>, smem, grid, g, c, s)
-                    : launch(map_tile_bwd_kernel<TPCF_M, false>, smem, grid, g, c, s);
-    }
-    if (what == TILE_TC) {
-        const size_t smem = tc_tile_bytes(g.K, TPCF_M, self);
-        return self ? launch(map_tile_tc_kernel<TPCF_M, true>, smem, grid, g, c, s)
-                    : launch(map_tile_tc_kernel<TPCF_M, false>, smem, grid, g, c, s);
+        return self ? launch(map_tile_bwd_kernel<TPCF_M, true, OCC>, smem, grid, g, c, s)
+                    : launch(map_tile_bwd_kernel<TPCF_M, false, OCC>, smem, grid, g, c, s);
     }
     const size_t smem = tile_floats_rt(g.K, TPCF_M) * sizeof(float);
+    return self ? launch(map_tile_fwd_kernel<TPCF_M, true, false, OCC>, smem, grid, g, c, s)
+                : launch(map_tile_fwd_kernel<TPCF_M, false, false, OCC>, smem, grid, g, c, s);
+}
+
+template <int OCC>
+static int tile_occupancy(int what, int K, bool self) {
+    if (what == TILE_BWD) {
+        const size_t smem = bwd_tile_floats_rt(K, TPCF_M) * sizeof(float);
+        return self ? occupancy(map_tile_bwd_kernel<TPCF_M, true, OCC>, smem)
+                    : occupancy(map_tile_bwd_kernel<TPCF_M, false, OCC>, smem);
+    }
+    const size_t smem = tile_floats_rt(K, TPCF_M) * sizeof(float);
+    return self ? occupancy(map_tile_fwd_kernel<TPCF_M, true, false, OCC>, smem)
+                : occupancy(map_tile_fwd_kernel<TPCF_M, false, false, OCC>, smem);
+}
+
+cudaError_t TPCF_CAT(map_tile_launch_m, TPCF_M)(const MapDev& g, const MapCall& c, int what, int variant, int grid,
+                                                cudaStream_t s) {
+    const bool self = c.self_subtract != 0;
+    const size_t smem = tile_floats_rt(g.K, TPCF_M) * sizeof(float);
+    if (what == TILE_TC) {
+        const size_t tcs = tc_tile_bytes(g.K, TPCF_M, self);
+        return self ? launch(map_tile_tc_kernel<TPCF_M, true>, tcs, grid, g, c, s)
+                    : launch(map_tile_tc_kernel<TPCF_M, false>, tcs, grid, g, c, s);
+    }
     if (what == TILE_GROUPED)  // (self pairs kept)
         return launch(map_tile_fwd_kernel<TPCF_M, false, false, 3, true>, smem, grid, g, c, s);
     if (what == TILE_DIRECT)  // the caller's delta and w, no packed copy
         return launch(map_tile_fwd_kernel<TPCF_M, false, true>, smem, grid, g, c, s);
-    return self ? launch(map_tile_fwd_kernel<TPCF_M, true, false>, smem, grid, g, c, s)
-                : launch(map_tile_fwd_kernel<TPCF_M, false, false>, smem, grid, g, c, s);
+    return variant == 2 ? tile_launch<2>(g, c, what, grid, s) : tile_launch<3>(g, c, what, grid, s);
 }
 
-int TPCF_CAT(map_tile_occupancy_m, TPCF_M)(int what, int K, int self) {
-    if (what == TILE_BWD) {
-        const size_t smem = bwd_tile_floats_rt(K, TPCF_M) * sizeof(float);
-        return self ? occupancy(map_tile_bwd_kernel<TPCF_M, true>, smem) : occupancy(map_tile_bwd_kernel<TPCF_M, false>, smem);
-    }
+int TPCF_CAT(map_tile_occupancy_m, TPCF_M)(int what, int variant, int K, int self) {
     if (what == TILE_TC) {
         const size_t smem = tc_tile_bytes(K, TPCF_M, self != 0);
         const int nb = self ? occupancy_by_resources(map_tile_tc_kernel<TPCF_M, true>, smem, NTHREADS)
                             : occupancy_by_resources(map_tile_tc_kernel<TPCF_M, false>, smem, NTHREADS);
         return nb < 512 / TC_TMEM_COLS ? nb : 512 / TC_TMEM_COLS;
     }
-    const size_t smem = tile_floats_rt(K, TPCF_M) * sizeof(float);
-    return self ? occupancy(map_tile_fwd_kernel<TPCF_M, true, false>, smem)
-                : occupancy(map_tile_fwd_kernel<TPCF_M, false, false>, smem);
+    return variant == 2 ? tile_occupancy<2>(what, K, self != 0) : tile_occupancy<3>(what, K, self != 0);
 }
 
 cudaError_t TPCF_CAT(map_tile_multi_launch_m, TPCF_M)(const MapDev& g, const MapCall& c, const float2* wdwB,

@@ -29,13 +29,13 @@
 
 namespace tpcf {
 
-#define TPCF_DECL_TILE(m) cudaError_t map_tile_launch_m##m(const MapDev&, const MapCall&, int, int, cudaStream_t);
+#define TPCF_DECL_TILE(m) cudaError_t map_tile_launch_m##m(const MapDev&, const MapCall&, int, int, int, cudaStream_t);
 TPCF_DECL_TILE(0) TPCF_DECL_TILE(1) TPCF_DECL_TILE(2) TPCF_DECL_TILE(3) TPCF_DECL_TILE(4) TPCF_DECL_TILE(5)
 TPCF_DECL_TILE(6) TPCF_DECL_TILE(7) TPCF_DECL_TILE(8) TPCF_DECL_TILE(9) TPCF_DECL_TILE(10) TPCF_DECL_TILE(11)
 TPCF_DECL_TILE(12) TPCF_DECL_TILE(13) TPCF_DECL_TILE(14) TPCF_DECL_TILE(15) TPCF_DECL_TILE(16)
 #undef TPCF_DECL_TILE
 
-typedef cudaError_t (*tile_fn)(const MapDev&, const MapCall&, int, int, cudaStream_t);
+typedef cudaError_t (*tile_fn)(const MapDev&, const MapCall&, int, int, int, cudaStream_t);
 static const tile_fn kTile[TPCF_MAX_M + 1] = {
     map_tile_launch_m0,  map_tile_launch_m1,  map_tile_launch_m2,  map_tile_launch_m3,  map_tile_launch_m4,
     map_tile_launch_m5,  map_tile_launch_m6,  map_tile_launch_m7,  map_tile_launch_m8,  map_tile_launch_m9,
@@ -121,7 +121,7 @@ extern "C" tpcf_status tpcf_forward_noalloc(tpcf_plan plan, const float* d_delta
     double* sums = (double*)(base + NOALLOC_HEADER);
     double* slots = (double*)(base + NOALLOC_HEADER + sums_bytes);
     const size_t room = (NOALLOC_SCRATCH_BYTES - NOALLOC_HEADER - sums_bytes) / slot_bytes;
-    const int64_t ctas = std::min<int64_t>(plan->map.ntiles, (int64_t)plan->num_sms * std::max(1, plan->tile_ctas[TILE_FWD]));
+    const int64_t ctas = std::min<int64_t>(plan->map.ntiles, (int64_t)plan->num_sms * std::max(1, plan->occ(TILE_FWD, 3)));
     const int grid = (int)std::min<size_t>((size_t)ctas, room);
     cudaStream_t s = (cudaStream_t)stream;
     plan->last_stream = s;
@@ -137,10 +137,11 @@ extern "C" tpcf_status tpcf_forward_noalloc(tpcf_plan plan, const float* d_delta
     c.status = plan->status;
     c.self_subtract = 0;
     c.norm = norm_of_flags(plan->flags);
-    c.flush = TILE_FLUSH;
+    c.flush = plan->tune_fwd.flush;
+    c.quad = plan->tune_fwd.quad;
     c.tile_lo = 0;  // every tile; those without a pivot in range return at once
     c.tile_hi = plan->map.ntiles;
-    TRY_CUDA(kTile[plan->M](plan->map, c, TILE_DIRECT, grid, s));
+    TRY_CUDA(kTile[plan->M](plan->map, c, TILE_DIRECT, 3, grid, s));
     reduce_slots_kernel<<<(plan->nent + 31) / 32, REDUCE_THREADS, 0, s>>>(slots, grid, plan->nent, sums);
     const int nout = (plan->M + 1) * plan->K * plan->K;
     finalize_kernel<<<(nout + 127) / 128, 128, 0, s>>>(sums, plan->K, plan->M, 0, 1.0, d_zeta, d_norm, nullptr);

@@ -47,18 +47,19 @@ struct tpcf_plan_s {
     float* ws = nullptr;  // workspace of the block kernels: ws_slots blocks of ws_floats
     int ws_slots = 0;
     size_t ws_floats = 0;
-    // launch configuration of the map pair kernels (defaults, or picked by the autotuner): pairs of
-    // CTAs per SM launched, and the entries summed in registers before they are added to the
-    // workspace, in units of 32; the register variant (3 or 2, one kernel serves both)
-    // and, for the forward, a tile-layout choice that is kept for callers that store configurations
-    // (the layout follows from the ring, map_block.cuh)
+    // launch configuration of the map pair kernels (defaults, or picked by the autotuner).  Tile
+    // kernels: register variant (sized for 3 or 2 CTAs per SM), CTAs per SM launched, rings summed in
+    // registers before a shared-memory flush, and for the forward the tile layout (1: quarter-turn
+    // runs).  Block kernels: the same share of their own CTAs, and the flush in units of 32 entries.
     struct Tune {
-        int variant = 2, ctas = 0, flush = 8, quad = 0;
+        int variant = 3, ctas = 0, flush = 8, quad = 0;
     } tune_fwd, tune_bwd;
     bool tuned = false;
-    // tile kernels of the map pair passes (map_tile.cuh): CTAs per SM by TileKernel; the largest share of
-    // the bins' area in one bin, and whether the rule of takes_blocks is overridden (1 tiles, 2 blocks)
-    int tile_ctas[4] = {0, 0, 0, 0};
+    // tile kernels of the map pair passes (map_tile.cuh): resident CTAs per SM by TileKernel and register
+    // variant (2, 3); the largest share of the bins' area in one bin, and whether the rule of
+    // takes_blocks is overridden (1 tiles, 2 blocks)
+    int tile_occ[4][2] = {};
+    int occ(int what, int variant) const { return tile_occ[what][variant - 2]; }
     double bin_share = 1.0;
     int route = 0;
     // per-call scratch

@@ -135,7 +135,6 @@ inline __host__ __device__ int n_entries_multi(int K, int M) { return 2 * (M + 1
 
 // The tile kernels (map_tile.cuh) that a call can take.
 enum TileKernel { TILE_FWD, TILE_GROUPED, TILE_TC, TILE_BWD, TILE_DIRECT };
-constexpr int TILE_FLUSH = 8;  // rings that a tile's registers sum
 constexpr int ROW = 512;  // floats per warp row buffer of the tile adjoint (wider rows: whole-ring or global adds)
 // Shared memory (floats) of a forward tile with runtime m_max mr: moments A[k][m][re/im][32],
 // W, Q, QW [k][32], the pivots' (w d, w).

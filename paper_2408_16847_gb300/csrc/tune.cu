@@ -1,11 +1,14 @@
 // Launch-configuration autotuner of the map pair kernels.
 //
-// The search space, per pass (forward, adjoint):
-//   * pairs of CTAs per SM launched: what the kernel's occupancy gives, or one fewer;
-//   * entries summed in registers before they are added to the workspace, in units of 32:
-//     4, 8, 16 or 32.
-// A stored configuration also names a register variant and a tile layout; one kernel
-// serves every value of both (map_block.cuh).
+// The search space, per pass (forward, adjoint), for the kernels that the pass takes over the
+// whole map (takes_blocks in api.cu).  Tile kernels:
+//   * register variant: compiled for 3 resident CTAs per SM (80 registers per thread, a few
+//     spills at large m_max) or for 2 (128 registers, none);
+//   * CTAs per SM launched: the variant's occupancy or one fewer;
+//   * rings summed in registers before a shared-memory flush: 4, 8, 16 or 32;
+//   * the forward's tile layout, at the best of these.
+// Block kernels: the share of their CTAs launched (by the same CTA count) and the entries summed in
+// registers before they go to the workspace, in units of 32: 4, 8, 16 or 32.
 // Each candidate runs the pass on a sample of pivots (slices at three latitudes, about
 // 0.5% of a large map, the whole map when it is small), once to warm up and then twice
 // timed with CUDA events; the fastest is kept in the plan.  Results are cached in the
@@ -25,8 +28,7 @@
 using namespace tpcf;
 
 namespace tpcf {
-int map_fwd_occupancy(int M);
-int map_bwd_occupancy(int M);
+int map_route(const tpcf_plan_s* P, bool bwd);
 
 static std::string tune_key(const tpcf_plan_s* P) {
     cudaDeviceProp prop;
@@ -44,7 +46,10 @@ static std::string tune_key(const tpcf_plan_s* P) {
     std::string name(prop.name);
     for (char& c : name)
         if (c == ' ') c = '_';
-    snprintf(buf, sizeof(buf), "v3 dev=%s sms=%d map nside=%d K=%d M=%d flags=%u edges=%016llx", name.c_str(),
+    // v2: configurations of the tile kernels, also those stored before there were blocks; v4: where a
+    // pass takes blocks (v3 had other meanings)
+    const int ver = map_route(P, false) == 1 && map_route(P, true) == 1 ? 2 : 4;
+    snprintf(buf, sizeof(buf), "v%d dev=%s sms=%d map nside=%d K=%d M=%d flags=%u edges=%016llx", ver, name.c_str(),
              P->num_sms, P->map.nside, P->K, P->M, P->flags, h);
     return buf;
 }
@@ -85,10 +90,7 @@ static void cache_store(const std::string& key, const tpcf_plan_s::Tune& f, cons
 static bool valid(const tpcf_plan_s* P, const tpcf_plan_s::Tune& t, bool bwd) {
     if (t.variant != 2 && t.variant != 3) return false;
     if (t.flush < 1 || t.flush > 64 || t.ctas < 1 || t.quad < 0 || t.quad > 1) return false;
-    // callers may name as many CTAs per SM as their variant stands for; the launch is cut to what
-    // fits (block_shape)
-    const int occ = bwd ? map_bwd_occupancy(P->M) : map_fwd_occupancy(P->M);
-    return t.ctas <= std::max(t.variant, (occ + 1) / 2);
+    return t.ctas <= P->occ(bwd ? TILE_BWD : TILE_FWD, t.variant);
 }
 
 // Applies a cached configuration to a new map plan (called at plan creation).
@@ -205,15 +207,27 @@ extern "C" tpcf_status tpcf_plan_autotune(tpcf_plan plan, const float* d_delta, 
                 best = T;
             }
         };
-        const int occ = ((bwd ? map_bwd_occupancy(M) : map_fwd_occupancy(M)) + 1) / 2;  // pairs
-        for (int ctas = occ; ctas >= std::max(1, occ - 1) && st == TPCF_OK; --ctas) {
-            const int flushes[4] = {4, 8, 16, 32};
-            for (int fi = 0; fi < 4 && st == TPCF_OK; ++fi) {
-                T.ctas = ctas;
-                T.flush = flushes[fi];
-                try_config();
+        const int what = bwd ? TILE_BWD : TILE_FWD;
+        const int route = P->route, tuned = map_route(P, bwd);
+        P->route = tuned;  // the sample's calls are shorter, but take the whole map's kernels
+        for (int variant = 3; variant >= (tuned == 1 ? 2 : 3) && st == TPCF_OK; --variant) {
+            const int occ = P->occ(what, variant);
+            for (int ctas = occ; ctas >= std::max(1, occ - 1) && st == TPCF_OK; --ctas) {
+                const int flushes[4] = {4, 8, 16, 32};
+                for (int fi = 0; fi < 4 && st == TPCF_OK; ++fi) {
+                    T.variant = variant;
+                    T.ctas = ctas;
+                    T.flush = flushes[fi];
+                    try_config();
+                }
             }
         }
+        if (!bwd && tuned == 1 && st == TPCF_OK) {  // the forward's tile layout, at the best shape
+            T = best;
+            T.quad = 1 - best.quad;
+            try_config();
+        }
+        P->route = route;
         T = st == TPCF_OK ? best : keep;
     }
     if (e0) cudaEventDestroy(e0);
