@@ -105,6 +105,14 @@ const char* tpcf_last_error(void);
  * section 3.3).  Builds, on the device and on `stream`, the ring geometry in FP64
  * and the per-ring-pair bin thresholds used by the exact ring-range neighbour
  * search.  On failure *out is left NULL and nothing is leaked.
+ *
+ * The plan holds its tables, 8 bytes per pixel and 8 bytes per sum and CTA (18 MB at 20 bins
+ * and m_max 10).  Large calls of map plans, and calls of catalogue plans, also take a
+ * workspace for the time they run (0.3 GB at 20 bins and m_max 10, three times that for three
+ * fields; 1 GB at most where a call has to hold all its pivots at once) from a pool that the
+ * device's plans share, in stream order: calls on other streams get memory of their own,
+ * at most 1 GB stays in the pool between calls, and it is freed with the last plan.  A call
+ * that is being captured into a graph uses a workspace that the plan allocates and keeps.
  */
 tpcf_status tpcf_plan_create_map(tpcf_plan* out, int64_t nside, const tpcf_bins* bins, void* stream);
 

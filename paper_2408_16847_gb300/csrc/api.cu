@@ -7,6 +7,7 @@
 #include <string.h>
 
 #include <atomic>
+#include <mutex>
 #include <new>
 #include <vector>
 
@@ -102,16 +103,17 @@ static std::atomic<long long> g_live_allocs{0};
 static std::atomic<long long> g_fail_countdown{0};
 
 namespace tpcf {
-cudaError_t dev_malloc(void** p, size_t bytes) {
+static bool injected_failure() {
     long long c = g_fail_countdown.load();
-    while (c > 0) {
-        if (g_fail_countdown.compare_exchange_weak(c, c - 1)) {
-            if (c == 1) {
-                *p = nullptr;
-                return cudaErrorMemoryAllocation;
-            }
-            break;
-        }
+    while (c > 0)
+        if (g_fail_countdown.compare_exchange_weak(c, c - 1)) return c == 1;
+    return false;
+}
+
+cudaError_t dev_malloc(void** p, size_t bytes) {
+    if (injected_failure()) {
+        *p = nullptr;
+        return cudaErrorMemoryAllocation;
     }
     cudaError_t e = cudaMalloc(p, bytes);
     if (e == cudaSuccess) ++g_live_allocs;
@@ -122,7 +124,93 @@ void dev_free(void* p) {
     cudaFree(p);
     --g_live_allocs;
 }
+
+// Workspaces of the block and catalogue kernels (up to 0.5 MB per CTA at 20 bins and m_max 10, 0.3 GB
+// in all).  A call takes one for the time its kernels run, from a pool per device that all plans
+// share: allocated and freed in stream order, so calls on other streams get memory of their own.
+// The pool keeps POOL_BYTES when idle and goes with the device's last plan.  A call that is being
+// captured into a graph, which may be replayed on any stream, uses memory that its plan keeps.
+// (With a workspace in every plan, 64 plans at 20 bins held 36 GB that only one call at a time used.)
+constexpr uint64_t POOL_BYTES = uint64_t(1) << 30;
+constexpr int POOL_DEVICES = 64;
+static std::mutex g_pool_mu;
+static cudaMemPool_t g_pool[POOL_DEVICES];
+static int g_pool_plans[POOL_DEVICES];
+
+static cudaError_t ws_pool(int dev, cudaMemPool_t* out) {
+    std::lock_guard<std::mutex> lock(g_pool_mu);
+    if (!g_pool[dev]) {
+        cudaMemPoolProps pr;
+        memset(&pr, 0, sizeof(pr));
+        pr.allocType = cudaMemAllocationTypePinned;
+        pr.location.type = cudaMemLocationTypeDevice;
+        pr.location.id = dev;
+        cudaMemPool_t pool = nullptr;
+        cudaError_t e = cudaMemPoolCreate(&pool, &pr);
+        if (e != cudaSuccess) return e;
+        uint64_t keep = POOL_BYTES;
+        int off = 0;
+        e = cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
+        // (otherwise a stream's call could be made to wait for another stream's)
+        if (e == cudaSuccess) e = cudaMemPoolSetAttribute(pool, cudaMemPoolReuseAllowInternalDependencies, &off);
+        if (e != cudaSuccess) {
+            cudaMemPoolDestroy(pool);
+            return e;
+        }
+        g_pool[dev] = pool;
+    }
+    *out = g_pool[dev];
+    return cudaSuccess;
+}
+
+void ws_count(tpcf_plan_s* P) {
+    if (P->device < 0 || P->device >= POOL_DEVICES) return;
+    std::lock_guard<std::mutex> lock(g_pool_mu);
+    ++g_pool_plans[P->device];
+    P->counted = true;
+}
+
+cudaError_t ws_take(tpcf_plan_s* P, size_t floats, cudaStream_t s, WsLease* w) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    cudaError_t e = cudaStreamIsCapturing(s, &cap);
+    if (e != cudaSuccess) return e;
+    if (cap == cudaStreamCaptureStatusNone && P->counted) {
+        cudaMemPool_t pool;
+        e = ws_pool(P->device, &pool);
+        if (e != cudaSuccess) return e;
+        if (injected_failure()) return cudaErrorMemoryAllocation;
+        void* q = nullptr;
+        e = cudaMallocFromPoolAsync(&q, floats * sizeof(float), pool, s);
+        if (e != cudaSuccess) return e;
+        w->p = (float*)q;
+        w->s = s;
+        w->pooled = true;
+        return cudaSuccess;
+    }
+    if (P->ws_graph_floats < floats) {  // (an earlier, smaller one stays: a graph may hold it)
+        cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;  // a plain allocation is no part of the graph
+        cudaThreadExchangeStreamCaptureMode(&mode);
+        float* q = nullptr;
+        e = P->alloc(&q, floats);
+        cudaThreadExchangeStreamCaptureMode(&mode);
+        if (e != cudaSuccess) return e;
+        P->ws_graph = q;
+        P->ws_graph_floats = floats;
+    }
+    w->p = P->ws_graph;
+    return cudaSuccess;
+}
 }  // namespace tpcf
+
+tpcf_plan_s::~tpcf_plan_s() {
+    for (void* p : allocs) tpcf::dev_free(p);
+    if (!counted) return;
+    std::lock_guard<std::mutex> lock(tpcf::g_pool_mu);
+    if (--tpcf::g_pool_plans[device] == 0 && tpcf::g_pool[device]) {
+        cudaMemPoolDestroy(tpcf::g_pool[device]);
+        tpcf::g_pool[device] = nullptr;
+    }
+}
 
 extern "C" void tpcf_test_fail_allocation(int64_t n) { g_fail_countdown.store(n > 0 ? n : 0); }
 
@@ -309,11 +397,9 @@ static tpcf_status build_map(tpcf_plan_s* P, int64_t nside, cudaStream_t s) {
     // slots for the largest grid any configuration launches
     P->fwd_grid = P->num_sms * ((occ_f + 1) / 2 * 2);
     P->bwd_grid = P->num_sms * ((occ_b + 1) / 2 * 2);
-    // workspace: a block per CTA, or (calls with few blocks) one per block, see block_shape
-    P->ws_slots = (int)std::max<int64_t>(1, std::min<int64_t>(2 * std::max(P->fwd_grid, P->bwd_grid), nlin + norb));
-    P->fwd_grid = (int)std::min<int64_t>(P->fwd_grid, 8 * (int64_t)P->ws_slots);
+    P->max_blocks = (int)std::max<int64_t>(1, std::min<int64_t>(2 * std::max(P->fwd_grid, P->bwd_grid), nlin + norb));
+    P->fwd_grid = (int)std::min<int64_t>(P->fwd_grid, 8 * (int64_t)P->max_blocks);
     P->ws_floats = block_floats(K, P->M, P->M, self != 0);
-    TRY_CUDA(P->alloc(&P->ws, P->ws_floats * P->ws_slots));
     for (int t = TILE_FWD; t <= TILE_BWD; ++t)
         for (int v = 2; v <= 3; ++v)
             if (t != TILE_GROUPED && t != (tc ? TILE_FWD : TILE_TC)) P->tile_occ[t][v - 2] = L.tile_occ(t, v, K, self);
@@ -326,7 +412,7 @@ static tpcf_status build_map(tpcf_plan_s* P, int64_t nside, cudaStream_t s) {
     widest(P->tune_fwd, fwd);
     widest(P->tune_bwd, TILE_BWD);
     P->nslots = (int)std::max<int64_t>(
-        P->fwd_grid, std::min<int64_t>(ntiles, (int64_t)P->num_sms * std::max(P->occ(fwd, 2), P->occ(fwd, 3))));
+        1, std::min<int64_t>(ntiles, (int64_t)P->num_sms * std::max(P->occ(fwd, 2), P->occ(fwd, 3))));
     P->bin_share = 0.0;
     auto area = [&](int e) { return pow(sin(0.5 * P->edges[e]), 2); };
     for (int k = 0; k < K; ++k) P->bin_share = std::max(P->bin_share, (area(k + 1) - area(k)) / (area(K) - area(0)));
@@ -334,10 +420,10 @@ static tpcf_status build_map(tpcf_plan_s* P, int64_t nside, cudaStream_t s) {
     TRY_CUDA(P->alloc(&P->wdw, g.npix + 1));  // and a zero after the last pixel
     TRY_CUDA(P->alloc(&P->slots, (size_t)P->nslots * P->nent));
     scratch.add(&P->sums, P->nent);
-    scratch.add(&P->counter, 4 + P->ws_slots);  // work counter (4 words), then finished parts per block
     scratch.add(&P->status, 4);
     scratch.add(&P->H, (size_t)(P->M + 1) * K * K * 2 + K);  // H, then cdiag (self-pair mode)
     TRY_CUDA(scratch.take(P));
+    TRY_CUDA(P->alloc(&P->counter, 4 + P->max_blocks));  // work counter (4 words), then finished parts per block
     TRY_CUDA(cudaMemsetAsync(P->status, 0, sizeof(int) * 4, s));
     TRY_CUDA(cudaStreamSynchronize(s));
     return TPCF_OK;
@@ -371,6 +457,7 @@ extern "C" tpcf_status tpcf_plan_create_map(tpcf_plan* out, int64_t nside, const
         delete P;
         return st;
     }
+    ws_count(P);
     tune_from_cache(P);
     // place tpcf_forward_noalloc's fixed scratch on this device now, during set-up;
     // on failure that call reports it, so clear the runtime's last-error state here
@@ -413,6 +500,7 @@ extern "C" tpcf_status tpcf_plan_create_catalog(tpcf_plan* out, const double* d_
         delete P;
         return st;
     }
+    ws_count(P);
     P->last_stream = s;
     *out = P;
     return TPCF_OK;
@@ -462,11 +550,14 @@ static void tile_range(const tpcf_plan_s* P, int64_t lo, int64_t hi, int64_t* tl
     *thi = P->tile_off_h[rb] + (hi - 1 - ring_first_pixel(nside, rb)) / TILE + 1;
 }
 
-// Blocks, parts and workspace of a forward over lin_list [lin_lo, lin_lo + nlin) and orb_list
-// [orb_lo, orb_lo + norb) (map_block.cuh); returns the grid.  Warp tiles go four to a block (one
+// Blocks and parts of a pass over lin_list [lin_lo, lin_lo + nlin) and orb_list [orb_lo, orb_lo + norb)
+// (map_block.cuh) for `fields` fields; returns the grid.  Warp tiles go four to a block (one
 // per warp), or two if that leaves fewer than four blocks per CTA of a full grid; a call with
-// fewer than three blocks per CTA splits each by bins, if the workspace has a slot for each block.
-static int block_shape(const tpcf_plan_s* P, const tpcf_plan_s::Tune& t, int occ, int cap, MapCall* c) {
+// fewer than three blocks per CTA splits each by bins.  The workspace then holds every block
+// at once: not beyond WS_PARTS bytes (1216 blocks at 20 bins and m_max 10 take 0.57 GB).
+constexpr double WS_PARTS = 1 << 30;
+
+static int block_shape(const tpcf_plan_s* P, const tpcf_plan_s::Tune& t, int occ, int cap, MapCall* c, int fields = 1) {
     // four CTAs of BT threads fit an SM; of `occ` tiles the configuration launches t.ctas
     const int64_t full = (int64_t)P->num_sms * std::max(1, std::min(4, (4 * t.ctas + occ - 1) / std::max(1, occ)));
     auto blocks = [&](int tiles) { return c->nlin + (c->norb + tiles - 1) / tiles; };
@@ -477,16 +568,25 @@ static int block_shape(const tpcf_plan_s* P, const tpcf_plan_s::Tune& t, int occ
         c->tiles = 1;
         c->slices = 4;
     }
+    c->ws_floats = fields * P->ws_floats;
     const int64_t n = blocks(c->tiles);
     c->parts = 1;
-    if (n < 3 * full && n <= P->ws_slots && n > 0)
+    if (n < 3 * full && n <= P->max_blocks && n > 0 && (double)n * c->ws_floats * sizeof(float) <= WS_PARTS)
         c->parts = (int)std::min<int64_t>(std::min(8, P->K), (4 * full + n - 1) / n);
-    c->ws = P->ws;
-    c->ws_floats = P->ws_floats;
     c->done = P->counter + 4;
-    int64_t grid = std::min<int64_t>(std::min<int64_t>(n * c->parts, full), cap);
-    if (c->parts == 1) grid = std::min<int64_t>(grid, P->ws_slots);
-    return (int)std::max<int64_t>(1, grid);
+    return (int)std::max<int64_t>(1, std::min<int64_t>(std::min<int64_t>(n * c->parts, full), cap));
+}
+
+// Takes the workspace of a pass by blocks and sets it in the call: `nent` sums per CTA (a forward's
+// slots), then a block per CTA, or one per block where blocks are split.
+static cudaError_t blocks_ws(tpcf_plan_s* P, MapCall* c, int grid, int nent, cudaStream_t s, WsLease* w) {
+    const int64_t blocks = c->parts > 1 ? c->nlin + (c->norb + c->tiles - 1) / c->tiles : grid;
+    const size_t slots = ((size_t)grid * nent * 2 + 63) / 64 * 64;  // floats
+    cudaError_t e = ws_take(P, slots + c->ws_floats * (size_t)blocks, s, w);
+    if (e != cudaSuccess) return e;
+    if (nent) c->slots = reinterpret_cast<double*>(w->p);
+    c->ws = w->p + slots;
+    return cudaSuccess;
 }
 
 // Whether a call goes to the block kernels (map_block.cuh) or to the tile kernels (map_tile.cuh), from
@@ -536,7 +636,7 @@ static void block_range(const tpcf_plan_s* P, int64_t lo, int64_t hi, MapCall* c
 }
 
 // Ints of P->counter a launch needs zeroed: the work counter, and the blocks' finished parts.
-static int n_counters(const tpcf_plan_s* P, const MapCall& c) { return 4 + (c.parts > 1 ? P->ws_slots : 0); }
+static int n_counters(const tpcf_plan_s* P, const MapCall& c) { return 4 + (c.parts > 1 ? P->max_blocks : 0); }
 
 namespace tpcf {
 // The kernels that a pass over the whole map takes (1 tiles, 2 blocks), for the autotuner (tune.cu).
@@ -592,7 +692,9 @@ static tpcf_status map_forward(tpcf_plan_s* P, const float* d_delta, const float
         }
         grid = tile_grid(P, c.tile_hi - c.tile_lo, t.ctas, P->nslots);
     }
-    fwd_prep_kernel<<<P->num_sms * 8, 256, 0, s>>>(d_delta, d_w, P->wdw, g.npix, P->slots, (int64_t)grid * P->nent,
+    WsLease ws;
+    if (blocks) TRY_CUDA(blocks_ws(P, &c, grid, P->nent, s, &ws));
+    fwd_prep_kernel<<<P->num_sms * 8, 256, 0, s>>>(d_delta, d_w, P->wdw, g.npix, c.slots, (int64_t)grid * P->nent,
                                                    P->counter, n_counters(P, c));
     if (!blocks)
         TRY_CUDA(kLaunch[P->M].tile(g, c, what, t.variant, grid, s));
@@ -600,7 +702,7 @@ static tpcf_status map_forward(tpcf_plan_s* P, const float* d_delta, const float
         TRY_CUDA(kLaunch[P->M].fwd_tc(g, c, grid, s));
     else
         TRY_CUDA(kLaunch[P->M].fwd(g, c, grid, s));
-    reduce_slots_kernel<<<n_blocks(P->nent, 32), REDUCE_THREADS, 0, s>>>(P->slots, grid, P->nent, P->sums);
+    reduce_slots_kernel<<<n_blocks(P->nent, 32), REDUCE_THREADS, 0, s>>>(c.slots, grid, P->nent, P->sums);
     const int nout = (P->M + 1) * P->K * P->K;
     finalize_kernel<<<n_blocks(nout, 128), 128, 0, s>>>(P->sums, P->K, P->M, c.self_subtract, 1.0, d_zeta,
                                                         d_norm, d_sums);
@@ -701,16 +803,13 @@ extern "C" tpcf_status tpcf_forward_multi(tpcf_plan plan, const float* d_delta_a
             return TPCF_ERR_UNSUPPORTED;
         }
         P->multi_ctas = kMulti[M].tiles_occ(K);
-        const int grid = P->num_sms * std::max(kMulti[M].blocks_occ(), P->multi_ctas);
+        const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(g.ntiles, (int64_t)P->num_sms * P->multi_ctas));
         float2 *b, *c;
         double *sl, *su;
         TRY_CUDA(P->alloc(&b, g.npix + 1));
         TRY_CUDA(P->alloc(&c, g.npix + 1));
         TRY_CUDA(P->alloc(&sl, (size_t)grid * nent));
         TRY_CUDA(P->alloc(&su, (size_t)nent));
-        float* w3;
-        TRY_CUDA(P->alloc(&w3, 3 * P->ws_floats * P->ws_slots));
-        P->ws3 = w3;
         P->wdw_c = c;
         P->mslots = sl;
         P->msums = su;
@@ -729,19 +828,19 @@ extern "C" tpcf_status tpcf_forward_multi(tpcf_plan plan, const float* d_delta_a
     c.flush = P->tune_fwd.flush;
     c.cells = LIN_CELLS;
     block_range(P, pivot_begin, pivot_end, &c);
-    int grid = std::min(block_shape(P, P->tune_fwd, P->occ(TILE_FWD, P->tune_fwd.variant), P->fwd_grid, &c), P->multi_grid);
-    c.ws = P->ws3;
-    c.ws_floats = 3 * P->ws_floats;
+    int grid = block_shape(P, P->tune_fwd, P->occ(TILE_FWD, P->tune_fwd.variant), P->fwd_grid, &c, 3);
     const bool blocks = takes_blocks(P, c, FILL_MULTI, P->multi_ctas);
     if (!blocks) {
         c.parts = 1;
         tile_range(P, pivot_begin, pivot_end, &c.tile_lo, &c.tile_hi, true);
         grid = tile_grid(P, c.tile_hi - c.tile_lo, P->multi_ctas, P->multi_grid);
     }
-    fwd_prep_kernel<<<P->num_sms * 8, 256, 0, s>>>(d_delta_a, d_w_a, P->wdw, g.npix, P->mslots, (int64_t)grid * nent,
+    WsLease ws;
+    if (blocks) TRY_CUDA(blocks_ws(P, &c, grid, nent, s, &ws));
+    fwd_prep_kernel<<<P->num_sms * 8, 256, 0, s>>>(d_delta_a, d_w_a, P->wdw, g.npix, c.slots, (int64_t)grid * nent,
                                                    P->counter, n_counters(P, c));
     TRY_CUDA((blocks ? kMulti[M].blocks : kMulti[M].tiles)(g, c, P->wdw_b, P->wdw_c, grid, s));
-    reduce_slots_kernel<<<n_blocks(nent, 32), REDUCE_THREADS, 0, s>>>(P->mslots, grid, nent, P->msums);
+    reduce_slots_kernel<<<n_blocks(nent, 32), REDUCE_THREADS, 0, s>>>(c.slots, grid, nent, P->msums);
     const int nout = (M + 1) * K * K;
     finalize_full_kernel<<<n_blocks(nout, 128), 128, 0, s>>>(P->msums, K, M, d_zeta, d_norm, d_sums);
     P->launches += 6;  // prep and two packs, the pair kernel, reduce, finalize
@@ -795,6 +894,8 @@ static tpcf_status map_backward(tpcf_plan_s* P, const float* d_delta, const floa
         tile_range(P, lo, hi, &c.tile_lo, &c.tile_hi);
         grid = tile_grid(P, c.tile_hi - c.tile_lo, t.ctas, P->num_sms * t.ctas);
     }
+    WsLease ws;
+    if (blocks) TRY_CUDA(blocks_ws(P, &c, grid, 0, s, &ws));
     bwd_prep_kernel<<<P->num_sms * 8, 256, 0, s>>>(d_delta, d_w, P->wdw, d_grad, g.npix, d_dL, d_norm, P->K, P->M, P->H,
                                                    self, P->counter, n_counters(P, c));
     if (!blocks) {

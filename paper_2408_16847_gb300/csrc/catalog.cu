@@ -342,8 +342,6 @@ tpcf_status build_catalog(tpcf_plan_s* P, const double* d_xyz, int64_t n, cudaSt
     P->bwd_grid = occ_b < 1 ? 0 : (int)std::max<int64_t>(1, std::min<int64_t>(g.ntiles, (int64_t)P->num_sms * occ_b));
     TRY_CUDA(P->alloc(&P->H, (size_t)(P->M + 1) * K * K * 2 + K));
     P->ws_floats = cat_slices(K) * sub_floats_rt(K, P->M, self != 0);
-    P->ws_slots = std::max(P->fwd_grid, P->bwd_grid);
-    TRY_CUDA(P->alloc(&P->ws, P->ws_floats * P->ws_slots));
     P->nent = n_entries(K, P->M);
     TRY_CUDA(P->alloc(&P->wdw, n));
     TRY_CUDA(P->alloc(&P->slots, (size_t)P->fwd_grid * P->nent));
@@ -397,8 +395,10 @@ tpcf_status catalog_backward(tpcf_plan_s* P, const float* d_delta, const float* 
     c.status = P->status;
     c.H = P->H;
     c.grad = d_grad;
-    c.ws = P->ws;
     c.ws_floats = P->ws_floats;
+    WsLease ws;
+    TRY_CUDA(ws_take(P, c.ws_floats * P->bwd_grid, s, &ws));
+    c.ws = ws.p;
     TRY_CUDA(kCat[P->M].bwd(g, c, P->bwd_grid, s));
     return TPCF_OK;
 }
@@ -426,9 +426,6 @@ tpcf_status catalog_forward_multi(tpcf_plan_s* P, const float* const* d_delta, c
         TRY_CUDA(P->alloc(&c, g.n));
         TRY_CUDA(P->alloc(&sl, (size_t)grid * nent));
         TRY_CUDA(P->alloc(&su, (size_t)nent));
-        float* w3;
-        TRY_CUDA(P->alloc(&w3, 3 * P->ws_floats * grid));
-        P->ws3 = w3;
         P->wdw_c = c;
         P->mslots = sl;
         P->msums = su;
@@ -447,8 +444,10 @@ tpcf_status catalog_forward_multi(tpcf_plan_s* P, const float* const* d_delta, c
     c.slots = P->mslots;
     c.counter = P->counter;
     c.status = P->status;
-    c.ws = P->ws3;
     c.ws_floats = 3 * P->ws_floats;
+    WsLease ws;
+    TRY_CUDA(ws_take(P, c.ws_floats * P->multi_grid, s, &ws));
+    c.ws = ws.p;
     TRY_CUDA(kCat[M].multi(g, c, P->wdw_b, P->wdw_c, P->multi_grid, s));
     reduce_slots_kernel<<<(nent + 31) / 32, REDUCE_THREADS, 0, s>>>(P->mslots, P->multi_grid, nent, P->msums);
     const int nout = (M + 1) * K * K;
@@ -474,8 +473,10 @@ tpcf_status catalog_forward(tpcf_plan_s* P, const float* d_delta, const float* d
     c.status = P->status;
     c.self_subtract = (P->flags & TPCF_SELF_PAIRS_SUBTRACT) ? 1 : 0;
     c.norm = norm_of_flags(P->flags);
-    c.ws = P->ws;
     c.ws_floats = P->ws_floats;
+    WsLease ws;
+    TRY_CUDA(ws_take(P, c.ws_floats * P->fwd_grid, s, &ws));
+    c.ws = ws.p;
     TRY_CUDA(kCat[P->M].fwd(g, c, P->fwd_grid, s));
     reduce_slots_kernel<<<(P->nent + 31) / 32, REDUCE_THREADS, 0, s>>>(P->slots, P->fwd_grid, P->nent, P->sums);
     const int nout = (P->M + 1) * P->K * P->K;

@@ -44,9 +44,11 @@ struct tpcf_plan_s {
     // ring has linear blocks (map_block.cuh)
     std::vector<int64_t> lin_off_h, orb_off_h;
     std::vector<unsigned char> lin_h;
-    float* ws = nullptr;  // workspace of the block kernels: ws_slots blocks of ws_floats
-    int ws_slots = 0;
-    size_t ws_floats = 0;
+    size_t ws_floats = 0;   // workspace of a block (catalogue plans: of a CTA), see ws_take
+    int max_blocks = 0;     // blocks that a call may split into parts
+    float* ws_graph = nullptr;  // workspace of calls that were captured into graphs
+    size_t ws_graph_floats = 0;
+    bool counted = false;   // among the plans that keep the workspaces' pool
     // launch configuration of the map pair kernels (defaults, or picked by the autotuner).  Tile
     // kernels: register variant (sized for 3 or 2 CTAs per SM), CTAs per SM launched, rings summed in
     // registers before a shared-memory flush, and for the forward the tile layout (1: quarter-turn
@@ -66,7 +68,7 @@ struct tpcf_plan_s {
     float2* wdw = nullptr;
     double* slots = nullptr;
     int fwd_grid = 0, bwd_grid = 0;
-    int nslots = 0;  // CTA slots: the largest grid of a forward
+    int nslots = 0;  // CTA slots: the largest grid of a forward by tiles
     int nent = 0;
     double* sums = nullptr;
     int* counter = nullptr;
@@ -75,7 +77,6 @@ struct tpcf_plan_s {
     // multi-field forward (allocated on its first call): packed fields B and C, slots
     float2* wdw_b = nullptr;
     float2* wdw_c = nullptr;
-    float* ws3 = nullptr;  // workspace: three fields per block
     double* mslots = nullptr;
     double* msums = nullptr;
     int multi_grid = 0, multi_ctas = 0;
@@ -121,7 +122,22 @@ struct tpcf_plan_s {
             return e;
         }
     };
-    ~tpcf_plan_s() {
-        for (void* p : allocs) tpcf::dev_free(p);
+    ~tpcf_plan_s();
+};
+
+namespace tpcf {
+// A call's workspace; given back, in stream order, when the call has enqueued its work.
+struct WsLease {
+    float* p = nullptr;
+    cudaStream_t s = nullptr;
+    bool pooled = false;
+    WsLease() = default;
+    WsLease(const WsLease&) = delete;
+    ~WsLease() {
+        if (pooled) cudaFreeAsync(p, s);
     }
 };
+cudaError_t ws_take(tpcf_plan_s* P, size_t floats, cudaStream_t s, WsLease* w);
+// counts a new plan among those that keep the pool
+void ws_count(tpcf_plan_s* P);
+}  // namespace tpcf
