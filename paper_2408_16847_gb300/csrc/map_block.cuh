@@ -678,13 +678,17 @@ __device__ __forceinline__ void orbit_bin(const MapDev& g, const PivotRing& P, i
 //
 // The subtiles are staged one at a time, a group of multipoles at once (all of them at 20
 // bins and m_max 10).  A thread takes a 4 x 4 block of bin pairs of one multipole: 17
-// shared-memory words feed 64 multiply-adds.  fp32 sums run over four subtiles
-// (128 pivots), then go through shared memory to the slot, in order.
-constexpr int CON_RUN = 4;            // subtiles summed in fp32
-// Pivots summed at a time before they are added to the run's sum: the two multiply-adds of a pivot
-// both round at the size of the sum, and short first sums keep that below one rounding per pivot of a
-// single chain, for 3% more instructions.
-constexpr int CON_FOLD = 16;
+// shared-memory words feed 64 multiply-adds.  fp32 sums run over two subtiles
+// (64 pivots; three fields: over the three products of two), then go through shared memory to the slot, in
+// order.
+constexpr int CON_RUN = 2;            // subtiles summed in fp32
+// Pivots summed at a time before they are added to the run's sum.  The two multiply-adds of a pivot both
+// round at the size of the sum, and the weight rounds before them; short first sums keep the error of a slot
+// below that of a chain of 32 with the finished products (map_tile.cuh).  Emulated, relative to the sum of
+// 128 pivots, for random moments and for moments of one sign: chain 1.07e-7 and 4.4e-8; runs of 64 with
+// first sums of 8 9.7e-8 and 3.8e-8 (of 16: 1.15e-7 and 4.2e-8); runs of 128 with first sums of 16,
+// as it was, 1.21e-7 and 5.8e-8.
+constexpr int CON_FOLD = 8;
 
 // Multipoles staged at once: the groups are of equal size, fit the stage and leave threads for D.
 __host__ __device__ inline int con_group(int K, int mr, int slices) {
@@ -769,7 +773,6 @@ __device__ __forceinline__ void block_contract(int K, int mr, const float* ws, s
             o2[i] = isD ? nm * K * 2 * TILE + k2 * TILE : (ml * K + k2) * 2 * TILE;
         }
         float2 tot[CB][CB], acc[CB][CB];
-        float q1 = 0.0f, q2 = 0.0f;  // self-pair diagonals of bin tid
 #pragma unroll
         for (int i = 0; i < CB; ++i)
 #pragma unroll
@@ -832,11 +835,14 @@ __device__ __forceinline__ void block_contract(int K, int mr, const float* ws, s
                 }
                 if (SELF && self && m0 == 0 && tid < K) {
                     const float* Q = sW + (K + tid) * TILE;
+                    float q1 = 0.0f, q2 = 0.0f;
                     for (int t = 0; t < TILE; ++t) {
                         const int l = (t + lane) & (TILE - 1);
                         q1 = fmaf(sPiv[l], Q[l], q1);
                         q2 = fmaf(sPiv[TILE + l], Q[K * TILE + l], q2);
                     }
+                    red_add_f32(slot + 2 * nS + P + tid, q1);
+                    red_add_f32(slot + 2 * nS + P + K + tid, q2);
                 }
                 ++run;
             }
@@ -862,11 +868,6 @@ __device__ __forceinline__ void block_contract(int K, int mr, const float* ws, s
                             }
                             tot[i][j] = make_float2(0.0f, 0.0f);
                         }
-                }
-                if (SELF && self && m0 == 0 && tid < K) {
-                    red_add_f32(slot + 2 * nS + P + tid, q1);
-                    red_add_f32(slot + 2 * nS + P + K + tid, q2);
-                    q1 = q2 = 0.0f;
                 }
                 __syncthreads();
                 for (int e = tid; e < 2 * nm * P; e += BT) red_add_f32(slot + 2 * m0 * P + e, out[e]);

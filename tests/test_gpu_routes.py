@@ -172,3 +172,72 @@ def test_small_calls_are_not_split():
     g = torch.ones(plan.zeta_shape(), dtype=torch.float64, device=d.device)
     assert _launches(plan, lambda: plan.backward(d, w, norm, g)) == 2
     plan.close()
+
+
+@pytest.mark.parametrize("bins", [2, 9])
+def test_small_contributions_reach_the_fp64_sums(bins):
+    """At most 64 pivots of a linear block are added up in fp32: 64 pivots of weight 2^-30 beside 64 of weight 1
+    keep their share of D, which sums in fp32 over 128 pivots lose."""
+    n = 12 * NSIDE * NSIDE
+    first = CAP + 4 * NSIDE * NSIDE  # pixel 0 of the equator: the block's first
+    w = np.ones(n, dtype=np.float32)
+    w[first + 64:first + 128] = 2.0 ** -30
+    d, w = to_dev(np.ones(n, dtype=np.float32)), to_dev(w)
+    plan = plan_on(BLOCKS, NSIDE, np.linspace(1.03, 5.9, bins + 1), 1)
+    whole, large, small = (plan.forward(d, w, (first + a, first + b))[1].cpu().numpy() for a, b in ((0, 128), (0, 64), (64, 128)))
+    plan.sync()
+    np.testing.assert_allclose(whole - large, small, rtol=1e-6)
+    plan.close()
+
+
+def test_linear_rings_of_several_blocks():
+    """Nside 256: four blocks to a ring, in the ring's middle (no row wraps) and across pixel 0."""
+    nside, m = 256, 6
+    edges = np.geomspace(0.31, 1.47, 6)
+    d = synth.bump_map(nside, 2000, (0.3, 2.0), 0.5, 0.05, seed=synth.BASE_SEED + 96).astype(np.float32)
+    w = synth.rng(97).uniform(0.5, 1.5, len(d)).astype(np.float32)
+    xyz = oracle.pix2vec_ring(nside)
+    plan = plan_on(BLOCKS, nside, edges, m)
+    ring = 2 * nside * (nside - 1) + 4 * nside * nside
+    for pivots in ((ring + 400, ring + 640), (ring + 511, ring + 514), (ring - 60, ring + 40)):
+        _check_step(plan, xyz, d, w, edges, m, pivots)
+    plan.close()
+
+
+def _exact_sums(nside, edges, m, field, pivots, cot):
+    """zeta, D and the gradient in 64 bits, from the workload file's direct sums over the pivots' rings."""
+    import importlib.util
+    import os
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    spec = importlib.util.spec_from_file_location("cases", os.path.join(root, "perf", "cases.py"))
+    cases = importlib.util.module_from_spec(spec)
+    spec.loader.exec_module(cases)
+    cases.edges_of = lambda case: np.array(edges)
+    case = dict(kind="map_host", k=len(edges) - 1, m=m, opt="default")
+    return cases.exact_sums(case, cases.Map(nside, np.radians(edges[-1])), [field], pivots, cot)
+
+
+# a warp's gradient rows fit its shared memory (reach 989 pixels), or go straight to the gradient (1018, 1054)
+@pytest.mark.parametrize("outer", [20.9, 21.5, 22.2])
+def test_wide_gradient_rows(outer):
+    nside, m = 4096, 3
+    edges = [outer - 0.1, outer - 0.04, outer]
+    n = 12 * nside * nside
+    first = 2 * nside * (nside - 1) + 4 * nside * nside + 5000
+    pivots = (first, first + 300)
+    g = torch.Generator(device="cuda:0")
+    g.manual_seed(98)
+    d = torch.randn(n, generator=g, device="cuda:0") + 0.3
+    w = 0.5 + torch.rand(n, generator=g, device="cuda:0")
+    cot = torch.randn(m + 1, 2, 2, 2, generator=g, device="cuda:0", dtype=torch.float64)
+    cot[..., 1] = 0.0
+    plan = plan_on(BLOCKS, nside, edges, m)
+    zeta, norm = plan.forward(d, w, pivots)
+    grad = plan.backward(d, w, norm, cot, pivots)
+    plan.sync()
+    plan.close()
+    ref = _exact_sums(nside, edges, m, (d, w), pivots, cot)
+    zref = torch.view_as_complex(ref["zeta"].contiguous()).cpu().numpy()
+    assert rel_err_per_m(_zeta(zeta), zref).max() < TOL
+    np.testing.assert_allclose(norm.cpu().numpy(), ref["norm"].cpu().numpy(), rtol=1e-6)
+    assert (grad.double() - ref["grad"]).abs().max() < TOL * ref["grad"].abs().max()
