@@ -265,9 +265,9 @@ tpcf_status tpcf_backward(tpcf_plan plan, const float* d_delta, const float* d_w
 /*
  * Exact number of in-bin ordered pairs (i, j) whose pivot i lies in
  * [pivot_begin, pivot_end) and has w_i != 0, whatever w_j (the units of the
- * throughput figure).  d_counts (device, int64[3]) receives: the total, the pairs
- * visited as mirror images (equatorial-belt symmetry), the pairs visited singly
- * (catalogue plans visit every pair singly).
+ * throughput figure).  d_counts (device, int64[3]) receives: the total, the pairs on
+ * rings with the pivot ring's pixel count less those on the pivot's meridian (mirror images
+ * of one another about it: equatorial-belt symmetry), the others (catalogue plans: all).
  */
 tpcf_status tpcf_count_pairs(tpcf_plan plan, const float* d_w, int64_t pivot_begin, int64_t pivot_end,
                              int64_t* d_counts, void* stream);

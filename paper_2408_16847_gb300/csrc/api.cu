@@ -359,7 +359,6 @@ static tpcf_status build_map(tpcf_plan_s* P, int64_t nside, cudaStream_t s) {
     tile_list_kernel<<<nrings, 128, 0, s>>>(nrings, lin_off, nlin_r, BT * np, lin_list);
     tile_list_kernel<<<nrings, 128, 0, s>>>(nrings, orb_off, norb_r, TILE, orb_list);
     TRY_CUDA(cudaGetLastError());
-    g.lin = lin;
     g.ring_reach = reach;
     g.rc = rc;
     g.lin_list = lin_list;
@@ -796,7 +795,8 @@ extern "C" tpcf_status tpcf_forward_multi(tpcf_plan plan, const float* d_delta_a
     const int K = P->K, M = P->M;
     const int nent = n_entries_multi(K, M);
     if (!P->wdw_b) {
-        // the three fields' moments of one tile have to fit an SM (as the catalogue's must)
+        // the three fields' moments of one tile have to fit an SM: the tile kernel's limit, and so the
+        // call's at every size (the blocks would take more)
         if (((size_t)3 * (K * (M + 1) * 2 + K) * TILE + 6 * TILE) * sizeof(float) > 232448 || kMulti[M].blocks_occ() < 1) {
             snprintf(g_last_error, sizeof(g_last_error),
                      "tpcf_forward_multi: three fields' moments (K=%d, m_max=%d) do not fit in shared memory", K, M);

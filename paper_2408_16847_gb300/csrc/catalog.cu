@@ -410,7 +410,8 @@ tpcf_status catalog_forward_multi(tpcf_plan_s* P, const float* const* d_delta, c
     const int K = P->K, M = P->M;
     const int nent = n_entries_multi(K, M);
     if (!P->wdw_b) {  // the second and third fields' packed values and the slots, on the first call
-        // the three fields' moments of one tile have to fit an SM's shared memory (the map's limit)
+        // the three fields' moments of one tile have to fit an SM's shared memory, as for maps (these
+        // kernels would take more)
         const int occ = kCat[M].multi_occ(K);
         if (((size_t)3 * (K * (M + 1) * 2 + K) * TILE + 6 * TILE) * sizeof(float) + 20480 > 232448 || occ < 1) {
             char msg[160];

@@ -14,15 +14,16 @@
 //     angle and runs the harmonic recurrence once for its images.
 //     A block is several warp tiles; its warps draw (tile, bin) items.
 // The sums of one bin stay in registers and go to the block's workspace in global memory
-// (it is read back soon, mostly from L2): no shared-memory atomics, no barrier per ring or bin.
-// Then the CTA stages the workspace 32 pivots at a time and contracts it.
+// (471 KB per CTA at 20 bins and m_max 10): no shared-memory atomics, no barrier per ring or bin.
+// Then the CTA stages the workspace 32 pivots at a time and contracts it.  Calls with too little work for
+// this split go to map_tile.cuh (takes_blocks in api.cu).
 //
 // A call with few blocks splits each into parts by bins, so that it still fills the GPU; the
 // part that finishes last contracts.
 //
-// Bound: FP32 and load/store issue.  Per call on a GB300, before (a ring at a time per pivot, sums by
-// shared-memory atomics) and now: Nside 512, 20 bins to 2 deg, m <= 10: 33.3 -> 11.1 ms; Nside 4096
-// polar slice (2 x 10^-3 of the pixels): 71.7 -> 47.6 ms; Nside 64: 328 -> 210 us.
+// Bound: FP32 and load/store issue.  Per call on a GB300, by tiles (a ring at a time per pivot, sums by
+// shared-memory atomics) and by blocks: Nside 512, 20 bins to 2 deg, m <= 10: 33.3 -> 11.8 ms; Nside 4096
+// polar slice (2 x 10^-3 of the pixels): 71.9 -> 46.9 ms; Nside 64, 10 bins: 328 -> 217 us.
 #pragma once
 
 namespace tpcf {

@@ -14,7 +14,7 @@
 // pixel.  Other rings: per-lane angles as in phase 1, one reduction per image and entry.
 //
 // Forward + adjoint before (each lane's own angles, a reduction per pixel and pivot) and now: Nside 4096
-// belt slice 126 -> 71 ms, masked Nside 1024 to 3 deg 1018 -> 522 ms.
+// belt slice 126 -> 74 ms, masked Nside 1024 to 3 deg 1018 -> 557 ms.
 #pragma once
 
 namespace tpcf {

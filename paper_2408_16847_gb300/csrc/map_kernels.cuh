@@ -2,31 +2,18 @@
 // section 3.1), templated on the largest multipole M.  Included by map_inst.cu,
 // which is compiled once per M.
 //
-// Work decomposition (forward):
-//   * a tile is 32 pivots of one HEALPix ring; a CTA of 8 warps owns one tile at a time
-//     (persistent CTAs pull tiles from an atomic counter).  Its moments come from the
-//     shared-angle walk (map_walk.cuh); the points below describe the per-lane walk, one
-//     pivot per lane, that shared neighbour lists and the adjoint use on rings without
-//     common angles;
-//   * for every radial bin k the warps split the neighbour rings that can hold bin-k
-//     pixels;
-//   * on a neighbour ring the bin-k pixels of a pivot form at most two contiguous
-//     runs, found from the per-ring-pair edge offsets T_e built by the plan (an
-//     exact ring-range disc query); each lane walks its own runs, so the bin is
-//     known without a per-pixel test and the (M+1) complex accumulators of the bin
-//     stay in registers across rings;
-//   * within a run e^{-i m phi} comes from a trig-free recurrence in m (the harmonic
-//     step the paper describes in Sec. 3.1 and 3.2, a few operations per m): Reinsch's
-//     stable form of the three-term relation on the angle folded into |psi| <= pi/2,
-//     with the neighbour weight folded into the start values and the cos and sin
-//     chains packed into f32x2 FMAs (see harmonics());
-//   * in the equatorial belt a neighbour ring has as many pixels as the pivot ring,
-//     so its pixels sit symmetrically about the pivot's meridian: the pixel at +phi
-//     and its mirror at -phi share one cos/sin evaluation and one recurrence;
-//   * after all bins, the tile's a_m^k(i) sit in shared memory and the CTA forms
-//     sum_i w_i d_i a^{k1} conj(a^{k2}) (eq. zetamEst2) and sum_i w_i W^{k1} W^{k2},
-//     adding them in FP64 into a slot owned by the CTA (FP32 pipe, or the tensor
-//     cores in map_fwd_tc_kernel).
+// What all map kernels share: positions of pivots and bin edges on a ring, the runs of a bin, the
+// position angle of a neighbour and its harmonics, data access, and the tensor-core contraction; then the
+// block kernels' entry points (map_block.cuh, map_block_bwd.cuh: large calls), the pair count, and the tile
+// kernels (map_tile.cuh: small calls).
+//   * on a neighbour ring the bin-k pixels of a pivot form at most two contiguous runs, found from
+//     the per-ring-pair edge offsets T_e built by the plan (an exact ring-range disc query);
+//   * within a run e^{-i m phi} comes from a trig-free recurrence in m (the harmonic step the paper
+//     describes in Sec. 3.1 and 3.2, a few operations per m): Reinsch's stable form of the
+//     three-term relation on the angle folded into |psi| <= pi/2, the cos and sin chains
+//     packed into f32x2 FMAs (fold_angle, harmonicsf);
+//   * a pivot's moments are contracted to sum_i w_i d_i a^{k1} conj(a^{k2}) (eq. zetamEst2) and
+//     sum_i w_i W^{k1} W^{k2}, added in FP64 into a slot owned by the CTA.
 #pragma once
 
 #include <math.h>
@@ -555,18 +542,6 @@ __device__ __forceinline__ bool tc_wait(uint32_t mbar, uint32_t phase) {
     }
 }
 
-__device__ __forceinline__ void tc_ld16(uint32_t taddr, float (&v)[16]) {
-    uint32_t r[16];
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-        : "r"(taddr));
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-    for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
-}
-
 __device__ __forceinline__ void tc_ld8(uint32_t taddr, float (&v)[8]) {
     uint32_t r[8];
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
@@ -927,9 +902,10 @@ __global__ void __launch_bounds__(BT, 4) map_fwd_multi_kernel(MapDev g, MapCall 
 
 // ------------------------------------------------------------- pair count
 #if defined(TPCF_M) && TPCF_M == 0  // one definition, in the M = 0 object
-// counts[0] += in-bin ordered pairs (i, j) of the pivots with w_i != 0 (any w_j);
-// counts[1] += those visited as mirror pairs, counts[2] += those visited singly.
-// Uses the same run construction as the forward, without touching pixel data.
+// counts[0] += in-bin ordered pairs (i, j) of the pivots with w_i != 0 (any w_j); counts[1] += those
+// on rings with the pivot ring's pixel count, where pixels are mirror images about the pivot's
+// meridian, counts[2] += the others and the pixels on the meridian.  The runs of the tile
+// kernels, without touching pixel data; the blocks' edges are the same positions (pos_edge).
 __global__ void __launch_bounds__(NTHREADS) map_count_kernel(MapDev g, const float2* __restrict__ wdw,
                                                              long long piv_lo, long long piv_hi,
                                                              long long tile_lo, long long tile_hi,
@@ -976,7 +952,7 @@ __global__ void __launch_bounds__(NTHREADS) map_count_kernel(MapDev g, const flo
 
 // val = sum_m (cos(m phi) hr_m + sin(m phi) hi_m): X the cosine part, Y the sine part.
 // h[m] = (hr_m, hi_m); the (cos, sin) chains run packed, in the folded frame psi, by
-// the recurrence of harmonics(); even and odd multipoles are summed apart and the odd
+// the recurrence of harmonicsf(); even and odd multipoles are summed apart and the odd
 // sum takes the sign sigma at the end.
 template <int M>
 __device__ __forceinline__ void adj_harmonicsf(const float2 (&h)[M + 1], const Fold& f, float& X, float& Y,

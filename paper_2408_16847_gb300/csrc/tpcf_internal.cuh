@@ -44,7 +44,6 @@ struct MapDev {
     int64_t ntiles;
     const int2* lin_list;       // linear blocks (ring, first pivot): BT walk_np consecutive pivots (map_block.cuh)
     const int2* orb_list;       // warp tiles (ring, first position) of the other rings: 32 positions and their turned images
-    const unsigned char* lin;   // [nrings] 1: linear walk tiles (every neighbour ring has n_i pixels)
     const int* ring_reach;      // [nrings] pixels that a linear tile's rows reach beyond a pivot
     const float4* rc;           // [2 * nrings] (s, s_lo, step, step_lo), (1/n, its lo, 2 n + shift, first)
     const double* E;            // [K+1] sin^2(theta_e / 2)
