@@ -80,3 +80,28 @@ def test_edges_of_small_bins_about_one_pivot(theta):
     got = [plan.count_pairs(wt, (i, i + 1))[0] for i in range(120)]
     assert [int(v) for v in got] == [int(v) for v in want]
     plan.close()
+
+
+@pytest.mark.parametrize("lo,hi,k", [(0.001, 20.0, 20), (0.01, 5.0, 32), (0.002, 30.0, 3)])
+def test_small_edges_in_wide_tiles(lo, hi, k):
+    """Sparse points with a partner each next to an edge: a tile of 32 spans tens of degrees, so its margins at the
+    small edges are wider than the table's cells."""
+    from paper_2408_16847_gb300 import tpcf
+    g = synth.rng(1110)
+    edges = np.geomspace(lo, hi, k + 1)
+    a = synth.uniform_sphere(700, g)
+    u = g.standard_normal(a.shape)
+    u -= (u * a).sum(1)[:, None] * a
+    u /= np.linalg.norm(u, axis=1)[:, None]
+    s = np.radians(edges[np.arange(700) % (k + 1)] * (1.0 + g.choice([-1e-5, -1e-6, 1e-6, 1e-5], 700)))[:, None]
+    b = np.cos(s) * a + np.sin(s) * u
+    xyz = np.concatenate([a, b / np.linalg.norm(b, axis=1)[:, None]])
+    d = (g.standard_normal(1400) + 0.3).astype(np.float32)
+    w = g.uniform(0.5, 1.5, 1400).astype(np.float32)
+    plan = tpcf.Plan.catalog(torch.from_numpy(xyz).to("cuda:0"), edges, 2)
+    ref = oracle.zeta(xyz, d.astype(np.float64), w.astype(np.float64), edges, 2)
+    assert ref["min_margin"] > 1e-9
+    assert int(plan.count_pairs(to_dev(w))[0]) == int(oracle.pair_counts(xyz, edges).sum())
+    _, norm = plan.forward(to_dev(d), to_dev(w))
+    np.testing.assert_allclose(norm.cpu().numpy(), ref["D"], rtol=1e-6, atol=1e-6 * np.abs(ref["D"]).max())
+    plan.close()
