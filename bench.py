@@ -139,27 +139,32 @@ def cat_flops_per_pair(M: int):
     return 35 + 6 * max(M - 1, 0)
 
 
-# DRAM bytes per pixel per launch of the map kernels, from the ncu capture of the
-# Nside 512 case (profiles/map_kernels_fullsky_nside512.md: dram__bytes_read.sum +
-# dram__bytes_write.sum / pixels), valid only for the kernel code it was taken on:
-# the key is a hash of map_kernels.cuh with comments and blank lines removed.
-TRAFFIC = {"map_bwd_kernel": (18.24, "b151b72319927b3f"), "map_fwd_kernel": (19.18, "263caf8e58838b4c")}
+# DRAM bytes per pixel per launch of the map kernels at 20 bins and m_max 10, from the ncu capture
+# of the Nside 512 case (profiles/map_block_kernels_fullsky_nside512.md: dram__bytes_read.sum +
+# dram__bytes_write.sum / pixels; nearly all of it the blocks' workspace, so it goes with the pivots),
+# valid only for the kernel code it was taken on: the key is a hash of the kernels' files with
+# comments and blank lines removed.
+TRAFFIC = {"map_bwd_kernel": (7487.7, "27bd9b53e467fe4f"), "map_fwd_kernel": (3933.1, "b2c3359be4a3fa7f")}
+TRAFFIC_FILES = {"map_fwd_kernel": ("map_kernels.cuh", "map_block.cuh"),
+                 "map_bwd_kernel": ("map_kernels.cuh", "map_block.cuh", "map_block_bwd.cuh")}
 
 
-def kernel_code_hash(path):
+def kernel_code_hash(*paths):
     import hashlib
     import re
-    src = open(path).read()
-    src = re.sub(r"/\*.*?\*/", "", src, flags=re.S)
-    src = re.sub(r"//[^\n]*", "", src)
-    src = "\n".join(line.rstrip() for line in src.splitlines() if line.strip())
-    return hashlib.sha256(src.encode()).hexdigest()[:16]
+    text = []
+    for path in paths:
+        src = open(path).read()
+        src = re.sub(r"/\*.*?\*/", "", src, flags=re.S)
+        src = re.sub(r"//[^\n]*", "", src)
+        text.append("\n".join(line.rstrip() for line in src.splitlines() if line.strip()))
+    return hashlib.sha256("\n".join(text).encode()).hexdigest()[:16]
 
 
-def traffic_per_launch(kernel, npix):
+def traffic_per_launch(kernel, npix, K, M):
     bpp, sha = TRAFFIC[kernel]
-    src = os.path.join(ROOT, "paper_2408_16847_gb300", "csrc", "map_kernels.cuh")
-    return bpp * npix if kernel_code_hash(src) == sha else None
+    files = [os.path.join(ROOT, "paper_2408_16847_gb300", "csrc", f) for f in TRAFFIC_FILES[kernel]]
+    return bpp * npix if (K, M) == (20, 10) and kernel_code_hash(*files) == sha else None
 
 
 def sm_count(dev=None):
@@ -420,9 +425,9 @@ def setup_map(args, dev, rank):
                 "implemented_note": "flops of the implemented loop (mirror pairs share one angle "
                                     "and one recurrence)",
                 "peak_note": "measured FMA throughput (tpcf_probe_fp32_peak, the larger of scalar and f32x2)",
-                "traffic": traffic_per_launch("map_fwd_kernel", 12 * wl.nside ** 2),
+                "traffic": traffic_per_launch("map_fwd_kernel", 12 * wl.nside ** 2, K, M),
                 "traffic_note": "DRAM bytes per launch scaled by pixels from the Nside 512 ncu capture "
-                                "(null when the kernel changed since)"}
+                                "(null when the kernel changed since, or at other bins and m_max)"}
 
     def roof_fb(ms_total, ms_fwd, clk, sms):
         ms_adj = ms_total - ms_fwd
@@ -432,7 +437,7 @@ def setup_map(args, dev, rank):
                 "flops_per_pair": alg_flops_per_pair(M, True),
                 "achieved_implemented": adj_impl / (ms_adj * 1e-3) / 1e12,
                 "step_achieved": fb_alg / (ms_total * 1e-3) / 1e12,
-                "traffic": traffic_per_launch("map_bwd_kernel", 12 * wl.nside ** 2)}
+                "traffic": traffic_per_launch("map_bwd_kernel", 12 * wl.nside ** 2, K, M)}
 
     config = {"workload": wl.name, "nside": wl.nside, "npix": 12 * wl.nside * wl.nside,
               "bins": "%d %s bins %.2f-%.2f deg" % (K, "lin" if wl.name == "map_nside64" else "log",
